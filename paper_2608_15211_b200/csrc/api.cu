@@ -142,7 +142,10 @@ static bool use_bwd_tc(const Geo& g) { return bwd_tc_supported(g) && !force_regi
 
 static bool use_bwd_kv64(const Geo& g) { return bwd_kv64_supported(g) && !force_register_path() && !small_window_128(g); }
 
+static bool use_bwd_onepass(const Geo& g) { return bwd_onepass_supported(g) && !force_register_path() && !small_windows(g); }
+
 static size_t delta_bytes(const Geo& g) {
+    if (use_bwd_onepass(g)) return align_up(bwd_onepass_plan(g).bytes, 256);
     if (use_bwd_tc(g)) return align_up(bwd_tc_workspace_bytes(g), 256);
     const size_t delta = align_up(sizeof(float) * (size_t)g.B * g.H * g.W * g.heads, 256);
     // the tcgen05 key-side kernel of the head-dim-64 regime also wants the prepared bias tables
@@ -256,6 +259,11 @@ static int bwd_call(const Geo& g, const void* q, const void* k, const void* v,
     rc = device_props(&sms);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
+    if (use_bwd_onepass(g)) {
+        cudaError_t et = g.f16 ? launch_bwd_onepass_f16(g, q, k, v, bias_table, o, lse, d_o, dq, dk, dv, dbias, workspace, sms, st)
+                               : launch_bwd_onepass(g, q, k, v, bias_table, o, lse, d_o, dq, dk, dv, dbias, workspace, sms, st);
+        return et == cudaSuccess ? TERRA_OK : cuda_fail(et, "terra_swin_attn_bwd");
+    }
     if (use_bwd_tc(g)) {
         cudaError_t et = g.f16 ? launch_bwd_tc_f16(g, q, k, v, bias_table, o, lse, d_o, dq, dk, dv, dbias, workspace, sms, st)
                                : launch_bwd_tc(g, q, k, v, bias_table, o, lse, d_o, dq, dk, dv, dbias, workspace, sms, st);
@@ -355,14 +363,16 @@ int terra_swin_check(void* stream) {
     e = read_bwd_q64_status(&timed_out_q);
     if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
     // the fp16 builds of the same kernels keep status words of their own
-    int t16[5] = {0, 0, 0, 0, 0};
+    int t16[7] = {0, 0, 0, 0, 0, 0, 0};
     e = read_tc_status_f16(&t16[0], (cudaStream_t)stream);
     if (e == cudaSuccess) e = read_bwd_tc_status_f16(&t16[1]);
     if (e == cudaSuccess) e = read_fwd_tc64_status_f16(&t16[2]);
     if (e == cudaSuccess) e = read_bwd_kv64_status_f16(&t16[3]);
     if (e == cudaSuccess) e = read_bwd_q64_status_f16(&t16[4]);
+    if (e == cudaSuccess) e = read_bwd_onepass_status_f16(&t16[5]);
+    if (e == cudaSuccess) e = read_bwd_onepass_status(&t16[6]);
     if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
-    const bool any16 = t16[0] || t16[1] || t16[2] || t16[3] || t16[4];
+    const bool any16 = t16[0] || t16[1] || t16[2] || t16[3] || t16[4] || t16[5] || t16[6];
     return (timed_out || timed_out_bwd || timed_out_64 || timed_out_kv || timed_out_q || any16) ? TERRA_ERR_DEVICE_TIMEOUT : TERRA_OK;
 }
 

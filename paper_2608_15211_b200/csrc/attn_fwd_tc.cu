@@ -27,6 +27,7 @@
 #include "swin_kernels.h"
 #include "tc_common.cuh"
 #include "tma_rows.cuh"
+#include "win_tiles.cuh"
 
 // fp16 build of this file (through attn_fwd_tc_f16.cu): the kernel, its launcher and its status word get names of
 // their own; the element-independent helpers below are compiled in the bf16 build only
@@ -937,6 +938,20 @@ bool make_col_map4(CUtensorMap* map, const Geo& g, const void* base, int token_s
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// one map of win_tiles.cuh: [heads * d][nb columns][ncols windows][token rows] from `base` on
+bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_stride, int nb, int ncols, int box_ch, int box_b, int box_rows) {
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return false;
+    const cuuint64_t ts = (cuuint64_t)token_stride * 2;
+    const cuuint64_t dims[4] = {(cuuint64_t)g.heads * g.d, (cuuint64_t)nb, (cuuint64_t)ncols, (cuuint64_t)g.B * g.H};
+    const cuuint64_t strides[3] = {ts, ts * g.w, ts * g.W};
+    const cuuint32_t box[4] = {(cuuint32_t)box_ch, (cuuint32_t)box_b, 1u, (cuuint32_t)box_rows};
+    const cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               box_ch == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 bool make_row_maps3(RowMaps3* maps, const Geo& g, const void* base, int token_stride) {

@@ -94,6 +94,25 @@ cudaError_t launch_bwd_q64(const Geo& g, const void* q, const void* k, const voi
                            const float* lse, const float* delta, void* dq, float* dbias, int sm_count, cudaStream_t stream);
 cudaError_t read_bwd_q64_status(int* timed_out);
 
+// One-pass tcgen05 backward for windows of more than 64 tokens and side <= 32, every head dim, any grid.
+struct OnePassPlan {
+    int rw;                  // slots per window row
+    int npad, rmax;          // slots of a window rounded up to 128; window rows rounded up to whole key tiles
+    int split_log2;          // a window's key tiles are shared by 1 << split_log2 units
+    long long units;
+    size_t off_bias0, off_bias1, off_acc, off_slabs, bytes;      // workspace
+};
+constexpr int kPlanSms = 148;          // SM count the plan is made for
+constexpr int kMaxCtas = 160;          // CTAs whose dQ slabs fit the workspace
+bool bwd_onepass_supported(const Geo& g);
+OnePassPlan bwd_onepass_plan(const Geo& g);
+cudaError_t launch_bwd_onepass(const Geo& g, const void* q, const void* k, const void* v, const float* bias, const void* o, const float* lse,
+                               const void* d_o, void* dq, void* dk, void* dv, float* dbias, void* workspace, int sm_count, cudaStream_t stream);
+cudaError_t launch_bwd_onepass_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias, const void* o, const float* lse,
+                                   const void* d_o, void* dq, void* dk, void* dv, float* dbias, void* workspace, int sm_count, cudaStream_t stream);
+cudaError_t read_bwd_onepass_status(int* timed_out);
+cudaError_t read_bwd_onepass_status_f16(int* timed_out);
+
 cudaError_t launch_bounded_wait_selftest(long long limit_cycles, cudaStream_t stream);
 cudaError_t launch_bias_prep(const Geo& g, const float* bias, float* prep, cudaStream_t stream);
 

@@ -1,0 +1,86 @@
+// Windows as tiles of slots, loaded by tiled bulk copies (TMA) on ANY grid: shared by the one-pass backward kernel and
+// its host side.
+//
+// A window's slots are laid out RW to a window row (RW = 16 for window sides 9 .. 16, 32 for 17 .. 32): slot = RW a + b.
+// Slots with b at or beyond the window's width, or a at or beyond its height, hold no token; the copies fill them with
+// zeros.  A tensor is described as [heads * d channels][w columns of a window][window columns][token rows], based at
+// the first token of the shifted frame, so that a box of RW columns reads past the w columns of its window only into
+// the zero fill.  64 slots (64 / RW window rows) of one channel part are one copy (4 or 8 KB) wherever the rows are
+// consecutive.  What the description cannot hold gets maps of its own: window columns that lie wholly behind the
+// longitude seam, the one that the seam cuts (two pieces per window row) and a truncated last column.
+#pragma once
+#include <cuda.h>
+
+#include "swin_common.cuh"
+#include "tc_common.cuh"
+
+namespace terra {
+
+struct WinMaps {
+    CUtensorMap group;       // columns in front of the seam, 64 / RW window rows per copy
+    CUtensorMap row;         // the same, one window row per copy
+    CUtensorMap wrapped;     // columns behind the seam, one window row
+    CUtensorMap seam_a;      // the column cut by the seam: its tokens in front of the seam ...
+    CUtensorMap seam_b;      // ... and behind it, up to slot RW
+    CUtensorMap last;        // a truncated last column (when the seam does not cut it)
+};
+
+struct WinCols {
+    int seam;                // window column cut by the seam (-1: none), n1 of its tokens lie in front of it
+    int n1;
+    int first_wrapped;       // columns >= this one start behind the seam
+    int last;                // truncated last column that needs the map of its own (-1: none)
+    int skip;                // 64-byte rows and an odd n1: slot n1 of the seam column is copied by the loading warp itself
+                             // (a bulk copy must start on a 128-byte boundary), seam_b starts one token later
+};
+
+constexpr int kMaxOnePassW = 32;
+inline int win_row_slots(const Geo& g) { return g.w <= 16 ? 16 : 32; }
+
+// host (attn_fwd_tc.cu, beside the driver's encoder)
+bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_stride, int nb, int ncols, int box_ch, int box_b, int box_rows);
+// host (attn_bwd_onepass.cu): false if the driver's encoder is not available
+bool make_win_cols(WinCols* c, const Geo& g);
+bool make_win_maps(WinMaps* m, const WinCols& c, const Geo& g, const void* base, int token_stride);
+
+// device: 64 slots from window row `a0` on, channels [ch, ch + part) of every token, to `dst` (rows of ROWB bytes, 1 KB
+// aligned); the bytes are counted on `bar` (64 * ROWB, less ROWB per window row for a seam column with c.skip).
+template <int RW, int ROWB>
+__device__ __forceinline__ void load_win_group(const WinMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
+                                               int a0, int ch, uint32_t bar) {
+    constexpr int G = 64 / RW;
+    int u = wr * g.w + a0 + g.sh;
+    if (u >= g.H) u -= g.H;
+    const bool special = wc == c.seam || wc >= c.first_wrapped || wc == c.last;
+    if (!special && a0 + G <= eh && u + G <= g.H) {
+        tc::tma_load_4d(dst, &m.group, ch, 0, wc, b * g.H + u, bar);
+        return;
+    }
+#pragma unroll
+    for (int r = 0; r < G; ++r) {
+        const int y = a0 + r < eh ? b * g.H + u : g.B * g.H;       // behind the last row: zeros
+        const uint32_t d = dst + r * RW * ROWB;
+        if (wc == c.seam) {
+            tc::tma_load_4d(d, &m.seam_a, ch, 0, 0, y, bar);
+            if (c.n1 + c.skip < RW) tc::tma_load_4d(d + (c.n1 + c.skip) * ROWB, &m.seam_b, ch, c.skip, 0, y, bar);
+        } else if (wc == c.last) {
+            tc::tma_load_4d(d, &m.last, ch, 0, 0, y, bar);
+        } else if (wc >= c.first_wrapped) {
+            tc::tma_load_4d(d, &m.wrapped, ch, 0, wc - c.first_wrapped, y, bar);
+        } else {
+            tc::tma_load_4d(d, &m.row, ch, 0, wc, y, bar);
+        }
+        if (++u >= g.H) u -= g.H;
+    }
+}
+
+// slot (a, b) of a window -> grid token
+__device__ __forceinline__ int win_token(const Geo& g, int wr, int wc, int a, int b) {
+    int u = wr * g.w + a + g.sh;
+    if (u >= g.H) u -= g.H;
+    int v = wc * g.w + b + g.sw;
+    if (v >= g.W) v -= g.W;
+    return u * g.W + v;
+}
+
+}  // namespace terra
