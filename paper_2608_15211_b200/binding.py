@@ -1,6 +1,6 @@
 """Thin Python binding of the C ABI declared in include/terra.h.
 
-Argument marshalling only: tensors must already live on the GPU; every step of the path
+Argument marshalling only (the attention calls' in native code, csrc/host_module.cpp): tensors must already live on the GPU; every step of the path
 (route, gather, attention, scatter) runs in the library's kernels.  There is no CPU
 fallback: if the shared library is missing or no CUDA device is present, calls raise.
 PyTorch is used for device memory and streams.
@@ -12,7 +12,7 @@ import os
 
 import torch
 
-from .build import LIB_PATH
+from .build import HOST_PATH, LIB_PATH
 
 TERRA_OK = 0
 EXPORTS = ("terra_route_sizes", "terra_window_route", "terra_swin_workspace_bytes", "terra_swin_attn_fwd",
@@ -81,8 +81,30 @@ def load_library(path: str | None = None) -> ctypes.CDLL:
         getattr(lib, n).argtypes = [vp, vp] + [ctypes.c_int32] * 5 + [ctypes.c_int64, vp]
         getattr(lib, n).restype = ctypes.c_int
     if path is None:
+        _bind_host(lib)
         _lib = lib
     return lib
+
+
+_host = None
+
+
+def _bind_host(lib) -> None:
+    """The native module that checks and marshals the attention calls' arguments gets the library's entry points."""
+    global _host
+    if not os.path.exists(HOST_PATH):
+        raise FileNotFoundError(f"{HOST_PATH} not found: build it with `python -m paper_2608_15211_b200.build`")
+    from . import _host as module
+    module.bind(*[ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in
+                  ("terra_swin_workspace_bytes", "terra_swin_attn_fwd", "terra_swin_attn_bwd", "terra_swin_attn_fwd_packed",
+                   "terra_swin_attn_bwd_packed", "terra_swin_attn_fwd_noalloc")], _check)
+    _host = module
+
+
+def _native():
+    if _host is None:
+        load_library()
+    return _host
 
 
 def make_desc(cfg, scale: float = 0.0, dtype=torch.bfloat16) -> terra_swin_desc:
@@ -93,10 +115,6 @@ def make_desc(cfg, scale: float = 0.0, dtype=torch.bfloat16) -> terra_swin_desc:
     return terra_swin_desc(cfg.B, cfg.H, cfg.W, cfg.heads, cfg.head_dim, cfg.window, cfg.shift_h, cfg.shift_w,
                            cfg.periodic_h, cfg.periodic_w, float(scale),
                            TERRA_DTYPE_F16 if dtype == torch.float16 else TERRA_DTYPE_BF16)
-
-
-def _act_dtype(desc):
-    return torch.float16 if desc.dtype == TERRA_DTYPE_F16 else torch.bfloat16
 
 
 def _check(status: int) -> None:
@@ -191,110 +209,34 @@ def terra_swin_workspace_bytes(desc: terra_swin_desc, backward: bool) -> int:
     return int(n.value)
 
 
-def _expect(t, dtype, numel, name):
-    if t.dtype != dtype or t.numel() != numel:
-        raise ValueError(f"terra: {name} must be {dtype} with {numel} elements, got {t.dtype} x {t.numel()}")
-
-
 def terra_swin_attn_fwd(desc, q, k, v, bias_table, o=None, lse=None, workspace=None):
     """Forward.  q, k, v bf16 [B, H, W, heads, head_dim]; bias_table fp32 [(2w-1)^2, heads].
     Returns (o bf16 like q, lse fp32 [B, H, W, heads]); pass o / lse / workspace to reuse buffers."""
-    n = desc.B * desc.H * desc.W * desc.heads
-    for name, t in (("q", q), ("k", k), ("v", v)):
-        _expect(t, _act_dtype(desc), n * desc.head_dim, name)
-    _expect(bias_table, torch.float32, (2 * desc.window - 1) ** 2 * desc.heads, "bias_table")
-    if o is None:
-        o = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((desc.B, desc.H, desc.W, desc.heads), dtype=torch.float32, device=q.device)
-    _expect(o, _act_dtype(desc), n * desc.head_dim, "o")
-    _expect(lse, torch.float32, n, "lse")
-    if workspace is None:
-        need = terra_swin_workspace_bytes(desc, False)
-        workspace = torch.empty(need, dtype=torch.uint8, device=q.device) if need else None
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load_library().terra_swin_attn_fwd(ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(bias_table),
-                                              _ptr(o), _ptr(lse), _ptr(workspace), ws_bytes, _stream()))
-    return o, lse
+    return (_host or _native()).fwd(desc, q, k, v, bias_table, o, lse, workspace)
 
 
 def terra_swin_attn_fwd_noalloc(desc, q, k, v, bias_table, o, lse):
     """Forward into caller-provided o / lse with no workspace: the library's built-in scratch is used and
     nothing is allocated, by this binding or by the library (see include/terra.h for who needs this and
     for its limits: at most TERRA_NOALLOC_MAX_HEADS heads, calls on one device must not overlap)."""
-    n = desc.B * desc.H * desc.W * desc.heads
-    for name, t in (("q", q), ("k", k), ("v", v), ("o", o)):
-        _expect(t, _act_dtype(desc), n * desc.head_dim, name)
-    _expect(bias_table, torch.float32, (2 * desc.window - 1) ** 2 * desc.heads, "bias_table")
-    _expect(lse, torch.float32, n, "lse")
-    _check(load_library().terra_swin_attn_fwd_noalloc(ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(bias_table),
-                                                      _ptr(o), _ptr(lse), _stream()))
-    return o, lse
+    return (_host or _native()).fwd_noalloc(desc, q, k, v, bias_table, o, lse)
 
 
 def terra_swin_attn_bwd(desc, q, k, v, bias_table, o, lse, d_o, dq=None, dk=None, dv=None, dbias=None,
                         workspace=None):
     """Backward.  Returns (dq, dk, dv bf16 like q, dbias fp32 like bias_table)."""
-    n = desc.B * desc.H * desc.W * desc.heads
-    for name, t in (("q", q), ("k", k), ("v", v), ("o", o), ("d_o", d_o)):
-        _expect(t, _act_dtype(desc), n * desc.head_dim, name)
-    _expect(lse, torch.float32, n, "lse")
-    _expect(bias_table, torch.float32, (2 * desc.window - 1) ** 2 * desc.heads, "bias_table")
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(q) if dk is None else dk
-    dv = torch.empty_like(q) if dv is None else dv
-    dbias = torch.empty_like(bias_table) if dbias is None else dbias
-    for name, t in (("dq", dq), ("dk", dk), ("dv", dv)):
-        _expect(t, _act_dtype(desc), n * desc.head_dim, name)
-    _expect(dbias, torch.float32, bias_table.numel(), "dbias")
-    if workspace is None:
-        workspace = torch.empty(terra_swin_workspace_bytes(desc, True), dtype=torch.uint8, device=q.device)
-    ws_bytes = workspace.numel() * workspace.element_size()
-    _check(load_library().terra_swin_attn_bwd(ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(bias_table),
-                                              _ptr(o), _ptr(lse), _ptr(d_o), _ptr(dq), _ptr(dk), _ptr(dv),
-                                              _ptr(dbias), _ptr(workspace), ws_bytes, _stream()))
-    return dq, dk, dv, dbias
+    return (_host or _native()).bwd(desc, q, k, v, bias_table, o, lse, d_o, dq, dk, dv, dbias, workspace)
 
 
 def terra_swin_attn_fwd_packed(desc, qkv, bias_table, o=None, lse=None, workspace=None):
     """Forward on the packed projection output.  qkv bf16 [B, H, W, 3, heads, head_dim] (q, k, v in that order);
     returns (o bf16 [B, H, W, heads, head_dim], lse fp32 [B, H, W, heads])."""
-    n = desc.B * desc.H * desc.W * desc.heads
-    _expect(qkv, _act_dtype(desc), 3 * n * desc.head_dim, "qkv")
-    _expect(bias_table, torch.float32, (2 * desc.window - 1) ** 2 * desc.heads, "bias_table")
-    if o is None:
-        o = torch.empty((desc.B, desc.H, desc.W, desc.heads, desc.head_dim), dtype=_act_dtype(desc), device=qkv.device)
-    if lse is None:
-        lse = torch.empty((desc.B, desc.H, desc.W, desc.heads), dtype=torch.float32, device=qkv.device)
-    _expect(o, _act_dtype(desc), n * desc.head_dim, "o")
-    _expect(lse, torch.float32, n, "lse")
-    if workspace is None:
-        need = terra_swin_workspace_bytes(desc, False)
-        workspace = torch.empty(need, dtype=torch.uint8, device=qkv.device) if need else None
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(load_library().terra_swin_attn_fwd_packed(ctypes.byref(desc), _ptr(qkv), _ptr(bias_table), _ptr(o), _ptr(lse),
-                                                     _ptr(workspace), ws_bytes, _stream()))
-    return o, lse
+    return (_host or _native()).fwd_packed(desc, qkv, bias_table, o, lse, workspace)
 
 
 def terra_swin_attn_bwd_packed(desc, qkv, bias_table, o, lse, d_o, dqkv=None, dbias=None, workspace=None):
     """Backward on the packed layout.  Returns (dqkv bf16 like qkv, dbias fp32 like bias_table)."""
-    n = desc.B * desc.H * desc.W * desc.heads
-    _expect(qkv, _act_dtype(desc), 3 * n * desc.head_dim, "qkv")
-    for name, t in (("o", o), ("d_o", d_o)):
-        _expect(t, _act_dtype(desc), n * desc.head_dim, name)
-    _expect(lse, torch.float32, n, "lse")
-    _expect(bias_table, torch.float32, (2 * desc.window - 1) ** 2 * desc.heads, "bias_table")
-    dqkv = torch.empty_like(qkv) if dqkv is None else dqkv
-    dbias = torch.empty_like(bias_table) if dbias is None else dbias
-    _expect(dqkv, _act_dtype(desc), 3 * n * desc.head_dim, "dqkv")
-    _expect(dbias, torch.float32, bias_table.numel(), "dbias")
-    if workspace is None:
-        workspace = torch.empty(terra_swin_workspace_bytes(desc, True), dtype=torch.uint8, device=qkv.device)
-    ws_bytes = workspace.numel() * workspace.element_size()
-    _check(load_library().terra_swin_attn_bwd_packed(ctypes.byref(desc), _ptr(qkv), _ptr(bias_table), _ptr(o), _ptr(lse),
-                                                     _ptr(d_o), _ptr(dqkv), _ptr(dbias), _ptr(workspace), ws_bytes, _stream()))
-    return dqkv, dbias
+    return (_host or _native()).bwd_packed(desc, qkv, bias_table, o, lse, d_o, dqkv, dbias, workspace)
 
 
 def padded_extent(extent: int, window: int) -> int:

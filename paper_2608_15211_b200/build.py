@@ -1,13 +1,16 @@
-"""Builds the CUDA library in-tree for sm_100a with nvcc (cross-compiles without a GPU)."""
+"""Builds the CUDA library in-tree for sm_100a with nvcc (cross-compiles without a GPU), and the binding's native module."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libterra_swin.so")
+HOST_SRC = os.path.join(CSRC, "host_module.cpp")
+HOST_PATH = os.path.join(PKG_DIR, "_host.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--shared", "-Xcompiler", "-fPIC", "-lcuda"]
@@ -26,8 +29,27 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > built for p in deps)
 
 
+def build_host(force: bool = False) -> str:
+    """Compile csrc/host_module.cpp, the attention calls' argument handling, against the installed torch."""
+    header = os.path.join(os.path.dirname(PKG_DIR), "include", "terra.h")
+    if not force and os.path.exists(HOST_PATH) and os.path.getmtime(HOST_PATH) >= max(os.path.getmtime(HOST_SRC), os.path.getmtime(header)):
+        return HOST_PATH
+    import torch
+    from torch.utils import cpp_extension
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cuda = cpp_extension.CUDA_HOME or "/usr/local/cuda"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-o", HOST_PATH, HOST_SRC]
+    cmd += ["-I" + d for d in cpp_extension.include_paths() + [sysconfig.get_paths()["include"], os.path.join(cuda, "include")]]
+    cmd += ["-L" + lib, "-Wl,-rpath," + lib, "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
+    proc = subprocess.run(cmd, capture_output=True, text=True)
+    if proc.returncode != 0:
+        raise RuntimeError("g++ failed:\n" + proc.stdout + proc.stderr)
+    return HOST_PATH
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile csrc/*.cu into libterra_swin.so next to this file; returns its path."""
+    """Compile csrc/*.cu into libterra_swin.so and the native module next to this file; returns the library's path."""
+    build_host(force)
     if not force and not _stale():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "nvcc")

@@ -16,10 +16,11 @@ static std::atomic<long long> g_launches{0};
 
 struct ProfEntry { const char* name; cudaEvent_t begin, end; bool closed; };
 static std::mutex g_prof_mutex;
-static bool g_prof_on = false;
+static std::atomic<bool> g_prof_on{false};
 static std::vector<ProfEntry> g_prof;
 
 void prof_begin(const char* name, cudaStream_t stream) {
+    if (!g_prof_on.load(std::memory_order_relaxed)) return;
     std::lock_guard<std::mutex> lock(g_prof_mutex);
     if (!g_prof_on) return;
     ProfEntry e{name, nullptr, nullptr, false};
@@ -30,6 +31,7 @@ void prof_begin(const char* name, cudaStream_t stream) {
 
 void count_launch(cudaStream_t stream) {
     g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (!g_prof_on.load(std::memory_order_relaxed)) return;
     std::lock_guard<std::mutex> lock(g_prof_mutex);
     if (g_prof_on && !g_prof.empty() && !g_prof.back().closed) {
         cudaEventRecord(g_prof.back().end, stream);
@@ -47,6 +49,37 @@ static thread_local char g_cuda_error[256] = "";
 static int cuda_fail(cudaError_t e, const char* where) {
     std::snprintf(g_cuda_error, sizeof g_cuda_error, "%s: %s", where, cudaGetErrorString(e));
     return TERRA_ERR_CUDA;
+}
+
+cudaError_t prepare_kernel(const void* kernel, size_t smem, int threads, int* occupancy) {
+    struct Known { const void* kernel; size_t smem; int device, threads, occupancy; };
+    constexpr int kKnown = 16;
+    static thread_local Known known[kKnown] = {};
+    static thread_local int next = 0;
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    for (const Known& k : known)
+        if (k.kernel == kernel && k.smem == smem && k.device == device && (!occupancy || k.threads == threads)) {
+            if (occupancy) *occupancy = k.occupancy;
+            return cudaSuccess;
+        }
+    {
+        // only ever raised: another size of the same kernel may be remembered, here or by another thread
+        static std::mutex raise;
+        std::lock_guard<std::mutex> lock(raise);
+        cudaFuncAttributes attr;
+        e = cudaFuncGetAttributes(&attr, kernel);
+        if (e == cudaSuccess && (int)smem > attr.maxDynamicSharedSizeBytes)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    }
+    int occ = 0;
+    if (e == cudaSuccess && occupancy) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem);
+    if (e != cudaSuccess) return e;
+    known[next] = {kernel, smem, device, occupancy ? threads : 0, occ};
+    next = (next + 1) % kKnown;
+    if (occupancy) *occupancy = occ;
+    return cudaSuccess;
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -217,7 +250,7 @@ static int fwd_call(const Geo& g, const void* q, const void* k, const void* v,
         e = g.f16 ? launch_fwd_tc_f16(g, q, k, v, bias_table, o, lse, workspace, sms, st)
                   : launch_fwd_tc(g, q, k, v, bias_table, o, lse, workspace, sms, st);
     else
-        e = g.f16 ? launch_fwd_mma_f16(g, q, k, v, bias_table, o, lse, st) : launch_fwd_mma(g, q, k, v, bias_table, o, lse, st);
+        e = g.f16 ? launch_fwd_mma_f16(g, q, k, v, bias_table, o, lse, sms, st) : launch_fwd_mma(g, q, k, v, bias_table, o, lse, sms, st);
     return e == cudaSuccess ? TERRA_OK : cuda_fail(e, "terra_swin_attn_fwd");
 }
 

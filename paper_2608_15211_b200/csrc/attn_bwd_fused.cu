@@ -1081,7 +1081,7 @@ cudaError_t launch_bwd_tc(const Geo& g, const void* q, const void* k, const void
             default: kern = swin_bwd_fused_kernel<15>; break;
         }
     }
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    e = prepare_kernel((const void*)kern, kSmemBytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_bwd_fused_kernel", stream);
     kern<<<grid, kThreads, kSmemBytes, stream>>>(

@@ -973,7 +973,7 @@ static cudaError_t launch_kv64(const Geo& g, const void* q, const void* k, const
     auto kern = g.d == 64 ? (qside ? swin_bwd_kv64_kernel<64, 3> : rows ? swin_bwd_kv64_kernel<64, 2> : tma ? swin_bwd_kv64_kernel<64, 1> : swin_bwd_kv64_kernel<64, 0>)
                           : (qside ? swin_bwd_kv64_kernel<128, 3> : rows ? swin_bwd_kv64_kernel<128, 2> : tma ? swin_bwd_kv64_kernel<128, 1> : swin_bwd_kv64_kernel<128, 0>);
     const int smem_bytes = g.d == 64 ? Lay<64>::kSmemBytes : Lay<128>::kSmemBytes;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    cudaError_t e = prepare_kernel((const void*)kern, smem_bytes);
     if (e != cudaSuccess) return e;
     prof_begin(qside ? "swin_bwd_kv64_kernel<query side>" : "swin_bwd_kv64_kernel", stream);
     kern<<<(unsigned)(cph * g.heads), kThreads, smem_bytes, stream>>>(

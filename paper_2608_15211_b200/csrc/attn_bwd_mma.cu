@@ -744,10 +744,8 @@ cudaError_t launch_one_sized(const Geo& g, const void* q, const void* k, const v
                        cudaStream_t stream) {
     auto kern = swin_bwd_mma_kernel<D, KV, BIG>;
     const size_t smem = bwd_smem_bytes(g, !KV);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NTHREADS, smem);
+    cudaError_t e = prepare_kernel((const void*)kern, smem, NTHREADS, &occ);
     if (e != cudaSuccess) return e;
     if (occ < 1) occ = 1;
     const int tiles = (g.nmax + BM - 1) / BM;
@@ -791,10 +789,8 @@ cudaError_t TERRA_ELEM_FN(launch_bwd_small)(const Geo& g, const void* q, const v
     if (e != cudaSuccess) return e;
     auto kern = g.d == 32 ? swin_bwd_small_kernel<32> : g.d == 64 ? swin_bwd_small_kernel<64> : swin_bwd_small_kernel<128>;
     const size_t smem = bwd_small_smem_bytes(g);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int occ = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NTHREADS, smem);
+    e = prepare_kernel((const void*)kern, smem, NTHREADS, &occ);
     if (e != cudaSuccess) return e;
     if (occ < 1) occ = 1;
     const long long items = (long long)g.B * g.Mh * g.Mw;

@@ -1104,7 +1104,7 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     swin_bwd_onepass_prep_kernel<D, RW><<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
         const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, stat);
     count_launch(stream);
-    cudaError_t e = cudaFuncSetAttribute(swin_bwd_onepass_kernel<D, RW>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kSmemBytes);
+    cudaError_t e = prepare_kernel((const void*)swin_bwd_onepass_kernel<D, RW>, L::kSmemBytes);
     if (e != cudaSuccess) return e;
     const int ctas = sm_count < kMaxCtas ? sm_count : kMaxCtas;
     const unsigned grid = (unsigned)(pl.units < ctas ? pl.units : ctas);

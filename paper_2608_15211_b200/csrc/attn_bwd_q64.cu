@@ -772,7 +772,7 @@ cudaError_t launch_bwd_q64(const Geo& g, const void* q, const void* k, const voi
     maps.k4_ok = (tma && !k4_off && make_col_map4(&maps.k4, g, k, g.ts) && make_col_map4(&maps.v4, g, v, g.ts)) ? 1 : 0;
     auto kern = g.d == 64 ? swin_bwd_q64_kernel<64, false> : (tma ? swin_bwd_q64_kernel<128, true> : swin_bwd_q64_kernel<128, false>);
     const int smem_bytes = g.d == 64 ? Lay<64>::kSmemBytes : Lay<128>::kSmemBytes;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    e = prepare_kernel((const void*)kern, smem_bytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_bwd_q64_kernel", stream);
     kern<<<(unsigned)(cph * g.heads), kThreads, smem_bytes, stream>>>(

@@ -466,22 +466,18 @@ size_t fwd_smem_bytes(const Geo& g) {
 }  // namespace
 
 cudaError_t TERRA_ELEM_FN(launch_fwd_mma)(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
-                           void* o, float* lse, cudaStream_t stream) {
+                           void* o, float* lse, int sm_count, cudaStream_t stream) {
     if (g.nmax <= BN && g.w <= 32) {
         // windows of at most 64 tokens: the persistent double-buffered kernel
         auto kern = g.d == 32 ? swin_fwd_small_kernel<32> : g.d == 64 ? swin_fwd_small_kernel<64> : swin_fwd_small_kernel<128>;
         const int nbias = (2 * g.w - 1) * (2 * g.w - 1);
         const size_t smem = (((size_t)BN * 16 + (size_t)nbias * 4 + 127) / 128) * 128 + 6 * (size_t)BN * g.d * 2;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        int occ = 0, dev = 0, sms = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, NTHREADS, smem);
-        if (e == cudaSuccess) e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        int occ = 0;
+        cudaError_t e = prepare_kernel((const void*)kern, smem, NTHREADS, &occ);
         if (e != cudaSuccess) return e;
         if (occ < 1) occ = 1;
         const long long items = (long long)g.B * g.Mh * g.Mw;
-        long long cph = ((long long)sms * occ) / g.heads;
+        long long cph = ((long long)sm_count * occ) / g.heads;
         if (cph < 1) cph = 1;
         if (cph > items) cph = items;
         prof_begin("swin_fwd_small_kernel", stream);
@@ -495,7 +491,7 @@ cudaError_t TERRA_ELEM_FN(launch_fwd_mma)(const Geo& g, const void* q, const voi
     const size_t smem = fwd_smem_bytes(g);
     auto kern = g.w > 32 ? ((g.d == 32) ? swin_fwd_mma_kernel<32, true> : (g.d == 64) ? swin_fwd_mma_kernel<64, true> : swin_fwd_mma_kernel<128, true>)
                          : ((g.d == 32) ? swin_fwd_mma_kernel<32, false> : (g.d == 64) ? swin_fwd_mma_kernel<64, false> : swin_fwd_mma_kernel<128, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = prepare_kernel((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     prof_begin("swin_fwd_mma_kernel", stream);
     kern<<<(unsigned)items, NTHREADS, smem, stream>>>(g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k,

@@ -1010,7 +1010,7 @@ cudaError_t launch_fwd_tc(const Geo& g, const void* q, const void* k, const void
             default: kern = swin_fwd_tc_kernel<false, false, 15>; break;
         }
     }
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    e = prepare_kernel((const void*)kern, kSmemBytes);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(items < sm_count ? items : sm_count);
     prof_begin("swin_fwd_tc_kernel", stream);

@@ -1109,7 +1109,7 @@ cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const vo
     auto kern = g.d == 64 ? (rows ? swin_fwd_tc64_kernel<64, 2> : tma ? swin_fwd_tc64_kernel<64, 1> : swin_fwd_tc64_kernel<64, 0>)
                           : (rows ? swin_fwd_tc64_kernel<128, 2> : tma ? swin_fwd_tc64_kernel<128, 1> : swin_fwd_tc64_kernel<128, 0>);
     const int smem_bytes = g.d == 64 ? Lay<64>::kSmemBytes : Lay<128>::kSmemBytes;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    e = prepare_kernel((const void*)kern, smem_bytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_fwd_tc64_kernel", stream);
     kern<<<grid, kThreads, smem_bytes, stream>>>(g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, prep,

@@ -70,8 +70,8 @@ extern "C" int terra_swin_attn_fwd_noalloc(const terra_swin_desc* desc, const vo
                   : launch_fwd_tc(g, q, k, v, bias_table, o, lse, scratch, sms, (cudaStream_t)stream);
     } else {
         // this kernel needs no scratch
-        e = g.f16 ? launch_fwd_mma_f16(g, q, k, v, bias_table, o, lse, (cudaStream_t)stream)
-                  : launch_fwd_mma(g, q, k, v, bias_table, o, lse, (cudaStream_t)stream);
+        e = g.f16 ? launch_fwd_mma_f16(g, q, k, v, bias_table, o, lse, sms, (cudaStream_t)stream)
+                  : launch_fwd_mma(g, q, k, v, bias_table, o, lse, sms, (cudaStream_t)stream);
     }
     return e == cudaSuccess ? TERRA_OK : report_cuda_failure(e, "terra_swin_attn_fwd_noalloc");
 }

@@ -13,14 +13,19 @@ void count_launch(cudaStream_t stream);   // after every launch: bumps the launc
 // count_launch closes.  Does nothing unless profiling is enabled.
 void prof_begin(const char* name, cudaStream_t stream);
 
+// Before a kernel's launch: allows it `smem` bytes of dynamic shared memory on the current device and, where `occupancy` is
+// given, says how many CTAs of `threads` threads fit an SM.  Each thread remembers its last few kernels: the two runtime
+// calls cost more host time than the launch of a small kernel.
+cudaError_t prepare_kernel(const void* kernel, size_t smem, int threads = 0, int* occupancy = nullptr);
+
 cudaError_t launch_route(const Geo& g, int32_t* perm, int32_t* inv_perm, int32_t* win_offsets,
                          int32_t* pos, int32_t* label, cudaStream_t stream);
 
 cudaError_t launch_fwd_mma(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
-                           void* o, float* lse, cudaStream_t stream);
+                           void* o, float* lse, int sm_count, cudaStream_t stream);
 // the register-tile kernels for fp16 activations and gradients (same arguments)
 cudaError_t launch_fwd_mma_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
-                               void* o, float* lse, cudaStream_t stream);
+                               void* o, float* lse, int sm_count, cudaStream_t stream);
 bool bwd_small_supported_f16(const Geo& g);
 cudaError_t launch_bwd_small_f16(const Geo& g, const void* q, const void* k, const void* v, const void* o, const void* d_o,
                                  const float* bias, const float* lse, void* dq, void* dk, void* dv, float* dbias,
