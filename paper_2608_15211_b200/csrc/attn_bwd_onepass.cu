@@ -27,7 +27,7 @@
 //
 // Roles (512 threads): warps 0-3 / 4-7 elementwise on the even / odd half chunks, warps 8-11 read accumulators out of
 // TMEM (dQ, dK, dV), warp 12 issues the products (dV, dK, dQ), warp 14 the scores (S^T, dP^T), warp 13 every copy, warp 15
-// walks over the units and hands the others a descriptor per key tile.  Half chunks are numbered through the CTA's run and
+// walks over the units, hands the others a descriptor per key tile and copies the tables.  Half chunks are numbered through the CTA's run and
 // use TMEM buffer (number mod 2).  Shared-memory slots for K, V and query half chunks come from one pool in FIFO order, so
 // the next tile's K and V are on their way while the current tile's last half chunks are worked on.
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, all roles leave their loops, TMEM is
@@ -292,20 +292,21 @@ __device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][
     }
 }
 
-// One half chunk of a warp (32 keys x 64 queries): scores in TMEM to P and dS in their places, in four steps of 16 queries with the
-// next step's loads in flight.  `t_s`: S^T (dP^T 64 columns behind it); `t_p`: P^T (dS^T kDsOff behind it); `tab_b`, `tab_s` / `bp`,
-// `sp`: where the tables are (shared / global memory); `pc` holds the first piece's.
+// One half chunk of a warp (32 keys x 64 queries): scores in TMEM to P and dS in their places, in four steps of 16 queries.
+// `t_s`: S^T (dP^T 64 columns behind it); `t_p`: P^T (dS^T kDsOff behind it).  Head dims 32 and 64: the next step's scores are
+// loaded ahead, pc[0] holds the first piece's tables and the second's follow from shared memory (`tab_b`, `tab_s`).  Head dim
+// 128: pc holds both pieces' tables, whose trip to L2 is the longer one.
 template <int D, int RW, int MASK>
-__device__ __forceinline__ void half_chunk(uint32_t t_s, uint32_t t_p, uint32_t st_addr, Piece<RW>& pc, uint32_t tab_b, uint32_t tab_s, const float* bp,
-                                           const float4* sp, const uint32_t (&okm)[2][4], float scale, float2 (&sum)[2][Piece<RW>::kSums], int lane,
-                                           uint32_t bar_sfree) {
+__device__ __forceinline__ void half_chunk(uint32_t t_s, uint32_t t_p, uint32_t st_addr, Piece<RW> (&pc)[2], uint32_t tab_b, uint32_t tab_s,
+                                           const uint32_t (&okm)[2][4], float scale, float2 (&sum)[2][Piece<RW>::kSums], int lane, uint32_t bar_sfree) {
     using L = Lay<D, RW>;
-    uint32_t rs[2][2][8], rp[2][2][8];
+    constexpr int kAhead = L::kTables ? 1 : 0;
+    uint32_t rs[1 + kAhead][2][8], rp[1 + kAhead][2][8];
     auto ld = [&](int i) {
 #pragma unroll
         for (int hl = 0; hl < 2; ++hl) {
-            tmem_ld_frag16(t_s + 16 * i + ((uint32_t)(16 * hl) << 16), rs[i & 1][hl]);
-            tmem_ld_frag16(t_s + 64 + 16 * i + ((uint32_t)(16 * hl) << 16), rp[i & 1][hl]);
+            tmem_ld_frag16(t_s + 16 * i + ((uint32_t)(16 * hl) << 16), rs[i & kAhead][hl]);
+            tmem_ld_frag16(t_s + 64 + 16 * i + ((uint32_t)(16 * hl) << 16), rp[i & kAhead][hl]);
         }
     };
     ld(0);
@@ -316,21 +317,20 @@ __device__ __forceinline__ void half_chunk(uint32_t t_s, uint32_t t_p, uint32_t 
 #pragma unroll
             for (int x = 0; x < Piece<RW>::kSums; ++x) sum[j][x] = make_float2(0.f, 0.f);
         }
+        if (!kAhead && i > 0) ld(i);
         tmem_ld_wait();
-        if (i < 3) ld(i + 1);
+        if (kAhead && i < 3) ld(i + 1);
         if (L::kOwnP && i == 3) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_sfree);
         }
         const uint32_t tp = t_p + L::kPieceP * j, sa = st_addr ^ (64u * j);
-        if ((i & 1) == 0) step_math<RW, MASK, 0>(rs[i & 1], rp[i & 1], tp, tp + L::kDsOff, sa, pc, okm[j], scale, sum[j]);
-        else step_math<RW, MASK, 1>(rs[i & 1], rp[i & 1], tp, tp + L::kDsOff, sa, pc, okm[j], scale, sum[j]);
-        if (i == 1) {
-            // the second piece: 32 / RW row differences further
-            if (L::kTables) pc.load(tab_b + (32 / RW) * 2 * RW * 4, tab_s + 256);
-            else pc.load(bp + (32 / RW) * 2 * RW, sp + 16);
-        }
+        const Piece<RW>& pj = pc[L::kTables ? 0 : j];
+        if ((i & 1) == 0) step_math<RW, MASK, 0>(rs[i & kAhead], rp[i & kAhead], tp, tp + L::kDsOff, sa, pj, okm[j], scale, sum[j]);
+        else step_math<RW, MASK, 1>(rs[i & kAhead], rp[i & kAhead], tp, tp + L::kDsOff, sa, pj, okm[j], scale, sum[j]);
+        // the second piece: 32 / RW row differences further
+        if (L::kTables && i == 1) pc[0].load(tab_b + (32 / RW) * 2 * RW * 4, tab_s + 256);
     }
 }
 
@@ -419,7 +419,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         // in a staged table: piece 0's row difference 0 is row 128 / RW - 1 - (the warp's first key row in the tile)
         const uint32_t tab_b0 = smem0 + L::kOffTab + ((gl & 1) ? L::kOffCopy1 : L::kOffCopy0) + ((kTile / RW - 1 - (RW == 32 ? wq : 2 * wq)) * 2 * RW + lane_e) * 4;
         const uint32_t tab_s0 = smem0 + L::kOffTab + t * 16;
-        Piece<RW> pc;
+        Piece<RW> pc[2];
         // the next tile: what its half chunks have in common
         auto enter_tile = [&]() {
             if (!next_tile()) return false;
@@ -448,7 +448,11 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         auto bias_ptr = [&]() { return tbl + row0 + hc * kG * (2 * RW); };
         auto stat_ptr = [&]() { return p.rowstat + (size_t)sp * (p.npad / 2) + (hc * 32 + t); };
         bool live = enter_tile();
-        if (live && !L::kTables) pc.load(bias_ptr(), stat_ptr());
+        auto load_tables = [&]() {
+            pc[0].load(bias_ptr(), stat_ptr());
+            pc[1].load(bias_ptr() + (32 / RW) * 2 * RW, stat_ptr() + 16);
+        };
+        if (live && !L::kTables) load_tables();
         while (live) {
             float2 sum[2][Piece<RW>::kSums];
             const uint32_t st_addr = smem0 + L::kOffDs + (D == 128 ? (uint32_t)b : 2 * (n & 1) + b) * L::kDsB + st_off;
@@ -456,15 +460,15 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             const uint32_t tb = tab_b0 + ti * L::kTabB, ts = tab_s0 + ti * L::kTabB;
             if (L::kTables) {
                 if (!mbar_wait_all(bar(kBTab + ti), tuse & 1, cta_abort)) break;
-                pc.load(tb, ts);
+                pc[0].load(tb, ts);
             }
             if (!mbar_wait_all(bar(kBSdp + b), n & 1, cta_abort)) break;
             tc_fence_after();
             uint32_t okm[2][4] = {{rowbits, 0, 0, 0}, {rowbits, 0, 0, 0}};
             if (mode == 0) {
-                half_chunk<D, RW, 0>(t_s, t_p, st_addr, pc, tb, ts, bias_ptr(), stat_ptr(), okm, scale, sum, lane, bar(kBSFree + b));
+                half_chunk<D, RW, 0>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
             } else if (mode == 1) {
-                half_chunk<D, RW, 1>(t_s, t_p, st_addr, pc, tb, ts, bias_ptr(), stat_ptr(), okm, scale, sum, lane, bar(kBSFree + b));
+                half_chunk<D, RW, 1>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
             } else {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
@@ -477,7 +481,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                         okm[j][m] = (rowbits & (1u << m)) ? ((rowbits & (16u << m)) ? qbits : ~qbits) & rows : 0u;
                     }
                 }
-                half_chunk<D, RW, 2>(t_s, t_p, st_addr, pc, tb, ts, bias_ptr(), stat_ptr(), okm, scale, sum, lane, bar(kBSFree + b));
+                half_chunk<D, RW, 2>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
             }
             fence_proxy_async();
             tmem_st_wait();
@@ -491,7 +495,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             float* acc = p.dbias_acc + row0 + hc * kG * (2 * RW);
             hc += 2;
             if (hc >= nh) live = enter_tile();
-            if (live && !L::kTables) pc.load(bias_ptr(), stat_ptr());
+            if (live && !L::kTables) load_tables();
             // The bias gradient, while the products are computed.  Head dim 128 has no shared memory to spare: the sums go
             // through the warp's own rows of the dS^T tile once the dQ product has read them.
             if (D == 128 && !mbar_wait_all(bar(kBDq + b), n & 1, cta_abort)) break;
@@ -562,15 +566,26 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
 #pragma unroll
                             for (int jr = 0; jr < 32 / RW; ++jr) {
                                 const int a = s0 / RW + jr;
-                                if (a < td.eh) {
-                                    int v = td.wc * g.w + g.sw;
-                                    if (v >= g.W) v -= g.W;
-                                    __nv_bfloat16* base = dq + (sample + (size_t)win_token(g, td.wr, td.wc, a, 0) - v) * g.ts + td.head * D + row;
+                                if (a >= td.eh) continue;
+                                int v = td.wc * g.w + g.sw;
+                                if (v >= g.W) v -= g.W;
+                                __nv_bfloat16* base = dq + (sample + (size_t)win_token(g, td.wr, td.wc, a, 0) - v) * g.ts + td.head * D;
+                                if (v + td.ew <= g.W && td.ew == RW) {
+                                    // two lanes exchange halves, so that each stores two channels of every other query
+                                    uint32_t* d2 = reinterpret_cast<uint32_t*>(base + (size_t)(v + (row & 1)) * g.ts + (row & ~1));
+#pragma unroll
+                                    for (int i = 0; i < RW; i += 2) {
+                                        const float x0 = __uint_as_float(r[hh][jr * RW + i]) * out_scale, x1 = __uint_as_float(r[hh][jr * RW + i + 1]) * out_scale;
+                                        const float y = __shfl_xor_sync(0xffffffffu, (row & 1) ? x0 : x1, 1);
+                                        *d2 = (row & 1) ? pack_elem(y, x1) : pack_elem(x0, y);
+                                        d2 += g.ts;                       // two tokens of ts 16-bit elements
+                                    }
+                                } else {
 #pragma unroll
                                     for (int i = 0; i < RW; ++i) {
                                         if (i < td.ew) {
                                             const uint32_t pkd = pack_elem(__uint_as_float(r[hh][jr * RW + i]) * out_scale, 0.f);
-                                            *reinterpret_cast<uint16_t*>(base + (size_t)v * g.ts) = (uint16_t)pkd;
+                                            *reinterpret_cast<uint16_t*>(base + (size_t)v * g.ts + row) = (uint16_t)pkd;
                                         }
                                         if (++v >= g.W) v = 0;
                                     }
@@ -654,21 +669,49 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 __syncwarp();
                 ++i;
             };
+            // The tables of the tile in front of the last one put: each of its copies takes this warp a few hundred cycles, and
+            // the loading warp has as many of its own (with both on one warp it was what the score warp waited for).
+            unsigned n = 0;                          // half chunks so far
+            int t_head = 0, t_kt = 0, t_nch = 0, t_win = 0;
+            auto tables = [&]() {
+                // bias rows of half chunk hc: row differences from hc kG - (kt + 1) (128 / RW) + 1 on
+                const size_t rows0 = ((size_t)t_head * 2 * p.rmax + p.rmax + 1 - (t_kt + 1) * (kTile / RW)) * (2 * RW);
+                const float4* stat = p.rowstat + ((size_t)t_win * g.heads + t_head) * (p.npad / 2);
+                for (int hc = 0; ok && hc < 2 * t_nch; ++hc, ++n) {
+                    const int r = (int)(n % L::kTabs);
+                    ok = mbar_wait_all(bar(kBTabFree + r), ((n / L::kTabs) & 1) ^ 1u, cta_abort);
+                    if (!ok) break;
+                    const uint32_t dst = smem0 + L::kOffTab + r * L::kTabB;
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(bar(kBTab + r), 512 + 2 * L::kCopyB);
+                        bulk_load(dst, stat + hc * 32, 512, bar(kBTab + r));
+                        bulk_load(dst + L::kOffCopy0, p.bias0 + rows0 + hc * kG * (2 * RW), L::kCopyB, bar(kBTab + r));
+                        bulk_load(dst + L::kOffCopy1, p.bias1 + rows0 + hc * kG * (2 * RW), L::kCopyB, bar(kBTab + r));
+                    }
+                    __syncwarp();
+                }
+            };
             for (long long u = blockIdx.x; ok && u < p.units; u += gridDim.x) {
                 const int head = cur.head >> p.split_log2, split = cur.head - (head << p.split_log2);
                 const int eh = min(g.w, g.H - cur.wr * g.w), ew = min(g.w, g.W - cur.wc * g.w), nch = (eh * RW + kTile - 1) / kTile;
                 const int kt0 = (split * nch) >> p.split_log2, kt1 = ((split + 1) * nch) >> p.split_log2;
-                for (int kt = kt0; ok && kt < kt1; ++kt) put(1 | (kt == kt0 ? 2 : 0) | (kt == kt1 - 1 ? 4 : 0), head, eh, ew, kt, nch, (int)u);
+                for (int kt = kt0; ok && kt < kt1; ++kt) {
+                    put(1 | (kt == kt0 ? 2 : 0) | (kt == kt1 - 1 ? 4 : 0), head, eh, ew, kt, nch, (int)u);
+                    if (L::kTables) {
+                        tables();
+                        t_head = head; t_kt = kt; t_nch = nch; t_win = (cur.b * g.Mh + cur.wr) * g.Mw + cur.wc;
+                    }
+                }
                 cursor_advance(cur, g.heads << p.split_log2, g.Mw, g.Mh);
             }
             if (ok) put(0, 0, 0, 0, 0, 0, 0);
+            if (L::kTables) tables();
         } else if (warp == kLoaderWarp) {
             // -------------------------------------------------------------- copies.  One warp fills every slot: a wait names a
             // barrier's phase by parity, so a slot's next use may only be waited for by who has filled its last one
             SlotQueue<L::kSlots> sq;
             sq.init();
             uint32_t use = 0;                        // bit per slot: parity of the slot's fills
-            unsigned n = 0;                          // half chunks so far
             bool ok = true;
             // lane -> (second half of a tile's rows / second tensor, channel part)
             const int part = lane % kParts, second = lane / kParts;
@@ -693,11 +736,28 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     fence_proxy_async();
                     __syncwarp();
                 }
-                if (lane == 0) mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB - (fix ? 2 * kG * kRowB : 0));
-                if (second < 2) {
-                    const uint32_t dst = smem0 + s * L::kSlotB + (two ? second * kHalf * D * 2 + part * kHalf * kRowB : part * kTile * kRowB + second * kHalf * kRowB);
-                    load_win_group<RW, kRowB>(second ? m1 : m0, p.cols, dst, g, td.b, td.wr, td.wc, td.eh, a0 + (two ? 0 : second * kG),
-                                              td.head * D + part * L::kPartCh, bar(kBFull + s));
+                const uint32_t base = smem0 + s * L::kSlotB;
+                if (win_group_whole<RW>(p.cols, g, td.wr, td.wc, td.eh, a0, two ? 1 : 2)) {
+                    // the common case: one thread, one copy per group and channel part
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB);
+                        int y0 = td.wr * g.w + a0 + g.sh;
+                        if (y0 >= g.H) y0 -= g.H;
+                        y0 += td.b * g.H;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int pt = 0; pt < kParts; ++pt)
+                                tma_load_4d(base + (two ? h * kHalf * D * 2 + pt * kHalf * kRowB : pt * kTile * kRowB + h * kHalf * kRowB), &(h ? m1 : m0).group,
+                                            td.head * D + pt * L::kPartCh, 0, td.wc, y0 + (two ? 0 : h * kG), bar(kBFull + s));
+                    }
+                } else {
+                    if (lane == 0) mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB - (fix ? 2 * kG * kRowB : 0));
+                    if (second < 2) {
+                        const uint32_t dst = base + (two ? second * kHalf * D * 2 + part * kHalf * kRowB : part * kTile * kRowB + second * kHalf * kRowB);
+                        load_win_rows<RW, kRowB>(second ? m1 : m0, p.cols, dst, g, td.b, td.wr, td.wc, td.eh, a0 + (two ? 0 : second * kG),
+                                                 td.head * D + part * L::kPartCh, bar(kBFull + s));
+                    }
                 }
                 __syncwarp();
             };
@@ -705,24 +765,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 const int sk = sq.pop(), sv = sq.pop();
                 fill(sk, mk, mk, p.k, p.k, td.kt * 2 * kG, false);
                 if (ok) fill(sv, mv, mv, p.v, p.v, td.kt * 2 * kG, false);
-                // bias rows of half chunk hc: row differences from hc kG - (kt + 1) (128 / RW) + 1 on
-                const size_t rows0 = ((size_t)td.head * 2 * p.rmax + p.rmax + 1 - (td.kt + 1) * (kTile / RW)) * (2 * RW);
-                const float4* stat = p.rowstat + (((size_t)td.b * g.Mh * g.Mw + td.wr * g.Mw + td.wc) * g.heads + td.head) * (p.npad / 2);
-                for (int hc = 0; ok && hc < 2 * td.nch; ++hc) {
-                    if (L::kTables) {
-                        const int i = (int)(n % L::kTabs);
-                        ok = mbar_wait_all(bar(kBTabFree + i), ((n / L::kTabs) & 1) ^ 1u, cta_abort);
-                        if (!ok) break;
-                        const uint32_t dst = smem0 + L::kOffTab + i * L::kTabB;
-                        if (lane == 0) mbar_arrive_expect_tx(bar(kBTab + i), 512 + 2 * L::kCopyB);
-                        if (lane == 1) bulk_load(dst, stat + hc * 32, 512, bar(kBTab + i));
-                        if (lane == 2) bulk_load(dst + L::kOffCopy0, p.bias0 + rows0 + hc * kG * (2 * RW), L::kCopyB, bar(kBTab + i));
-                        if (lane == 3) bulk_load(dst + L::kOffCopy1, p.bias1 + rows0 + hc * kG * (2 * RW), L::kCopyB, bar(kBTab + i));
-                        __syncwarp();
-                        ++n;
-                    }
-                    fill(sq.take_half(), mq, mg, p.q, p.d_o, hc * kG, true);
-                }
+                for (int hc = 0; ok && hc < 2 * td.nch; ++hc) fill(sq.take_half(), mq, mg, p.q, p.d_o, hc * kG, true);
                 sq.end_tile(sk, sv);
             }
         } else if (warp == kScoreWarp) {

@@ -43,19 +43,22 @@ bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_
 bool make_win_cols(WinCols* c, const Geo& g);
 bool make_win_maps(WinMaps* m, const WinCols& c, const Geo& g, const void* base, int token_stride);
 
-// device: 64 slots from window row `a0` on, channels [ch, ch + part) of every token, to `dst` (rows of ROWB bytes, 1 KB
-// aligned); the bytes are counted on `bar` (64 * ROWB, less ROWB per window row for a seam column with c.skip).
+// device: whether the `groups` 64-slot groups from window row `a0` on are one copy each (map `group`)
+template <int RW>
+__device__ __forceinline__ bool win_group_whole(const WinCols& c, const Geo& g, int wr, int wc, int eh, int a0, int groups) {
+    int u = wr * g.w + a0 + g.sh;
+    if (u >= g.H) u -= g.H;
+    return wc != c.seam && wc < c.first_wrapped && wc != c.last && a0 + groups * (64 / RW) <= eh && u + groups * (64 / RW) <= g.H;
+}
+
+// device: 64 slots from window row `a0` on, a copy per window row, channels [ch, ch + part) of every token, to `dst` (rows of
+// ROWB bytes, 1 KB aligned); the bytes are counted on `bar` (64 * ROWB, less ROWB per window row for a seam column with c.skip).
 template <int RW, int ROWB>
-__device__ __forceinline__ void load_win_group(const WinMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
-                                               int a0, int ch, uint32_t bar) {
+__device__ __forceinline__ void load_win_rows(const WinMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
+                                              int a0, int ch, uint32_t bar) {
     constexpr int G = 64 / RW;
     int u = wr * g.w + a0 + g.sh;
     if (u >= g.H) u -= g.H;
-    const bool special = wc == c.seam || wc >= c.first_wrapped || wc == c.last;
-    if (!special && a0 + G <= eh && u + G <= g.H) {
-        tc::tma_load_4d(dst, &m.group, ch, 0, wc, b * g.H + u, bar);
-        return;
-    }
 #pragma unroll
     for (int r = 0; r < G; ++r) {
         const int y = a0 + r < eh ? b * g.H + u : g.B * g.H;       // behind the last row: zeros
