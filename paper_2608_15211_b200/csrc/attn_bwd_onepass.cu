@@ -107,6 +107,10 @@ struct Params {
     int split_log2;                  // key tiles of a window are shared by 1 << split_log2 units
     int npad;                        // slots of a full window, rounded up to 128
     int rmax;                        // window rows rounded up to whole key tiles: bias-table rows run from -rmax to rmax - 1
+    // The launch's units: first those of the windows (row >= row1, any column), then of (row < row1, column >= col1); a launch of
+    // the inner windows has the units of (row < row1, column < col1).
+    int row1, col1, inner;
+    int slab0;                       // first slab of the launch (two launches may overlap)
     long long units;
     const float4* rowstat;           // per (b, window, head) and slot pair: (-lse log2 e) x 2, delta x 2
     const float* bias0;              // [head][2 rmax][2 RW]: bias log2 e at (da + rmax, db + RW), 0 outside the table
@@ -138,7 +142,7 @@ struct TileDesc {
     int eh, ew, kt, nch;
     int ha, hb;            // window rows >= ha / columns >= hb carry the other shift-mask label (far outside: none do)
     int flags;             // 1: a tile (0: the end), 2: the unit's first, 4: its last
-    int unit;
+    int slab;
 };
 
 __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
@@ -211,7 +215,7 @@ __device__ __forceinline__ void store_scaled32(uint4* dst, const uint32_t (&r)[3
 
 // One step (32 keys x 16 queries, columns k = 2 U and 2 U + 1 of the piece): P = exp2(S scale + bias - lse), dS = P (dP - delta);
 // packed P and dS go to TMEM, dS also to its shared-memory tile, and the piece's sums per diagonal grow.
-// MASK 0: every pair counts.  1: rows m with bit m of ok[0] clear hold no key.  2: bit 2 k + e of ok[m] allows the pair.
+// MASK: bit 2 k + e of ok[m] allows the pair.
 template <int RW, int MASK, int U>
 __device__ __forceinline__ void step_math(const uint32_t (&rs)[2][8], const uint32_t (&rp)[2][8], uint32_t t_p, uint32_t t_ds, uint32_t st_addr,
                                           const Piece<RW>& pc, const uint32_t (&ok)[4], float scale, float2 (&sum)[Piece<RW>::kSums]) {
@@ -224,10 +228,7 @@ __device__ __forceinline__ void step_math(const uint32_t (&rs)[2][8], const uint
             float x0, x1, t0, t1, d0, d1;
             fma2(x0, x1, __uint_as_float(rs[hl][4 * kk + 2 * mi]), __uint_as_float(rs[hl][4 * kk + 2 * mi + 1]), scale, pc.bias[i].x, pc.bias[i].y);
             add2vv(x0, x1, x0, x1, pc.st[k].x, pc.st[k].y);
-            if (MASK == 1) {
-                x0 = (ok[0] & (1u << m)) ? x0 : -INFINITY;
-                x1 = (ok[0] & (1u << m)) ? x1 : -INFINITY;
-            } else if (MASK == 2) {
+            if (MASK) {
                 x0 = (ok[m] & (1u << (2 * k))) ? x0 : -INFINITY;
                 x1 = (ok[m] & (2u << (2 * k))) ? x1 : -INFINITY;
             }
@@ -334,7 +335,11 @@ __device__ __forceinline__ void half_chunk(uint32_t t_s, uint32_t t_p, uint32_t 
     }
 }
 
-template <int D, int RW>
+// KIND 0: windows whose slots all hold tokens and whose tokens share one mask label.  1: windows that need the mask.  2: both (head
+// dim 128).  Two launches instead of a branch: with both bodies in one kernel the unmasked one ran 1.14 times as long (the
+// elementwise warps are sensitive to what the compiler and the instruction caches make of them), at head dim 128 it is not
+// what bounds the kernel.
+template <int D, int RW, int KIND>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk,
                         __nv_bfloat16* __restrict__ dv, const __grid_constant__ WinMaps mq, const __grid_constant__ WinMaps mk,
@@ -393,12 +398,15 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         const int4 d0 = src[0], d1 = src[1], d2 = src[2];
         td.head = d0.x; td.b = d0.y; td.wr = d0.z; td.wc = d0.w;
         td.eh = d1.x; td.ew = d1.y; td.kt = d1.z; td.nch = d1.w;
-        td.ha = d2.x; td.hb = d2.y; td.flags = d2.z; td.unit = d2.w;
+        td.ha = d2.x; td.hb = d2.y; td.flags = d2.z; td.slab = d2.w;
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kBDescFree + i));
         ++desc_n;
         return (td.flags & 1) != 0;
     };
+
+    // the launch of the masked windows may take the SMs that this one leaves (it waits for this one's end before its own)
+    if (KIND == 0) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 
     if (warp < kWorkWarps) {
         // ------------------------------------------------------------------ elementwise: the half chunks of buffer b
@@ -412,7 +420,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         const uint32_t st_off = (uint32_t)((32 * wq + 8 * (lane >> 4) + (lane & 7)) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4));
         const uint32_t scr0 = D == 128 ? smem0 + L::kOffDs + b * L::kDsB + 32 * wq * 128 : smem0 + L::kOffScr + warp * L::kScrB;
         unsigned n = 0;                                      // half chunks of this buffer so far
-        int a_k0, nh, ha, mode, row0, hc = 0;
+        int a_k0, nh, ha, row0, hc = 0;
+        bool masked;
         uint32_t rowbits, qbits, sp;
         const int lane_e = 2 * t - gl - (gl & 1) + RW;       // the thread's entry within a table row (even: both copies are read in pairs)
         const float* tbl = ((gl & 1) ? p.bias1 : p.bias0) + lane_e;
@@ -428,10 +437,10 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             ha = td.ha;
             a_k0 = td.kt * (kTile / RW) + (RW == 32 ? wq : 2 * wq);
             const bool labels = (ha > 0 && ha < td.eh) || (td.hb > 0 && td.hb < td.ew);
-            mode = labels ? 2 : (td.ew < RW || (td.kt + 1) * (kTile / RW) > td.eh) ? 1 : 0;
+            masked = KIND == 1 || (KIND == 2 && (labels || td.ew < RW || (td.kt + 1) * (kTile / RW) > td.eh));
             rowbits = 0;                                     // bits m: the row holds a key; bits 4 + m: it lies behind hb
             qbits = 0;
-            if (mode) {
+            if (masked) {
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     const int a = a_k0 + (RW == 32 ? 0 : m >> 1), bb = gl + 8 * (RW == 32 ? m : m & 1);
@@ -464,11 +473,9 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             }
             if (!mbar_wait_all(bar(kBSdp + b), n & 1, cta_abort)) break;
             tc_fence_after();
-            uint32_t okm[2][4] = {{rowbits, 0, 0, 0}, {rowbits, 0, 0, 0}};
-            if (mode == 0) {
-                half_chunk<D, RW, 0>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
-            } else if (mode == 1) {
-                half_chunk<D, RW, 1>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
+            uint32_t okm[2][4] = {};
+            if (!masked) {
+                half_chunk<D, RW, KIND == 1 ? 1 : 0>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
             } else {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
@@ -481,7 +488,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                         okm[j][m] = (rowbits & (1u << m)) ? ((rowbits & (16u << m)) ? qbits : ~qbits) & rows : 0u;
                     }
                 }
-                half_chunk<D, RW, 2>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
+                half_chunk<D, RW, KIND == 0 ? 0 : 1>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
             }
             fence_proxy_async();
             tmem_st_wait();
@@ -543,7 +550,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         while (ok && next_tile()) {
             const bool first = td.flags & 2, last = td.flags & 4;
             const size_t sample = (size_t)td.b * g.H * g.W;
-            float4* slab = p.slabs + (size_t)(split ? td.unit : (int)blockIdx.x) * ((size_t)p.npad * D / 4) + row;
+            float4* slab = p.slabs + (size_t)td.slab * ((size_t)p.npad * D / 4) + row;
             if (D == 128) {
                 // dQ^T: lanes = channels, columns = the half chunk's queries
                 for (int hc = 0; hc < 2 * td.nch; ++hc, ++n) {
@@ -653,17 +660,17 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsOther));
         if (warp == kPlanWarp) {
             // -------------------------------------------------------------- tiles in the order every role meets them
-            ItemCursor cur = cursor_init(blockIdx.x, gridDim.x, g.heads << p.split_log2, g.Mw, g.Mh);
+            struct { int b, wr, wc; } cur = {0, 0, 0};
             unsigned i = 0;
             bool ok = true;
-            auto put = [&](int flags, int head, int eh, int ew, int kt, int nch, int unit) {
+            auto put = [&](int flags, int head, int eh, int ew, int kt, int nch, int slab) {
                 ok = mbar_wait_all(bar(kBDescFree + i % kDescs), ((i / kDescs) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
                 if (lane == 0) {
                     int4* dst = reinterpret_cast<int4*>(smem + L::kOffDesc + (i % kDescs) * 64);
                     dst[0] = make_int4(head, cur.b, cur.wr, cur.wc);
                     dst[1] = make_int4(eh, ew, kt, nch);
-                    dst[2] = make_int4((!g.ph && g.sh > 0) ? g.H - g.sh - cur.wr * g.w : (1 << 20), (!g.pw && g.sw > 0) ? g.W - g.sw - cur.wc * g.w : (1 << 20), flags, unit);
+                    dst[2] = make_int4((!g.ph && g.sh > 0) ? g.H - g.sh - cur.wr * g.w : (1 << 20), (!g.pw && g.sw > 0) ? g.W - g.sw - cur.wc * g.w : (1 << 20), flags, slab);
                     mbar_arrive(bar(kBDesc + i % kDescs));
                 }
                 __syncwarp();
@@ -692,17 +699,32 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 }
             };
             for (long long u = blockIdx.x; ok && u < p.units; u += gridDim.x) {
-                const int head = cur.head >> p.split_log2, split = cur.head - (head << p.split_log2);
+                // unit -> head and share, window, sample (the windows of the launch: see Params)
+                const unsigned hs = (unsigned)g.heads << p.split_log2, bottom = (unsigned)(g.Mh - p.row1) * g.Mw;
+                const unsigned per_row = p.inner ? p.col1 : g.Mw - p.col1, per_sample = p.row1 * per_row + (p.inner ? 0u : bottom);
+                const unsigned wi = (unsigned)u / hs, hd = (unsigned)u - wi * hs;
+                cur.b = wi / per_sample;
+                unsigned r = wi - cur.b * per_sample;
+                if (!p.inner && r < bottom) {
+                    cur.wr = p.row1 + r / g.Mw;
+                    cur.wc = r % g.Mw;
+                } else {
+                    if (!p.inner) r -= bottom;
+                    cur.wr = r / per_row;
+                    cur.wc = (p.inner ? 0 : p.col1) + r % per_row;
+                }
+                const int head = hd >> p.split_log2, split = hd - (head << p.split_log2);
                 const int eh = min(g.w, g.H - cur.wr * g.w), ew = min(g.w, g.W - cur.wc * g.w), nch = (eh * RW + kTile - 1) / kTile;
                 const int kt0 = (split * nch) >> p.split_log2, kt1 = ((split + 1) * nch) >> p.split_log2;
+                // a slab per CTA; where windows are split, per unit in the order of all windows
+                const int slab = p.split_log2 ? (int)((((long long)(cur.b * g.Mh + cur.wr) * g.Mw + cur.wc) * hs) + hd) : p.slab0 + (int)blockIdx.x;
                 for (int kt = kt0; ok && kt < kt1; ++kt) {
-                    put(1 | (kt == kt0 ? 2 : 0) | (kt == kt1 - 1 ? 4 : 0), head, eh, ew, kt, nch, (int)u);
+                    put(1 | (kt == kt0 ? 2 : 0) | (kt == kt1 - 1 ? 4 : 0), head, eh, ew, kt, nch, slab);
                     if (L::kTables) {
                         tables();
                         t_head = head; t_kt = kt; t_nch = nch; t_win = (cur.b * g.Mh + cur.wr) * g.Mw + cur.wc;
                     }
                 }
-                cursor_advance(cur, g.heads << p.split_log2, g.Mw, g.Mh);
             }
             if (ok) put(0, 0, 0, 0, 0, 0, 0);
             if (L::kTables) tables();
@@ -915,6 +937,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
     __syncthreads();
     tc_fence_after();
     if (warp == kProductWarp) tmem_dealloc(tmem, 512);
+    if (KIND == 1) asm volatile("griddepcontrol.wait;\n" ::: "memory");
     if (tid == 0 && *cta_abort) atomicExch(&g_bwd_onepass_timeout, 1);
 }
 
@@ -1063,7 +1086,8 @@ OnePassPlan bwd_onepass_plan(const Geo& g) {
         if (ls == 0 || t < 0.875 * best) { best = t; p.split_log2 = ls; }
     }
     p.units = items << p.split_log2;
-    const size_t slabs = p.split_log2 ? (size_t)p.units : p.units < kMaxCtas ? (size_t)p.units : (size_t)kMaxCtas;
+    const size_t ctas = p.units < 2 * kMaxCtas ? (size_t)p.units : (size_t)(2 * kMaxCtas);       // of both launches
+    const size_t slabs = p.split_log2 ? (size_t)p.units : ctas;
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t table = up(sizeof(float) * (size_t)g.heads * 2 * p.rmax * 2 * p.rw);
     p.off_bias0 = up(sizeof(float4) * (size_t)g.B * g.Mh * g.Mw * g.heads * (p.npad / 2));
@@ -1133,7 +1157,6 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     p.split_log2 = pl.split_log2;
     p.npad = pl.npad;
     p.rmax = pl.rmax;
-    p.units = pl.units;
     p.rowstat = reinterpret_cast<const float4*>(ws);
     p.bias0 = reinterpret_cast<const float*>(ws + pl.off_bias0);
     p.bias1 = reinterpret_cast<const float*>(ws + pl.off_bias1);
@@ -1147,13 +1170,49 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     swin_bwd_onepass_prep_kernel<D, RW><<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
         const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, stat);
     count_launch(stream);
-    cudaError_t e = prepare_kernel((const void*)swin_bwd_onepass_kernel<D, RW>, L::kSmemBytes);
-    if (e != cudaSuccess) return e;
     const int ctas = sm_count < kMaxCtas ? sm_count : kMaxCtas;
-    const unsigned grid = (unsigned)(pl.units < ctas ? pl.units : ctas);
-    prof_begin("swin_bwd_onepass_kernel", stream);
-    swin_bwd_onepass_kernel<D, RW><<<grid, kThreads, L::kSmemBytes, stream>>>(p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
-    count_launch(stream);
+    auto launch = [&](auto kernel, bool inner, long long windows, int slab0, bool overlap) {
+        p.inner = inner;
+        p.units = windows * g.B * g.heads << pl.split_log2;
+        p.slab0 = slab0;
+        cudaError_t err = prepare_kernel((const void*)kernel, L::kSmemBytes);
+        if (err != cudaSuccess) return err;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(p.units < ctas ? p.units : ctas));
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = L::kSmemBytes;
+        cfg.stream = stream;
+        // the second launch needs nothing of the first: its CTAs take the SMs as the first one's leave them
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = overlap ? 1 : 0;
+        prof_begin(overlap ? "swin_bwd_onepass_kernel<masked>" : "swin_bwd_onepass_kernel", stream);
+        err = cudaLaunchKernelEx(&cfg, kernel, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
+        if (err == cudaSuccess) count_launch(stream);
+        return err;
+    };
+    const long long all = (long long)g.Mh * g.Mw;
+    cudaError_t e = cudaSuccess;
+    if constexpr (D == 128) {
+        p.row1 = g.Mh;
+        p.col1 = g.Mw;
+        e = launch(swin_bwd_onepass_kernel<D, RW, 2>, true, all, 0, false);
+    } else {
+        // the windows in front of the first row and column that need the mask
+        p.row1 = g.w == RW ? g.H / g.w : 0;
+        p.col1 = g.w == RW ? g.W / g.w : 0;
+        if (!g.ph && g.sh > 0 && (g.H - g.sh) % g.w && (g.H - g.sh) / g.w < p.row1) p.row1 = (g.H - g.sh) / g.w;
+        if (!g.pw && g.sw > 0 && (g.W - g.sw) % g.w && (g.W - g.sw) / g.w < p.col1) p.col1 = (g.W - g.sw) / g.w;
+        if (p.row1 == 0 || p.col1 == 0) p.row1 = p.col1 = 0;
+        const long long inner = (long long)p.row1 * p.col1;
+        const long long units0 = inner * g.B * g.heads << pl.split_log2;
+        const int slabs0 = (int)(units0 < ctas ? units0 : ctas);
+        if (inner > 0) e = launch(swin_bwd_onepass_kernel<D, RW, 0>, true, inner, 0, false);
+        if (e == cudaSuccess && inner < all) e = launch(swin_bwd_onepass_kernel<D, RW, 1>, false, all - inner, slabs0, inner > 0);
+    }
+    if (e != cudaSuccess) return e;
     const int nw = 2 * g.w - 1;
     const unsigned bias_blocks = (unsigned)((nw * nw * g.heads + 255) / 256);
     const long long sum_blocks = pl.split_log2 ? (pl.units >> pl.split_log2) * ((pl.npad * D / 4 + 255) / 256) : 0;
