@@ -1,0 +1,734 @@
+// Forward shifted-window attention on the tcgen05 tensor cores: window sides 9 .. 32 at head dims 32, 64 and 128, any grid.
+//
+// A unit is a pair of 128-row query tiles of one (sample, window, head); a persistent CTA per SM walks over units and streams
+// the window's keys through shared memory in chunks of 128 slots (see win_tiles.cuh: 16 or 32 slots to a window row).  Per
+// chunk and query tile:
+//   S = Q K^T (+ E_q E_k^T, see below), 128 x 128 in TMEM;
+//   the softmax warps, 32 query rows each, take the rows' 128 scores into registers in one go, add the bias, take their exact
+//   maximum, raise the row's reference m when the chunk exceeds it by more than 8 octaves (rare; O and the row sum are
+//   scaled down then), and write P = exp2(S scale + bias - m) over S in 16 bits;
+//   O += P V, accumulated in TMEM.
+// Masks cost the softmax threads nothing: where a window's slots differ in shift-mask label or hold no token, one more
+// 16-wide step of the score product adds -2^30 (fp16) or -2^100 (bf16) to the pairs that must not see one another.  E_q holds
+// a one at the query's label, E_k the penalty at every label but the key's.  One body serves every window: the elementwise
+// code is what bounds the kernel, and two copies of it in one kernel run slower than one.
+// Scores and P share three TMEM buffers (head dim 128: two), so that the products of other chunks run under the softmax.
+//
+// What bounds it: MUFU, 16 exponentials per clock and SM (0.40 ms for the 510 x 1080 grid with 12 heads and 16 x 16 windows).
+//
+// Roles (512 threads): warps 0-3 / 4-7 softmax of the pair's first / second tile, warps 8-11 read O out of TMEM, normalise
+// and store it, warp 12 issues the PV products, warp 13 every copy, warp 14 the scores, warp 15 walks over the units.
+// Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, all roles leave their loops, TMEM is released and
+// the host reads the device status word.
+#include "swin_common.cuh"
+#include "swin_kernels.h"
+#include "tc_common.cuh"
+#include "win_tiles.cuh"
+
+// fp16 build of this file (through the _f16 wrapper file): names of its own
+#ifdef TERRA_ELEM_F16
+#define g_fwd_win_timeout g_fwd_win_timeout_f16
+#define launch_fwd_win launch_fwd_win_f16
+#define read_fwd_win_status read_fwd_win_status_f16
+#endif
+
+namespace terra {
+
+__device__ int g_fwd_win_timeout = 0;   // set when a bounded wait expired in any CTA of the kernel below
+
+namespace {
+
+using namespace tc;
+
+constexpr int kThreads = 512;
+constexpr int kSoftWarps = 8, kReadWarp0 = 8, kPvWarp = 12, kLoaderWarp = 13, kScoreWarp = 14, kPlanWarp = 15;
+constexpr int kRegsLaunch = 128, kRegsSoft = 184, kRegsOther = 72;
+static_assert(2 * kRegsSoft + 2 * kRegsOther <= 4 * kRegsLaunch, "register hand-over does not balance");
+constexpr int kTile = 128, kDescs = 8;
+#ifdef TERRA_ELEM_F16
+constexpr uint32_t kMaskQ = 0x7800, kMaskK = 0xF800;           // 2^15, -2^15
+#else
+constexpr uint32_t kMaskQ = 0x5880, kMaskK = 0xD880;           // 2^50, -2^50
+#endif
+
+// The bias table by row difference, twice: copy c starts at column difference c - (RW - 1), so that a thread's pairs of keys
+// are read aligned, from the copy of its row's parity; the copies lie 16 banks apart.
+template <int RW>
+struct Tab {
+    static constexpr int kCopyF = RW == 16 ? 48 : 80, kRowF = 2 * kCopyF;
+    static constexpr int kFront = RW == 16;                   // a row in front of the first difference: two query rows share their reads
+    static __host__ __device__ constexpr int rows(int w) { return 2 * w + 2 * kFront; }
+};
+
+enum { kBFull = 0, kBEmpty = 16, kBS = 32, kBP = 35, kBFree = 38, kBPv = 41, kBO = 43, kBOFree = 45, kBStat = 47, kBTab = 49, kBBias = 51, kBOne = 52,
+       kBDesc = 54, kBDescFree = kBDesc + kDescs, kBCount = kBDescFree + kDescs };
+
+template <int D, int RW>
+struct Lay {
+    static constexpr int kParts = D == 128 ? 2 : 1, kRowB = D >= 64 ? 128 : 64, kPartCh = kRowB / 2;
+    static constexpr int kSlotB = kTile * D * 2;                                    // a Q, K or V tile
+    static constexpr int kSlots = D == 128 ? (RW == 16 ? 6 : 5) : D == 64 ? 10 : 14;
+    static constexpr int kBufs = D == 128 ? 2 : 3, kColO = 128 * kBufs;
+    static constexpr int kOffE = kSlots * kSlotB;                                   // E operands, 64 bytes a slot: E_q, then E_k
+    static constexpr int kOffTab = kOffE + 256 * 64;
+    static constexpr int kOffStat = kOffTab + Tab<RW>::rows(RW) * Tab<RW>::kRowF * 4;          // per row of both tiles: m, row sum
+    static constexpr int kOffDesc = kOffStat + 2 * kTile * 8;
+    static constexpr int kOffBars = kOffDesc + kDescs * 64;
+    static constexpr int kSmemBytes = kOffBars + 8 * kBCount + 16;
+};
+
+struct Params {
+    Geo g;
+    WinCols cols;
+    const __nv_bfloat16 *q, *k, *v;
+    const float* tables;         // [head][Tab::rows][Tab::kRowF]
+    int pairs;                   // query tile pairs of a full window
+    int head_slow;               // units in head-major order, a run per CTA; else the head is the fastest digit, strided
+    long long units;
+};
+
+struct Unit {
+    int head, b, wr, wc;
+    int eh, ew, tile0, ntq;      // first query tile, 1 or 2 of them
+    int ku, nch, ha, hb;         // 32-slot key units, chunks; window rows >= ha / columns >= hb carry the other mask label
+    int flags;                   // 1: a unit (0: the end), 2: another head than before, 4: the scores need the mask step
+};
+
+// FIFO of shared-memory slots: two held for a unit (Q tiles), the others cycle (K, V chunks)
+template <int N>
+struct SlotQueue {
+    uint64_t q;
+    __device__ __forceinline__ void init() {
+        q = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) q |= (uint64_t)i << (4 * i);
+    }
+    __device__ __forceinline__ int pop() { const int s = (int)(q & 15); q >>= 4; return s; }
+    __device__ __forceinline__ int take() { const int s = pop(); q |= (uint64_t)s << (4 * (N - 3)); return s; }
+    __device__ __forceinline__ void end_unit(int s0, int s1) { q |= ((uint64_t)s0 << (4 * (N - 2))) | ((uint64_t)s1 << (4 * (N - 1))); }
+};
+
+__device__ __forceinline__ float2 lds_f2(uint32_t addr) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+    return v;
+}
+
+// The thread's scores of one 32-slot key unit (32 query rows x 32 keys a warp; thread 4 g + t holds rows g + 8 m, keys
+// 8 k + 2 t + e) -> S scale + bias in place, and the rows' maxima.  Pairs on one diagonal share their bias: 7 or 9 reads
+// for 32 scores.  (A thread per row read each score's own entry: the shared-memory pipe then bound the kernel, 1300 to 2500
+// of 4100 to 6800 cycles per 128 x 128 scores and tile.)  `bias`: shared address of the entry of rows g, keys 2 t.
+template <int RW>
+__device__ __forceinline__ void add_bias(uint32_t (&x)[2][16], uint32_t bias, float scale, float (&mx)[4]) {
+    constexpr int kRowB = Tab<RW>::kRowF * 4;
+    float2 bv[9];
+#pragma unroll
+    for (int i = 0; i < (RW == 32 ? 7 : 9); ++i)
+        bv[i] = lds_f2(bias + (RW == 32 ? 32 * (i - 3) : (i / 3 - 1) * kRowB + 32 * (i % 3 - 1)));
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            uint32_t* v = &x[m >> 1][4 * k + 2 * (m & 1)];
+            const float2 b = bv[RW == 32 ? k - m + 3 : 3 * ((k >> 1) - (m >> 1) + 1) + (k & 1) - (m & 1) + 1];
+            float x0, x1;
+            fma2(x0, x1, __uint_as_float(v[0]), __uint_as_float(v[1]), scale, b.x, b.y);
+            v[0] = __float_as_uint(x0);
+            v[1] = __float_as_uint(x1);
+            mx[m] = max3(mx[m], x0, x1);
+        }
+}
+
+template <int D, int RW>
+__global__ void __launch_bounds__(kThreads, 1)
+swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
+                    const __grid_constant__ WinMaps mq, const __grid_constant__ WinMaps mk, const __grid_constant__ WinMaps mv) {
+    using L = Lay<D, RW>;
+    constexpr int kParts = L::kParts, kRowB = L::kRowB, kG = 64 / RW, NB = L::kBufs, kTileRows = kTile / RW;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const uint32_t smem0 = smem_u32(smem), bar0 = smem0 + L::kOffBars;
+    auto bar = [&](int i) { return bar0 + 8u * i; };
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kOffBars + 8 * kBCount);
+    volatile int* cta_abort = reinterpret_cast<volatile int*>(smem + L::kOffBars + 8 * kBCount + 8);
+    const Geo& g = p.g;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+    if (tid == 0) {
+        for (int s = 0; s < L::kSlots; ++s) {
+            mbar_init(bar(kBFull + s), 1);
+            mbar_init(bar(kBEmpty + s), 1);
+        }
+        for (int b = 0; b < NB; ++b) {
+            mbar_init(bar(kBS + b), 1);            // scores of a chunk are in buffer b
+            mbar_init(bar(kBP + b), 4);            // ... and P has taken their place
+            mbar_init(bar(kBFree + b), 1);         // ... and been read by the product
+        }
+        for (int t = 0; t < 2; ++t) {
+            mbar_init(bar(kBPv + t), 1);           // a chunk's product of tile t is done
+            mbar_init(bar(kBO + t), 1);            // ... the unit's last one
+            mbar_init(bar(kBOFree + t), 4);        // O and the statistics of tile t have been read
+            mbar_init(bar(kBStat + t), 4);         // the rows' m and sums are in shared memory
+            mbar_init(bar(kBTab + t), kSoftWarps); // the softmax of a unit is done (even / odd units)
+            mbar_init(bar(kBOne + t), 4);          // ... of a unit of one tile (even / odd ones): the other warps keep in step
+        }
+        mbar_init(bar(kBBias), 1);                 // the head's bias table is in shared memory
+        for (int i = 0; i < kDescs; ++i) {
+            mbar_init(bar(kBDesc + i), 1);
+            mbar_init(bar(kBDescFree + i), kSoftWarps + 7);
+        }
+        *cta_abort = 0;
+        fence_barrier_init();
+    }
+    if (warp == kPvWarp) {
+        tmem_alloc(smem_u32(tmem_slot), 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    unsigned desc_n = 0;
+    Unit td;
+    // the next unit; false at the end of the run (or after an expired wait)
+    auto next_unit = [&]() {
+        const unsigned i = desc_n % kDescs;
+        if (!mbar_wait_all(bar(kBDesc + i), (desc_n / kDescs) & 1, cta_abort)) return false;
+        const int4* src = reinterpret_cast<const int4*>(smem + L::kOffDesc + i * 64);
+        const int4 d0 = src[0], d1 = src[1], d2 = src[2];
+        td.head = d0.x; td.b = d0.y; td.wr = d0.z; td.wc = d0.w;
+        td.eh = d1.x; td.ew = d1.y; td.tile0 = d1.z; td.ntq = d1.w;
+        td.ku = d2.x; td.nch = d2.y; td.ha = d2.z; td.hb = d2.w;
+        td.flags = src[3].x;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kBDescFree + i));
+        ++desc_n;
+        return (td.flags & 1) != 0;
+    };
+
+    if (warp < kSoftWarps) {
+        // ------------------------------------------------------------------ softmax of tile t
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kRegsSoft));
+        const int t = warp >> 2, wq = warp & 3, gl = lane >> 2, ql = lane & 3;
+        const uint32_t tq = tmem + ((uint32_t)(32 * wq) << 16), t_o = tq + L::kColO + D * t;
+        const float scale = g.scale_log2e;
+        const int i0 = RW - 1 + 2 * ql - gl;                 // table column of row g, key 2 t
+        const uint32_t tab0 = smem0 + L::kOffTab + 4u * ((i0 & 1) * Tab<RW>::kCopyF + (i0 & ~1));
+        float2* stat = reinterpret_cast<float2*>(smem + L::kOffStat) + t * kTile + 32 * wq + gl;
+        unsigned n = 0, pv = 0, units = 0, mine = 0, heads = 0, ones = 0;   // chunks of the CTA, of this tile; units, those with this tile; tables; 1-tile units
+        bool ok = true;
+        while (ok && next_unit()) {
+            if (td.flags & 2) ok = mbar_wait_all(bar(kBBias), heads++ & 1, cta_abort);
+            if (ok && t < td.ntq) {
+                const int aq = min((td.tile0 + t) * kTileRows + wq * (32 / RW), td.eh - 1);
+                uint32_t bias = tab0 + 4u * (g.w - 1 - aq + Tab<RW>::kFront) * Tab<RW>::kRowF;
+                float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                float2 sum[4] = {};
+                for (int c = 0; c < td.nch; ++c, ++pv) {
+                    const unsigned idx = n + c * td.ntq + t, buf = idx % NB;
+                    const uint32_t t_s = tq + 128u * buf;
+                    const int nu = min(4, td.ku - 4 * c);
+                    ok = mbar_wait_all(bar(kBS + buf), (idx / NB) & 1, cta_abort);
+                    if (!ok) break;
+                    tc_fence_after();
+                    auto load = [&](int u, uint32_t (&x)[2][16]) {
+                        tmem_ld_frag32(t_s + 32 * u, x[0]);
+                        tmem_ld_frag32(t_s + (16u << 16) + 32 * u, x[1]);
+                    };
+                    auto work = [&](int u, uint32_t (&x)[2][16]) {
+                        float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                        add_bias<RW>(x, bias, scale, top);
+                        bias += 4u * (32 / RW) * Tab<RW>::kRowF;
+                        if (__any_sync(0xffffffffu, top[0] - m[0] > 8.f || top[1] - m[1] > 8.f || top[2] - m[2] > 8.f || top[3] - m[3] > 8.f)) {
+                            // raise the reference: the sums, the chunk's P so far and, once its products are done, O are scaled down
+                            float f[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                top[i] = fmaxf(top[i], __shfl_xor_sync(0xffffffffu, top[i], 1));
+                                top[i] = fmaxf(top[i], __shfl_xor_sync(0xffffffffu, top[i], 2));
+                                const float up = top[i] - m[i] > 8.f ? top[i] : m[i];
+                                f[i] = fast_exp2(m[i] - up);
+                                m[i] = up;
+                                sum[i].x *= f[i];
+                                sum[i].y *= f[i];
+                            }
+                            if (u > 0) {
+                                tmem_st_wait();
+#pragma unroll 1
+                                for (int col = 0; col < 16 * u; col += 16)
+#pragma unroll
+                                    for (int h = 0; h < 2; ++h) {
+                                        uint32_t r[8];
+                                        tmem_ld_frag_packed16(t_s + ((16u * h) << 16) + col, r);
+                                        tmem_ld_wait();
+#pragma unroll
+                                        for (int i = 0; i < 8; ++i) {
+                                            const float2 v = elem2_to_float2(r[i]);
+                                            r[i] = pack_elem(v.x * f[2 * h + (i & 1)], v.y * f[2 * h + (i & 1)]);
+                                        }
+                                        tmem_st_frag_packed16(t_s + ((16u * h) << 16) + col, r);
+                                    }
+                            }
+                            if (c > 0) {
+                                ok = mbar_wait_all(bar(kBPv + t), (pv - 1) & 1, cta_abort);
+                                if (ok) tc_fence_after();
+#pragma unroll 1
+                                for (int col = 0; ok && col < D; col += 16)
+#pragma unroll
+                                    for (int h = 0; h < 2; ++h) {
+                                        uint32_t r[8];
+                                        tmem_ld_frag16(t_o + ((16u * h) << 16) + col, r);
+                                        tmem_ld_wait();
+#pragma unroll
+                                        for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f[2 * h + ((i >> 1) & 1)]);
+                                        tmem_st_frag16(t_o + ((16u * h) << 16) + col, r);
+                                    }
+                            }
+                        }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t pk[8];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                                for (int mi = 0; mi < 2; ++mi) {
+                                    const int i = 2 * h + mi;
+                                    float x0, x1;
+                                    add2(x0, x1, __uint_as_float(x[h][4 * k + 2 * mi]), __uint_as_float(x[h][4 * k + 2 * mi + 1]), -m[i]);
+                                    x0 = fast_exp2(x0);
+                                    x1 = fast_exp2(x1);
+                                    add2vv(sum[i].x, sum[i].y, sum[i].x, sum[i].y, x0, x1);
+                                    pk[2 * k + mi] = pack_elem(x0, x1);
+                                }
+                            tmem_st_frag_packed16(t_s + ((16u * h) << 16) + 16 * u, pk);
+                        }
+                    };
+                    // the next unit's scores come while this one's are worked on.  A loop of two units: the code has to stay
+                    // small, a chunk in one piece ran at a fetch-bound 12 cycles an instruction
+                    uint32_t xa[2][16], xb[2][16];
+                    load(0, xa);
+#pragma unroll 1
+                    for (int u = 0; u < nu; u += 2) {
+                        tmem_ld_wait();
+                        if (u + 1 < nu) load(u + 1, xb);
+                        work(u, xa);
+                        if (u + 1 < nu) {
+                            tmem_ld_wait();
+                            if (u + 2 < nu) load(u + 2, xa);
+                            work(u + 1, xb);
+                        }
+                    }
+                    if (!ok) break;
+                    tmem_st_wait();
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kBP + buf));
+                }
+                if (ok) {
+                    // the last unit's statistics have been read
+                    ok = mbar_wait_all(bar(kBOFree + t), (mine & 1) ^ 1u, cta_abort);
+                    ++mine;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float s = sum[i].x + sum[i].y;
+                        s += __shfl_xor_sync(0xffffffffu, s, 1);
+                        s += __shfl_xor_sync(0xffffffffu, s, 2);
+                        if (ql == 0) stat[8 * i] = make_float2(m[i], s);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(kBStat + t));
+                }
+            }
+            if (td.ntq == 1) {
+                // barriers are waited for by parity: warps that skip units must not be ahead of the scores or the tables
+                if (t == 0) {
+                    if (lane == 0) mbar_arrive(bar(kBOne + (ones & 1)));
+                } else {
+                    ok = ok && mbar_wait_all(bar(kBOne + (ones & 1)), (ones >> 1) & 1, cta_abort);
+                }
+                ++ones;
+            }
+            if (lane == 0) mbar_arrive(bar(kBTab + (units & 1)));
+            ++units;
+            n += td.nch * td.ntq;
+        }
+    } else if (warp < kPvWarp) {
+        // ------------------------------------------------------------------ O: normalise and store
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsOther));
+        const int wq = warp - kReadWarp0, row = 32 * wq + lane;
+        const uint32_t t_o = tmem + ((uint32_t)(32 * wq) << 16) + L::kColO;
+        unsigned done[2] = {0, 0};
+        bool ok = true;
+        while (ok && next_unit()) {
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (t >= td.ntq) break;
+                const int slot = (td.tile0 + t) * kTile + row, a = slot / RW, bb = slot % RW;
+                ok = mbar_wait_all(bar(kBStat + t), done[t] & 1, cta_abort) && mbar_wait_all(bar(kBO + t), done[t] & 1, cta_abort);
+                if (!ok) break;
+                ++done[t];
+                tc_fence_after();
+                const float2 st = reinterpret_cast<const float2*>(smem + L::kOffStat)[t * kTile + row];
+                const float inv = 1.f / st.y;
+                const bool live = a < td.eh && bb < td.ew;
+                const size_t tok = live ? (size_t)td.b * g.H * g.W + win_token(g, td.wr, td.wc, a, bb) : 0;
+                uint4* dst = reinterpret_cast<uint4*>(o + (tok * g.heads + td.head) * D);
+#pragma unroll
+                for (int col = 0; col < D; col += 32) {
+                    uint32_t r[32];
+                    tmem_ld32(t_o + D * t + col, r);
+                    tmem_ld_wait();
+                    if (col + 32 == D) {
+                        // all of it is in registers
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(kBOFree + t));
+                    }
+                    if (live) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            uint32_t w[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) w[j] = pack_elem(__uint_as_float(r[8 * i + 2 * j]) * inv, __uint_as_float(r[8 * i + 2 * j + 1]) * inv);
+                            dst[col / 8 + i] = make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                    }
+                }
+                if (live) lse[tok * g.heads + td.head] = (st.x + log2f(st.y)) * kLn2;
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsOther));
+        if (warp == kPlanWarp) {
+            // -------------------------------------------------------------- units in the order every role meets them
+            unsigned i = 0;
+            int last_head = -1;
+            bool ok = true;
+            auto put = [&](int flags, int head, int b, int wr, int wc, int eh, int ew, int tile0) {
+                ok = mbar_wait_all(bar(kBDescFree + i % kDescs), ((i / kDescs) & 1) ^ 1u, cta_abort);
+                if (!ok) return;
+                if (lane == 0) {
+                    const int ha = (!g.ph && g.sh > 0) ? g.H - g.sh - wr * g.w : (1 << 20), hb = (!g.pw && g.sw > 0) ? g.W - g.sw - wc * g.w : (1 << 20);
+                    const int nqt = (eh * RW + kTile - 1) / kTile, ku = RW == 32 ? eh : (eh + 1) / 2;
+                    if (ew < RW || (ha > 0 && ha < eh) || (hb > 0 && hb < ew) || (RW == 16 && (eh & 1))) flags |= 4;
+                    int4* dst = reinterpret_cast<int4*>(smem + L::kOffDesc + (i % kDescs) * 64);
+                    dst[0] = make_int4(head, b, wr, wc);
+                    dst[1] = make_int4(eh, ew, tile0, min(2, nqt - tile0));
+                    dst[2] = make_int4(ku, (ku + 3) / 4, ha, hb);
+                    dst[3] = make_int4(flags, 0, 0, 0);
+                    mbar_arrive(bar(kBDesc + i % kDescs));
+                }
+                __syncwarp();
+                ++i;
+            };
+            const long long lo = p.head_slow ? p.units * blockIdx.x / gridDim.x : blockIdx.x, hi = p.head_slow ? p.units * (blockIdx.x + 1) / gridDim.x : p.units;
+            const int step = p.head_slow ? 1 : gridDim.x;
+            const unsigned per_head = (unsigned)(p.units / g.heads);
+            for (long long u = lo; ok && u < hi; u += step) {
+                unsigned rest, head;
+                if (p.head_slow) { head = (unsigned)u / per_head; rest = (unsigned)u - head * per_head; }
+                else { rest = (unsigned)u / g.heads; head = (unsigned)u - rest * g.heads; }
+                const unsigned win = rest / p.pairs, pair = rest - win * p.pairs, r2 = win / g.Mw, wc = win - r2 * g.Mw, b = r2 / g.Mh, wr = r2 - b * g.Mh;
+                const int eh = min(g.w, g.H - (int)wr * g.w), ew = min(g.w, g.W - (int)wc * g.w);
+                if ((int)pair * 2 * kTileRows >= eh) continue;            // a truncated window has fewer query tiles
+                put(1 | ((int)head != last_head ? 2 : 0), head, b, wr, wc, eh, ew, pair * 2);
+                last_head = head;
+            }
+            if (ok) put(0, 0, 0, 0, 0, 1, 1, 0);
+        } else if (warp == kLoaderWarp) {
+            // -------------------------------------------------------------- copies, bias tables, mask operands
+            SlotQueue<L::kSlots> sq;
+            sq.init();
+            uint32_t use = 0;                        // bit per slot: parity of the slot's fills
+            unsigned units = 0;
+            int e_key = -1, q0 = -1, q1 = -1;        // what the mask operands are made for; Q slots of the last unit
+            bool ok = true;
+            const int part = lane % kParts, second = lane / kParts;
+            auto fill = [&](int s, const WinMaps& m, const __nv_bfloat16* src, int a0) {
+                ok = ok && mbar_wait_all(bar(kBEmpty + s), ((use >> s) & 1) ^ 1u, cta_abort);
+                if (!ok) return;
+                use ^= 1u << s;
+                const bool fix = D == 32 && p.cols.skip && td.wc == p.cols.seam;
+                if (D == 32 && fix) {
+                    // the seam column's slot n1 cannot be the start of a bulk copy of 64-byte rows (128-byte alignment)
+                    for (int i = lane; i < 2 * kG * 4; i += 32) {
+                        const int r = i >> 2, ch = i & 3, a = a0 + r;
+                        uint4 val = make_uint4(0, 0, 0, 0);
+                        if (a < td.eh && p.cols.n1 < td.ew)
+                            val = __ldg(reinterpret_cast<const uint4*>(src + ((size_t)td.b * g.H * g.W + win_token(g, td.wr, td.wc, a, p.cols.n1)) * g.ts + td.head * D) + ch);
+                        *reinterpret_cast<uint4*>(smem + s * L::kSlotB + tile_off<32>(r * RW + p.cols.n1, ch)) = val;
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                }
+                const uint32_t base = smem0 + s * L::kSlotB;
+                if (win_group_whole<RW>(p.cols, g, td.wr, td.wc, td.eh, a0, 2)) {
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB);
+                        int y0 = td.wr * g.w + a0 + g.sh;
+                        if (y0 >= g.H) y0 -= g.H;
+                        y0 += td.b * g.H;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int pt = 0; pt < kParts; ++pt)
+                                tma_load_4d(base + pt * kTile * kRowB + h * 64 * kRowB, &m.group, td.head * D + pt * L::kPartCh, 0, td.wc, y0 + h * kG, bar(kBFull + s));
+                    }
+                } else {
+                    if (lane == 0) mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB - (fix ? 2 * kG * kRowB : 0));
+                    __syncwarp();
+                    if (second < 2)
+                        load_win_rows<RW, kRowB>(m, p.cols, base + part * kTile * kRowB + second * 64 * kRowB, g, td.b, td.wr, td.wc, td.eh, a0 + second * kG,
+                                                 td.head * D + part * L::kPartCh, bar(kBFull + s));
+                }
+                __syncwarp();
+            };
+            while (ok && next_unit()) {
+                // at most two units ahead of the softmax: the barriers of even and odd units are waited for once per use
+                if (units >= 2) ok = mbar_wait_all(bar(kBTab + (units & 1)), ((units - 2) >> 1) & 1, cta_abort);
+                if (ok && (td.flags & 2)) {
+                    if (units >= 1) ok = mbar_wait_all(bar(kBTab + ((units - 1) & 1)), ((units - 1) >> 1) & 1, cta_abort);
+                    if (ok && elect_one()) {
+                        const uint32_t bytes = Tab<RW>::rows(g.w) * Tab<RW>::kRowF * 4;
+                        mbar_arrive_expect_tx(bar(kBBias), bytes);
+                        bulk_load(smem0 + L::kOffTab, p.tables + (size_t)td.head * Tab<RW>::rows(g.w) * Tab<RW>::kRowF, bytes, bar(kBBias));
+                    }
+                    __syncwarp();
+                }
+                if (ok && (td.flags & 4)) {
+                    // 32 slots to a row: rows 0-3 carry the first row label, 4-7 the second; a tile starts where its rows change
+                    const int ha = min(max(td.ha, 0), td.eh), hb = min(max(td.hb, 0), td.ew);
+                    const int key = RW == 32 ? td.ew | hb << 6 : td.ew | hb << 6 | td.eh << 12 | ha << 18;
+                    if (key != e_key) {
+                        e_key = key;
+                        // the last unit's scores are done when its Q slots are free
+                        if (q0 >= 0) ok = ok && mbar_wait_all(bar(kBEmpty + q0), ((use >> q0) & 1) ^ 1u, cta_abort);
+                        if (q1 >= 0) ok = ok && mbar_wait_all(bar(kBEmpty + q1), ((use >> q1) & 1) ^ 1u, cta_abort);
+                        if (ok) {
+                            for (int s = lane; s < 256; s += 32) {
+                                const int a = s / RW, b = s % RW;
+                                const bool valid = b < td.ew && (RW == 32 || a < td.eh);
+                                const int label = 2 * (RW == 32 ? a >= 4 : a >= ha) + (b >= hb);
+                                uint32_t eq[2] = {0, 0}, ek[2] = {kMaskK | kMaskK << 16, kMaskK | kMaskK << 16};
+                                if (valid) {
+                                    const uint32_t half = (label & 1) ? 0xffff0000u : 0xffffu;
+#pragma unroll
+                                    for (int i = 0; i < 2; ++i)
+                                        if (i == label >> 1) { eq[i] = (kMaskQ | kMaskQ << 16) & half; ek[i] &= ~half; }
+                                }
+                                unsigned char* e = smem + L::kOffE;
+                                *reinterpret_cast<uint4*>(e + tile_off<32>(s, 0)) = make_uint4(eq[0], eq[1], 0, 0);
+                                *reinterpret_cast<uint4*>(e + tile_off<32>(s, 1)) = make_uint4(0, 0, 0, 0);
+                                *reinterpret_cast<uint4*>(e + tile_off<32>(s, 2)) = make_uint4(ek[0], ek[1], 0, 0);
+                                *reinterpret_cast<uint4*>(e + tile_off<32>(s, 3)) = make_uint4(0, 0, 0, 0);
+                            }
+                            fence_proxy_async();
+                            __syncwarp();
+                        }
+                    }
+                }
+                q0 = sq.pop();
+                q1 = sq.pop();
+                fill(q0, mq, p.q, td.tile0 * kTileRows);
+                for (int c = 0; ok && c < td.nch; ++c) {
+                    fill(sq.take(), mk, p.k, c * kTileRows);
+                    if (c == 0 && td.ntq == 2) fill(q1, mq, p.q, (td.tile0 + 1) * kTileRows);
+                    fill(sq.take(), mv, p.v, c * kTileRows);
+                }
+                sq.end_unit(q0, q1);
+                if (td.ntq < 2) q1 = -1;
+                ++units;
+            }
+        } else if (warp == kScoreWarp) {
+            // -------------------------------------------------------------- S = Q K^T
+            constexpr uint32_t kIdS = make_idesc_elem(128, 0, 0, 0);
+            const uint64_t d_k = D == 32 ? make_sdesc_sw64(smem0, 512) : make_sdesc_sw128(smem0);
+            const uint64_t d_e = make_sdesc_sw64(smem0 + L::kOffE, 512);
+            const uint32_t hi = sdesc_hi(d_k), lo = sdesc_lo(d_k), hi_e = sdesc_hi(d_e), lo_e = sdesc_lo(d_e);
+            constexpr int kPerPart = L::kPartCh / 16;
+            SlotQueue<L::kSlots> sq;
+            sq.init();
+            uint32_t full_use = 0;
+            unsigned idx = 0;
+            bool ok = true;
+            auto wait_full = [&](int s) {
+                ok = ok && mbar_wait_all(bar(kBFull + s), (full_use >> s) & 1, cta_abort);
+                full_use ^= 1u << s;
+            };
+            // where the rows from window row a0 on start among the mask operands (16-byte units)
+            auto mask_rows = [&](int a0) {
+                return RW == 16 ? (uint32_t)a0 * (RW * 64 / 16) : (uint32_t)min(max(4 - (td.ha - a0), 0), 4) * (RW * 64 / 16);
+            };
+            while (ok && next_unit()) {
+                const int s_q[2] = {sq.pop(), sq.pop()};
+                for (int c = 0; ok && c < td.nch; ++c) {
+                    const int sk = sq.take(), sv = sq.take();
+                    full_use ^= 1u << sv;
+                    const uint32_t id = kIdS + ((uint32_t)(4 * min(4, td.ku - 4 * c)) << 17);
+                    if (c == 0) wait_full(s_q[0]);
+                    wait_full(sk);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        if (t >= td.ntq) break;
+                        const unsigned buf = idx % NB;
+                        if (t == 1 && c == 0) wait_full(s_q[1]);
+                        ok = ok && mbar_wait_all(bar(kBFree + buf), ((idx / NB) & 1) ^ 1u, cta_abort);
+                        if (!ok) break;
+                        ++idx;
+                        tc_fence_after();
+                        const uint32_t a = lo + s_q[t] * (L::kSlotB >> 4), b = lo + sk * (L::kSlotB >> 4), dst = tmem + 128u * buf;
+                        const uint32_t ea = lo_e + mask_rows((td.tile0 + t) * kTileRows), eb = lo_e + mask_rows(c * kTileRows) + 2;
+                        if (elect_one()) {
+#pragma unroll
+                            for (int ks = 0; ks < D / 16; ++ks) {
+                                const uint32_t off = (ks / kPerPart) * (kTile * kRowB / 16) + (ks % kPerPart) * 2;
+                                if (ks == 0) mma_ss_h<false>(dst, a + off, b + off, hi, id);
+                                else mma_ss_h<true>(dst, a + off, b + off, hi, id);
+                            }
+                            if (td.flags & 4) mma_ss_h<true>(dst, ea, eb, hi_e, id);
+                            mma_commit(bar(kBS + buf));
+                            if (c == td.nch - 1) mma_commit(bar(kBEmpty + s_q[t]));
+                            if (t == td.ntq - 1) mma_commit(bar(kBEmpty + sk));
+                        }
+                        __syncwarp();
+                    }
+                }
+                sq.end_unit(s_q[0], s_q[1]);
+            }
+        } else if (warp == kPvWarp) {
+            // -------------------------------------------------------------- O += P V
+            constexpr uint32_t kIdO = make_idesc_elem(128, D, 0, 1);
+            const uint64_t d_v = D == 32 ? make_sdesc_sw64_mn(smem0, 512, 512) : make_sdesc_sw128(smem0, kTile * kRowB);
+            const uint32_t hi = sdesc_hi(d_v), lo = sdesc_lo(d_v);
+            constexpr uint32_t kStep = 16 * kRowB / 16;
+            SlotQueue<L::kSlots> sq;
+            sq.init();
+            uint32_t full_use = 0;
+            unsigned idx = 0, opened[2] = {0, 0};
+            bool ok = true;
+            while (ok && next_unit()) {
+                const int s_q[2] = {sq.pop(), sq.pop()};
+                for (int t = 0; t < td.ntq; ++t) full_use ^= 1u << s_q[t];
+                for (int c = 0; ok && c < td.nch; ++c) {
+                    const int sk = sq.take(), sv = sq.take();
+                    full_use ^= 1u << sk;
+                    ok = mbar_wait_all(bar(kBFull + sv), (full_use >> sv) & 1, cta_abort);
+                    full_use ^= 1u << sv;
+                    const int steps = 2 * min(4, td.ku - 4 * c);
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        if (t >= td.ntq) break;
+                        const unsigned buf = idx % NB;
+                        ok = ok && mbar_wait_all(bar(kBP + buf), (idx / NB) & 1, cta_abort);
+                        if (c == 0) {
+                            ok = ok && mbar_wait_all(bar(kBOFree + t), (opened[t] & 1) ^ 1u, cta_abort);
+                            ++opened[t];
+                        }
+                        if (!ok) break;
+                        ++idx;
+                        tc_fence_after();
+                        const uint32_t dst = tmem + L::kColO + D * t, a = tmem + 128u * buf, b = lo + sv * (L::kSlotB >> 4);
+                        if (elect_one()) {
+                            if (c == 0) mma_ts_h<false>(dst, a, b, hi, kIdO);
+                            else mma_ts_h<true>(dst, a, b, hi, kIdO);
+                            mma_ts_h<true>(dst, a + 8, b + kStep, hi, kIdO);
+#pragma unroll
+                            for (int ks = 2; ks < 8; ++ks)
+                                if (ks < steps) mma_ts_h<true>(dst, a + 8 * ks, b + ks * kStep, hi, kIdO);
+                            mma_commit(bar(kBFree + buf));
+                            mma_commit(bar(kBPv + t));
+                            if (c == td.nch - 1) mma_commit(bar(kBO + t));
+                            if (t == td.ntq - 1) mma_commit(bar(kBEmpty + sv));
+                        }
+                        __syncwarp();
+                    }
+                }
+                sq.end_unit(s_q[0], s_q[1]);
+            }
+        }
+    }
+
+    // teardown: every role ends up here, also after an expired wait
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == kPvWarp) tmem_dealloc(tmem, 512);
+    if (tid == 0 && *cta_abort) atomicExch(&g_fwd_win_timeout, 1);
+}
+
+// The bias tables of all heads as the softmax threads read them: bias log2 e by row and column difference, two copies.
+template <int RW>
+__global__ void swin_fwd_win_prep_kernel(const Geo g, const float* __restrict__ bias, float* __restrict__ tables) {
+    const int per_head = Tab<RW>::rows(g.w) * Tab<RW>::kRowF, total = per_head * g.heads, nw = 2 * g.w - 1;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+        const int head = i / per_head, e = i - head * per_head, row = e / Tab<RW>::kRowF, f = e - row * Tab<RW>::kRowF;
+        const int c = f / Tab<RW>::kCopyF, da = row - Tab<RW>::kFront - (g.w - 1), db = f - c * Tab<RW>::kCopyF + c - (RW - 1);    // key minus query
+        const bool in = da > -g.w && da < g.w && db > -g.w && db < g.w;
+        tables[i] = in ? bias[((size_t)(g.w - 1 - da) * nw + (g.w - 1 - db)) * g.heads + head] * kLog2e : 0.f;
+    }
+}
+
+}  // namespace
+
+cudaError_t read_fwd_win_status(int* timed_out) {
+    int zero = 0;
+    cudaError_t e = cudaMemcpyFromSymbol(timed_out, g_fwd_win_timeout, sizeof(int));
+    if (e != cudaSuccess) return e;
+    if (*timed_out) e = cudaMemcpyToSymbol(g_fwd_win_timeout, &zero, sizeof(int));
+    return e;
+}
+
+#ifndef TERRA_ELEM_F16
+bool fwd_win_supported(const Geo& g) {
+    return (g.d == 32 || g.d == 64 || g.d == 128) && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
+           (long long)g.B * g.Mh * g.Mw * g.heads * 4 < 0x7fffffffLL;
+}
+
+size_t fwd_win_workspace_bytes(const Geo& g) {
+    return sizeof(float) * (size_t)g.heads * (win_row_slots(g) == 16 ? Tab<16>::rows(g.w) * Tab<16>::kRowF : Tab<32>::rows(g.w) * Tab<32>::kRowF);
+}
+#endif
+
+namespace {
+template <int D, int RW>
+cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
+                       int sm_count, cudaStream_t stream) {
+    using L = Lay<D, RW>;
+    Params p;
+    p.g = g;
+    WinMaps mq, mk, mv;
+    if (!make_win_cols(&p.cols, g) || !make_win_maps(&mq, p.cols, g, q, g.ts) || !make_win_maps(&mk, p.cols, g, k, g.ts) || !make_win_maps(&mv, p.cols, g, v, g.ts))
+        return cudaErrorNotSupported;
+    p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v;
+    p.tables = (const float*)workspace;
+    const int tiles = ((g.w < g.H ? g.w : g.H) * RW + kTile - 1) / kTile;
+    p.pairs = (tiles + 1) / 2;
+    p.units = (long long)g.B * g.Mh * g.Mw * g.heads * p.pairs;
+    // A CTA keeps to one head where that leaves no more than 1 SM in 20 idle: neighbouring CTAs then read the heads of the same
+    // tokens at the same time.  Otherwise each CTA takes a run of the units in head-major order.
+    const int bound = sm_count / g.heads * g.heads;
+    p.head_slow = bound * 20 < sm_count * 19 && p.units > bound;
+    const long long ctas = p.head_slow ? sm_count : bound > 0 ? bound : sm_count;
+    const int total = g.heads * Tab<RW>::rows(g.w) * Tab<RW>::kRowF;
+    prof_begin("swin_fwd_win_prep_kernel", stream);
+    swin_fwd_win_prep_kernel<RW><<<total / 512 + 1 < 592 ? total / 512 + 1 : 592, 256, 0, stream>>>(g, bias, (float*)workspace);
+    count_launch(stream);
+    cudaError_t e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW>, L::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    prof_begin("swin_fwd_win_kernel", stream);
+    swin_fwd_win_kernel<D, RW><<<(unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream>>>(p, (__nv_bfloat16*)o, lse, mq, mk, mv);
+    count_launch(stream);
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_fwd_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
+                           int sm_count, cudaStream_t stream) {
+    const bool wide = win_row_slots(g) == 32;
+    switch (g.d) {
+        case 32: return (wide ? launch_win<32, 32> : launch_win<32, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+        case 64: return (wide ? launch_win<64, 32> : launch_win<64, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+        default: return (wide ? launch_win<128, 32> : launch_win<128, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+    }
+}
+
+}  // namespace terra

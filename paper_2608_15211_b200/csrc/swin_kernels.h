@@ -72,6 +72,15 @@ bool tma_row_shape(const Geo& g);
 bool make_row_map(void* cu_tensor_map, const Geo& g, const void* base, int token_stride, int box_tokens);
 
 // tcgen05 forward path for head dim 64 and windows of up to 1024 tokens (keys streamed in chunks, two passes)
+// windows of side 9 .. 32 on any grid (attn_fwd_win.cu)
+bool fwd_win_supported(const Geo& g);
+size_t fwd_win_workspace_bytes(const Geo& g);
+cudaError_t launch_fwd_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
+                           int sm_count, cudaStream_t stream);
+cudaError_t launch_fwd_win_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
+                               int sm_count, cudaStream_t stream);
+cudaError_t read_fwd_win_status(int* timed_out);
+cudaError_t read_fwd_win_status_f16(int* timed_out);
 bool fwd_tc64_supported(const Geo& g);
 size_t fwd_tc64_workspace_bytes(const Geo& g);
 cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
