@@ -60,15 +60,15 @@ struct Tab {
     static __host__ __device__ constexpr int rows(int w) { return 2 * w + 2 * kFront; }
 };
 
-enum { kBFull = 0, kBEmpty = 16, kBS = 32, kBP = 35, kBFree = 38, kBPv = 41, kBO = 43, kBOFree = 45, kBStat = 47, kBTab = 49, kBBias = 51, kBOne = 52,
-       kBDesc = 54, kBDescFree = kBDesc + kDescs, kBCount = kBDescFree + kDescs };
+enum { kBFull = 0, kBEmpty = 16, kBS = 32, kBP = 38, kBFree = 44, kBO = 50, kBOFree = 52, kBStat = 54, kBTab = 56, kBBias = 58,
+       kBOne = 59, kBDesc = 61, kBDescFree = kBDesc + kDescs, kBCount = kBDescFree + kDescs };
 
 template <int D, int RW>
 struct Lay {
     static constexpr int kParts = D == 128 ? 2 : 1, kRowB = D >= 64 ? 128 : 64, kPartCh = kRowB / 2;
     static constexpr int kSlotB = kTile * D * 2;                                    // a Q, K or V tile
     static constexpr int kSlots = D == 128 ? (RW == 16 ? 6 : 5) : D == 64 ? 10 : 14;
-    static constexpr int kBufs = D == 128 ? 2 : 3, kColO = 128 * kBufs;
+    static constexpr int kBufs = D == 128 ? 4 : 6, kColO = 64 * kBufs;
     static constexpr int kOffE = kSlots * kSlotB;                                   // E operands, 64 bytes a slot: E_q, then E_k
     static constexpr int kOffTab = kOffE + 256 * 64;
     static constexpr int kOffStat = kOffTab + Tab<RW>::rows(RW) * Tab<RW>::kRowF * 4;          // per row of both tiles: m, row sum
@@ -119,7 +119,7 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
 // for 32 scores.  (A thread per row read each score's own entry: the shared-memory pipe then bound the kernel, 1300 to 2500
 // of 4100 to 6800 cycles per 128 x 128 scores and tile.)  `bias`: shared address of the entry of rows g, keys 2 t.
 template <int RW>
-__device__ __forceinline__ void add_bias(uint32_t (&x)[2][16], uint32_t bias, float scale, float (&mx)[4]) {
+__device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, uint32_t bias, float scale, float (&mx)[4]) {
     constexpr int kRowB = Tab<RW>::kRowF * 4;
     float2 bv[9];
 #pragma unroll
@@ -129,7 +129,7 @@ __device__ __forceinline__ void add_bias(uint32_t (&x)[2][16], uint32_t bias, fl
     for (int m = 0; m < 4; ++m)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            uint32_t* v = &x[m >> 1][4 * k + 2 * (m & 1)];
+            uint32_t* v = &x[m >> 1][16 * u + 4 * k + 2 * (m & 1)];
             const float2 b = bv[RW == 32 ? k - m + 3 : 3 * ((k >> 1) - (m >> 1) + 1) + (k & 1) - (m & 1) + 1];
             float x0, x1;
             fma2(x0, x1, __uint_as_float(v[0]), __uint_as_float(v[1]), scale, b.x, b.y);
@@ -159,12 +159,11 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             mbar_init(bar(kBEmpty + s), 1);
         }
         for (int b = 0; b < NB; ++b) {
-            mbar_init(bar(kBS + b), 1);            // scores of a chunk are in buffer b
+            mbar_init(bar(kBS + b), 1);            // scores of a half chunk are in buffer b
             mbar_init(bar(kBP + b), 4);            // ... and P has taken their place
             mbar_init(bar(kBFree + b), 1);         // ... and been read by the product
         }
         for (int t = 0; t < 2; ++t) {
-            mbar_init(bar(kBPv + t), 1);           // a chunk's product of tile t is done
             mbar_init(bar(kBO + t), 1);            // ... the unit's last one
             mbar_init(bar(kBOFree + t), 4);        // O and the statistics of tile t have been read
             mbar_init(bar(kBStat + t), 4);         // the rows' m and sums are in shared memory
@@ -214,7 +213,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
         const int i0 = RW - 1 + 2 * ql - gl;                 // table column of row g, key 2 t
         const uint32_t tab0 = smem0 + L::kOffTab + 4u * ((i0 & 1) * Tab<RW>::kCopyF + (i0 & ~1));
         float2* stat = reinterpret_cast<float2*>(smem + L::kOffStat) + t * kTile + 32 * wq + gl;
-        unsigned n = 0, pv = 0, units = 0, mine = 0, heads = 0, ones = 0;   // chunks of the CTA, of this tile; units, those with this tile; tables; 1-tile units
+        unsigned n = 0, units = 0, mine = 0, heads = 0, ones = 0;   // half chunks of the CTA; units, those with this tile; tables; 1-tile units
         bool ok = true;
         while (ok && next_unit()) {
             if (td.flags & 2) ok = mbar_wait_all(bar(kBBias), heads++ & 1, cta_abort);
@@ -223,101 +222,76 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 uint32_t bias = tab0 + 4u * (g.w - 1 - aq + Tab<RW>::kFront) * Tab<RW>::kRowF;
                 float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
                 float2 sum[4] = {};
-                for (int c = 0; c < td.nch; ++c, ++pv) {
-                    const unsigned idx = n + c * td.ntq + t, buf = idx % NB;
-                    const uint32_t t_s = tq + 128u * buf;
-                    const int nu = min(4, td.ku - 4 * c);
+                for (int j = 0; 2 * j < td.ku; ++j) {
+                    const unsigned idx = n + j * td.ntq + t, buf = idx % NB;
+                    const uint32_t t_s = tq + 64u * buf;
                     ok = mbar_wait_all(bar(kBS + buf), (idx / NB) & 1, cta_abort);
                     if (!ok) break;
                     tc_fence_after();
-                    auto load = [&](int u, uint32_t (&x)[2][16]) {
-                        tmem_ld_frag32(t_s + 32 * u, x[0]);
-                        tmem_ld_frag32(t_s + (16u << 16) + 32 * u, x[1]);
-                    };
-                    auto work = [&](int u, uint32_t (&x)[2][16]) {
-                        float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                        add_bias<RW>(x, bias, scale, top);
+                    uint32_t x[2][32];                       // [rows g + 16 h, + 8]
+                    tmem_ld_frag64(t_s, x[0]);
+                    tmem_ld_frag64(t_s + (16u << 16), x[1]);
+                    tmem_ld_wait();
+                    float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                    add_bias<RW>(x, 0, bias, scale, top);
+                    bias += 4u * (32 / RW) * Tab<RW>::kRowF;
+                    if (2 * j + 1 < td.ku) {
+                        add_bias<RW>(x, 1, bias, scale, top);
                         bias += 4u * (32 / RW) * Tab<RW>::kRowF;
-                        if (__any_sync(0xffffffffu, top[0] - m[0] > 8.f || top[1] - m[1] > 8.f || top[2] - m[2] > 8.f || top[3] - m[3] > 8.f)) {
-                            // raise the reference: the sums, the chunk's P so far and, once its products are done, O are scaled down
-                            float f[4];
+                    } else {
+                        // 32 slots that do not exist
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                top[i] = fmaxf(top[i], __shfl_xor_sync(0xffffffffu, top[i], 1));
-                                top[i] = fmaxf(top[i], __shfl_xor_sync(0xffffffffu, top[i], 2));
-                                const float up = top[i] - m[i] > 8.f ? top[i] : m[i];
-                                f[i] = fast_exp2(m[i] - up);
-                                m[i] = up;
-                                sum[i].x *= f[i];
-                                sum[i].y *= f[i];
-                            }
-                            if (u > 0) {
-                                tmem_st_wait();
-#pragma unroll 1
-                                for (int col = 0; col < 16 * u; col += 16)
+                        for (int i = 16; i < 32; ++i) x[0][i] = x[1][i] = 0xff800000u;
+                    }
+                    if (__any_sync(0xffffffffu, top[0] - m[0] > 8.f || top[1] - m[1] > 8.f || top[2] - m[2] > 8.f || top[3] - m[3] > 8.f)) {
+                        // raise the reference; O and the sums so far are scaled down, once the products so far are done
+                        float f[4];
 #pragma unroll
-                                    for (int h = 0; h < 2; ++h) {
-                                        uint32_t r[8];
-                                        tmem_ld_frag_packed16(t_s + ((16u * h) << 16) + col, r);
-                                        tmem_ld_wait();
-#pragma unroll
-                                        for (int i = 0; i < 8; ++i) {
-                                            const float2 v = elem2_to_float2(r[i]);
-                                            r[i] = pack_elem(v.x * f[2 * h + (i & 1)], v.y * f[2 * h + (i & 1)]);
-                                        }
-                                        tmem_st_frag_packed16(t_s + ((16u * h) << 16) + col, r);
-                                    }
-                            }
-                            if (c > 0) {
-                                ok = mbar_wait_all(bar(kBPv + t), (pv - 1) & 1, cta_abort);
-                                if (ok) tc_fence_after();
-#pragma unroll 1
-                                for (int col = 0; ok && col < D; col += 16)
-#pragma unroll
-                                    for (int h = 0; h < 2; ++h) {
-                                        uint32_t r[8];
-                                        tmem_ld_frag16(t_o + ((16u * h) << 16) + col, r);
-                                        tmem_ld_wait();
-#pragma unroll
-                                        for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f[2 * h + ((i >> 1) & 1)]);
-                                        tmem_st_frag16(t_o + ((16u * h) << 16) + col, r);
-                                    }
-                            }
+                        for (int i = 0; i < 4; ++i) {
+                            top[i] = fmaxf(top[i], __shfl_xor_sync(0xffffffffu, top[i], 1));
+                            top[i] = fmaxf(top[i], __shfl_xor_sync(0xffffffffu, top[i], 2));
+                            const float up = top[i] - m[i] > 8.f ? top[i] : m[i];
+                            f[i] = fast_exp2(m[i] - up);
+                            m[i] = up;
+                            sum[i].x *= f[i];
+                            sum[i].y *= f[i];
                         }
+                        if (j > 0) {
+                            // (the buffer of the last product cannot be freed again before this half chunk's product)
+                            const unsigned last = idx - td.ntq;
+                            ok = mbar_wait_all(bar(kBFree + last % NB), (last / NB) & 1, cta_abort);
+                            if (!ok) break;
+                            tc_fence_after();
+#pragma unroll 1
+                            for (int col = 0; col < D; col += 16)
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            uint32_t pk[8];
+                                for (int h = 0; h < 2; ++h) {
+                                    uint32_t r[8];
+                                    tmem_ld_frag16(t_o + ((16u * h) << 16) + col, r);
+                                    tmem_ld_wait();
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-#pragma unroll
-                                for (int mi = 0; mi < 2; ++mi) {
-                                    const int i = 2 * h + mi;
-                                    float x0, x1;
-                                    add2(x0, x1, __uint_as_float(x[h][4 * k + 2 * mi]), __uint_as_float(x[h][4 * k + 2 * mi + 1]), -m[i]);
-                                    x0 = fast_exp2(x0);
-                                    x1 = fast_exp2(x1);
-                                    add2vv(sum[i].x, sum[i].y, sum[i].x, sum[i].y, x0, x1);
-                                    pk[2 * k + mi] = pack_elem(x0, x1);
+                                    for (int i = 0; i < 8; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * f[2 * h + ((i >> 1) & 1)]);
+                                    tmem_st_frag16(t_o + ((16u * h) << 16) + col, r);
                                 }
-                            tmem_st_frag_packed16(t_s + ((16u * h) << 16) + 16 * u, pk);
-                        }
-                    };
-                    // the next unit's scores come while this one's are worked on.  A loop of two units: the code has to stay
-                    // small, a chunk in one piece ran at a fetch-bound 12 cycles an instruction
-                    uint32_t xa[2][16], xb[2][16];
-                    load(0, xa);
-#pragma unroll 1
-                    for (int u = 0; u < nu; u += 2) {
-                        tmem_ld_wait();
-                        if (u + 1 < nu) load(u + 1, xb);
-                        work(u, xa);
-                        if (u + 1 < nu) {
-                            tmem_ld_wait();
-                            if (u + 2 < nu) load(u + 2, xa);
-                            work(u + 1, xb);
                         }
                     }
-                    if (!ok) break;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        uint32_t pk[16];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+#pragma unroll
+                            for (int mi = 0; mi < 2; ++mi) {
+                                const int i = 2 * h + mi;
+                                float x0, x1;
+                                add2(x0, x1, __uint_as_float(x[h][4 * k + 2 * mi]), __uint_as_float(x[h][4 * k + 2 * mi + 1]), -m[i]);
+                                x0 = fast_exp2(x0);
+                                x1 = fast_exp2(x1);
+                                add2vv(sum[i].x, sum[i].y, sum[i].x, sum[i].y, x0, x1);
+                                pk[2 * k + mi] = pack_elem(x0, x1);
+                            }
+                        tmem_st_frag_packed32(t_s + ((16u * h) << 16), pk);
+                    }
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
@@ -349,7 +323,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             }
             if (lane == 0) mbar_arrive(bar(kBTab + (units & 1)));
             ++units;
-            n += td.nch * td.ntq;
+            n += ((td.ku + 1) >> 1) * td.ntq;
         }
     } else if (warp < kPvWarp) {
         // ------------------------------------------------------------------ O: normalise and store
@@ -563,33 +537,36 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 for (int c = 0; ok && c < td.nch; ++c) {
                     const int sk = sq.take(), sv = sq.take();
                     full_use ^= 1u << sv;
-                    const uint32_t id = kIdS + ((uint32_t)(4 * min(4, td.ku - 4 * c)) << 17);
                     if (c == 0) wait_full(s_q[0]);
                     wait_full(sk);
+                    for (int hf = 0; hf < 2 && 4 * c + 2 * hf < td.ku; ++hf) {
+                        const int left = td.ku - (4 * c + 2 * hf);
+                        const uint32_t id = kIdS + ((left > 1 ? 8u : 4u) << 17);
 #pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        if (t >= td.ntq) break;
-                        const unsigned buf = idx % NB;
-                        if (t == 1 && c == 0) wait_full(s_q[1]);
-                        ok = ok && mbar_wait_all(bar(kBFree + buf), ((idx / NB) & 1) ^ 1u, cta_abort);
-                        if (!ok) break;
-                        ++idx;
-                        tc_fence_after();
-                        const uint32_t a = lo + s_q[t] * (L::kSlotB >> 4), b = lo + sk * (L::kSlotB >> 4), dst = tmem + 128u * buf;
-                        const uint32_t ea = lo_e + mask_rows((td.tile0 + t) * kTileRows), eb = lo_e + mask_rows(c * kTileRows) + 2;
-                        if (elect_one()) {
+                        for (int t = 0; t < 2; ++t) {
+                            if (t >= td.ntq) break;
+                            const unsigned buf = idx % NB;
+                            if (t == 1 && c == 0 && hf == 0) wait_full(s_q[1]);
+                            ok = ok && mbar_wait_all(bar(kBFree + buf), ((idx / NB) & 1) ^ 1u, cta_abort);
+                            if (!ok) break;
+                            ++idx;
+                            tc_fence_after();
+                            const uint32_t a = lo + s_q[t] * (L::kSlotB >> 4), b = lo + sk * (L::kSlotB >> 4) + hf * (64 * kRowB / 16), dst = tmem + 64u * buf;
+                            const uint32_t ea = lo_e + mask_rows((td.tile0 + t) * kTileRows), eb = lo_e + mask_rows((2 * c + hf) * kG) + 2;
+                            if (elect_one()) {
 #pragma unroll
-                            for (int ks = 0; ks < D / 16; ++ks) {
-                                const uint32_t off = (ks / kPerPart) * (kTile * kRowB / 16) + (ks % kPerPart) * 2;
-                                if (ks == 0) mma_ss_h<false>(dst, a + off, b + off, hi, id);
-                                else mma_ss_h<true>(dst, a + off, b + off, hi, id);
+                                for (int ks = 0; ks < D / 16; ++ks) {
+                                    const uint32_t oa = (ks / kPerPart) * (kTile * kRowB / 16) + (ks % kPerPart) * 2;
+                                    if (ks == 0) mma_ss_h<false>(dst, a + oa, b + oa, hi, id);
+                                    else mma_ss_h<true>(dst, a + oa, b + oa, hi, id);
+                                }
+                                if (td.flags & 4) mma_ss_h<true>(dst, ea, eb, hi_e, id);
+                                mma_commit(bar(kBS + buf));
+                                if (c == td.nch - 1 && left <= 2) mma_commit(bar(kBEmpty + s_q[t]));
+                                if (t == td.ntq - 1 && (hf == 1 || left <= 2)) mma_commit(bar(kBEmpty + sk));
                             }
-                            if (td.flags & 4) mma_ss_h<true>(dst, ea, eb, hi_e, id);
-                            mma_commit(bar(kBS + buf));
-                            if (c == td.nch - 1) mma_commit(bar(kBEmpty + s_q[t]));
-                            if (t == td.ntq - 1) mma_commit(bar(kBEmpty + sk));
+                            __syncwarp();
                         }
-                        __syncwarp();
                     }
                 }
                 sq.end_unit(s_q[0], s_q[1]);
@@ -613,33 +590,36 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     full_use ^= 1u << sk;
                     ok = mbar_wait_all(bar(kBFull + sv), (full_use >> sv) & 1, cta_abort);
                     full_use ^= 1u << sv;
-                    const int steps = 2 * min(4, td.ku - 4 * c);
+                    for (int hf = 0; hf < 2 && 4 * c + 2 * hf < td.ku; ++hf) {
+                        const int left = td.ku - (4 * c + 2 * hf);
 #pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        if (t >= td.ntq) break;
-                        const unsigned buf = idx % NB;
-                        ok = ok && mbar_wait_all(bar(kBP + buf), (idx / NB) & 1, cta_abort);
-                        if (c == 0) {
-                            ok = ok && mbar_wait_all(bar(kBOFree + t), (opened[t] & 1) ^ 1u, cta_abort);
-                            ++opened[t];
+                        for (int t = 0; t < 2; ++t) {
+                            if (t >= td.ntq) break;
+                            const unsigned buf = idx % NB;
+                            const bool first = c == 0 && hf == 0;
+                            ok = ok && mbar_wait_all(bar(kBP + buf), (idx / NB) & 1, cta_abort);
+                            if (first) {
+                                ok = ok && mbar_wait_all(bar(kBOFree + t), (opened[t] & 1) ^ 1u, cta_abort);
+                                ++opened[t];
+                            }
+                            if (!ok) break;
+                            ++idx;
+                            tc_fence_after();
+                            const uint32_t dst = tmem + L::kColO + D * t, a = tmem + 64u * buf, b = lo + sv * (L::kSlotB >> 4) + hf * 4 * kStep;
+                            if (elect_one()) {
+                                if (first) mma_ts_h<false>(dst, a, b, hi, kIdO);
+                                else mma_ts_h<true>(dst, a, b, hi, kIdO);
+                                mma_ts_h<true>(dst, a + 8, b + kStep, hi, kIdO);
+                                if (left > 1) {
+                                    mma_ts_h<true>(dst, a + 16, b + 2 * kStep, hi, kIdO);
+                                    mma_ts_h<true>(dst, a + 24, b + 3 * kStep, hi, kIdO);
+                                }
+                                mma_commit(bar(kBFree + buf));
+                                if (c == td.nch - 1 && left <= 2) mma_commit(bar(kBO + t));
+                                if (t == td.ntq - 1 && (hf == 1 || left <= 2)) mma_commit(bar(kBEmpty + sv));
+                            }
+                            __syncwarp();
                         }
-                        if (!ok) break;
-                        ++idx;
-                        tc_fence_after();
-                        const uint32_t dst = tmem + L::kColO + D * t, a = tmem + 128u * buf, b = lo + sv * (L::kSlotB >> 4);
-                        if (elect_one()) {
-                            if (c == 0) mma_ts_h<false>(dst, a, b, hi, kIdO);
-                            else mma_ts_h<true>(dst, a, b, hi, kIdO);
-                            mma_ts_h<true>(dst, a + 8, b + kStep, hi, kIdO);
-#pragma unroll
-                            for (int ks = 2; ks < 8; ++ks)
-                                if (ks < steps) mma_ts_h<true>(dst, a + 8 * ks, b + ks * kStep, hi, kIdO);
-                            mma_commit(bar(kBFree + buf));
-                            mma_commit(bar(kBPv + t));
-                            if (c == td.nch - 1) mma_commit(bar(kBO + t));
-                            if (t == td.ntq - 1) mma_commit(bar(kBEmpty + sv));
-                        }
-                        __syncwarp();
                     }
                 }
                 sq.end_unit(s_q[0], s_q[1]);
@@ -679,7 +659,8 @@ cudaError_t read_fwd_win_status(int* timed_out) {
 
 #ifndef TERRA_ELEM_F16
 bool fwd_win_supported(const Geo& g) {
-    return (g.d == 32 || g.d == 64 || g.d == 128) && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
+    // (head dim 32 with sides up to 16 has a kernel of its own, 0.77 against 1.16 ms on the 510 x 1080 grid with 12 heads)
+    return (g.d == 64 || g.d == 128 || (g.d == 32 && g.w > 16)) && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 4 < 0x7fffffffLL;
 }
 
@@ -725,7 +706,7 @@ cudaError_t launch_fwd_win(const Geo& g, const void* q, const void* k, const voi
                            int sm_count, cudaStream_t stream) {
     const bool wide = win_row_slots(g) == 32;
     switch (g.d) {
-        case 32: return (wide ? launch_win<32, 32> : launch_win<32, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+        case 32: return launch_win<32, 32>(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
         case 64: return (wide ? launch_win<64, 32> : launch_win<64, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
         default: return (wide ? launch_win<128, 32> : launch_win<128, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
     }
