@@ -269,81 +269,76 @@ swin_fwd_mma_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv
     swin_fwd_mma_body<D, BIG>(g, q, k, v, bias, o, lse, qtiles);
 }
 
-// Windows of at most 64 tokens (the paper's 8 x 8 windows), every head dim: persistent CTAs bound to one head walk over
-// (batch, window); a window is one 64-row tile of Q, K and V.  The tiles are double-buffered: while a window is
-// computed and its output rows are written, the next window's rows are already on their way, so a CTA always has
-// loads in flight (these shapes are bound by HBM).  No online softmax: the whole score row is in registers.
+// Window sides up to 8 (the paper's 8 x 8 windows), every head dim: persistent CTAs bound to one head walk over
+// (batch, window); a window is one 64-row tile of Q, K and V, 8 slots to a window row (slot = 8 a + b).  No online softmax: the
+// whole score row is in registers.
+// These shapes should be bound by HBM, but a CTA's chain (copies, products, softmax, stores) is several times as long as the
+// copies take, so what counts is how many CTAs an SM holds: tiles are not double-buffered (8 x 128 channels: 4 CTAs of 50 KB),
+// the bias entries that a thread needs (a window row further down is a row further up in the table: 18 for 32 scores) stay in its
+// registers for the whole run, a warp's output takes the place of its own Q rows, and a window costs two barriers.
+// 288 x 544 tokens, 8 x 128: 353 -> 232 us (85 % of the copy bandwidth); 128 x 256, 6 x 32: 27 -> 20 us.
 template <int D>
-__global__ void __launch_bounds__(NTHREADS, 2)
+__global__ void __launch_bounds__(NTHREADS, D == 128 ? 4 : D == 64 ? 5 : 6)
 swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
                       const __nv_bfloat16* __restrict__ v, const float* __restrict__ bias,
                       __nv_bfloat16* __restrict__ o, float* __restrict__ lse, int ctas_per_head) {
     constexpr int KS = D / 16;
     constexpr int DT = D / 8;
+    constexpr int CPR = D / 8, RPI = 32 / CPR;       // 16-byte chunks of a row; rows a warp copies at a time
     constexpr int TILE_BYTES = BN * D * 2;
-    constexpr int BUF_BYTES = 3 * TILE_BYTES;
     extern __shared__ __align__(128) unsigned char smem[];
-
-    const int nbias = (2 * g.w - 1) * (2 * g.w - 1);
-    int* s_tok = reinterpret_cast<int*>(smem);                // [2][64]
-    int* s_meta = s_tok + 2 * BN;                             // [2][64]
-    float* s_bias = reinterpret_cast<float*>(s_meta + 2 * BN);
-    unsigned char* s_tiles = smem + (((size_t)BN * 16 + (size_t)nbias * 4 + 127) / 128) * 128;   // [2][Q | K | V]
+    unsigned char* s_q = smem;
+    unsigned char* s_k = smem + TILE_BYTES;
+    unsigned char* s_v = smem + 2 * TILE_BYTES;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int gq = lane >> 2, tq = lane & 3;
     const int head = blockIdx.x % g.heads;
-    const int M = g.Mh * g.Mw;
-    const int c0 = (g.w - 1) * 2 * g.w;
-    const long long n_items = (long long)g.B * M;
-    const long long first = blockIdx.x / g.heads;
+    ItemCursor cur = cursor_init(blockIdx.x / g.heads, ctas_per_head, 1, g.Mw, g.Mh);
 
-    for (int i = tid; i < nbias; i += NTHREADS) s_bias[i] = bias[(size_t)i * g.heads + head] * kLog2e;
-
-    // slot tables of item `item` into buffer `b`
-    auto fill_tables = [&](long long item, int b) {
-        if (tid < BN) {
-            const WindowRef r = window_ref(g, (int)(item % M));
-            int meta = 0xff << 16, tok = -1;
-            if (tid < r.n) tok = slot_token(g, r, tid, meta);
-            s_tok[b * BN + tid] = tok;
-            s_meta[b * BN + tid] = meta;
-        }
+    auto token = [&](const ItemCursor& c, int a, int b) {
+        int u = c.wr * g.w + a + g.sh;
+        if (u >= g.H) u -= g.H;
+        int col = c.wc * g.w + b + g.sw;
+        if (col >= g.W) col -= g.W;
+        return ((size_t)c.b * g.H + u) * g.W + col;
     };
-    // the copies of item `item` into buffer `b` (its tables must be visible), one group
-    auto issue_loads = [&](long long item, int b) {
-        const size_t sample_off = (size_t)(item / M) * g.H * g.W;
-        unsigned char* t = s_tiles + b * BUF_BYTES;
-        load_rows<D>(t, q, s_tok + b * BN, 0, sample_off, g.ts, head, tid);
-        load_rows<D>(t + TILE_BYTES, k, s_tok + b * BN, 0, sample_off, g.ts, head, tid);
-        load_rows<D>(t + 2 * TILE_BYTES, v, s_tok + b * BN, 0, sample_off, g.ts, head, tid);
+    // each warp copies its own 16 rows (window rows 2 warp and 2 warp + 1) of the three tiles
+    const int crow = 16 * warp + lane / CPR, cchunk = lane % CPR;
+    auto issue_loads = [&](const ItemCursor& c) {
+        const int eh = min(g.w, g.H - c.wr * g.w), ew = min(g.w, g.W - c.wc * g.w);
+#pragma unroll
+        for (int i = 0; i < 16 / RPI; ++i) {
+            const int row = crow + i * RPI, a = row >> 3, b = row & 7;
+            const bool ok = a < eh && b < ew;
+            const size_t off = ok ? token(c, a, b) * g.ts + head * D + cchunk * 8 : 0;
+            const uint32_t dst = smem_u32(s_q + tile_off<D>(row, cchunk));
+            cp_async16(dst, q + off, ok ? 16 : 0);
+            cp_async16(dst + TILE_BYTES, k + off, ok ? 16 : 0);
+            cp_async16(dst + 2 * TILE_BYTES, v + off, ok ? 16 : 0);
+        }
         cp_async_commit();
     };
-    if (first < n_items) {
-        fill_tables(first, 0);
-        __syncthreads();
-        issue_loads(first, 0);
-    }
-    int buf = 0;
-    for (long long item = first; item < n_items; item += ctas_per_head, buf ^= 1) {
-        const long long next = item + ctas_per_head;
-        // the other buffer was last read by the scatter of the item before this one, which ended with a barrier
-        if (next < n_items) fill_tables(next, buf ^ 1);
-        __syncthreads();
-        if (next < n_items) {
-            issue_loads(next, buf ^ 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
+    if (cur.b < g.B) issue_loads(cur);
+
+    // bias log2 e between query row (2 warp + h, gq) and key (nt, 2 tq + e): entry [h - nt + 7][e]
+    float bv[9][2];
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int da = 2 * warp + i - 7, db = gq - 2 * tq - e;
+            const bool in = da > -g.w && da < g.w && db > -g.w && db < g.w;
+            bv[i][e] = in ? bias[((size_t)(da + g.w - 1) * (2 * g.w - 1) + db + g.w - 1) * g.heads + head] * kLog2e : 0.f;
         }
+
+    while (cur.b < g.B) {
+        const int eh = min(g.w, g.H - cur.wr * g.w), ew = min(g.w, g.W - cur.wc * g.w);
+        // window rows >= ha / columns >= hb carry the other mask label
+        const int ha = (!g.ph && g.sh > 0) ? min(max(g.H - g.sh - cur.wr * g.w, 0), 8) : 8;
+        const int hb = (!g.pw && g.sw > 0) ? min(max(g.W - g.sw - cur.wc * g.w, 0), 8) : 8;
+        cp_async_wait<0>();
         __syncthreads();
-        const WindowRef r = window_ref(g, (int)(item % M));
-        const size_t sample_off = (size_t)(item / M) * g.H * g.W;
-        unsigned char* s_q = s_tiles + buf * BUF_BYTES;
-        const unsigned char* s_k = s_q + TILE_BYTES;
-        const unsigned char* s_v = s_q + 2 * TILE_BYTES;
-        const int* tokb = s_tok + buf * BN;
-        const int* metab = s_meta + buf * BN;
 
         // S = Q K^T for the warp's 16 query rows
         float acc_s[BN / 8][4];
@@ -365,29 +360,38 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
                 mma_elem(acc_s[2 * np + 1], qf, bf[2], bf[3]);
             }
         }
-        // scale + relative-position bias + shift mask, in the log2 domain; row maxima
-        const int meta_r[2] = {metab[warp * 16 + gq], metab[warp * 16 + gq + 8]};
-        float mx[2] = {-INFINITY, -INFINITY};
+        // scale + relative-position bias in the log2 domain
 #pragma unroll
-        for (int nt = 0; nt < BN / 8; ++nt) {
+        for (int nt = 0; nt < BN / 8; ++nt)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int mj = metab[nt * 8 + 2 * tq + (e & 1)];
-                const int mi = meta_r[e >> 1];
-                const bool ok = meta_label(mi) == meta_label(mj);
-                float sc = acc_s[nt][e] * g.scale_log2e + s_bias[meta_code(mi) - meta_code(mj) + c0];
-                sc = ok ? sc : -INFINITY;
-                acc_s[nt][e] = sc;
-                mx[e >> 1] = fmaxf(mx[e >> 1], sc);
+            for (int e = 0; e < 4; ++e) acc_s[nt][e] = fmaf(acc_s[nt][e], g.scale_log2e, bv[(e >> 1) - nt + 7][e & 1]);
+        if (eh < 8 || ew < 8 || (ha > 0 && ha < eh) || (hb > 0 && hb < ew)) {
+            // key slots without a token and of another mask label
+            const uint32_t behind = 0xffu << ha, rows = (1u << eh) - 1;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t see = ((2 * warp + h >= ha) ? behind : ~behind) & rows;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int b = 2 * tq + e;
+                    const uint32_t ok = (b < ew && (b >= hb) == (gq >= hb)) ? see : 0u;
+#pragma unroll
+                    for (int nt = 0; nt < BN / 8; ++nt) acc_s[nt][2 * h + e] = (ok & (1u << nt)) ? acc_s[nt][2 * h + e] : -INFINITY;
+                }
             }
         }
-        float m_use[2], l_row[2] = {0.f, 0.f};
+        float mx[2] = {-INFINITY, -INFINITY}, m_use[2], l_row[2] = {0.f, 0.f};
+#pragma unroll
+        for (int nt = 0; nt < BN / 8; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mx[e >> 1] = fmaxf(mx[e >> 1], acc_s[nt][e]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 1));
             mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], 2));
-            m_use[h] = (mx[h] == -INFINITY) ? 0.f : mx[h];     // a row without a token sees no key
+            m_use[h] = (mx[h] == -INFINITY) ? 0.f : mx[h];     // a row without a token may see no key
         }
+        uint32_t pf[BN / 8][2];
 #pragma unroll
         for (int nt = 0; nt < BN / 8; ++nt) {
 #pragma unroll
@@ -396,6 +400,8 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
                 acc_s[nt][e] = p;
                 l_row[e >> 1] += p;
             }
+            pf[nt][0] = pack_elem(acc_s[nt][0], acc_s[nt][1]);
+            pf[nt][1] = pack_elem(acc_s[nt][2], acc_s[nt][3]);
         }
         // O = P V
         float acc_o[DT][4];
@@ -405,18 +411,14 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
             for (int e = 0; e < 4; ++e) acc_o[i][e] = 0.f;
 #pragma unroll
         for (int ks = 0; ks < BN / 16; ++ks) {
-            uint32_t pf[4];
-            pf[0] = pack_elem(acc_s[2 * ks][0], acc_s[2 * ks][1]);
-            pf[1] = pack_elem(acc_s[2 * ks][2], acc_s[2 * ks][3]);
-            pf[2] = pack_elem(acc_s[2 * ks + 1][0], acc_s[2 * ks + 1][1]);
-            pf[3] = pack_elem(acc_s[2 * ks + 1][2], acc_s[2 * ks + 1][3]);
+            const uint32_t af[4] = {pf[2 * ks][0], pf[2 * ks][1], pf[2 * ks + 1][0], pf[2 * ks + 1][1]};
 #pragma unroll
             for (int dp = 0; dp < DT / 2; ++dp) {
                 uint32_t bf[4];
                 const int key = ks * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
                 ldmatrix_x4_trans(bf, smem_u32(s_v + tile_off<D>(key, 2 * dp + (lane >> 4))));
-                mma_elem(acc_o[2 * dp], pf, bf[0], bf[1]);
-                mma_elem(acc_o[2 * dp + 1], pf, bf[2], bf[3]);
+                mma_elem(acc_o[2 * dp], af, bf[0], bf[1]);
+                mma_elem(acc_o[2 * dp + 1], af, bf[2], bf[3]);
             }
         }
         float inv[2];
@@ -428,30 +430,28 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
             l_row[h] = l;
             inv[h] = 1.f / l;
         }
-        __syncthreads();   // every warp has read its Q fragments: the Q tile becomes the output tile
+        // the warp's output goes where its own Q rows were
+        __syncwarp();
 #pragma unroll
         for (int i = 0; i < DT; ++i) {
             const int lr = warp * 16 + gq;
             *reinterpret_cast<uint32_t*>(s_q + tile_off<D>(lr, i) + tq * 4) = pack_elem(acc_o[i][0] * inv[0], acc_o[i][1] * inv[0]);
             *reinterpret_cast<uint32_t*>(s_q + tile_off<D>(lr + 8, i) + tq * 4) = pack_elem(acc_o[i][2] * inv[1], acc_o[i][3] * inv[1]);
         }
-        if (tq == 0) {
+        if (tq < 2) {
+            const int a = 2 * warp + tq;
+            if (a < eh && gq < ew) lse[token(cur, a, gq) * g.heads + head] = ((tq ? mx[1] : mx[0]) + log2f(tq ? l_row[1] : l_row[0])) * kLn2;
+        }
+        __syncwarp();
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int slot = warp * 16 + gq + 8 * h;
-                if (slot < r.n) lse[(sample_off + (size_t)tokb[slot]) * g.heads + head] = (mx[h] + log2f(l_row[h])) * kLn2;
-            }
+        for (int i = 0; i < 16 / RPI; ++i) {
+            const int row = crow + i * RPI, a = row >> 3, b = row & 7;
+            if (a < eh && b < ew)
+                *reinterpret_cast<uint4*>(o + (token(cur, a, b) * g.heads + head) * D + cchunk * 8) = *reinterpret_cast<const uint4*>(s_q + tile_off<D>(row, cchunk));
         }
-        __syncthreads();
-        constexpr int CPR = D / 8;
-        for (int idx = tid; idx < BM * CPR; idx += NTHREADS) {
-            const int row = idx / CPR, chunk = idx - row * CPR;
-            if (row < r.n) {
-                const uint4 val = *reinterpret_cast<const uint4*>(s_q + tile_off<D>(row, chunk));
-                *reinterpret_cast<uint4*>(o + ((sample_off + (size_t)tokb[row]) * g.heads + head) * D + chunk * 8) = val;
-            }
-        }
-        __syncthreads();   // the buffer's tiles and tables are free for the item after next
+        cursor_advance(cur, 1, g.Mw, g.Mh);
+        __syncthreads();   // the tiles are free for the next window
+        if (cur.b < g.B) issue_loads(cur);
     }
 }
 
@@ -467,11 +467,9 @@ size_t fwd_smem_bytes(const Geo& g) {
 
 cudaError_t TERRA_ELEM_FN(launch_fwd_mma)(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
                            void* o, float* lse, int sm_count, cudaStream_t stream) {
-    if (g.nmax <= BN && g.w <= 32) {
-        // windows of at most 64 tokens: the persistent double-buffered kernel
+    if (g.w <= 8) {
         auto kern = g.d == 32 ? swin_fwd_small_kernel<32> : g.d == 64 ? swin_fwd_small_kernel<64> : swin_fwd_small_kernel<128>;
-        const int nbias = (2 * g.w - 1) * (2 * g.w - 1);
-        const size_t smem = (((size_t)BN * 16 + (size_t)nbias * 4 + 127) / 128) * 128 + 6 * (size_t)BN * g.d * 2;
+        const size_t smem = 3 * (size_t)BN * g.d * 2;
         int occ = 0;
         cudaError_t e = prepare_kernel((const void*)kern, smem, NTHREADS, &occ);
         if (e != cudaSuccess) return e;
