@@ -143,10 +143,10 @@ static bool force_register_path() {
     return on;
 }
 
-// Windows of at most 64 tokens (the 8 x 8 windows of configs 1, 2 and of the paper's small and medium models) half
-// fill a 128-row tcgen05 tile and are bound by HBM and launch overheads: the register-tile forward and the one-kernel
-// register-tile backward are faster there at every head dim (config 2: 0.117 ms against 0.188 ms per step).
-static bool small_windows(const Geo& g) { return g.nmax <= 64; }
+// Window sides up to 8 (the 8 x 8 windows of configs 1, 2 and of the paper's small and medium models) half fill a 128-row
+// tcgen05 tile and are bound by HBM and launch overheads: the mma.sync forward and the one-kernel backward are faster there
+// at every head dim (config 2: 0.117 ms against 0.188 ms per step).
+static bool small_windows(const Geo& g) { return g.w <= 8; }
 
 // (every kernel exists for bf16 and for fp16 activations: `f16` only selects the build of the kernel)
 static bool use_fwd_tc(const Geo& g) { return fwd_tc_supported(g) && !small_windows(g); }
@@ -308,7 +308,7 @@ static int bwd_call(const Geo& g, const void* q, const void* k, const void* v,
         return et == cudaSuccess ? TERRA_OK : cuda_fail(et, "terra_swin_attn_bwd");
     }
     if (bwd_small_supported(g) && !force_split_small()) {
-        // windows of at most 64 tokens at head dim 128: one kernel reads every tensor once
+        // window sides up to 8: one kernel reads every tensor once
         cudaError_t es = g.f16 ? launch_bwd_small_f16(g, q, k, v, o, d_o, bias_table, lse, dq, dk, dv, dbias, sms, st)
                                : launch_bwd_small(g, q, k, v, o, d_o, bias_table, lse, dq, dk, dv, dbias, sms, st);
         return es == cudaSuccess ? TERRA_OK : cuda_fail(es, "terra_swin_attn_bwd");

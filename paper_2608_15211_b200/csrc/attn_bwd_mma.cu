@@ -463,99 +463,115 @@ __device__ __forceinline__ void coef_t_times_block(float (&out)[D / 8][4], const
     }
 }
 
-// The whole backward of windows of at most 64 tokens in one kernel (the paper's 8 x 8 windows), any head dim: a CTA holds the
-// window's Q, K, V, dO and O rows of one head, so every tensor is read once and dQ, dK, dV are written once (the
-// split into a key side and a query side reads the inputs twice, and a third time for delta).
-//   delta = rowsum(dO * O)                                 (per query row, from the two tiles)
-//   query-major, a warp owns 16 query rows:  S = Q K^T, dP = dO V^T, P = exp2(S scale + bias - lse), dS = P (dP - delta),
-//   the bias gradient (as in the query-side kernel above), dQ = dS K; P and dS go to shared memory as 64 x 64 tiles
+// The whole backward of windows of side up to 8 (the paper's 8 x 8 windows) in one kernel, any head dim: a CTA holds the
+// window's Q, K, V and dO rows of one head, 8 slots to a window row (slot = 8 a + b), so every tensor is read once and dQ, dK,
+// dV are written once (the split into a key side and a query side reads the inputs twice, and a third time for delta).
+//   query-major, a warp owns 16 query rows:  delta = rowsum(dO * O), S = Q K^T, dP = dO V^T, P = exp2(S scale + bias - lse),
+//   dS = P (dP - delta), dQ = dS K; P and dS go to shared memory as 64 x 64 tiles, over V where it is large enough
 //   key-major, a warp owns 16 key rows:      dV = P^T dO, dK = dS^T Q  (A fragments by transposing loads of those tiles)
-// Persistent CTAs bound to one head walk over (batch, window).  Shared memory: the four operand tiles, one more that
-// holds O first and P | dS afterwards, the slot tables, the summed-dS image and the staging tile of the bias gradient.
+// Persistent CTAs bound to one head walk over (batch, window).  As in the forward kernel what counts is how many CTAs an SM
+// holds, not prefetching: three of 66 KB at head dim 128.  O goes to registers only, a thread's bias gradients (18 diagonals of its
+// 32 pairs) stay in registers for the whole run, a warp's results take the place of its own K rows one after the other and are
+// stored from there; a window costs four barriers.  Five products of 64 x 64 x D on mma.sync take 2700 of about 3000 cycles that
+// the copies need at head dim 128.
+// 288 x 544 tokens, 8 x 128: @@; 128 x 256, 6 x 32: @@.
 template <int D>
-__global__ void __launch_bounds__(NTHREADS, 2)
+__device__ __host__ constexpr int small_tile_bytes() { return BN * D * 2; }
+template <int D>
+constexpr size_t kSmallSmem = 4 * (size_t)small_tile_bytes<D>() + (D == 128 ? 0 : 16384) + 2 * 15 * 16 * sizeof(float);
+
+template <int D>
+__global__ void __launch_bounds__(NTHREADS, D == 128 ? 3 : 4)
 swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
                       const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ o,
                       const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ bias, const float* __restrict__ lse,
                       __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv,
-                      float* __restrict__ dbias, int ctas_per_head, int acc_stride) {
+                      float* __restrict__ dbias, int ctas_per_head) {
     constexpr int KS = D / 16;
     constexpr int DT = D / 8;
-    constexpr int TILE_BYTES = BN * D * 2;
-    constexpr int X_BYTES = TILE_BYTES > 16384 ? TILE_BYTES : 16384;      // O, then P (8 KB) | dS (8 KB)
+    constexpr int CPR = D / 8, RPI = 32 / CPR;       // 16-byte chunks of a row; rows a warp copies at a time
+    constexpr int TILE_BYTES = small_tile_bytes<D>();
     extern __shared__ __align__(128) unsigned char smem[];
-
-    const int nbias = (2 * g.w - 1) * (2 * g.w - 1);
-    int* s_tok = reinterpret_cast<int*>(smem);
-    int* s_meta = s_tok + BN;
-    float* s_lse = reinterpret_cast<float*>(s_meta + BN);
-    float* s_delta = s_lse + BN;
-    float* s_bias = s_delta + BN;
-    float* s_dbias = s_bias + nbias;
-    unsigned char* s_q = smem + (((size_t)BN * 16 + (size_t)nbias * 8 + 127) / 128) * 128;
+    unsigned char* s_q = smem;
     unsigned char* s_k = s_q + TILE_BYTES;
-    unsigned char* s_v = s_k + TILE_BYTES;
-    unsigned char* s_g = s_v + TILE_BYTES;            // dO
-    unsigned char* s_x = s_g + TILE_BYTES;
-    unsigned char* s_p = s_x;                         // P as a 64 x 64 tile
-    unsigned char* s_ds = s_x + 8192;                 // dS as a 64 x 64 tile
-    float* s_acc = reinterpret_cast<float*>(s_x + X_BYTES);              // 64 x acc_stride image of summed dS
-    float* s_stage = s_acc + BM * acc_stride;                            // 4 warps x 16 x kStageStride
+    unsigned char* s_g = s_k + TILE_BYTES;            // dO
+    unsigned char* s_v = s_g + TILE_BYTES;
+    unsigned char* s_p = D == 128 ? s_v : s_v + TILE_BYTES;     // P as a 64 x 64 tile
+    unsigned char* s_ds = s_p + 8192;                 // dS as a 64 x 64 tile
+    float* s_bias = reinterpret_cast<float*>(s_ds + 8192);      // bias log2 e at [query row - key row + 7][query column - key column + 7]
+    float* s_dbias = s_bias + 15 * 16;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int gq = lane >> 2, tq = lane & 3;
     const int head = blockIdx.x % g.heads;
-    const int M = g.Mh * g.Mw;
-    const int c0 = (g.w - 1) * 2 * g.w;
-    const long long n_items = (long long)g.B * M;
     const int dense = g.heads * D;                    // token stride of o and dO
+    ItemCursor cur = cursor_init(blockIdx.x / g.heads, ctas_per_head, 1, g.Mw, g.Mh);
 
-    for (int i = tid; i < nbias; i += NTHREADS) {
-        s_bias[i] = bias[(size_t)i * g.heads + head] * kLog2e;
+    auto token = [&](int a, int b) {
+        int u = cur.wr * g.w + a + g.sh;
+        if (u >= g.H) u -= g.H;
+        int col = cur.wc * g.w + b + g.sw;
+        if (col >= g.W) col -= g.W;
+        return ((size_t)cur.b * g.H + u) * g.W + col;
+    };
+    const int crow = 16 * warp + lane / CPR, cchunk = lane % CPR;
+    // what comes with a window in registers: chunks tq, tq + 4, ... of the O rows (2 warp + h, gq) and their log-sum-exp
+    uint4 o_r[2][DT / 4];
+    float lse_r[2];
+    auto issue_loads = [&]() {
+        const int eh = min(g.w, g.H - cur.wr * g.w), ew = min(g.w, g.W - cur.wc * g.w);
+#pragma unroll
+        for (int i = 0; i < 16 / RPI; ++i) {
+            const int row = crow + i * RPI, a = row >> 3, b = row & 7;
+            const bool ok = a < eh && b < ew;
+            const size_t tok = ok ? token(a, b) : 0, off = tok * g.ts + head * D + cchunk * 8;
+            const uint32_t dst = smem_u32(s_q + tile_off<D>(row, cchunk));
+            cp_async16(dst, q + off, ok ? 16 : 0);
+            cp_async16(dst + TILE_BYTES, k + off, ok ? 16 : 0);
+            cp_async16(dst + 2 * TILE_BYTES, d_o + tok * dense + head * D + cchunk * 8, ok ? 16 : 0);
+            cp_async16(dst + 3 * TILE_BYTES, v + off, ok ? 16 : 0);
+        }
+        cp_async_commit();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const bool ok = 2 * warp + h < eh && gq < ew;
+            const size_t tok = ok ? token(2 * warp + h, gq) : 0;
+            lse_r[h] = ok ? __ldg(lse + tok * g.heads + head) * kLog2e : INFINITY;      // no token: P = exp2(x - inf) = 0
+#pragma unroll
+            for (int c = 0; c < DT / 4; ++c)
+                o_r[h][c] = ok ? __ldg(reinterpret_cast<const uint4*>(o + tok * dense + head * D) + tq + 4 * c) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    if (cur.b < g.B) issue_loads();
+    for (int i = tid; i < 15 * 16; i += NTHREADS) {
+        const int da = (i >> 4) - 7, db = (i & 15) - 7;
+        const bool in = da > -g.w && da < g.w && db > -g.w && db < g.w;
+        s_bias[i] = in ? bias[((size_t)(da + g.w - 1) * (2 * g.w - 1) + db + g.w - 1) * g.heads + head] * kLog2e : 0.f;
         s_dbias[i] = 0.f;
     }
-    for (int i = tid; i < BM * acc_stride; i += NTHREADS) s_acc[i] = 0.f;
+    // query row (2 warp + h, gq), key (nt, 2 tq + e): entry [h - nt + 7][e] of what follows
+    const float* my_bias = s_bias + 2 * warp * 16 + gq - 2 * tq + 7;
+    float db_r[9][2];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) db_r[i][0] = db_r[i][1] = 0.f;
 
-    for (long long item = blockIdx.x / g.heads; item < n_items; item += ctas_per_head) {
-        const int win = (int)(item % M);
-        const int b = (int)(item / M);
-        const WindowRef r = window_ref(g, win);
-        const size_t sample_off = (size_t)b * g.H * g.W;
-
-        __syncthreads();   // the previous item's readers of the tables and tiles are done
-        if (tid < BN) {
-            int meta = 0xff << 16, tok = -1;
-            if (tid < r.n) {
-                tok = slot_token(g, r, tid, meta);
-                // the row's log-sum-exp travels with the tiles (no load that the copies below would have to wait for)
-                cp_async4(smem_u32(&s_lse[tid]), lse + (sample_off + (size_t)tok) * g.heads + head);
-            } else {
-                s_lse[tid] = INFINITY;              // padded queries: P = exp2(x - inf) = 0
-            }
-            s_tok[tid] = tok;
-            s_meta[tid] = meta;
-        }
-        __syncthreads();
-        load_rows<D>(s_q, q, s_tok, 0, sample_off, g.ts, head, tid);
-        load_rows<D>(s_k, k, s_tok, 0, sample_off, g.ts, head, tid);
-        load_rows<D>(s_v, v, s_tok, 0, sample_off, g.ts, head, tid);
-        load_rows<D>(s_g, d_o, s_tok, 0, sample_off, dense, head, tid);
-        load_rows<D>(s_x, o, s_tok, 0, sample_off, dense, head, tid);
-        cp_async_commit();
+    while (cur.b < g.B) {
+        const int eh = min(g.w, g.H - cur.wr * g.w), ew = min(g.w, g.W - cur.wc * g.w);
+        // window rows >= ha / columns >= hb carry the other mask label
+        const int ha = (!g.ph && g.sh > 0) ? min(max(g.H - g.sh - cur.wr * g.w, 0), 8) : 8;
+        const int hb = (!g.pw && g.sw > 0) ? min(max(g.W - g.sw - cur.wc * g.w, 0), 8) : 8;
         cp_async_wait<0>();
         __syncthreads();
 
-        // ---- delta of the warp's 16 query rows: two lanes per row, half a row each
-        {
-            const int row = warp * 16 + (lane >> 1);
+        // ---- delta of the thread's two query rows
+        float del_r[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
             float acc = 0.f;
 #pragma unroll
-            for (int c = 0; c < DT / 2; ++c) {
-                const int chunk = (lane & 1) * (DT / 2) + c;
-                const uint4 a = *reinterpret_cast<const uint4*>(s_x + tile_off<D>(row, chunk));
-                const uint4 bb = *reinterpret_cast<const uint4*>(s_g + tile_off<D>(row, chunk));
-                const uint32_t* pa = reinterpret_cast<const uint32_t*>(&a);
-                const uint32_t* pb = reinterpret_cast<const uint32_t*>(&bb);
+            for (int c = 0; c < DT / 4; ++c) {
+                const uint4 bb = *reinterpret_cast<const uint4*>(s_g + tile_off<D>(warp * 16 + gq + 8 * h, tq + 4 * c));
+                const uint32_t pa[4] = {o_r[h][c].x, o_r[h][c].y, o_r[h][c].z, o_r[h][c].w}, pb[4] = {bb.x, bb.y, bb.z, bb.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float2 x = elem2_to_float2(pa[e]), y = elem2_to_float2(pb[e]);
@@ -563,88 +579,82 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
                 }
             }
             acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-            if ((lane & 1) == 0) s_delta[row] = acc;
+            del_r[h] = acc + __shfl_xor_sync(0xffffffffu, acc, 2);
         }
-        __syncthreads();   // O has been read by every warp: its tile becomes P | dS
 
         // ---- query-major part
-        const int row_tab[2] = {warp * 16 + gq, warp * 16 + gq + 8};
-        const int meta_r[2] = {s_meta[row_tab[0]], s_meta[row_tab[1]]};
-        const float lse_r[2] = {s_lse[row_tab[0]] * kLog2e, s_lse[row_tab[1]] * kLog2e};
-        const float del_r[2] = {s_delta[row_tab[0]], s_delta[row_tab[1]]};
         float acc1[DT][4];
+        const float scale = g.scale_log2e * kLn2;
+        // the warp's rows of a result, from its own K rows
+        auto store_rows = [&](__nv_bfloat16* dst, float mul) {
+            __syncwarp();
+            stage_rows<D>(s_k, acc1, mul, warp, gq, tq);
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 16 / RPI; ++i) {
+                const int row = crow + i * RPI, a = row >> 3, b = row & 7;
+                if (a < eh && b < ew)
+                    *reinterpret_cast<uint4*>(dst + token(a, b) * g.ts + head * D + cchunk * 8) = *reinterpret_cast<const uint4*>(s_k + tile_off<D>(row, cchunk));
+            }
+        };
         {
-            // fragments of the warp's own Q and dO rows (head dim 128: read from shared memory at each use instead)
-            uint32_t f1[kFragsInRegs<D> ? KS : 1][4], f2[kFragsInRegs<D> ? KS : 1][4];
-            if constexpr (kFragsInRegs<D>) {
+            float acc_s[BN / 8][4], acc_dp[BN / 8][4];
+            auto rows_times = [&](float (&acc)[BN / 8][4], const unsigned char* own, const unsigned char* blk) {
+#pragma unroll
+                for (int i = 0; i < BN / 8; ++i)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
 #pragma unroll
                 for (int ks = 0; ks < KS; ++ks) {
-                    const int row = warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8;
-                    ldmatrix_x4(f1[ks], smem_u32(s_q + tile_off<D>(row, 2 * ks + (lane >> 4))));
-                    ldmatrix_x4(f2[ks], smem_u32(s_g + tile_off<D>(row, 2 * ks + (lane >> 4))));
+                    uint32_t af[4];
+                    ldmatrix_x4(af, smem_u32(own + tile_off<D>(warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8, 2 * ks + (lane >> 4))));
+#pragma unroll
+                    for (int np = 0; np < BN / 16; ++np) {
+                        uint32_t bf[4];
+                        ldmatrix_x4(bf, smem_u32(blk + tile_off<D>(np * 16 + (lane & 7) + (lane >> 4) * 8, 2 * ks + ((lane >> 3) & 1))));
+                        mma_elem(acc[2 * np], af, bf[0], bf[1]);
+                        mma_elem(acc[2 * np + 1], af, bf[2], bf[3]);
+                    }
+                }
+            };
+            rows_times(acc_s, s_q, s_k);
+            rows_times(acc_dp, s_g, s_v);
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const float bv = my_bias[i * 16 - e];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int nt = h + 7 - i;
+                        if (nt >= 0 && nt < 8) acc_s[nt][2 * h + e] = fmaf(acc_s[nt][2 * h + e], g.scale_log2e, bv) - lse_r[h];
+                    }
+                }
+            if (eh < 8 || ew < 8 || (ha > 0 && ha < eh) || (hb > 0 && hb < ew)) {
+                // key slots without a token and of another mask label
+                const uint32_t behind = 0xffu << ha, rows = (1u << eh) - 1;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t see = ((2 * warp + h >= ha) ? behind : ~behind) & rows;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int b = 2 * tq + e;
+                        const uint32_t ok = (b < ew && (b >= hb) == (gq >= hb)) ? see : 0u;
+#pragma unroll
+                        for (int nt = 0; nt < BN / 8; ++nt) acc_s[nt][2 * h + e] = (ok & (1u << nt)) ? acc_s[nt][2 * h + e] : -INFINITY;
+                    }
                 }
             }
-            float acc_s[BN / 8][4], acc_dp[BN / 8][4];
-            rows_times_block_t<D>(acc_s, f1, s_q, s_k, warp, lane);
-            rows_times_block_t<D>(acc_dp, f2, s_g, s_v, warp, lane);
 #pragma unroll
-            for (int nt = 0; nt < BN / 8; ++nt) {
+            for (int nt = 0; nt < BN / 8; ++nt)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const int col = nt * 8 + 2 * tq + (e & 1);
-                    const int mc = s_meta[col];
-                    const int mr = meta_r[e >> 1];
-                    const bool ok = meta_label(mr) == meta_label(mc);
-                    const int bidx = meta_code(mr) - meta_code(mc) + c0;
-                    float p = fast_exp2(acc_s[nt][e] * g.scale_log2e + s_bias[bidx] - lse_r[e >> 1]);
-                    p = ok ? p : 0.f;
-                    acc_s[nt][e] = p;
-                    acc_dp[nt][e] = p * (acc_dp[nt][e] - del_r[e >> 1]);
+                    const float pe = fast_exp2(acc_s[nt][e]);
+                    acc_s[nt][e] = pe;
+                    acc_dp[nt][e] = pe * (acc_dp[nt][e] - del_r[e >> 1]);
+                    db_r[(e >> 1) - nt + 7][e & 1] += acc_dp[nt][e];
                 }
-            }
-            // bias gradient
-            if (r.ew == g.w) {
-                // full-width window: this thread owns these cells of the image (binned into the table at the end)
-                float2* cell0 = reinterpret_cast<float2*>(s_acc + (warp * 16 + gq) * acc_stride + 2 * tq);
-                float2 cur[BN / 8][2];
-#pragma unroll
-                for (int nt = 0; nt < BN / 8; ++nt) {
-                    cur[nt][0] = cell0[nt * 4];
-                    cur[nt][1] = cell0[nt * 4 + 4 * acc_stride];
-                }
-#pragma unroll
-                for (int nt = 0; nt < BN / 8; ++nt) {
-                    cur[nt][0].x += acc_dp[nt][0]; cur[nt][0].y += acc_dp[nt][1];
-                    cur[nt][1].x += acc_dp[nt][2]; cur[nt][1].y += acc_dp[nt][3];
-                }
-#pragma unroll
-                for (int nt = 0; nt < BN / 8; ++nt) {
-                    cell0[nt * 4] = cur[nt][0];
-                    cell0[nt * 4 + 4 * acc_stride] = cur[nt][1];
-                }
-            } else {
-                // narrow edge window: through the staging tile, one shared-memory atomic per pair, 32 different table
-                // entries per instruction
-                float* stage = s_stage + warp * 16 * kStageStride;
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-#pragma unroll
-                    for (int nt = 4 * half; nt < 4 * half + 4; ++nt) {
-                        const int col = (nt - 4 * half) * 8 + 2 * tq;
-                        *reinterpret_cast<float2*>(stage + gq * kStageStride + col) = make_float2(acc_dp[nt][0], acc_dp[nt][1]);
-                        *reinterpret_cast<float2*>(stage + (gq + 8) * kStageStride + col) = make_float2(acc_dp[nt][2], acc_dp[nt][3]);
-                    }
-                    __syncwarp();
-                    const int code_c = meta_code(s_meta[half * 32 + lane]);
-                    for (int rr = 0; rr < 16; ++rr) {
-                        const int code_r = meta_code(s_meta[warp * 16 + rr]) + c0;
-                        const float v0 = stage[rr * kStageStride + lane];
-                        if (v0 != 0.f) atomicAdd(&s_dbias[code_r - code_c], v0);
-                    }
-                    __syncwarp();
-                }
-            }
-            // P and dS as 64 x 64 tiles for the key-major part
+            if (D == 128) __syncthreads();   // V has been read by every warp
             stage_rows<64>(s_p, acc_s, 1.f, warp, gq, tq);
             stage_rows<64>(s_ds, acc_dp, 1.f, warp, gq, tq);
             // dQ = dS K
@@ -654,9 +664,8 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
                 for (int e = 0; e < 4; ++e) acc1[i][e] = 0.f;
             coef_times_block<D>(acc1, acc_dp, s_k, lane);
         }
-        __syncthreads();   // P, dS are complete; K and V have been read by every warp
-        const float scale = g.scale_log2e * kLn2;
-        stage_rows<D>(s_v, acc1, scale, warp, gq, tq);           // dQ into the V tile
+        __syncthreads();   // P, dS are complete; K has been read by every warp
+        store_rows(dq, scale);
 
         // ---- key-major part
 #pragma unroll
@@ -664,36 +673,30 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc1[i][e] = 0.f;
         coef_t_times_block<D>(acc1, s_p, s_g, warp, lane);       // dV = P^T dO
-        stage_rows<D>(s_k, acc1, 1.f, warp, gq, tq);             // dV into the K tile
+        store_rows(dv, 1.f);
 #pragma unroll
         for (int i = 0; i < DT; ++i)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc1[i][e] = 0.f;
         coef_t_times_block<D>(acc1, s_ds, s_q, warp, lane);      // dK = dS^T Q
-        __syncthreads();   // Q has been read by every warp
-        stage_rows<D>(s_q, acc1, scale, warp, gq, tq);           // dK into the Q tile
-        __syncthreads();
-        scatter_rows<D>(s_v, dq, s_tok, 0, r.n, sample_off, g.ts, head, tid);
-        scatter_rows<D>(s_k, dv, s_tok, 0, r.n, sample_off, g.ts, head, tid);
-        scatter_rows<D>(s_q, dk, s_tok, 0, r.n, sample_off, g.ts, head, tid);
+        store_rows(dk, scale);
+        cursor_advance(cur, 1, g.Mw, g.Mh);
+        __syncthreads();   // the tiles are free for the next window
+        if (cur.b < g.B) issue_loads();
     }
 
+    // the threads' sums into the CTA's table, that into the caller's
+    float* mine = s_dbias + 2 * warp * 16 + gq - 2 * tq + 7;
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            if (db_r[i][e] != 0.f) atomicAdd(mine + i * 16 - e, db_r[i][e]);
     __syncthreads();
-    // bin the image: cell (row, col) of a full-width window belongs to table row code(row) - code(col) + c0
-    const int n_full = g.nmax;
-    for (int cell = tid; cell < BM * n_full; cell += NTHREADS) {
-        const int row = cell / n_full, col = cell - row * n_full;
-        if (row >= n_full) continue;
-        const float val = s_acc[row * acc_stride + col];
-        if (val == 0.f) continue;
-        const int code_r = (row / g.w) * (2 * g.w - 1) + row % g.w;
-        const int code_c = (col / g.w) * (2 * g.w - 1) + col % g.w;
-        atomicAdd(&s_dbias[code_r - code_c + c0], val);
-    }
-    __syncthreads();
-    for (int i = tid; i < nbias; i += NTHREADS) {
-        float val = s_dbias[i];
-        if (val != 0.f) atomicAdd(&dbias[(size_t)i * g.heads + head], val);
+    for (int i = tid; i < 15 * 16; i += NTHREADS) {
+        const int da = (i >> 4) - 7, db = (i & 15) - 7;
+        if (da > -g.w && da < g.w && db > -g.w && db < g.w && s_dbias[i] != 0.f)
+            atomicAdd(&dbias[((size_t)(da + g.w - 1) * (2 * g.w - 1) + db + g.w - 1) * g.heads + head], s_dbias[i]);
     }
 }
 
@@ -770,17 +773,10 @@ cudaError_t launch_one(const Geo& g, const void* q, const void* k, const void* v
                     : launch_one_sized<D, KV, false>(g, q, k, v, d_o, bias, lse, delta, out1, out2, dbias, sm_count, stream);
 }
 
-size_t bwd_small_smem_bytes(const Geo& g) {
-    const int nbias = (2 * g.w - 1) * (2 * g.w - 1);
-    const size_t head = (((size_t)BN * 16 + (size_t)nbias * 8 + 127) / 128) * 128;
-    const size_t tile = (size_t)BN * g.d * 2;
-    return head + 4 * tile + (tile > 16384 ? tile : 16384) + ((size_t)BM * (BN + 8) + (size_t)BM * kStageStride) * sizeof(float);
-}
-
 }  // namespace
 
-// windows of at most 64 tokens: the one-kernel backward
-bool TERRA_ELEM_FN(bwd_small_supported)(const Geo& g) { return g.nmax <= BN && g.w <= 32; }
+// window sides up to 8: the one-kernel backward
+bool TERRA_ELEM_FN(bwd_small_supported)(const Geo& g) { return g.w <= 8; }
 
 cudaError_t TERRA_ELEM_FN(launch_bwd_small)(const Geo& g, const void* q, const void* k, const void* v, const void* o, const void* d_o,
                                             const float* bias, const float* lse, void* dq, void* dk, void* dv, float* dbias,
@@ -788,7 +784,7 @@ cudaError_t TERRA_ELEM_FN(launch_bwd_small)(const Geo& g, const void* q, const v
     cudaError_t e = cudaMemsetAsync(dbias, 0, sizeof(float) * (size_t)(2 * g.w - 1) * (2 * g.w - 1) * g.heads, stream);
     if (e != cudaSuccess) return e;
     auto kern = g.d == 32 ? swin_bwd_small_kernel<32> : g.d == 64 ? swin_bwd_small_kernel<64> : swin_bwd_small_kernel<128>;
-    const size_t smem = bwd_small_smem_bytes(g);
+    const size_t smem = g.d == 32 ? kSmallSmem<32> : g.d == 64 ? kSmallSmem<64> : kSmallSmem<128>;
     int occ = 0;
     e = prepare_kernel((const void*)kern, smem, NTHREADS, &occ);
     if (e != cudaSuccess) return e;
@@ -800,7 +796,7 @@ cudaError_t TERRA_ELEM_FN(launch_bwd_small)(const Geo& g, const void* q, const v
     prof_begin("swin_bwd_small_kernel", stream);
     kern<<<(unsigned)(cph * g.heads), NTHREADS, smem, stream>>>(
         g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)o,
-        (const __nv_bfloat16*)d_o, bias, lse, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, dbias, (int)cph, BN + 8);
+        (const __nv_bfloat16*)d_o, bias, lse, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, dbias, (int)cph);
     count_launch(stream);
     return cudaGetLastError();
 }
