@@ -472,9 +472,10 @@ __device__ __forceinline__ void coef_t_times_block(float (&out)[D / 8][4], const
 // Persistent CTAs bound to one head walk over (batch, window).  As in the forward kernel what counts is how many CTAs an SM
 // holds, not prefetching: three of 66 KB at head dim 128.  O goes to registers only, a thread's bias gradients (18 diagonals of its
 // 32 pairs) stay in registers for the whole run, a warp's results take the place of its own K rows one after the other and are
-// stored from there; a window costs four barriers.  Five products of 64 x 64 x D on mma.sync take 2700 of about 3000 cycles that
+// stored from there; a window costs four barriers; the next window's rows are prefetched into L2 meanwhile (752 -> 575 us at head
+// dim 128; the forward kernel, with four CTAs, gains nothing by it: 232 -> 240 us).  Five products of 64 x 64 x D on mma.sync take 2700 of about 3000 cycles that
 // the copies need at head dim 128.
-// 288 x 544 tokens, 8 x 128: @@; 128 x 256, 6 x 32: @@.
+// 288 x 544 tokens, 8 x 128: 770 -> 575 us (68 % of the copy bandwidth); 128 x 256, 6 x 32: 55 -> 40 us.
 template <int D>
 __device__ __host__ constexpr int small_tile_bytes() { return BN * D * 2; }
 template <int D>
@@ -507,12 +508,12 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
     const int dense = g.heads * D;                    // token stride of o and dO
     ItemCursor cur = cursor_init(blockIdx.x / g.heads, ctas_per_head, 1, g.Mw, g.Mh);
 
-    auto token = [&](int a, int b) {
-        int u = cur.wr * g.w + a + g.sh;
+    auto token = [&](const ItemCursor& c, int a, int b) {
+        int u = c.wr * g.w + a + g.sh;
         if (u >= g.H) u -= g.H;
-        int col = cur.wc * g.w + b + g.sw;
+        int col = c.wc * g.w + b + g.sw;
         if (col >= g.W) col -= g.W;
-        return ((size_t)cur.b * g.H + u) * g.W + col;
+        return ((size_t)c.b * g.H + u) * g.W + col;
     };
     const int crow = 16 * warp + lane / CPR, cchunk = lane % CPR;
     // what comes with a window in registers: chunks tq, tq + 4, ... of the O rows (2 warp + h, gq) and their log-sum-exp
@@ -524,7 +525,7 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
         for (int i = 0; i < 16 / RPI; ++i) {
             const int row = crow + i * RPI, a = row >> 3, b = row & 7;
             const bool ok = a < eh && b < ew;
-            const size_t tok = ok ? token(a, b) : 0, off = tok * g.ts + head * D + cchunk * 8;
+            const size_t tok = ok ? token(cur, a, b) : 0, off = tok * g.ts + head * D + cchunk * 8;
             const uint32_t dst = smem_u32(s_q + tile_off<D>(row, cchunk));
             cp_async16(dst, q + off, ok ? 16 : 0);
             cp_async16(dst + TILE_BYTES, k + off, ok ? 16 : 0);
@@ -535,11 +536,23 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const bool ok = 2 * warp + h < eh && gq < ew;
-            const size_t tok = ok ? token(2 * warp + h, gq) : 0;
+            const size_t tok = ok ? token(cur, 2 * warp + h, gq) : 0;
             lse_r[h] = ok ? __ldg(lse + tok * g.heads + head) * kLog2e : INFINITY;      // no token: P = exp2(x - inf) = 0
 #pragma unroll
             for (int c = 0; c < DT / 4; ++c)
                 o_r[h][c] = ok ? __ldg(reinterpret_cast<const uint4*>(o + tok * dense + head * D) + tq + 4 * c) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    // a window ahead of the copies: its rows into L2, half a row a thread
+    auto prefetch = [&](const ItemCursor& c) {
+        const int a = tid >> 4, b = (tid >> 1) & 7;
+        if (a < min(g.w, g.H - c.wr * g.w) && b < min(g.w, g.W - c.wc * g.w)) {
+            const size_t tok = token(c, a, b), off = tok * g.ts + head * D + (tid & 1) * (D / 2), offd = tok * dense + head * D + (tid & 1) * (D / 2);
+            prefetch_l2(q + off);
+            prefetch_l2(k + off);
+            prefetch_l2(v + off);
+            prefetch_l2(d_o + offd);
+            prefetch_l2(o + offd);
         }
     };
     if (cur.b < g.B) issue_loads();
@@ -562,6 +575,9 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
         const int hb = (!g.pw && g.sw > 0) ? min(max(g.W - g.sw - cur.wc * g.w, 0), 8) : 8;
         cp_async_wait<0>();
         __syncthreads();
+        ItemCursor next = cur;
+        cursor_advance(next, 1, g.Mw, g.Mh);
+        if (next.b < g.B) prefetch(next);
 
         // ---- delta of the thread's two query rows
         float del_r[2];
@@ -594,7 +610,7 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
             for (int i = 0; i < 16 / RPI; ++i) {
                 const int row = crow + i * RPI, a = row >> 3, b = row & 7;
                 if (a < eh && b < ew)
-                    *reinterpret_cast<uint4*>(dst + token(a, b) * g.ts + head * D + cchunk * 8) = *reinterpret_cast<const uint4*>(s_k + tile_off<D>(row, cchunk));
+                    *reinterpret_cast<uint4*>(dst + token(cur, a, b) * g.ts + head * D + cchunk * 8) = *reinterpret_cast<const uint4*>(s_k + tile_off<D>(row, cchunk));
             }
         };
         {
@@ -680,7 +696,7 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
             for (int e = 0; e < 4; ++e) acc1[i][e] = 0.f;
         coef_t_times_block<D>(acc1, s_ds, s_q, warp, lane);      // dK = dS^T Q
         store_rows(dk, scale);
-        cursor_advance(cur, 1, g.Mw, g.Mh);
+        cur = next;
         __syncthreads();   // the tiles are free for the next window
         if (cur.b < g.B) issue_loads();
     }
