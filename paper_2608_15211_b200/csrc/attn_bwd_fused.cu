@@ -497,13 +497,14 @@ swin_bwd_fused_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
         *cta_abort = 0;
         fence_barrier_init();
     }
-    // the head's prepared bias table, and zeroed bias-gradient tables
-    for (int i = tid; i < kFwdBiasFloats; i += kThreads)
-        reinterpret_cast<float*>(smem + kOffBias)[i] = bias_prep[(size_t)head * kFwdBiasFloats + i];
+    // zeroed bias-gradient tables, and the head's prepared bias table
     for (int i = tid; i < 8 * kDBiasFloats; i += kThreads) reinterpret_cast<float*>(smem + kOffDBias)[i] = 0.f;
     // the shared dS tile starts finite: columns that no block writes only reach dQ rows that are never stored
     for (int i = tid; i < 4 * kDSGroupBytes / 4; i += kThreads) reinterpret_cast<uint32_t*>(smem + kOffDS)[i] = 0u;
     fence_proxy_async();
+    wait_for_prerequisites();      // delta, the bias tables
+    for (int i = tid; i < kFwdBiasFloats; i += kThreads)
+        reinterpret_cast<float*>(smem + kOffBias)[i] = bias_prep[(size_t)head * kFwdBiasFloats + i];
     if (warp == kIssuerWarp) {
         tmem_alloc(smem_u32(tmem_slot), 512);
         tmem_relinquish();
@@ -1022,6 +1023,7 @@ swin_bwd_dbias_finalize_kernel(const float* __restrict__ parts, float* __restric
     const int nw = 2 * w - 1;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;       // (table row, head)
     if (i >= nw * nw * heads) return;
+    wait_for_prerequisites();
     const int head = i % heads, r = i / heads;
     const int e = margin + (r / nw) * cs + (r % nw);
     float acc = 0.f;
@@ -1084,17 +1086,15 @@ cudaError_t launch_bwd_tc(const Geo& g, const void* q, const void* k, const void
     e = prepare_kernel((const void*)kern, kSmemBytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_bwd_fused_kernel", stream);
-    kern<<<grid, kThreads, kSmemBytes, stream>>>(
-        g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)d_o, prep, lse, delta,
-        (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, parts, items, (int)cph);
+    e = launch_dependent(kern, grid, kThreads, kSmemBytes, stream, g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v,
+                         (const __nv_bfloat16*)d_o, prep, lse, delta, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, parts, items, (int)cph);
     count_launch(stream);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int nrows = (2 * g.w - 1) * (2 * g.w - 1) * g.heads;
-    swin_bwd_dbias_finalize_kernel<<<(nrows + 255) / 256, 256, 0, stream>>>(parts, dbias, g.w, g.heads, (int)cph, pad ? dbias_margin(g.w) : 0,
-                                                                            pad ? 48 : g.w + 32);
+    e = launch_dependent(swin_bwd_dbias_finalize_kernel, (nrows + 255) / 256, 256, 0, stream, parts, dbias, g.w, g.heads, (int)cph,
+                         pad ? dbias_margin(g.w) : 0, pad ? 48 : g.w + 32);
     count_launch(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace terra

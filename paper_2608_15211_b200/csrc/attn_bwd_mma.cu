@@ -476,6 +476,12 @@ __device__ __forceinline__ void coef_t_times_block(float (&out)[D / 8][4], const
 // dim 128; the forward kernel, with four CTAs, gains nothing by it: 232 -> 240 us).  Five products of 64 x 64 x D on mma.sync take 2700 of about 3000 cycles that
 // the copies need at head dim 128.
 // 288 x 544 tokens, 8 x 128: 770 -> 575 us (68 % of the copy bandwidth); 128 x 256, 6 x 32: 55 -> 40 us.
+__global__ void swin_bwd_small_zero_kernel(float* __restrict__ dbias, int n) {
+    let_dependents_start();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) dbias[i] = 0.f;
+}
+
 template <int D>
 __device__ __host__ constexpr int small_tile_bytes() { return BN * D * 2; }
 template <int D>
@@ -709,6 +715,7 @@ swin_bwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
         for (int e = 0; e < 2; ++e)
             if (db_r[i][e] != 0.f) atomicAdd(mine + i * 16 - e, db_r[i][e]);
     __syncthreads();
+    wait_for_prerequisites();      // the zeroed table
     for (int i = tid; i < 15 * 16; i += NTHREADS) {
         const int da = (i >> 4) - 7, db = (i & 15) - 7;
         if (da > -g.w && da < g.w && db > -g.w && db < g.w && s_dbias[i] != 0.f)
@@ -722,6 +729,7 @@ __global__ void __launch_bounds__(256)
 swin_bwd_delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
                       float* __restrict__ delta, long long rows) {
     constexpr int LPR = D / 8;   // lanes per row, each lane takes one 16-byte chunk
+    let_dependents_start();
     long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long row = gid / LPR;
     int chunk = (int)(gid % LPR);
@@ -797,7 +805,10 @@ bool TERRA_ELEM_FN(bwd_small_supported)(const Geo& g) { return g.w <= 8; }
 cudaError_t TERRA_ELEM_FN(launch_bwd_small)(const Geo& g, const void* q, const void* k, const void* v, const void* o, const void* d_o,
                                             const float* bias, const float* lse, void* dq, void* dk, void* dv, float* dbias,
                                             int sm_count, cudaStream_t stream) {
-    cudaError_t e = cudaMemsetAsync(dbias, 0, sizeof(float) * (size_t)(2 * g.w - 1) * (2 * g.w - 1) * g.heads, stream);
+    const int entries = (2 * g.w - 1) * (2 * g.w - 1) * g.heads;
+    swin_bwd_small_zero_kernel<<<(entries + 255) / 256, 256, 0, stream>>>(dbias, entries);
+    count_launch(stream);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     auto kern = g.d == 32 ? swin_bwd_small_kernel<32> : g.d == 64 ? swin_bwd_small_kernel<64> : swin_bwd_small_kernel<128>;
     const size_t smem = g.d == 32 ? kSmallSmem<32> : g.d == 64 ? kSmallSmem<64> : kSmallSmem<128>;
@@ -810,11 +821,11 @@ cudaError_t TERRA_ELEM_FN(launch_bwd_small)(const Geo& g, const void* q, const v
     if (cph < 1) cph = 1;
     if (cph > items) cph = items;
     prof_begin("swin_bwd_small_kernel", stream);
-    kern<<<(unsigned)(cph * g.heads), NTHREADS, smem, stream>>>(
-        g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (const __nv_bfloat16*)o,
-        (const __nv_bfloat16*)d_o, bias, lse, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, dbias, (int)cph);
+    e = launch_dependent(kern, (unsigned)(cph * g.heads), NTHREADS, smem, stream, g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k,
+                         (const __nv_bfloat16*)v, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, bias, lse, (__nv_bfloat16*)dq,
+                         (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, dbias, (int)cph);
     count_launch(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t TERRA_ELEM_FN(launch_bwd_delta)(const Geo& g, const void* o, const void* d_o, float* delta, cudaStream_t stream) {

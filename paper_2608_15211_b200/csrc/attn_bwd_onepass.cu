@@ -111,6 +111,7 @@ struct Params {
     // the inner windows has the units of (row < row1, column < col1).
     int row1, col1, inner;
     int slab0;                       // first slab of the launch (two launches may overlap)
+    int overlap;                     // the launch runs beside the one before it, which started when its prerequisites were complete
     long long units;
     const float4* rowstat;           // per (b, window, head) and slot pair: (-lse log2 e) x 2, delta x 2
     const float* bias0;              // [head][2 rmax][2 RW]: bias log2 e at (da + rmax, db + RW), 0 outside the table
@@ -406,7 +407,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
     };
 
     // the launch of the masked windows may take the SMs that this one leaves (it waits for this one's end before its own)
-    if (KIND == 0) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (KIND == 0) let_dependents_start();
 
     if (warp < kWorkWarps) {
         // ------------------------------------------------------------------ elementwise: the half chunks of buffer b
@@ -937,7 +938,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
     __syncthreads();
     tc_fence_after();
     if (warp == kProductWarp) tmem_dealloc(tmem, 512);
-    if (KIND == 1) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    if (KIND == 1 && p.overlap) wait_for_prerequisites();
     if (tid == 0 && *cta_abort) atomicExch(&g_bwd_onepass_timeout, 1);
 }
 
@@ -1010,6 +1011,7 @@ template <int D, int RW>
 __global__ void __launch_bounds__(256)
 swin_bwd_onepass_finish_kernel(const Geo g, const float* __restrict__ dbias_acc, float* __restrict__ dbias, const float4* __restrict__ slabs,
                                __nv_bfloat16* __restrict__ dq, int npad, int rmax, int split_log2, unsigned bias_blocks) {
+    wait_for_prerequisites();
     if (blockIdx.x < bias_blocks) {
         const int nw = 2 * g.w - 1, i = blockIdx.x * 256 + threadIdx.x;
         if (i >= nw * nw * g.heads) return;
@@ -1175,21 +1177,19 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         p.inner = inner;
         p.units = windows * g.B * g.heads << pl.split_log2;
         p.slab0 = slab0;
+        p.overlap = overlap;
         cudaError_t err = prepare_kernel((const void*)kernel, L::kSmemBytes);
         if (err != cudaSuccess) return err;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(p.units < ctas ? p.units : ctas));
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = L::kSmemBytes;
-        cfg.stream = stream;
-        // the second launch needs nothing of the first: its CTAs take the SMs as the first one's leave them
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = overlap ? 1 : 0;
         prof_begin(overlap ? "swin_bwd_onepass_kernel<masked>" : "swin_bwd_onepass_kernel", stream);
-        err = cudaLaunchKernelEx(&cfg, kernel, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
+        const unsigned grid = (unsigned)(p.units < ctas ? p.units : ctas);
+        if (overlap) {
+            // needs nothing of the launch before it: its CTAs take the SMs as that one's leave them
+            err = launch_dependent(kernel, grid, kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
+        } else {
+            // (brought up beside the statistics kernel its CTAs are spread less well: 64 x 128 tokens, 8 x 64, 32 x 32 windows 211 instead of 168 us a step)
+            kernel<<<grid, kThreads, L::kSmemBytes, stream>>>(p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
+            err = cudaGetLastError();
+        }
         if (err == cudaSuccess) count_launch(stream);
         return err;
     };
@@ -1217,10 +1217,10 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     const unsigned bias_blocks = (unsigned)((nw * nw * g.heads + 255) / 256);
     const long long sum_blocks = pl.split_log2 ? (pl.units >> pl.split_log2) * ((pl.npad * D / 4 + 255) / 256) : 0;
     prof_begin("swin_bwd_onepass_finish_kernel", stream);
-    swin_bwd_onepass_finish_kernel<D, RW><<<(unsigned)(bias_blocks + sum_blocks), 256, 0, stream>>>(g, p.dbias_acc, dbias, p.slabs, (__nv_bfloat16*)dq,
-                                                                                                  pl.npad, pl.rmax, pl.split_log2, bias_blocks);
+    e = launch_dependent(swin_bwd_onepass_finish_kernel<D, RW>, (unsigned)(bias_blocks + sum_blocks), 256, 0, stream, g, p.dbias_acc, dbias, p.slabs,
+                         (__nv_bfloat16*)dq, pl.npad, pl.rmax, pl.split_log2, bias_blocks);
     count_launch(stream);
-    return cudaGetLastError();
+    return e;
 }
 }  // namespace
 

@@ -464,6 +464,7 @@ swin_fwd_tc_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    wait_for_prerequisites();                // the prepared bias tables
 
     const int cs = code_stride(g.w, PAD);
     const int c0 = (g.w - 1) * (cs + 1);     // code of the last in-window offset; bias index = code_q - code_k + c0
@@ -826,6 +827,7 @@ swin_fwd_tc_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_
 //   more than 64 octaves: the forward kernel then takes exact row maxima).
 __global__ void __launch_bounds__(256)
 swin_fwd_bias_prep_kernel(const float* __restrict__ bias, float* __restrict__ prep, int w, int heads, int cs) {
+    let_dependents_start();
     const int head = blockIdx.x;
     const int nw = 2 * w - 1;
     const int c0 = (w - 1) * (cs + 1);
@@ -857,6 +859,7 @@ swin_fwd_bias_prep_kernel(const float* __restrict__ bias, float* __restrict__ pr
         for (int i = 1; i < 8; ++i) { mx = fmaxf(mx, red[i]); mn = fminf(mn, red_mn[i]); }
         dst[kFwdBiasFloats - 1] = (mx - mn <= 64.f) ? mx : INFINITY;
     }
+    wait_for_prerequisites();      // what depends on this launch also depends on the one before it
 }
 
 }  // namespace
@@ -1014,10 +1017,10 @@ cudaError_t launch_fwd_tc(const Geo& g, const void* q, const void* k, const void
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)(items < sm_count ? items : sm_count);
     prof_begin("swin_fwd_tc_kernel", stream);
-    kern<<<grid, kThreads, kSmemBytes, stream>>>(g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, prep,
-                                                 (__nv_bfloat16*)o, lse, items, maps);
+    e = launch_dependent(kern, grid, kThreads, kSmemBytes, stream, g, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k,
+                         (const __nv_bfloat16*)v, prep, (__nv_bfloat16*)o, lse, items, maps);
     count_launch(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 #ifndef TERRA_ELEM_F16
@@ -1043,11 +1046,11 @@ cudaError_t launch_bounded_wait_selftest(long long limit_cycles, cudaStream_t st
     return cudaGetLastError();
 }
 
-// prepared bias tables for every head (also used by the backward kernels)
+// prepared bias tables for every head, for the backward; complete only when the launch before it (delta) is
 cudaError_t launch_bias_prep(const Geo& g, const float* bias, float* prep, cudaStream_t stream) {
-    swin_fwd_bias_prep_kernel<<<g.heads, 256, 0, stream>>>(bias, prep, g.w, g.heads, pad16_layout(g) ? 48 : g.w + 32);
+    const cudaError_t e = launch_dependent(swin_fwd_bias_prep_kernel, g.heads, 256, 0, stream, bias, prep, g.w, g.heads, pad16_layout(g) ? 48 : g.w + 32);
     count_launch(stream);
-    return cudaGetLastError();
+    return e;
 }
 
 #endif  // !TERRA_ELEM_F16

@@ -186,6 +186,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    wait_for_prerequisites();                      // the bias tables
     unsigned desc_n = 0;
     Unit td;
     // the next unit; false at the end of the run (or after an expired wait)
@@ -638,6 +639,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
 // The bias tables of all heads as the softmax threads read them: bias log2 e by row and column difference, two copies.
 template <int RW>
 __global__ void swin_fwd_win_prep_kernel(const Geo g, const float* __restrict__ bias, float* __restrict__ tables) {
+    let_dependents_start();
     const int per_head = Tab<RW>::rows(g.w) * Tab<RW>::kRowF, total = per_head * g.heads, nw = 2 * g.w - 1;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int head = i / per_head, e = i - head * per_head, row = e / Tab<RW>::kRowF, f = e - row * Tab<RW>::kRowF;
@@ -696,9 +698,9 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
     cudaError_t e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW>, L::kSmemBytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_fwd_win_kernel", stream);
-    swin_fwd_win_kernel<D, RW><<<(unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream>>>(p, (__nv_bfloat16*)o, lse, mq, mk, mv);
+    e = launch_dependent(swin_fwd_win_kernel<D, RW>, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
     count_launch(stream);
-    return cudaGetLastError();
+    return e;
 }
 }  // namespace
 

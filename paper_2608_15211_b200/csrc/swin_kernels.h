@@ -13,6 +13,24 @@ void count_launch(cudaStream_t stream);   // after every launch: bumps the launc
 // count_launch closes.  Does nothing unless profiling is enabled.
 void prof_begin(const char* name, cudaStream_t stream);
 
+// Launches `kernel` so that it may be brought up (barriers, tensor memory, shared memory) while the launch before it in the stream is
+// still running; the kernel calls wait_for_prerequisites() before it touches what that launch reads or writes.  A chain of
+// small kernels loses 2 to 3 us less at each joint.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A&&... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Before a kernel's launch: allows it `smem` bytes of dynamic shared memory on the current device and, where `occupancy` is
 // given, says how many CTAs of `threads` threads fit an SM.  Each thread remembers its last few kernels: the two runtime
 // calls cost more host time than the launch of a small kernel.
