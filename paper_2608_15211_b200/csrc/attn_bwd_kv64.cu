@@ -1,6 +1,5 @@
-// Key side of the backward pass (dK, dV) on the tcgen05 tensor cores for head dims 64 and 128 and windows of up to
-// 1024 tokens (window side <= 32).  The query side (dQ, dBias) of this regime runs its own tcgen05 kernel on grids of
-// complete 32 x 32 windows and the register-tile kernel otherwise.
+// Backward pass of complete windows of side 64 and 128 (4096 and 16 384 tokens) on the tcgen05 tensor cores, head dims 64 and
+// 128: the key side (dK, dV), and with the tensors' roles exchanged the query side (dQ, dBias).
 //
 // One persistent CTA per SM, bound to one head, walks over (batch, window, 128-key tile) items.  The tile's K and V
 // rows stay in shared memory; the window's queries stream through a ring of slots in chunks of 128 (Q, dO rows and
@@ -12,9 +11,8 @@
 //   dV += P^T dO_c, dK += dS^T Q_c                                   (A from TMEM, B = the chunk's rows, MN-major)
 // P is recomputed from the saved log-sum-exp, so the chunks are independent.
 // Roles: warps 0-7 elementwise (warps w and w + 4 share TMEM lane quarter w & 3 and take the chunk's first / second
-// 64 query columns), warp 8 issues every MMA, warps 9-11 load rows (bulk copies from warp 9 on grids of complete
-// windows, else cp.async gathers from all three).  A row is kept as head dim / 32 parts of 32 columns in the
-// 64-byte-swizzled operand layout, as in the forward kernel of this regime.
+// 64 query columns), warp 8 issues every MMA, warp 9 loads rows by bulk copies.  A row is kept as head dim / 32 parts of 32
+// columns in the 64-byte-swizzled operand layout, as in the forward kernel of this regime.
 // Half chunks rotate through TMEM buffers (S^T 64 columns | dP^T 64 columns): three at head dim 64, so that the scores of
 // a group's next half chunk are issued while it still works on the current one, two at head dim 128, where the
 // accumulators dV and dK (head dim columns each, behind the buffers) take the rest of the 512 columns.
@@ -47,7 +45,6 @@ using namespace tc;
 
 constexpr int kMmaWarp = 8;
 constexpr int kLoaderWarp0 = 9;
-constexpr int kLoaderThreads = 96;
 constexpr int kThreads = 384;
 constexpr int kWorkThreads = 256;
 constexpr int kRegsLaunch = 168, kRegsWork = 208, kRegsOther = 80;
@@ -157,23 +154,15 @@ __device__ __forceinline__ int lds_i32(uint32_t addr) {
 // 16 query columns [c, c + 16) of one key row: P = exp2(S scale + bias - lse), dS = P (dP - delta), packed to bf16.
 // `bias_row` = shared address of the bias table + the key row's part of the index (the -inf zone if the row has no
 // token); a query column without a token has lse = +inf, so its P is 0.
-// ROW32: the window is 32 tokens wide, so the group's 16 queries sit in one window row and their bias codes are
-// consecutive: `code4` = 4 * code of column c, no per-query code table is read.
+// The group's 16 queries sit in one window row and their bias entries are consecutive from bias_row + code4 on.
 // `sl_a` = shared address of the slot's per-query tables (code, label, lse, delta: TAB bytes each); c counts within the slot.
-template <bool MASKED, bool ROW32, int TAB>
+template <bool MASKED, int TAB>
 __device__ __forceinline__ void cols16(const uint32_t (&rs)[16], const uint32_t (&rp)[16], int c, uint32_t bias_row, int klabel,
-                                       uint32_t sl_a, float scale, uint32_t (&pk_p)[8], uint32_t (&pk_ds)[8], int code4 = 0) {
-    constexpr int kOffQCode = 0, kOffQLab = TAB, kOffQLse = 2 * TAB, kOffQDelta = 3 * TAB;
+                                       uint32_t sl_a, float scale, uint32_t (&pk_p)[8], uint32_t (&pk_ds)[8], int code4) {
+    constexpr int kOffQLab = TAB, kOffQLse = 2 * TAB, kOffQDelta = 3 * TAB;
     // all table loads first (they are issued in program order), then the gathers that depend on them, then the math
-    int co[16], ql[16];
+    int ql[16];
     float l2[16], dl[16], bv[16];
-    if (!ROW32) {
-#pragma unroll
-        for (int e4 = 0; e4 < 4; ++e4) {
-            const int4 c4 = lds_i4(sl_a + kOffQCode + 4 * (c + e4 * 4));
-            co[e4 * 4] = c4.x; co[e4 * 4 + 1] = c4.y; co[e4 * 4 + 2] = c4.z; co[e4 * 4 + 3] = c4.w;
-        }
-    }
 #pragma unroll
     for (int e4 = 0; e4 < 4; ++e4) {
         const float4 a = lds_f4(sl_a + kOffQLse + 4 * (c + e4 * 4));
@@ -189,7 +178,7 @@ __device__ __forceinline__ void cols16(const uint32_t (&rs)[16], const uint32_t 
         }
     }
 #pragma unroll
-    for (int e = 0; e < 16; ++e) bv[e] = ROW32 ? lds_f32(bias_row + code4 + 4 * e) : lds_f32(bias_row + co[e]);
+    for (int e = 0; e < 16; ++e) bv[e] = lds_f32(bias_row + code4 + 4 * e);
     // two-wide fp32 operations: one instruction per pair of columns
     float p[16], ds[16];
 #pragma unroll
@@ -262,17 +251,12 @@ struct KvMaps64 {
     RowMaps3 q, k, v, g;      // g: the output gradient dO
 };
 
-// TMA: complete windows of side 16 or 32 and a longitude shift that is a multiple of 8: one loader warp fetches every
-// window row with tiled bulk copies (per-query lse and delta by 4-byte cp.async copies tied to the same barrier);
-// otherwise three loader warps gather the rows with 16-byte cp.async copies.  (Gathering the dO rows with the two
-// idle warps next to the bulk copies, as the forward kernel does with V, was measured and is slightly slower here.)
-//
-// MODE 0: gathered rows.  MODE 1: bulk-copied rows, window side 16 or 32, the head's whole bias table in shared memory.
-// MODE 2: bulk-copied rows, complete windows of side 64 or 128: the table does not fit, and the loader warp stages,
-// with every query chunk, the 2 kr - 1 table rows (kr = 128 / w window rows per 128 slots) that the chunk's queries
-// need against the item's key tile; in the prepared layout (2 w floats per table row) they are one contiguous block,
-// and the 16 queries of a column group read consecutive entries, as in the 32-wide case.
-// MODE 3: MODE 2 put to use for the query side (dQ, dBias) of such windows.  The host hands over the tensors with the
+// Complete windows of side 64 and 128 and a longitude shift that is a multiple of 8: one loader warp fetches every
+// window row with tiled bulk copies (per-query lse and delta by 4-byte cp.async copies tied to the same barrier).  The bias table
+// does not fit shared memory; the loader warp stages, with every query chunk, the 2 kr - 1 table rows (kr = 128 / w window
+// rows per 128 slots) that the chunk's queries need against the item's key tile; in the prepared layout (2 w floats per
+// table row) they are one contiguous block, and the 16 queries of a column group read consecutive entries.
+// QS: the kernel put to use for the query side (dQ, dBias) of such windows.  The host hands over the tensors with the
 // roles exchanged (Q and dO as the "key tile", K and V as the streamed "queries") and the bias table reflected through
 // its centre, so that rows are queries and columns keys: S = Q K_c^T, dP = dO V_c^T, dS as above with the row's own
 // lse and delta, and the accumulator that is dK in the key-side use is dQ = dS K_c; the other one is not computed.
@@ -281,7 +265,7 @@ struct KvMaps64 {
 // The block has 95 diagonals; each is summed in one of three accumulators of one lane: a column's 32 values reach
 // their diagonals' lanes with one rotation of the warp (one shuffle per element, no chain between columns), and after
 // the half chunk the lanes add their accumulators to the global gradient: 95 float atomics per warp and half chunk.
-template <int D, int MODE>
+template <int D, bool QS>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
                      const __nv_bfloat16* __restrict__ v, const __nv_bfloat16* __restrict__ d_o,
@@ -289,8 +273,7 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                      __nv_bfloat16* __restrict__ dk, __nv_bfloat16* __restrict__ dv, float* __restrict__ dbias, long long n_items,
                      int ctas_per_head, int max_tiles, const __grid_constant__ KvMaps64 maps) {
     using L = Lay<D>;
-    constexpr bool TMA = MODE >= 1, ROWS = MODE >= 2, QS = MODE == 3;
-    constexpr int kStageBytes = 1536;                 // MODE 2: the staged table rows of one query slot
+    constexpr int kStageBytes = 1536;                 // the staged table rows of one query slot
     constexpr int kHPS = L::kHPS, kSlotQ = L::kSlotQ, kSPart = L::kSPart, kTab = L::kTab;
     constexpr int kParts = L::kParts, kKvStages = L::kKvStages, kSlots = L::kSlots;
     constexpr int kOffK = L::kOffK, kOffV = L::kOffV, kOffKCode = L::kOffKCode, kOffKLab = L::kOffKLab, kOffKTok = L::kOffKTok;
@@ -323,11 +306,11 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
 
     if (tid == 0) {
         for (int s = 0; s < kKvStages; ++s) {
-            mbar_init(bar_kvfull(s), TMA ? 32 : kLoaderThreads);
+            mbar_init(bar_kvfull(s), 32);
             mbar_init(bar_kvempty(s), 1 + kWorkThreads);   // the issuer's commit + every elementwise thread
         }
         for (int s = 0; s < kSlots; ++s) {
-            mbar_init(bar_qfull(s), TMA ? 32 : kLoaderThreads);
+            mbar_init(bar_qfull(s), 32);
             mbar_init(bar_qempty(s), 1);
         }
         for (int b = 0; b < kBufs; ++b) {
@@ -338,10 +321,6 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
         mbar_init(bar_accfree, kWorkThreads);
         *cta_abort = 0;
         fence_barrier_init();
-    }
-    if (!ROWS) {
-        for (int i = tid; i < kBiasFloats; i += kThreads)
-            reinterpret_cast<float*>(smem + kOffBias)[i] = bias_prep[(size_t)head * kBiasFloats + i];
     }
     fence_proxy_async();
     if (warp == kMmaWarp) {
@@ -359,8 +338,8 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
 
     if (warp >= kMmaWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsOther));
-    if (TMA && warp >= kLoaderWarp0) {
-        // ------------------------------------------------------------------ loader warp (TMA); the other two have no work
+    if (warp >= kLoaderWarp0) {
+        // ------------------------------------------------------------------ loader warp; the other two have no work
         if (warp == kLoaderWarp0) {
             const int wrows = max(1, kTile / g.w);            // window rows per 128 slots
             int kuse = 0;
@@ -391,21 +370,12 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                         reinterpret_cast<int*>(st + kOffKTok)[row] = tok;
                     }
                     const uint32_t sb = smem0 + ks * kKvStageBytes;
-                    if (!ROWS && g.w == 32) {
-                        // one lane per tensor and part: the tile's four window rows, in groups where the copies allow it
-                        for (int i = lane; i < 2 * kParts; i += 32) {
-                            const int tsr = i >= kParts ? 1 : 0, part = i - tsr * kParts;
-                            bulk_copy_window_rows(tsr ? maps.v : maps.k, sb + (tsr ? kOffV : kOffK) + part * kPart, g, x.b, x.r.wr, v0,
-                                                  x.kt * wrows, wrows, head * D + part * 32, bar_kvfull(ks));
-                        }
-                    } else {
-                        const int per_tensor = wrows * kParts;
-                        for (int i = lane; i < 2 * per_tensor; i += 32) {
-                            const int tsr = i >= per_tensor ? 1 : 0, rem = i - tsr * per_tensor;
-                            const int ar = rem / kParts, part = rem - ar * kParts;
-                            bulk_copy_window_row(tsr ? maps.v : maps.k, sb + (tsr ? kOffV : kOffK) + part * kPart + ar * g.w * kPartBytes, g,
-                                                 x.b, x.r.wr, v0, x.kt * wrows + ar, head * D + part * 32, bar_kvfull(ks));
-                        }
+                    const int per_tensor = wrows * kParts;
+                    for (int i = lane; i < 2 * per_tensor; i += 32) {
+                        const int tsr = i >= per_tensor ? 1 : 0, rem = i - tsr * per_tensor;
+                        const int ar = rem / kParts, part = rem - ar * kParts;
+                        bulk_copy_window_row(tsr ? maps.v : maps.k, sb + (tsr ? kOffV : kOffK) + part * kPart + ar * g.w * kPartBytes, g,
+                                             x.b, x.r.wr, v0, x.kt * wrows + ar, head * D + part * 32, bar_kvfull(ks));
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive_expect_tx(bar_kvfull(ks), (uint32_t)(kTile * D * 2 * 2));
@@ -434,23 +404,14 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                         reinterpret_cast<int*>(sl + kOffQCode)[row] = 4 * code;
                         reinterpret_cast<int*>(sl + kOffQLab)[row] = label;
                     }
-                    if (!ROWS && g.w == 32) {
-                        // whole window rows: one lane per tensor and part, groups of window rows where the copies allow it
-                        for (int j = lane; j < 2 * kParts; j += 32) {
-                            const int tsr = j >= kParts ? 1 : 0, part = j - tsr * kParts;
-                            bulk_copy_window_rows(tsr ? maps.g : maps.q, sb + (tsr ? kOffG : kOffQ) + part * kSPart, g, x.b, x.r.wr, v0,
-                                                  slot0 / 32, runs, head * D + part * 32, bar_qfull(s));
-                        }
-                    } else {
-                        for (int j = lane; j < 2 * runs * kParts; j += 32) {
-                            const int tsr = j >= runs * kParts ? 1 : 0, rem = j - tsr * runs * kParts;
-                            const int rr = rem / kParts, part = rem - rr * kParts;
-                            const int rslot = slot0 + rr * n_run, a = rslot / g.w;
-                            bulk_copy_window_run(tsr ? maps.g : maps.q, sb + (tsr ? kOffG : kOffQ) + part * kSPart + rr * n_run * kPartBytes, g,
-                                                 x.b, x.r.wr, v0, a, rslot - a * g.w, n_run, head * D + part * 32, bar_qfull(s));
-                        }
+                    for (int j = lane; j < 2 * runs * kParts; j += 32) {
+                        const int tsr = j >= runs * kParts ? 1 : 0, rem = j - tsr * runs * kParts;
+                        const int rr = rem / kParts, part = rem - rr * kParts;
+                        const int rslot = slot0 + rr * n_run, a = rslot / g.w;
+                        bulk_copy_window_run(tsr ? maps.g : maps.q, sb + (tsr ? kOffG : kOffQ) + part * kSPart + rr * n_run * kPartBytes, g,
+                                             x.b, x.r.wr, v0, a, rslot - a * g.w, n_run, head * D + part * 32, bar_qfull(s));
                     }
-                    if (ROWS && lane == 0) {
+                    if (lane == 0) {
                         // the table rows that this slot's ur window rows need against the key tile's kr window rows
                         const int lw = 31 - __clz(g.w), kr = kTile >> lw, ur = max(1, kSlotQ >> lw);
                         const int r0 = (slot0 >> lw) - x.kt * kr - (kr - 1) + g.w - 1;
@@ -466,121 +427,6 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                 }
                 ++kuse;
             }
-        }
-    } else if (warp >= kLoaderWarp0) {
-        // ------------------------------------------------------------------ loaders
-        // D / 32 lanes per row (one 32-column part of the row each, four 16-byte copies).  A thread never waits for
-        // data: its arrival on a stage's or slot's barrier is tied to the completion of the copies it has issued.
-        const int lt = (warp - kLoaderWarp0) * 32 + lane;
-        const int hf = lt % kParts;
-        const int lrow = lt / kParts;
-        constexpr int kRowsPerIter = kLoaderThreads / kParts;
-        int kuse = 0;
-        unsigned ru = 0;                                      // half chunks so far
-        bool ok = true;
-        auto acquire = [&](uint32_t bar, uint32_t parity) -> bool { return mbar_wait_all(bar, parity, cta_abort); };
-        // the thread's table entries are visible to the CTA before its arrival, which follows its copies
-        auto issued = [&](uint32_t bar) {
-            __threadfence_block();
-            cp_async_mbar_arrive_noinc(bar);
-        };
-        ItemCursor cur = cursor_init(cta_in_head, ctas_per_head, max_tiles, g.Mw, g.Mh);
-        for (long long it = cta_in_head; ok && it < n_items; it += ctas_per_head, cursor_advance(cur, max_tiles, g.Mw, g.Mh)) {
-            const Item x = make_item(g, cur);
-            if (!x.has) continue;
-            const int ks = kuse % kKvStages;
-            ok = acquire(bar_kvempty(ks), ((kuse / kKvStages) & 1) ^ 1);
-            if (!ok) break;
-            const size_t sample_off = (size_t)x.b * HW;
-            const int ew = x.r.ew;
-            const int q_r = kRowsPerIter / ew, r_r = kRowsPerIter - q_r * ew;
-            // ---- the key tile: K, V rows (rows without a token as zeros) and the key tables
-            {
-                unsigned char* st = smem + ks * kKvStageBytes;
-                const uint32_t sb = smem0 + ks * kKvStageBytes + hf * kPart;
-                const int slot0 = x.kt * kTile;
-                for (int row = lt; row < kTile; row += kLoaderThreads) {
-                    const int slot = slot0 + row;
-                    int code = 0, label = 0xff, tok = -1;
-                    if (slot < x.r.n) {
-                        const int a = slot / ew;
-                        tok = offset_token(g, x.r, a, slot - a * ew, code, label);
-                    }
-                    reinterpret_cast<int*>(st + kOffKCode)[row] = 4 * code;
-                    reinterpret_cast<int*>(st + kOffKLab)[row] = label;
-                    reinterpret_cast<int*>(st + kOffKTok)[row] = tok;
-                }
-                int a_r = (slot0 + lrow) / ew, b_r = (slot0 + lrow) - a_r * ew;
-                for (int row = lrow; row < kTile; row += kRowsPerIter, a_r += q_r, b_r += r_r) {
-                    if (b_r >= ew) { b_r -= ew; ++a_r; }
-                    const __nv_bfloat16 *sk = k, *sv = v;
-                    int bytes = 0;
-                    if (slot0 + row < x.r.n) {
-                        int code, label;
-                        const int tok = offset_token(g, x.r, a_r, b_r, code, label);
-                        const size_t off = (sample_off + (size_t)tok) * g.ts + head * D + hf * 32;
-                        sk = k + off; sv = v + off;
-                        bytes = 16;
-                    }
-#pragma unroll
-                    for (int c4 = 0; c4 < 4; ++c4) {
-                        const uint32_t so = tile_off<32>(row, c4);
-                        cp_async16(sb + kOffK + so, bytes ? sk + c4 * 8 : sk, bytes);
-                        cp_async16(sb + kOffV + so, bytes ? sv + c4 * 8 : sv, bytes);
-                    }
-                }
-                issued(bar_kvfull(ks));
-            }
-            // ---- the window's queries, slot by slot (the last one may be partly filled)
-            const int nu = (x.npad + kSlotQ - 1) / kSlotQ;
-            for (int i = 0; i < nu; ++i, ++ru) {
-                const int s = (int)(ru % kSlots);
-                ok = acquire(bar_qempty(s), (uint32_t)((ru / kSlots) & 1) ^ 1u);
-                if (!ok) break;
-                unsigned char* sl = smem + kOffSlots + s * kSlotBytes;
-                const uint32_t sb = smem0 + kOffSlots + s * kSlotBytes + hf * kSPart;
-                const int slot0 = i * kSlotQ;
-                const int ncols = min(kSlotQ, x.npad - slot0);
-                for (int row = lt; row < kSlotQ; row += kLoaderThreads) {
-                    const int slot = slot0 + row;
-                    int code = 0, label = 0xff;
-                    if (slot < x.r.n) {
-                        // lse and delta travel with the rows (no load the loader would have to wait for)
-                        const int a = slot / ew;
-                        const int tok = offset_token(g, x.r, a, slot - a * ew, code, label);
-                        const size_t li = (sample_off + (size_t)tok) * g.heads + head;
-                        cp_async4(smem0 + kOffSlots + s * kSlotBytes + kOffQLse + 4 * row, lse + li);
-                        cp_async4(smem0 + kOffSlots + s * kSlotBytes + kOffQDelta + 4 * row, delta + li);
-                    } else {
-                        reinterpret_cast<float*>(sl + kOffQLse)[row] = INFINITY;   // no token: P = exp2(.. - inf) = 0
-                        reinterpret_cast<float*>(sl + kOffQDelta)[row] = 0.f;
-                    }
-                    reinterpret_cast<int*>(sl + kOffQCode)[row] = 4 * code;
-                    reinterpret_cast<int*>(sl + kOffQLab)[row] = label;
-                }
-                const int slot_first = slot0 + lrow;
-                int a_r = slot_first / ew, b_r = slot_first - a_r * ew;
-                for (int row = lrow; row < ncols; row += kRowsPerIter, a_r += q_r, b_r += r_r) {
-                    if (b_r >= ew) { b_r -= ew; ++a_r; }
-                    const __nv_bfloat16 *sq = q, *sg = d_o;
-                    int bytes = 0;
-                    if (slot0 + row < x.r.n) {
-                        int code, label;
-                        const int tok = offset_token(g, x.r, a_r, b_r, code, label);
-                        sq = q + (sample_off + (size_t)tok) * g.ts + head * D + hf * 32;
-                        sg = d_o + ((sample_off + (size_t)tok) * g.heads + head) * D + hf * 32;
-                        bytes = 16;
-                    }
-#pragma unroll
-                    for (int c4 = 0; c4 < 4; ++c4) {
-                        const uint32_t so = tile_off<32>(row, c4);
-                        cp_async16(sb + kOffQ + so, bytes ? sq + c4 * 8 : sq, bytes);
-                        cp_async16(sb + kOffG + so, bytes ? sg + c4 * 8 : sg, bytes);
-                    }
-                }
-                issued(bar_qfull(s));
-            }
-            ++kuse;
         }
     } else {
         // ------------------------------------------------------------------ MMA issuer
@@ -731,7 +577,7 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
             const int klabel = lds_i32(st_a + kOffKLab + 4 * krow);
             const int ktok = lds_i32(st_a + kOffKTok + 4 * krow);
             mbar_arrive(bar_kvempty(ks));                 // this thread has what it needs from the key stage
-            // MODE 3: the row is a query; its lse and delta
+            // QS: the row is a query; its lse and delta
             float neg_l2 = 0.f, row_dl = 0.f;
             if (QS) {
                 const size_t li = ((size_t)x.b * HW + (size_t)ktok) * g.heads + head;
@@ -740,13 +586,10 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
             }
             // bias index = code_query - code_key + c0; a key row without a token reads the table's -inf zone
             uint32_t bias_row = smem0 + kOffBias + (ktok >= 0 ? 4 * c0 - kcode4 : 4 * (2 * c0 + 1));
-            const bool row32 = ROWS || x.r.ew == 32;
             const int lw = 31 - __clz(g.w);
-            if (ROWS) {
-                // relative to a slot's stage: this key's window row within the tile and its column
-                const int kslot = x.kt * kTile + krow, kr = kTile >> lw;
-                bias_row = smem0 + kOffBias + (kr - 1 - ((kslot >> lw) - ((x.kt * kTile) >> lw))) * 8 * g.w + 4 * (g.w - 1 - (kslot & (g.w - 1)));
-            }
+            // relative to a slot's stage: this key's window row within the tile and its column
+            const int kslot = x.kt * kTile + krow, kr = kTile >> lw;
+            bias_row = smem0 + kOffBias + (kr - 1 - ((kslot >> lw) - ((x.kt * kTile) >> lw))) * 8 * g.w + 4 * (g.w - 1 - (kslot & (g.w - 1)));
             for (int c = 0; c < x.nch && ok; ++c) {
                 const int ncols = min(kTile, x.npad - c * kTile);
                 if (ncols <= 64 * hcol) continue;          // this group's half of the chunk does not exist
@@ -762,10 +605,9 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                 const uint32_t t_s = tmem_base + lane_addr + kBufCols * buf, t_dp = t_s + 64;
                 const int col_end = min(ncols - 64 * hcol, 64);
                 // 4 * bias code of query column `col` of this half chunk in a 32-wide window: slot = 128 c + 64 hcol + col = 32 a + b
-                // (MODE 2: the offset into the slot's staged table rows; the half chunk lies in one window row)
+                // (the offset into the slot's staged table rows; the half chunk lies in one window row)
                 auto code4_of = [&](int col) {
-                    return ROWS ? s * kStageBytes + (((sc0 + col) >> lw) * 2 * g.w + ((64 * hcol + col) & (g.w - 1))) * 4
-                                : 4 * ((4 * c + 2 * hcol + (col >> 5)) * cs + (col & 31));
+                    return s * kStageBytes + (((sc0 + col) >> lw) * 2 * g.w + ((64 * hcol + col) & (g.w - 1))) * 4;
                 };
                 // groups of 16 columns; the next group's S^T / dP^T travel from TMEM while this one is worked on
                 uint32_t rs[16], rp[16], rs2[16], rp2[16], pk_p[8], pk_ds[8];
@@ -822,10 +664,8 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                         tmem_ld16(t_s + cc + 16, rs2);
                         tmem_ld16(t_dp + cc + 16, rp2);
                     }
-                    if (ROWS && x.masked) cols16<true, true, kTab>(rs, rp, cc, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc));
-                    else if (x.masked) cols16<true, false, kTab>(rs, rp, cc, bias_row, klabel, sl_a, scale, pk_p, pk_ds);
-                    else if (row32) cols16<false, true, kTab>(rs, rp, cc, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc));
-                    else cols16<false, false, kTab>(rs, rp, cc, bias_row, klabel, sl_a, scale, pk_p, pk_ds);
+                    if (x.masked) cols16<true, kTab>(rs, rp, cc, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc));
+                    else cols16<false, kTab>(rs, rp, cc, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc));
                     tmem_st8(t_s + cc, pk_p);              // 16 queries -> 8 packed columns at the group's own place
                     tmem_st8(t_dp + cc, pk_ds);
                     if (cc + 16 < col_end) {
@@ -834,10 +674,8 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                             tmem_ld16(t_s + cc + 32, rs);
                             tmem_ld16(t_dp + cc + 32, rp);
                         }
-                        if (ROWS && x.masked) cols16<true, true, kTab>(rs2, rp2, cc + 16, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc + 16));
-                        else if (x.masked) cols16<true, false, kTab>(rs2, rp2, cc + 16, bias_row, klabel, sl_a, scale, pk_p, pk_ds);
-                        else if (row32) cols16<false, true, kTab>(rs2, rp2, cc + 16, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc + 16));
-                        else cols16<false, false, kTab>(rs2, rp2, cc + 16, bias_row, klabel, sl_a, scale, pk_p, pk_ds);
+                        if (x.masked) cols16<true, kTab>(rs2, rp2, cc + 16, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc + 16));
+                        else cols16<false, kTab>(rs2, rp2, cc + 16, bias_row, klabel, sl_a, scale, pk_p, pk_ds, code4_of(cc + 16));
                         tmem_st8(t_s + cc + 16, pk_p);
                         tmem_st8(t_dp + cc + 16, pk_ds);
                     }
@@ -913,24 +751,14 @@ cudaError_t read_bwd_kv64_status(int* timed_out) {
     return e;
 }
 
-namespace {
-bool no_tma_env() {
-    static const bool off = [] { const char* e_ = std::getenv("TERRA_NO_TMA"); return e_ && e_[0] == '1'; }();
-    return off;
-}
-}  // namespace
-
 #ifndef TERRA_ELEM_F16
-// window sides up to 32 on any grid; sides 64 and 128 on grids of complete windows that the bulk-copy loader serves
+// window sides 64 and 128 on grids of complete windows that the bulk-copy loader serves
 bool bwd_kv64_supported(const Geo& g) {
-    if (!(g.d == 64 || g.d == 128) || g.heads > 148) return false;
-    if (g.w <= 32) return g.nmax <= 1024;
-    return (g.w == 64 || g.w == 128) && bulk_rows_shape(g);
+    return (g.d == 64 || g.d == 128) && g.heads <= 148 && (g.w == 64 || g.w == 128) && bulk_rows_shape(g);
 }
 #endif  // !TERRA_ELEM_F16
 
-// `prep` = the prepared bias tables of the head-dim-64 forward kernel (kBiasFloats per head; for window sides 64 and
-// 128 its layout of whole table rows), filled by the caller
+// `prep` = the prepared bias tables of the head-dim-64 forward kernel (whole table rows), filled by the caller
 static cudaError_t launch_kv64(const Geo& g, const void* q, const void* k, const void* v, const void* d_o, const float* prep,
                                const float* lse, const float* delta, void* dk, void* dv, float* dbias, bool qside, int sm_count,
                                cudaStream_t stream);
@@ -946,7 +774,6 @@ cudaError_t launch_bwd_kv64(const Geo& g, const void* q, const void* k, const vo
 cudaError_t launch_bwd_kv64_qside(const Geo& g, const void* q, const void* k, const void* v, const void* d_o,
                                   const float* prep_reflected, const float* lse, const float* delta, void* dq, float* dbias,
                                   int sm_count, cudaStream_t stream) {
-    if (g.w <= 32) return cudaErrorNotSupported;
     cudaError_t e = cudaMemsetAsync(dbias, 0, sizeof(float) * (size_t)(2 * g.w - 1) * (2 * g.w - 1) * g.heads, stream);
     if (e != cudaSuccess) return e;
     return launch_kv64(g, q, k, v, d_o, prep_reflected, lse, delta, dq, nullptr, dbias, true, sm_count, stream);
@@ -962,16 +789,15 @@ static cudaError_t launch_kv64(const Geo& g, const void* q, const void* k, const
     if (cph > items) cph = items;
     KvMaps64 maps;
     std::memset(&maps, 0, sizeof maps);
-    const bool rows = g.w > 32;
     // the kernel's tile rows ("k", "v") and streamed rows ("q", "g"); the query side exchanges the roles
-    const bool tma = (!no_tma_env() || rows) && bulk_rows_shape(g) &&
+    const bool tma = bulk_rows_shape(g) &&
                      (qside ? make_row_maps3(&maps.k, g, q, g.ts) && make_row_maps3(&maps.v, g, d_o, g.heads * g.d) &&
                                   make_row_maps3(&maps.q, g, k, g.ts) && make_row_maps3(&maps.g, g, v, g.ts)
                             : make_row_maps3(&maps.q, g, q, g.ts) && make_row_maps3(&maps.k, g, k, g.ts) &&
                                   make_row_maps3(&maps.v, g, v, g.ts) && make_row_maps3(&maps.g, g, d_o, g.heads * g.d));
-    if ((rows || qside) && !tma) return cudaErrorNotSupported;       // windows of side 64 and 128 have no gathering loader
-    auto kern = g.d == 64 ? (qside ? swin_bwd_kv64_kernel<64, 3> : rows ? swin_bwd_kv64_kernel<64, 2> : tma ? swin_bwd_kv64_kernel<64, 1> : swin_bwd_kv64_kernel<64, 0>)
-                          : (qside ? swin_bwd_kv64_kernel<128, 3> : rows ? swin_bwd_kv64_kernel<128, 2> : tma ? swin_bwd_kv64_kernel<128, 1> : swin_bwd_kv64_kernel<128, 0>);
+    if (!tma) return cudaErrorNotSupported;
+    auto kern = g.d == 64 ? (qside ? swin_bwd_kv64_kernel<64, true> : swin_bwd_kv64_kernel<64, false>)
+                          : (qside ? swin_bwd_kv64_kernel<128, true> : swin_bwd_kv64_kernel<128, false>);
     const int smem_bytes = g.d == 64 ? Lay<64>::kSmemBytes : Lay<128>::kSmemBytes;
     cudaError_t e = prepare_kernel((const void*)kern, smem_bytes);
     if (e != cudaSuccess) return e;

@@ -5,8 +5,8 @@
 // Roll, window gather, shift mask, relative-position bias, softmax, PV and the scatter back to the
 // contiguous grid all happen here; nothing window-major is ever written to global memory.
 // The file is compiled for bf16 and, through attn_fwd_mma_f16.cu, for fp16 activations.
-// This path covers every window class (truncated edges, the split latitude-wrap row, w up to 32,
-// head dim 32 / 64 / 128; head dim 128, the width of the paper's Table V models, runs here only).
+// The first kernel covers every window class (truncated edges, the split latitude-wrap row, every side and head dim); what runs
+// there is sides 33 .. 128 that the tcgen05 kernels do not take.
 #include "swin_common.cuh"
 #include "swin_kernels.h"
 

@@ -1,6 +1,5 @@
-// Forward shifted-window attention on the tcgen05 tensor cores for head dims 64 and 128 in the large-window regime,
-// where a score row no longer fits tensor memory: windows of up to 1024 tokens (window side <= 32) on any grid, and
-// complete windows of side 64 and 128 (4096 and 16 384 tokens) whose rows the bulk-copy loader can fetch.
+// Forward shifted-window attention on the tcgen05 tensor cores for head dims 64 and 128 and complete windows of side 64 and
+// 128 (4096 and 16 384 tokens) whose rows the bulk-copy loader can fetch.
 //
 // One persistent CTA per SM, bound to one head, walks over (batch, window, pair of 128-row query tiles) items.
 // The window's keys are streamed once, in chunks of 128, through a ring of shared-memory slots.  Per chunk:
@@ -14,11 +13,9 @@
 //   ones behind V make the accumulator's columns 64..79 carry the row sums; at head dim 128 tensor memory has no
 //   columns left for them and the softmax threads add the row sums themselves).
 // Roles: warps 0-3 / 4-7 softmax warpgroups (one thread per query row of the pair's first / second tile),
-// warp 8 issues every tcgen05.mma (whole warp runs the loop, one elected lane issues), warps 9-11 load rows, undoing
-// the roll: on grids of complete windows warp 9 fetches Q and K rows with tiled bulk copies, and the V rows come from
-// warp 10 by bulk copies of large boxes (window sides 32, 64, 128: four window rows, or one, per copy) or are gathered
-// by warps 10-11 with cp.async (window side 16); otherwise all three gather with cp.async.  A row is kept as head dim / 32 parts of 32 columns in
-// the 64-byte-swizzled operand layout of the small-window kernels, so that the same descriptors serve.
+// warp 8 issues every tcgen05.mma (whole warp runs the loop, one elected lane issues), warp 9 fetches Q and K rows, warp 10
+// the V rows, with tiled bulk copies, undoing the roll; warp 11 has no work.  A row is kept as head dim / 32 parts of 32
+// columns in the 64-byte-swizzled operand layout.
 // TMEM: columns [256 t, 256 t + 256) belong to query tile t of the pair: S chunk (fp32, 128 columns), overwritten
 // in place by bf16 P (64 columns); the O accumulator at +128.
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, all roles leave their loops, TMEM is
@@ -49,7 +46,6 @@ using namespace tc;
 
 constexpr int kMmaWarp = 8;
 constexpr int kLoaderWarp0 = 9;
-constexpr int kLoaderThreads = 96;
 constexpr int kThreads = 384;
 constexpr int kRegsLaunch = 168, kRegsSoftmax = 216, kRegsOther = 72;
 static_assert(2 * (kRegsSoftmax - kRegsLaunch) <= (kRegsLaunch - kRegsOther), "register hand-over does not balance");
@@ -58,7 +54,7 @@ constexpr int kPartBytes = 64;                        // one 32-column part of a
 constexpr int kQRows = 256, kChunk = 128;
 constexpr int kQPart = kQRows * kPartBytes;           // 16384: the region of one 32-column part of the Q rows
 constexpr int kKPart = kChunk * kPartBytes;           // 8192:  ... of a key chunk
-constexpr int kBiasFloats = 6048;                     // 3 c0 + 3 with c0 = 31 * 65 (window side 32)
+constexpr int kBiasFloats = 6048;                     // place of the staged table rows
 constexpr int kColO = 128;
 
 // Shared-memory plan per head dim D (64 or 128): a row is kept as D / 32 parts of 32 columns, each part a region in the
@@ -137,43 +133,6 @@ __device__ __forceinline__ int lds_i32(uint32_t addr) {
     return v;
 }
 
-// P for N consecutive key columns of the chunk starting at local column c: exp2(raw * scale + bias - m), packed
-// (SUM: also adds the values, before rounding, onto `sum`)
-template <int N, bool MASKED, bool SUM>
-__device__ __forceinline__ void softmax_cols(const uint32_t (&r)[N], uint32_t (&pk)[N / 2], int c, uint32_t bias_i,
-                                             uint32_t a_kc, uint32_t a_klab, int label_i, float scale, float neg_m,
-                                             float (&sum)[2]) {
-#pragma unroll
-    for (int e4 = 0; e4 < N / 4; ++e4) {
-        const int4 kc4 = lds_i4(a_kc + 4 * (c + e4 * 4));
-        const int kc[4] = {kc4.x, kc4.y, kc4.z, kc4.w};
-        int kl[4] = {0, 0, 0, 0};
-        if (MASKED) {
-            const int4 kl4 = lds_i4(a_klab + 4 * (c + e4 * 4));
-            kl[0] = kl4.x; kl[1] = kl4.y; kl[2] = kl4.z; kl[3] = kl4.w;
-        }
-        float p[4], bv[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) bv[e] = lds_f32(bias_i + kc[e]);
-#pragma unroll
-        for (int e = 0; e < 4; e += 2) {
-            float x0, x1;
-            fma2(x0, x1, __uint_as_float(r[e4 * 4 + e]), __uint_as_float(r[e4 * 4 + e + 1]), scale, bv[e], bv[e + 1]);
-            add2(x0, x1, x0, x1, neg_m);
-            if (MASKED && kl[e] != label_i) x0 = -INFINITY;
-            if (MASKED && kl[e + 1] != label_i) x1 = -INFINITY;
-            p[e] = fast_exp2(x0);
-            p[e + 1] = fast_exp2(x1);
-        }
-        pk[e4 * 2] = pack_elem(p[0], p[1]);
-        pk[e4 * 2 + 1] = pack_elem(p[2], p[3]);
-        if (SUM) {
-            sum[0] += p[0] + p[2];
-            sum[1] += p[1] + p[3];
-        }
-    }
-}
-
 template <int OFF>
 __device__ __forceinline__ float lds_f32_at(uint32_t addr) {
     float v;
@@ -242,26 +201,6 @@ __device__ __forceinline__ void softmax_cols32_row(const uint32_t (&r)[32], uint
     }
 }
 
-// exact maximum of scale * raw + bias over the keys of N columns that the row may see (others, and slots without a
-// token, give -inf)
-template <int N>
-__device__ __forceinline__ float score_max_cols(const uint32_t* r, int c, uint32_t bias_i, uint32_t a_kc, uint32_t a_klab,
-                                                int label_i, float scale, float mx) {
-#pragma unroll
-    for (int e4 = 0; e4 < N / 4; ++e4) {
-        const int4 kc4 = lds_i4(a_kc + 4 * (c + e4 * 4));
-        const int4 kl4 = lds_i4(a_klab + 4 * (c + e4 * 4));
-        const int kc[4] = {kc4.x, kc4.y, kc4.z, kc4.w};
-        const int kl[4] = {kl4.x, kl4.y, kl4.z, kl4.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float xv = fmaf(__uint_as_float(r[e4 * 4 + e]), scale, lds_f32(bias_i + kc[e]));
-            mx = fmaxf(mx, kl[e] == label_i ? xv : -INFINITY);
-        }
-    }
-    return mx;
-}
-
 // the same for 32 key columns whose bias entries are consecutive (see softmax_cols32_row)
 __device__ __forceinline__ float score_max_cols32_row(const uint32_t (&r)[32], uint32_t top, uint32_t a_klab, int label_i, float scale,
                                                       float mx) {
@@ -307,25 +246,20 @@ struct FwdMaps64 {
     RowMaps3 q, k, v;
 };
 
-// TMA: the grid consists of complete windows of side 16 or 32 and the longitude shift is a multiple of 8: a window row
-// is then one run of tokens (two where it wraps around the longitude seam), and one loader warp fetches every row with
-// tiled bulk copies; otherwise three loader warps gather the rows with 16-byte cp.async copies.
-//
-// MODE 0: gathered rows.  MODE 1: bulk-copied Q and K rows, window side 16 or 32, the head's whole bias table in
-// shared memory.  MODE 2: bulk-copied rows, window side 64 or 128 (complete windows of 4096 or 16384 tokens): the bias
-// table no longer fits, and the bulk-copy warp stages, per chunk and query tile, the table rows the tile's rows need.
+// The grid consists of complete windows of side 64 or 128 (4096 or 16384 tokens) and the longitude shift is a multiple of 8:
+// a window row is one run of tokens (two where it wraps around the longitude seam), fetched by tiled bulk copies.  The bias
+// table does not fit shared memory; the warp that copies K stages, per chunk and query tile, the table rows the tile's rows need.
 // A chunk's 128 keys are kr = 128 / w window rows and a tile's 128 queries qr = kr window rows, so the row offsets
 // between them span 2 kr - 1 table rows; in the prepared layout (2 w floats per table row) those are one contiguous
-// block, and within a 32-key group the entries a query row needs are consecutive, as in the 32-wide case.
-template <int D, int MODE>
+// block, and within a 32-key group the entries a query row needs are consecutive.
+template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
                      const __nv_bfloat16* __restrict__ v, const float* __restrict__ bias_prep,
                      __nv_bfloat16* __restrict__ o, float* __restrict__ lse, long long n_items, int ctas_per_head,
                      int max_pairs, const __grid_constant__ FwdMaps64 maps) {
     using L = Lay<D>;
-    constexpr bool TMA = MODE >= 1, ROWS = MODE == 2;
-    constexpr int kStageBytes = 4096, kStageTile = 1536;      // MODE 2: ring of four bias stages, two tiles each
+    constexpr int kStageBytes = 4096, kStageTile = 1536;      // ring of four bias stages, two tiles each
     static_assert(4 * kStageBytes <= (kBiasFloats - 1) * 4, "bias stages lie below the table's last float");
     constexpr int kParts = L::kParts, kQStages = L::kQStages, kSlots = L::kSlots, kQStageBytes = L::kQStageBytes;
     constexpr int kOffK = L::kOffK, kOffV = L::kOffV, kSlotBytes = L::kSlotBytes, kOffSlots = L::kOffSlots;
@@ -358,13 +292,12 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
 
     if (tid == 0) {
         for (int s = 0; s < kQStages; ++s) {
-            mbar_init(bar_qfull(s), TMA ? 32 : kLoaderThreads);
+            mbar_init(bar_qfull(s), 32);
             mbar_init(bar_qempty(s), 1 + 256);        // the issuer's commit + every softmax thread
         }
         for (int s = 0; s < kSlots; ++s) {
-            mbar_init(bar_kfull(s), TMA ? 32 : kLoaderThreads);       // TMA: the bulk-copy warp's lanes
-            // TMA: the 64 threads that gather V rows; MODE 2 and 32-wide windows: the lanes of the warp that bulk-copies them
-            mbar_init(bar_vfull(s), (ROWS || (TMA && g.w == 32)) ? 32 : TMA ? 64 : kLoaderThreads);
+            mbar_init(bar_kfull(s), 32);       // the bulk-copy warp's lanes
+            mbar_init(bar_vfull(s), 32);
             mbar_init(bar_kempty(s), 1);
             mbar_init(bar_vempty(s), 1);
         }
@@ -378,14 +311,9 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
         fence_barrier_init();
     }
     // the head's prepared bias table; the ones block of every ring slot (first 16 bf16 of a row = 1)
-    const int lw = 31 - __clz(g.w);                         // MODE 2: w = 1 << lw
-    const int rows_floats = (2 * g.w - 1) * 2 * g.w + 4;    // MODE 2: floats of one head's prepared table
-    if (ROWS) {
-        if (tid == 0) reinterpret_cast<float*>(smem + kOffBias)[kBiasFloats - 1] = bias_prep[(size_t)(head + 1) * rows_floats - 1];
-    } else {
-        for (int i = tid; i < kBiasFloats; i += kThreads)
-            reinterpret_cast<float*>(smem + kOffBias)[i] = bias_prep[(size_t)head * kBiasFloats + i];
-    }
+    const int lw = 31 - __clz(g.w);                         // w = 1 << lw
+    const int rows_floats = (2 * g.w - 1) * 2 * g.w + 4;    // floats of one head's prepared table
+    if (tid == 0) reinterpret_cast<float*>(smem + kOffBias)[kBiasFloats - 1] = bias_prep[(size_t)(head + 1) * rows_floats - 1];
     if (L::kOnes) {
         for (int i = tid; i < kSlots * kChunk * 4; i += kThreads) {
             const int s = i / (kChunk * 4), rem = i - s * (kChunk * 4), row = rem >> 2, chunk = rem & 3;
@@ -413,8 +341,8 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
 
     if (warp >= kMmaWarp) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsOther));
-    if (TMA && warp >= kLoaderWarp0) {
-        // ------------------------------------------------------------------ loader warp (TMA); the other two have no work
+    if (warp >= kLoaderWarp0) {
+        // ------------------------------------------------------------------ loader warps
         if (warp == kLoaderWarp0) {
             const int wrows = kChunk / g.w;                   // window rows per 128 slots
             int v0 = 0;                                       // first token column of the current window's rows
@@ -484,7 +412,7 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                                 klab[row] = label;
                             }
                         }
-                        if (ROWS && lane < x.ntiles) {
+                        if (lane < x.ntiles) {
                             // the 2 kr - 1 table rows that tile `lane` of the pair needs against this chunk
                             const int kr = kChunk >> lw;
                             const int r0 = (((x.pair * kQRows + lane * 128) >> lw) - c * kr - (kr - 1)) + g.w - 1;
@@ -492,8 +420,7 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                                       bias_prep + (size_t)head * rows_floats + (size_t)r0 * 2 * g.w, (uint32_t)((2 * kr - 1) * 8 * g.w),
                                       bar_kfull(s));
                         }
-                        // K rows (the V rows are gathered by the other two loader warps: the bulk-copy
-                        // engine takes a fixed time per 64-byte row, and the two ways of loading run side by side)
+                        // K rows
                         const uint32_t sb = smem0 + kOffSlots + s * kSlotBytes;
                         for (int i = lane; i < wrows * kParts; i += 32) {
                             const int ar = i / kParts, part = i - ar * kParts;
@@ -501,182 +428,38 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                         }
                         __syncwarp();
                         if (lane == 0)
-                            mbar_arrive_expect_tx(bar_kfull(s), (uint32_t)(kChunk * D * 2 + (ROWS ? x.ntiles * (2 * (kChunk >> lw) - 1) * 8 * g.w : 0)));
+                            mbar_arrive_expect_tx(bar_kfull(s), (uint32_t)(kChunk * D * 2 + x.ntiles * (2 * (kChunk >> lw) - 1) * 8 * g.w));
                         else mbar_arrive(bar_kfull(s));
                     }
                 }
                 ++kuse;
             }
-        } else if (ROWS || g.w == 32) {
-            // ---- MODE 2 and 32-wide windows, warp 10: the V rows by bulk copies as well (a window row is one or two boxes of 64 or 128 tokens,
-            // which the copy engine moves at several times the rate of 32-token boxes); warp 11 has no work
-            if (warp == kLoaderWarp0 + 1) {
-                const int wrows = kChunk / g.w;
-                long long ru = 0;
-                bool ok = true;
-                ItemCursor cur = cursor_init(cta_in_head, ctas_per_head, max_pairs, g.Mw, g.Mh);
-                for (long long it = cta_in_head; ok && it < n_items; it += ctas_per_head, cursor_advance(cur, max_pairs, g.Mw, g.Mh)) {
-                    const Item x = make_item(g, cur);
-                    if (x.ntiles == 0) continue;
-                    int v0 = x.r.wc * g.w + g.sw;
-                    if (v0 >= g.W) v0 -= g.W;
-                    for (int c = 0; c < x.nch; ++c, ++ru) {
-                        const int s = (int)(ru % kSlots);
-                        ok = mbar_wait_all(bar_vempty(s), (uint32_t)((ru / kSlots) & 1) ^ 1u, cta_abort);
-                        if (!ok) break;
-                        const uint32_t sb = smem0 + kOffSlots + s * kSlotBytes;
-                        // (one lane per part: the chunk's window rows, in groups of 4 where a 32-wide window allows it)
-                        if (lane < kParts)
-                            bulk_copy_window_rows(maps.v, sb + kOffV + lane * kKPart, g, x.b, x.r.wr, v0, c * wrows, wrows, head * D + lane * 32,
-                                                  bar_vfull(s));
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_expect_tx(bar_vfull(s), (uint32_t)(kChunk * D * 2));
-                        else mbar_arrive(bar_vfull(s));
-                    }
-                }
-            }
-        } else {
-            // ---- warps 10, 11: the V rows with 16-byte cp.async copies; a thread's arrival on the chunk's
-            // barrier is tied to the completion of its copies, so it never waits for data
-            const int vt = (warp - kLoaderWarp0 - 1) * 32 + lane;      // 0 .. 63
-            const int part = vt % kParts, row0 = vt / kParts;
-            constexpr int kRowStep = 64 / kParts;
+        } else if (warp == kLoaderWarp0 + 1) {
+            // ---- the V rows (a window row is one or two boxes of 64 or 128 tokens); warp 11 has no work
+            const int wrows = kChunk / g.w;
             long long ru = 0;
             bool ok = true;
             ItemCursor cur = cursor_init(cta_in_head, ctas_per_head, max_pairs, g.Mw, g.Mh);
             for (long long it = cta_in_head; ok && it < n_items; it += ctas_per_head, cursor_advance(cur, max_pairs, g.Mw, g.Mh)) {
                 const Item x = make_item(g, cur);
                 if (x.ntiles == 0) continue;
-                const size_t sample_off = (size_t)x.b * HW;
-                const int ew = x.r.ew;
-                {
-                    for (int c = 0; c < x.nch; ++c, ++ru) {
-                        const int s = (int)(ru % kSlots);
-                        ok = mbar_wait_all(bar_vempty(s), (uint32_t)((ru / kSlots) & 1) ^ 1u, cta_abort);
-                        if (!ok) break;
-                        const uint32_t vb = smem0 + kOffSlots + s * kSlotBytes + kOffV + part * kKPart;
-                        for (int row = row0; row < kChunk; row += kRowStep) {
-                            const int slot = c * kChunk + row, a = slot / ew;
-                            int code, label;
-                            const int tok = offset_token(g, x.r, a, slot - a * ew, code, label);
-                            const __nv_bfloat16* src = v + (sample_off + (size_t)tok) * g.ts + head * D + part * 32;
-#pragma unroll
-                            for (int c4 = 0; c4 < 4; ++c4) cp_async16(vb + tile_off<32>(row, c4), src + c4 * 8, 16);
-                        }
-                        cp_async_mbar_arrive_noinc(bar_vfull(s));
-                    }
-                }
-            }
-        }
-    } else if (warp >= kLoaderWarp0) {
-        // ------------------------------------------------------------------ loaders
-        // D / 32 lanes per row: each takes one 32-column part of the row and issues its four 16-byte copies with one
-        // address computation.  A thread never waits for data: its arrival on a stage's or slot's barrier is tied to
-        // the completion of the copies it has issued, so as many chunks are in flight as the ring has free slots.
-        const int lt = (warp - kLoaderWarp0) * 32 + lane;
-        const int hf = lt % kParts;                       // which 32-column part of the row this thread copies
-        const int lrow = lt / kParts;
-        constexpr int kRowsPerIter = kLoaderThreads / kParts;
-        int kuse = 0;
-        long long ru = 0;                                 // ring uses so far
-        bool ok = true;
-        auto acquire = [&](uint32_t bar, uint32_t parity) -> bool { return mbar_wait_all(bar, parity, cta_abort); };
-        // the thread's table entries are visible to the CTA before its arrival, which follows its copies
-        auto issued = [&](uint32_t bar) {
-            __threadfence_block();
-            cp_async_mbar_arrive_noinc(bar);
-        };
-        ItemCursor cur = cursor_init(cta_in_head, ctas_per_head, max_pairs, g.Mw, g.Mh);
-        for (long long it = cta_in_head; ok && it < n_items; it += ctas_per_head, cursor_advance(cur, max_pairs, g.Mw, g.Mh)) {
-            const Item x = make_item(g, cur);
-            if (x.ntiles == 0) continue;
-            const int qs = kuse % kQStages;
-            ok = acquire(bar_qempty(qs), ((kuse / kQStages) & 1) ^ 1);
-            if (!ok) break;
-            const size_t sample_off = (size_t)x.b * HW;
-            const int ew = x.r.ew;
-            const int q_r = kRowsPerIter / ew, r_r = kRowsPerIter - q_r * ew;       // window-offset step of 48 slots
-            // ---- Q rows of the pair (rows without a token as zeros) and the row tables
-            {
-                const uint32_t qb = smem0 + qs * kQStageBytes + hf * kQPart;
-                int* rowmeta = reinterpret_cast<int*>(smem + kOffRowMeta + qs * 2048);
-                int* rowtok = rowmeta + 256;
-                const int slot0 = x.pair * kQRows;
-                for (int row = lt; row < kQRows; row += kLoaderThreads) {
-                    const int slot = slot0 + row;
-                    int code = 0, label = 0xff, tok = -1;
-                    if (slot < x.r.n) {
-                        const int a = slot / ew;
-                        tok = offset_token(g, x.r, a, slot - a * ew, code, label);
-                    }
-                    rowmeta[row] = code | (label << 16);
-                    rowtok[row] = tok;
-                }
-                const int nrows = x.ntiles * 128;
-                int a_r = (slot0 + lrow) / ew, b_r = (slot0 + lrow) - a_r * ew;
-                for (int row = lrow; row < nrows; row += kRowsPerIter, a_r += q_r, b_r += r_r) {
-                    if (b_r >= ew) { b_r -= ew; ++a_r; }
-                    const __nv_bfloat16* src = q;
-                    int bytes = 0;
-                    if (slot0 + row < x.r.n) {
-                        int code, label;
-                        const int tok = offset_token(g, x.r, a_r, b_r, code, label);
-                        src = q + (sample_off + (size_t)tok) * g.ts + head * D + hf * 32;
-                        bytes = 16;
-                    }
-#pragma unroll
-                    for (int c4 = 0; c4 < 4; ++c4) cp_async16(qb + tile_off<32>(row, c4), bytes ? src + c4 * 8 : src, bytes);
-                }
-                issued(bar_qfull(qs));
-            }
-            // ---- the key chunks: K and V rows and the key tables
-            {
+                int v0 = x.r.wc * g.w + g.sw;
+                if (v0 >= g.W) v0 -= g.W;
                 for (int c = 0; c < x.nch; ++c, ++ru) {
                     const int s = (int)(ru % kSlots);
-                    ok = acquire(bar_kempty(s), (uint32_t)((ru / kSlots) & 1) ^ 1u) && acquire(bar_vempty(s), (uint32_t)((ru / kSlots) & 1) ^ 1u);
+                    ok = mbar_wait_all(bar_vempty(s), (uint32_t)((ru / kSlots) & 1) ^ 1u, cta_abort);
                     if (!ok) break;
-                    const uint32_t sb = smem0 + kOffSlots + s * kSlotBytes + hf * kKPart;
-                    const int ncols = min(kChunk, x.npad - c * kChunk);
-                    {
-                        int* kcs = reinterpret_cast<int*>(smem + kOffKeyMeta + (int)(ru & 3) * 1024);
-                        int* klab = kcs + 128;
-                        for (int row = lt; row < kChunk; row += kLoaderThreads) {
-                            const int slot = c * kChunk + row;
-                            int code = 0, label = 0xff, kc = 4 * (2 * c0 + 1);
-                            if (slot < x.r.n) {
-                                const int a = slot / ew;
-                                offset_token(g, x.r, a, slot - a * ew, code, label);
-                                kc = 4 * (c0 - code);
-                            }
-                            kcs[row] = kc;
-                            klab[row] = label;
-                        }
+                    const uint32_t sb = smem0 + kOffSlots + s * kSlotBytes;
+                    for (int i = lane; i < wrows * kParts; i += 32) {
+                        const int ar = i / kParts, part = i - ar * kParts;
+                        bulk_copy_window_row(maps.v, sb + kOffV + part * kKPart + ar * g.w * kPartBytes, g, x.b, x.r.wr, v0, c * wrows + ar,
+                                             head * D + part * 32, bar_vfull(s));
                     }
-                    const int slot_first = c * kChunk + lrow;
-                    int a_r = slot_first / ew, b_r = slot_first - a_r * ew;
-                    for (int row = lrow; row < ncols; row += kRowsPerIter, a_r += q_r, b_r += r_r) {
-                        if (b_r >= ew) { b_r -= ew; ++a_r; }
-                        const __nv_bfloat16 *sk = k, *sv = v;
-                        int bytes = 0;
-                        if (c * kChunk + row < x.r.n) {
-                            int code, label;
-                            const int tok = offset_token(g, x.r, a_r, b_r, code, label);
-                            const size_t off = (sample_off + (size_t)tok) * g.ts + head * D + hf * 32;
-                            sk = k + off; sv = v + off;
-                            bytes = 16;
-                        }
-#pragma unroll
-                        for (int c4 = 0; c4 < 4; ++c4) {
-                            const uint32_t so = tile_off<32>(row, c4);
-                            cp_async16(sb + kOffK + so, bytes ? sk + c4 * 8 : sk, bytes);
-                            cp_async16(sb + kOffV + so, bytes ? sv + c4 * 8 : sv, bytes);
-                        }
-                    }
-                    issued(bar_kfull(s));
-                    cp_async_mbar_arrive_noinc(bar_vfull(s));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_expect_tx(bar_vfull(s), (uint32_t)(kChunk * D * 2));
+                    else mbar_arrive(bar_vfull(s));
                 }
             }
-            ++kuse;
         }
     } else {
         // ------------------------------------------------------------------ MMA issuer
@@ -818,10 +601,9 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
             const uint32_t bias_i = smem0 + kOffBias + 4 * meta_code(rmeta);
             const int label_i = meta_label(rmeta);
             const float bmax = lds_f32(smem0 + kOffBias + 4 * (kBiasFloats - 1));
-            const bool row32 = g.w == 32 && x.r.ew == 32 && !x.masked;       // then every key slot holds a token, too
             const bool exact = exact_max(x);
             bool ok = true;
-            // MODE 2: this row's window row within its tile, and the byte offset of its entry for key column 0 of a table row
+            // this row's window row within its tile, and the byte offset of its entry for key column 0 of a table row
             const int slot_q = x.pair * kQRows + wg * 128 + row;
             const int aq_l = (slot_q >> lw) - ((x.pair * kQRows + wg * 128) >> lw), kr = kChunk >> lw;
             const int colq = 4 * ((slot_q & (g.w - 1)) + g.w - 1);
@@ -838,7 +620,6 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
             float m = -INFINITY;
             float psum[2] = {0.f, 0.f};
             for (int c = 0; c < x.nch; ++c) {
-                const int ncols = min(kChunk, x.npad - c * kChunk);
                 const uint32_t a_kc = smem0 + kOffKeyMeta + (int)((ru0 + c) & 3) * 1024, a_klab = a_kc + 512;
                 const uint32_t stage = smem0 + kOffBias + (int)((ru0 + c) & 3) * kStageBytes;
                 ok = mbar_wait_all(bar_sready(wg), n_s & 1, cta_abort);
@@ -852,39 +633,20 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                     int cc = 0;
                     if (exact) {
                         float mxe = -INFINITY;
-                        for (; cc + 32 <= ncols; cc += 32) {
+                        for (; cc < kChunk; cc += 32) {
                             tmem_ld32(t_s + cc, ra);
                             tmem_ld_wait();
-                            if (ROWS) mxe = score_max_cols32_row(ra, row_top(stage, cc >> 5), a_klab + 4 * cc, label_i, scale, mxe);
-                            else mxe = score_max_cols<32>(ra, cc, bias_i, a_kc, a_klab, label_i, scale, mxe);
-                        }
-                        if (cc < ncols) {
-                            uint32_t rt[16];
-                            tmem_ld16(t_s + cc, rt);
-                            tmem_ld_wait();
-                            mxe = score_max_cols<16>(rt, cc, bias_i, a_kc, a_klab, label_i, scale, mxe);
+                            mxe = score_max_cols32_row(ra, row_top(stage, cc >> 5), a_klab + 4 * cc, label_i, scale, mxe);
                         }
                         mc = mxe;
                     } else {
                         float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                        for (; cc + 64 <= ncols; cc += 64) {
+                        for (; cc < kChunk; cc += 64) {
                             tmem_ld32(t_s + cc, ra);
                             tmem_ld32(t_s + cc + 32, rb);
                             tmem_ld_wait();
                             max_cols<32>(ra, mx4);
                             max_cols<32>(rb, mx4);
-                        }
-                        if (cc + 32 <= ncols) {
-                            tmem_ld32(t_s + cc, ra);
-                            tmem_ld_wait();
-                            max_cols<32>(ra, mx4);
-                            cc += 32;
-                        }
-                        if (cc < ncols) {
-                            uint32_t rt[16];
-                            tmem_ld16(t_s + cc, rt);
-                            tmem_ld_wait();
-                            max_cols<16>(rt, mx4);
                         }
                         mc = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * scale + bmax;
                     }
@@ -911,40 +673,22 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                 if (raise) m = mc;
                 const float neg_m = m == -INFINITY ? 0.f : -m;
                 // ---- P
-                const int nfull = ncols >> 5;
-                if (nfull > 0) tmem_ld32(t_s, ra);
-                // full-width 32-wide window without mask labels: 32-column group i of chunk c is key row 4 c + i
-                const uint32_t top_c = bias_i + 4 * (c0 - 4 * c * cs);
+                constexpr int nfull = kChunk / 32;
+                tmem_ld32(t_s, ra);
                 for (int i = 0; i < nfull; i += 2) {
                     uint32_t pk[16];
                     tmem_ld_wait();
                     if (i + 1 < nfull) tmem_ld32(t_s + 32 * (i + 1), rb);
-                    if (ROWS) {
-                        if (x.masked) softmax_cols32_row<kSum, true>(ra, pk, row_top(stage, i), scale, neg_m, psum, a_klab + 128 * i, label_i);
-                        else softmax_cols32_row<kSum>(ra, pk, row_top(stage, i), scale, neg_m, psum);
-                    } else if (row32) softmax_cols32_row<kSum>(ra, pk, top_c - 4 * i * cs, scale, neg_m, psum);
-                    else if (x.masked) softmax_cols<32, true, kSum>(ra, pk, 32 * i, bias_i, a_kc, a_klab, label_i, scale, neg_m, psum);
-                    else softmax_cols<32, false, kSum>(ra, pk, 32 * i, bias_i, a_kc, a_klab, label_i, scale, neg_m, psum);
+                    if (x.masked) softmax_cols32_row<kSum, true>(ra, pk, row_top(stage, i), scale, neg_m, psum, a_klab + 128 * i, label_i);
+                    else softmax_cols32_row<kSum>(ra, pk, row_top(stage, i), scale, neg_m, psum);
                     tmem_st16(t_s + 16 * i, pk);
                     if (i + 1 < nfull) {
                         tmem_ld_wait();
                         if (i + 2 < nfull) tmem_ld32(t_s + 32 * (i + 2), ra);
-                        if (ROWS) {
-                            if (x.masked) softmax_cols32_row<kSum, true>(rb, pk, row_top(stage, i + 1), scale, neg_m, psum, a_klab + 128 * (i + 1), label_i);
-                            else softmax_cols32_row<kSum>(rb, pk, row_top(stage, i + 1), scale, neg_m, psum);
-                        } else if (row32) softmax_cols32_row<kSum>(rb, pk, top_c - 4 * (i + 1) * cs, scale, neg_m, psum);
-                        else if (x.masked) softmax_cols<32, true, kSum>(rb, pk, 32 * (i + 1), bias_i, a_kc, a_klab, label_i, scale, neg_m, psum);
-                        else softmax_cols<32, false, kSum>(rb, pk, 32 * (i + 1), bias_i, a_kc, a_klab, label_i, scale, neg_m, psum);
+                        if (x.masked) softmax_cols32_row<kSum, true>(rb, pk, row_top(stage, i + 1), scale, neg_m, psum, a_klab + 128 * (i + 1), label_i);
+                        else softmax_cols32_row<kSum>(rb, pk, row_top(stage, i + 1), scale, neg_m, psum);
                         tmem_st16(t_s + 16 * (i + 1), pk);
                     }
-                }
-                if (ncols & 16) {
-                    uint32_t rt[16], pk[8];
-                    tmem_ld16(t_s + 32 * nfull, rt);
-                    tmem_ld_wait();
-                    if (x.masked) softmax_cols<16, true, kSum>(rt, pk, 32 * nfull, bias_i, a_kc, a_klab, label_i, scale, neg_m, psum);
-                    else softmax_cols<16, false, kSum>(rt, pk, 32 * nfull, bias_i, a_kc, a_klab, label_i, scale, neg_m, psum);
-                    tmem_st8(t_s + 16 * nfull, pk);
                 }
                 tmem_st_wait();
                 tc_fence_before();
@@ -1015,25 +759,20 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
 // floats, the last of which is the head's largest entry as above; `rows` = 2: the table reflected through its centre
 // (entry (r, c) holds T[2w - 2 - r][2w - 2 - c]), for the query-side use of the key-major backward kernel.
 __global__ void __launch_bounds__(256)
-swin_fwd_bias_prep64_kernel(const float* __restrict__ bias, float* __restrict__ prep, int w, int heads, int rows) {
+swin_fwd_bias_prep64_kernel(const float* __restrict__ bias, float* __restrict__ prep, int w, int heads, int reflect) {
     const int head = blockIdx.x;
-    const int cs = rows ? 2 * w : w + 32, nw = 2 * w - 1;
-    const int c0 = (w - 1) * (cs + 1);
-    const int total = rows ? nw * cs + 4 : kBiasFloats;
+    const int cs = 2 * w, nw = 2 * w - 1;
+    const int total = nw * cs + 4;
     float* dst = prep + (size_t)head * total;
     float mx = -INFINITY, mn = INFINITY;
     for (int e = threadIdx.x; e < total - 1; e += blockDim.x) {
         float val = 0.f;
-        if (!rows && e > 2 * c0) {
-            val = -INFINITY;
-        } else {
-            const int ra = e / cs, rb = e - ra * cs;
-            if (rb < nw && ra < nw) {
-                const int sa = rows == 2 ? nw - 1 - ra : ra, sb = rows == 2 ? nw - 1 - rb : rb;
-                val = bias[(size_t)(sa * nw + sb) * heads + head] * kLog2e;
-                mx = fmaxf(mx, val);
-                mn = fminf(mn, val);
-            }
+        const int ra = e / cs, rb = e - ra * cs;
+        if (rb < nw && ra < nw) {
+            const int sa = reflect ? nw - 1 - ra : ra, sb = reflect ? nw - 1 - rb : rb;
+            val = bias[(size_t)(sa * nw + sb) * heads + head] * kLog2e;
+            mx = fmaxf(mx, val);
+            mn = fminf(mn, val);
         }
         dst[e] = val;
     }
@@ -1064,24 +803,20 @@ cudaError_t read_fwd_tc64_status(int* timed_out) {
 }
 
 #ifndef TERRA_ELEM_F16
-// prepared bias tables for the kernels of the large-window regime: kBiasFloats = 6048 floats per head for window
-// sides up to 32, whole table rows for sides 64 and 128 (see the kernel above)
+// prepared bias tables for the kernels of window sides 64 and 128: whole table rows (see the kernel above)
 cudaError_t launch_bias_prep64(const Geo& g, const float* bias, float* prep, cudaStream_t stream, bool reflect) {
-    if (reflect && g.w <= 32) return cudaErrorNotSupported;
-    swin_fwd_bias_prep64_kernel<<<g.heads, 256, 0, stream>>>(bias, prep, g.w, g.heads, g.w > 32 ? (reflect ? 2 : 1) : 0);
+    swin_fwd_bias_prep64_kernel<<<g.heads, 256, 0, stream>>>(bias, prep, g.w, g.heads, reflect ? 1 : 0);
     count_launch(stream);
     return cudaGetLastError();
 }
 
-// window sides up to 32 on any grid; sides 64 and 128 on grids of complete windows that the bulk-copy loaders serve
+// window sides 64 and 128 on grids of complete windows that the bulk-copy loaders serve
 bool fwd_tc64_supported(const Geo& g) {
-    if (!(g.d == 64 || g.d == 128) || g.heads > 148) return false;
-    if (g.w <= 32) return g.nmax <= 1024;
-    return (g.w == 64 || g.w == 128) && bulk_rows_shape(g);
+    return (g.d == 64 || g.d == 128) && g.heads <= 148 && (g.w == 64 || g.w == 128) && bulk_rows_shape(g);
 }
 
 size_t fwd_tc64_workspace_bytes(const Geo& g) {
-    const size_t per_head = g.w <= 32 ? (size_t)kBiasFloats : (size_t)(2 * g.w - 1) * 2 * g.w + 4;
+    const size_t per_head = (size_t)(2 * g.w - 1) * 2 * g.w + 4;
     return (size_t)g.heads * per_head * sizeof(float);
 }
 #endif  // !TERRA_ELEM_F16
@@ -1089,8 +824,7 @@ size_t fwd_tc64_workspace_bytes(const Geo& g) {
 cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
                             void* o, float* lse, void* workspace, int sm_count, cudaStream_t stream) {
     float* prep = reinterpret_cast<float*>(workspace);
-    const bool rows = g.w > 32;
-    swin_fwd_bias_prep64_kernel<<<g.heads, 256, 0, stream>>>(bias, prep, g.w, g.heads, rows ? 1 : 0);
+    swin_fwd_bias_prep64_kernel<<<g.heads, 256, 0, stream>>>(bias, prep, g.w, g.heads, 0);
     count_launch(stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1102,12 +836,8 @@ cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const vo
     const unsigned grid = (unsigned)(cph * g.heads);
     FwdMaps64 maps;
     std::memset(&maps, 0, sizeof maps);
-    static const bool tma_off = [] { const char* e_ = std::getenv("TERRA_NO_TMA"); return e_ && e_[0] == '1'; }();
-    const bool tma = (!tma_off || rows) && bulk_rows_shape(g) && make_row_maps3(&maps.q, g, q, g.ts) && make_row_maps3(&maps.k, g, k, g.ts) &&
-                     make_row_maps3(&maps.v, g, v, g.ts);
-    if (rows && !tma) return cudaErrorNotSupported;       // windows of side 64 and 128 have no gathering loader
-    auto kern = g.d == 64 ? (rows ? swin_fwd_tc64_kernel<64, 2> : tma ? swin_fwd_tc64_kernel<64, 1> : swin_fwd_tc64_kernel<64, 0>)
-                          : (rows ? swin_fwd_tc64_kernel<128, 2> : tma ? swin_fwd_tc64_kernel<128, 1> : swin_fwd_tc64_kernel<128, 0>);
+    if (!make_row_maps3(&maps.q, g, q, g.ts) || !make_row_maps3(&maps.k, g, k, g.ts) || !make_row_maps3(&maps.v, g, v, g.ts)) return cudaErrorNotSupported;
+    auto kern = g.d == 64 ? swin_fwd_tc64_kernel<64> : swin_fwd_tc64_kernel<128>;
     const int smem_bytes = g.d == 64 ? Lay<64>::kSmemBytes : Lay<128>::kSmemBytes;
     e = prepare_kernel((const void*)kern, smem_bytes);
     if (e != cudaSuccess) return e;

@@ -65,14 +65,10 @@ cudaError_t read_bwd_kv64_status_f16(int* timed_out);
 cudaError_t launch_bwd_kv64_qside_f16(const Geo& g, const void* q, const void* k, const void* v, const void* d_o,
                                       const float* prep_reflected, const float* lse, const float* delta, void* dq, float* dbias,
                                       int sm_count, cudaStream_t stream);
-cudaError_t launch_bwd_q64_f16(const Geo& g, const void* q, const void* k, const void* v, const void* d_o, const float* prep,
-                               const float* lse, const float* delta, void* dq, float* dbias, int sm_count, cudaStream_t stream);
-cudaError_t read_bwd_q64_status_f16(int* timed_out);
 cudaError_t launch_bwd_delta_f16(const Geo& g, const void* o, const void* d_o, float* delta, cudaStream_t stream);
 cudaError_t launch_bwd_mma_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
                                const float* lse, const float* delta, const void* d_o,
-                               void* dq, void* dk, void* dv, float* dbias, int sm_count, cudaStream_t stream,
-                               bool query_side_only = false);
+                               void* dq, void* dk, void* dv, float* dbias, int sm_count, cudaStream_t stream);
 
 // tcgen05 forward path (head dim 32, window side <= 16)
 constexpr int kFwdBiasFloats = 2304;   // prepared bias table per head (padded rows, -inf zone, maximum in the last float)
@@ -119,13 +115,6 @@ cudaError_t launch_bwd_kv64_qside(const Geo& g, const void* q, const void* k, co
                                   const float* prep_reflected, const float* lse, const float* delta, void* dq, float* dbias,
                                   int sm_count, cudaStream_t stream);
 
-// tcgen05 query side (dQ, dBias) of the same regime for complete 32 x 32 windows (window side 32, grid extents
-// multiples of 32); dbias is overwritten
-bool bwd_q64_supported(const Geo& g);
-cudaError_t launch_bwd_q64(const Geo& g, const void* q, const void* k, const void* v, const void* d_o, const float* prep,
-                           const float* lse, const float* delta, void* dq, float* dbias, int sm_count, cudaStream_t stream);
-cudaError_t read_bwd_q64_status(int* timed_out);
-
 // One-pass tcgen05 backward for windows of more than 64 tokens and side <= 32, every head dim, any grid.
 struct OnePassPlan {
     int rw;                  // slots per window row
@@ -167,7 +156,6 @@ cudaError_t launch_bwd_delta(const Geo& g, const void* o, const void* d_o, float
 // dK, dV (key-tile CTAs) and dQ, dBias (query-tile CTAs)
 cudaError_t launch_bwd_mma(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
                            const float* lse, const float* delta, const void* d_o,
-                           void* dq, void* dk, void* dv, float* dbias, int sm_count, cudaStream_t stream,
-                           bool query_side_only = false);
+                           void* dq, void* dk, void* dv, float* dbias, int sm_count, cudaStream_t stream);
 
 }  // namespace terra
