@@ -11,8 +11,8 @@
 //   dV += P^T dO_c, dK += dS^T Q_c                                   (A from TMEM, B = the chunk's rows, MN-major)
 // P is recomputed from the saved log-sum-exp, so the chunks are independent.
 // Roles: warps 0-7 elementwise (warps w and w + 4 share TMEM lane quarter w & 3 and take the chunk's first / second
-// 64 query columns), warp 8 issues every MMA, warp 9 loads rows by bulk copies.  A row is kept as head dim / 32 parts of 32
-// columns in the 64-byte-swizzled operand layout, as in the forward kernel of this regime.
+// 64 query columns), warp 8 issues every MMA, warp 9 loads rows by bulk copies.  A row is kept as two parts in the
+// swizzled operand layout, as in the forward kernel of this regime.
 // Half chunks rotate through TMEM buffers (S^T 64 columns | dP^T 64 columns): three at head dim 64, so that the scores of
 // a group's next half chunk are issued while it still works on the current one, two at head dim 128, where the
 // accumulators dV and dK (head dim columns each, behind the buffers) take the rest of the 512 columns.
@@ -50,9 +50,7 @@ constexpr int kWorkThreads = 256;
 constexpr int kRegsLaunch = 168, kRegsWork = 208, kRegsOther = 80;
 static_assert(2 * (kRegsWork - kRegsLaunch) <= (kRegsLaunch - kRegsOther), "register hand-over does not balance");
 
-constexpr int kPartBytes = 64;                        // one 32-column part of a row
 constexpr int kTile = 128;                            // keys per item, queries per chunk
-constexpr int kPart = kTile * kPartBytes;             // 8192: the region of one 32-column part of 128 rows
 constexpr int kHalf = 64;                             // queries per half chunk
 constexpr int kBiasFloats = 6048;
 constexpr int kBufCols = 128;                         // TMEM buffer b: S^T of a half chunk at 128 b, dP^T at 128 b + 64
@@ -64,11 +62,14 @@ constexpr int kBufCols = 128;                         // TMEM buffer b: S^T of a
 // time; several smaller copies in flight hide the copy latency better.  At head dim 64 the same split was slower).
 template <int D>
 struct Lay {
-    static constexpr int kParts = D / 32;
+    // a row is two parts of 32 (64-byte swizzle) or 64 columns (128-byte swizzle: half as many, twice as large copies and
+    // the same MMAs: window side 128 27.7 + 28.1 -> 26.2 + 27.4 ms; the forward kernel gains nothing by it)
+    static constexpr int kParts = 2, kPartCols = D / 2, kPartBytes = D;
+    static constexpr int kPart = kTile * kPartBytes;  // the region of one part of 128 rows
     static constexpr int kKvStages = D == 64 ? 2 : 1, kSlots = D == 64 ? 3 : 4;
     static constexpr int kHPS = D == 64 ? 2 : 1;      // half chunks per ring slot
     static constexpr int kSlotQ = kHalf * kHPS;       // query rows per ring slot
-    static constexpr int kSPart = kSlotQ * kPartBytes;            // the region of one 32-column part of a slot's rows
+    static constexpr int kSPart = kSlotQ * kPartBytes;            // ... of a slot's rows
     static constexpr int kRows = 2 * kParts * kPart;  // two tensors' rows
     // key stage: K parts | V parts, then per key row: 4 * bias code, label, token
     static constexpr int kOffK = 0, kOffV = kParts * kPart;
@@ -275,6 +276,7 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
     using L = Lay<D>;
     constexpr int kStageBytes = 1536;                 // the staged table rows of one query slot
     constexpr int kHPS = L::kHPS, kSlotQ = L::kSlotQ, kSPart = L::kSPart, kTab = L::kTab;
+    constexpr int kPartBytes = L::kPartBytes, kPartCols = L::kPartCols, kPart = L::kPart;
     constexpr int kParts = L::kParts, kKvStages = L::kKvStages, kSlots = L::kSlots;
     constexpr int kOffK = L::kOffK, kOffV = L::kOffV, kOffKCode = L::kOffKCode, kOffKLab = L::kOffKLab, kOffKTok = L::kOffKTok;
     constexpr int kKvStageBytes = L::kKvStageBytes, kOffQ = L::kOffQ, kOffG = L::kOffG, kOffQCode = L::kOffQCode;
@@ -374,8 +376,8 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                     for (int i = lane; i < 2 * per_tensor; i += 32) {
                         const int tsr = i >= per_tensor ? 1 : 0, rem = i - tsr * per_tensor;
                         const int ar = rem / kParts, part = rem - ar * kParts;
-                        bulk_copy_window_row(tsr ? maps.v : maps.k, sb + (tsr ? kOffV : kOffK) + part * kPart + ar * g.w * kPartBytes, g,
-                                             x.b, x.r.wr, v0, x.kt * wrows + ar, head * D + part * 32, bar_kvfull(ks));
+                        bulk_copy_window_row<kPartBytes>(tsr ? maps.v : maps.k, sb + (tsr ? kOffV : kOffK) + part * kPart + ar * g.w * kPartBytes, g,
+                                             x.b, x.r.wr, v0, x.kt * wrows + ar, head * D + part * kPartCols, bar_kvfull(ks));
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive_expect_tx(bar_kvfull(ks), (uint32_t)(kTile * D * 2 * 2));
@@ -408,8 +410,8 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                         const int tsr = j >= runs * kParts ? 1 : 0, rem = j - tsr * runs * kParts;
                         const int rr = rem / kParts, part = rem - rr * kParts;
                         const int rslot = slot0 + rr * n_run, a = rslot / g.w;
-                        bulk_copy_window_run(tsr ? maps.g : maps.q, sb + (tsr ? kOffG : kOffQ) + part * kSPart + rr * n_run * kPartBytes, g,
-                                             x.b, x.r.wr, v0, a, rslot - a * g.w, n_run, head * D + part * 32, bar_qfull(s));
+                        bulk_copy_window_run<kPartBytes>(tsr ? maps.g : maps.q, sb + (tsr ? kOffG : kOffQ) + part * kSPart + rr * n_run * kPartBytes, g,
+                                             x.b, x.r.wr, v0, a, rslot - a * g.w, n_run, head * D + part * kPartCols, bar_qfull(s));
                     }
                     if (lane == 0) {
                         // the table rows that this slot's ur window rows need against the key tile's kr window rows
@@ -431,7 +433,9 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
     } else {
         // ------------------------------------------------------------------ MMA issuer
         const uint32_t idesc_acc = make_idesc_elem(128, D, 0, 1);        // A from TMEM, B = 16 rows x D (MN-major)
-        const uint32_t sd_hi = sdesc_hi(make_sdesc_sw64(smem0, 512));    // common high word of the K-major descriptors
+        auto k_major = [](uint32_t a) { return D == 64 ? make_sdesc_sw64(a, 512) : make_sdesc_sw128(a); };
+        auto mn_major = [](uint32_t a, uint32_t part) { return D == 64 ? make_sdesc_sw64_mn(a, part, 512) : make_sdesc_sw128(a, part); };
+        const uint32_t sd_hi = sdesc_hi(k_major(smem0));    // common high word of the K-major descriptors
         int kuse = 0;
         unsigned p0 = 0;                                  // half chunks before the current item
         unsigned u0 = 0;                                  // ring slots used before the current item; use u is in slot u % kSlots
@@ -453,31 +457,26 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                 return true;
             };
             // S^T = K Q^T, dP^T = V dO^T for the queries of the half chunk in ring slot `sb`
-            // (descriptor low words = start address in 16-byte units: + 2 per 32-byte K step, + region / 16 per 32-column part)
-            const uint32_t k_lo = sdesc_lo(make_sdesc_sw64(kb + kOffK, 512)), v_lo = sdesc_lo(make_sdesc_sw64(kb + kOffV, 512));
+            // (descriptor low words = start address in 16-byte units: + 2 per 32-byte K step, + region / 16 per part)
+            const uint32_t k_lo = sdesc_lo(k_major(kb + kOffK)), v_lo = sdesc_lo(k_major(kb + kOffV));
             // (`sb` = the address of the half chunk's first row in its slot)
             auto issue_sdp = [&](uint32_t sb, int nc, int buf) {
                 const uint32_t idesc = make_idesc_elem(128, nc, 0, 0);
-                const uint32_t q_lo = sdesc_lo(make_sdesc_sw64(sb + kOffQ, 512));
-                const uint32_t g_lo = sdesc_lo(make_sdesc_sw64(sb + kOffG, 512));
+                const uint32_t q_lo = sdesc_lo(k_major(sb + kOffQ));
+                const uint32_t g_lo = sdesc_lo(k_major(sb + kOffG));
                 const uint32_t t_s = tmem_base + kBufCols * buf, t_dp = t_s + 64;
                 constexpr uint32_t kNext = kPart >> 4, kNextH = kSPart >> 4;
+                constexpr int kSteps = kPartCols / 16;
                 tc_fence_after();
                 if (elect_one()) {
                     mma_ss_h<false>(t_s, k_lo, q_lo, sd_hi, idesc);
-                    mma_ss_h<true>(t_s, k_lo + 2, q_lo + 2, sd_hi, idesc);
 #pragma unroll
-                    for (int pt = 1; pt < kParts; ++pt) {
-                        mma_ss_h<true>(t_s, k_lo + pt * kNext, q_lo + pt * kNextH, sd_hi, idesc);
-                        mma_ss_h<true>(t_s, k_lo + pt * kNext + 2, q_lo + pt * kNextH + 2, sd_hi, idesc);
-                    }
+                    for (int ks = 1; ks < D / 16; ++ks)
+                        mma_ss_h<true>(t_s, k_lo + (ks / kSteps) * kNext + (ks % kSteps) * 2, q_lo + (ks / kSteps) * kNextH + (ks % kSteps) * 2, sd_hi, idesc);
                     mma_ss_h<false>(t_dp, v_lo, g_lo, sd_hi, idesc);
-                    mma_ss_h<true>(t_dp, v_lo + 2, g_lo + 2, sd_hi, idesc);
 #pragma unroll
-                    for (int pt = 1; pt < kParts; ++pt) {
-                        mma_ss_h<true>(t_dp, v_lo + pt * kNext, g_lo + pt * kNextH, sd_hi, idesc);
-                        mma_ss_h<true>(t_dp, v_lo + pt * kNext + 2, g_lo + pt * kNextH + 2, sd_hi, idesc);
-                    }
+                    for (int ks = 1; ks < D / 16; ++ks)
+                        mma_ss_h<true>(t_dp, v_lo + (ks / kSteps) * kNext + (ks % kSteps) * 2, g_lo + (ks / kSteps) * kNextH + (ks % kSteps) * 2, sd_hi, idesc);
                     mma_commit(bar_sdp(buf));
                 }
                 __syncwarp();
@@ -515,8 +514,8 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                 if (!ok) break;
                 tc_fence_after();
                 // dV += P^T dO, dK += dS^T Q over the half chunk's query columns
-                const uint64_t gd = make_sdesc_sw64_mn(sb + kOffG, kSPart, 512);
-                const uint64_t qd = make_sdesc_sw64_mn(sb + kOffQ, kSPart, 512);
+                const uint64_t gd = mn_major(sb + kOffG, kSPart);
+                const uint64_t qd = mn_major(sb + kOffQ, kSPart);
                 const uint32_t g_lo = sdesc_lo(gd), q_lo = sdesc_lo(qd), d_hi = sdesc_hi(gd);
                 const uint32_t t_p = tmem_base + kBufCols * buf, t_ds = t_p + 64;
                 const int nks = nc >> 4;
@@ -528,8 +527,8 @@ swin_bwd_kv64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                         j = 1;
                     }
                     for (; j < nks; ++j) {
-                        if (!QS) mma_ts_h<true>(tmem_base + kColDV, t_p + 16 * j, g_lo + 64 * j, d_hi, idesc_acc);
-                        mma_ts_h<true>(tmem_base + kColDK, t_ds + 16 * j, q_lo + 64 * j, d_hi, idesc_acc);
+                        if (!QS) mma_ts_h<true>(tmem_base + kColDV, t_p + 16 * j, g_lo + kPartBytes * j, d_hi, idesc_acc);
+                        mma_ts_h<true>(tmem_base + kColDK, t_ds + 16 * j, q_lo + kPartBytes * j, d_hi, idesc_acc);
                     }
                     // the slot's last readers were issued just above
                     if (kHPS == 1 || h == 1 || half_cols(c, 1) == 0) mma_commit(bar_qempty(s));
@@ -791,10 +790,10 @@ static cudaError_t launch_kv64(const Geo& g, const void* q, const void* k, const
     std::memset(&maps, 0, sizeof maps);
     // the kernel's tile rows ("k", "v") and streamed rows ("q", "g"); the query side exchanges the roles
     const bool tma = bulk_rows_shape(g) &&
-                     (qside ? make_row_maps3(&maps.k, g, q, g.ts) && make_row_maps3(&maps.v, g, d_o, g.heads * g.d) &&
-                                  make_row_maps3(&maps.q, g, k, g.ts) && make_row_maps3(&maps.g, g, v, g.ts)
-                            : make_row_maps3(&maps.q, g, q, g.ts) && make_row_maps3(&maps.k, g, k, g.ts) &&
-                                  make_row_maps3(&maps.v, g, v, g.ts) && make_row_maps3(&maps.g, g, d_o, g.heads * g.d));
+                     (qside ? make_row_maps3(&maps.k, g, q, g.ts, g.d / 2) && make_row_maps3(&maps.v, g, d_o, g.heads * g.d, g.d / 2) &&
+                                  make_row_maps3(&maps.q, g, k, g.ts, g.d / 2) && make_row_maps3(&maps.g, g, v, g.ts, g.d / 2)
+                            : make_row_maps3(&maps.q, g, q, g.ts, g.d / 2) && make_row_maps3(&maps.k, g, k, g.ts, g.d / 2) &&
+                                  make_row_maps3(&maps.v, g, v, g.ts, g.d / 2) && make_row_maps3(&maps.g, g, d_o, g.heads * g.d, g.d / 2));
     if (!tma) return cudaErrorNotSupported;
     auto kern = g.d == 64 ? (qside ? swin_bwd_kv64_kernel<64, true> : swin_bwd_kv64_kernel<64, false>)
                           : (qside ? swin_bwd_kv64_kernel<128, true> : swin_bwd_kv64_kernel<128, false>);

@@ -909,16 +909,16 @@ EncodeTiledFn encode_tiled_fn() {
 
 // [tokens][channels] bf16 with a token stride of `token_stride` elements; box = 32 channels x `box_tokens` tokens,
 // 64-byte swizzle.  `map` points to a CUtensorMap.
-bool make_row_map(void* map, const Geo& g, const void* base, int token_stride, int box_tokens) {
+bool make_row_map(void* map, const Geo& g, const void* base, int token_stride, int box_tokens, int box_ch) {
     CUtensorMap* m = reinterpret_cast<CUtensorMap*>(map);
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)g.heads * g.d, (cuuint64_t)g.B * g.H * g.W};
     const cuuint64_t strides[1] = {(cuuint64_t)token_stride * 2};
-    const cuuint32_t box[2] = {32u, (cuuint32_t)box_tokens};
+    const cuuint32_t box[2] = {(cuuint32_t)box_ch, (cuuint32_t)box_tokens};
     const cuuint32_t estr[2] = {1u, 1u};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+               box_ch == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // one map of win_tiles.cuh: [heads * d][nb columns][ncols windows][token rows] from `base` on
@@ -935,13 +935,13 @@ bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-bool make_row_maps3(RowMaps3* maps, const Geo& g, const void* base, int token_stride) {
+bool make_row_maps3(RowMaps3* maps, const Geo& g, const void* base, int token_stride, int part_cols) {
     for (int i = 0; i < 3; ++i)
-        if (!make_row_map(&maps->m[i], g, base, token_stride, 32 >> i)) return false;
+        if (!make_row_map(&maps->m[i], g, base, token_stride, 32 >> i, part_cols)) return false;
     // boxes of 64 and 128 tokens (a box may not be longer than the token axis)
     for (int i = 3; i < 5; ++i) {
         const int box = (long long)g.B * g.H * g.W >= (8 << i) ? (8 << i) : 32;
-        if (!make_row_map(&maps->m[i], g, base, token_stride, box)) return false;
+        if (!make_row_map(&maps->m[i], g, base, token_stride, box, part_cols)) return false;
     }
     return true;
 }

@@ -349,7 +349,7 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
             int xb = 0, xwr = 0;
             // the copies of window row `a`, part `part` of a row: w consecutive slots from `dst` on
             auto copy_row = [&](const RowMaps3& m3, uint32_t dst, int a, int part, uint32_t bar) {
-                bulk_copy_window_row(m3, dst, g, xb, xwr, v0, a, head * D + part * 32, bar);
+                bulk_copy_window_row<kPartBytes>(m3, dst, g, xb, xwr, v0, a, head * D + part * 32, bar);
             };
             int kuse = 0;
             long long ru = 0;
@@ -452,7 +452,7 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                     const uint32_t sb = smem0 + kOffSlots + s * kSlotBytes;
                     for (int i = lane; i < wrows * kParts; i += 32) {
                         const int ar = i / kParts, part = i - ar * kParts;
-                        bulk_copy_window_row(maps.v, sb + kOffV + part * kKPart + ar * g.w * kPartBytes, g, x.b, x.r.wr, v0, c * wrows + ar,
+                        bulk_copy_window_row<kPartBytes>(maps.v, sb + kOffV + part * kKPart + ar * g.w * kPartBytes, g, x.b, x.r.wr, v0, c * wrows + ar,
                                              head * D + part * 32, bar_vfull(s));
                     }
                     __syncwarp();
@@ -836,7 +836,7 @@ cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const vo
     const unsigned grid = (unsigned)(cph * g.heads);
     FwdMaps64 maps;
     std::memset(&maps, 0, sizeof maps);
-    if (!make_row_maps3(&maps.q, g, q, g.ts) || !make_row_maps3(&maps.k, g, k, g.ts) || !make_row_maps3(&maps.v, g, v, g.ts)) return cudaErrorNotSupported;
+    if (!make_row_maps3(&maps.q, g, q, g.ts, 32) || !make_row_maps3(&maps.k, g, k, g.ts, 32) || !make_row_maps3(&maps.v, g, v, g.ts, 32)) return cudaErrorNotSupported;
     auto kern = g.d == 64 ? swin_fwd_tc64_kernel<64> : swin_fwd_tc64_kernel<128>;
     const int smem_bytes = g.d == 64 ? Lay<64>::kSmemBytes : Lay<128>::kSmemBytes;
     e = prepare_kernel((const void*)kern, smem_bytes);

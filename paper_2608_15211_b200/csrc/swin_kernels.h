@@ -83,7 +83,7 @@ cudaError_t read_tc_status(int* timed_out, cudaStream_t stream);
 // TMA variants of the two kernels above (grids of 16-wide windows whose window rows are runs of consecutive tokens):
 // the shape test, and the encoder of a [tokens][channels] tensor map with a box of 32 channels x box_tokens tokens
 bool tma_row_shape(const Geo& g);
-bool make_row_map(void* cu_tensor_map, const Geo& g, const void* base, int token_stride, int box_tokens);
+bool make_row_map(void* cu_tensor_map, const Geo& g, const void* base, int token_stride, int box_tokens, int box_ch = 32);
 
 // tcgen05 forward path for head dim 64 and windows of up to 1024 tokens (keys streamed in chunks, two passes)
 // windows of side 9 .. 32 on any grid (attn_fwd_win.cu)

@@ -14,12 +14,12 @@
 namespace terra {
 
 struct RowMaps3 {
-    // boxes of 32, 16, 8, 64 and 128 tokens
+    // boxes of 32, 16, 8, 64 and 128 tokens x one part of a row: 32 columns (64-byte swizzle) or 64 columns (128-byte swizzle)
     CUtensorMap m[5];
 };
 
-// host: the three maps of one tensor (`token_stride` in elements); false if the driver's encoder is not available
-bool make_row_maps3(RowMaps3* maps, const Geo& g, const void* base, int token_stride);
+// host: the maps of one tensor (`token_stride` in elements, parts of `part_cols` columns); false if the driver's encoder is not available
+bool make_row_maps3(RowMaps3* maps, const Geo& g, const void* base, int token_stride, int part_cols);
 
 // host: the geometry the bulk-copy loaders are written for
 inline bool bulk_rows_shape(const Geo& g) {
@@ -27,10 +27,11 @@ inline bool bulk_rows_shape(const Geo& g) {
            (long long)g.B * g.H * g.W < 0x7fffffffLL;
 }
 
-// device: the copies of `n_run` slots (a multiple of 8) of window row `a`, from window column `b0` (a multiple of 8) on,
-// of window row-index `wr` in sample `b`: 64 bytes per slot from `dst` on (a multiple of 512 bytes into a swizzled
-// region), columns [xc, xc + 32) of every token; `v0` = the window's first token column after the roll.  The bytes
+// device (ROWB = bytes of a part's row: 64 or 128): the copies of `n_run` slots (a multiple of 8) of window row `a`, from window column `b0` (a multiple of 8) on,
+// of window row-index `wr` in sample `b`: ROWB bytes per slot from `dst` on (a multiple of 8 rows into a swizzled
+// region), columns from xc on of every token; `v0` = the window's first token column after the roll.  The bytes
 // are counted on `bar`.
+template <int ROWB>
 __device__ __forceinline__ void bulk_copy_window_run(const RowMaps3& m3, uint32_t dst, const Geo& g, int b, int wr, int v0, int a,
                                                      int b0, int n_run, int xc, uint32_t bar) {
     int u = wr * g.w + a + g.sh;
@@ -42,19 +43,20 @@ __device__ __forceinline__ void bulk_copy_window_run(const RowMaps3& m3, uint32_
     int y = y0 + vs, n = n1;
 #pragma unroll
     for (int seg = 0; seg < 2; ++seg) {
-        while (n >= 128) { tc::tma_load_2d(dst, &m3.m[4], xc, y, bar); dst += 128 * 64; y += 128; n -= 128; }
-        if (n >= 64) { tc::tma_load_2d(dst, &m3.m[3], xc, y, bar); dst += 64 * 64; y += 64; n -= 64; }
-        while (n >= 32) { tc::tma_load_2d(dst, &m3.m[0], xc, y, bar); dst += 32 * 64; y += 32; n -= 32; }
-        if (n >= 16) { tc::tma_load_2d(dst, &m3.m[1], xc, y, bar); dst += 16 * 64; y += 16; n -= 16; }
-        if (n >= 8) { tc::tma_load_2d(dst, &m3.m[2], xc, y, bar); dst += 8 * 64; }
+        while (n >= 128) { tc::tma_load_2d(dst, &m3.m[4], xc, y, bar); dst += 128 * ROWB; y += 128; n -= 128; }
+        if (n >= 64) { tc::tma_load_2d(dst, &m3.m[3], xc, y, bar); dst += 64 * ROWB; y += 64; n -= 64; }
+        while (n >= 32) { tc::tma_load_2d(dst, &m3.m[0], xc, y, bar); dst += 32 * ROWB; y += 32; n -= 32; }
+        if (n >= 16) { tc::tma_load_2d(dst, &m3.m[1], xc, y, bar); dst += 16 * ROWB; y += 16; n -= 16; }
+        if (n >= 8) { tc::tma_load_2d(dst, &m3.m[2], xc, y, bar); dst += 8 * ROWB; }
         y = y0;
         n = n_run - n1;
     }
 }
 // the whole window row
+template <int ROWB>
 __device__ __forceinline__ void bulk_copy_window_row(const RowMaps3& m3, uint32_t dst, const Geo& g, int b, int wr, int v0, int a,
                                                      int xc, uint32_t bar) {
-    bulk_copy_window_run(m3, dst, g, b, wr, v0, a, 0, g.w, xc, bar);
+    bulk_copy_window_run<ROWB>(m3, dst, g, b, wr, v0, a, 0, g.w, xc, bar);
 }
 
 }  // namespace terra
