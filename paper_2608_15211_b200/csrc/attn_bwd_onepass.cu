@@ -736,8 +736,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             sq.init();
             uint32_t use = 0;                        // bit per slot: parity of the slot's fills
             bool ok = true;
-            // lane -> (second half of a tile's rows / second tensor, channel part)
-            const int part = lane % kParts, second = lane / kParts;
+            // lane -> channel part, window row of a tile or of the two half chunks
+            const int part = lane % kParts, row = lane / kParts;
             // one slot; `two`: Q and dO of a half chunk (else the two 64-slot groups of a K or V tile); a0 = first window row
             auto fill = [&](int s, const WinMaps& m0, const WinMaps& m1, const __nv_bfloat16* x0, const __nv_bfloat16* x1, int a0, bool two) {
                 ok = mbar_wait_all(bar(kBEmpty + s), ((use >> s) & 1) ^ 1u, cta_abort);
@@ -776,10 +776,12 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     }
                 } else {
                     if (lane == 0) mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB - (fix ? 2 * kG * kRowB : 0));
-                    if (second < 2) {
-                        const uint32_t dst = base + (two ? second * kHalf * D * 2 + part * kHalf * kRowB : part * kTile * kRowB + second * kHalf * kRowB);
-                        load_win_rows<RW, kRowB>(second ? m1 : m0, p.cols, dst, g, td.b, td.wr, td.wc, td.eh, a0 + (two ? 0 : second * kG),
-                                                 td.head * D + part * L::kPartCh, bar(kBFull + s));
+                    __syncwarp();
+                    if (row < 2 * kG) {
+                        const int second = row / kG, r = row % kG;
+                        const uint32_t dst = base + r * RW * kRowB + (two ? second * kHalf * D * 2 + part * kHalf * kRowB : part * kTile * kRowB + second * kHalf * kRowB);
+                        load_win_row<RW, kRowB>(second ? m1 : m0, p.cols, dst, g, td.b, td.wr, td.wc, td.eh, a0 + (two ? r : row),
+                                                td.head * D + part * L::kPartCh, bar(kBFull + s));
                     }
                 }
                 __syncwarp();

@@ -417,7 +417,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             unsigned units = 0;
             int e_key = -1, q0 = -1, q1 = -1;        // what the mask operands are made for; Q slots of the last unit
             bool ok = true;
-            const int part = lane % kParts, second = lane / kParts;
+            const int part = lane % kParts, row = lane / kParts;      // lane -> channel part, window row of a tile
             auto fill = [&](int s, const WinMaps& m, const __nv_bfloat16* src, int a0) {
                 ok = ok && mbar_wait_all(bar(kBEmpty + s), ((use >> s) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
@@ -451,9 +451,9 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 } else {
                     if (lane == 0) mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB - (fix ? 2 * kG * kRowB : 0));
                     __syncwarp();
-                    if (second < 2)
-                        load_win_rows<RW, kRowB>(m, p.cols, base + part * kTile * kRowB + second * 64 * kRowB, g, td.b, td.wr, td.wc, td.eh, a0 + second * kG,
-                                                 td.head * D + part * L::kPartCh, bar(kBFull + s));
+                    if (row < 2 * kG)
+                        load_win_row<RW, kRowB>(m, p.cols, base + part * kTile * kRowB + row * RW * kRowB, g, td.b, td.wr, td.wc, td.eh, a0 + row,
+                                                td.head * D + part * L::kPartCh, bar(kBFull + s));
                 }
                 __syncwarp();
             };

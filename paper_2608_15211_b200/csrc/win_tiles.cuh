@@ -51,29 +51,24 @@ __device__ __forceinline__ bool win_group_whole(const WinCols& c, const Geo& g, 
     return wc != c.seam && wc < c.first_wrapped && wc != c.last && a0 + groups * (64 / RW) <= eh && u + groups * (64 / RW) <= g.H;
 }
 
-// device: 64 slots from window row `a0` on, a copy per window row, channels [ch, ch + part) of every token, to `dst` (rows of
-// ROWB bytes, 1 KB aligned); the bytes are counted on `bar` (64 * ROWB, less ROWB per window row for a seam column with c.skip).
+// device: the RW slots of window row `a`, channels [ch, ch + part) of every token, to `dst` (rows of ROWB bytes); the bytes are
+// counted on `bar` (RW * ROWB, less ROWB for a seam column with c.skip).  A lane per row: a lane's copies follow one another at
+// 250 cycles each, those of different lanes overlap.
 template <int RW, int ROWB>
-__device__ __forceinline__ void load_win_rows(const WinMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
-                                              int a0, int ch, uint32_t bar) {
-    constexpr int G = 64 / RW;
-    int u = wr * g.w + a0 + g.sh;
+__device__ __forceinline__ void load_win_row(const WinMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
+                                             int a, int ch, uint32_t bar) {
+    int u = wr * g.w + a + g.sh;
     if (u >= g.H) u -= g.H;
-#pragma unroll
-    for (int r = 0; r < G; ++r) {
-        const int y = a0 + r < eh ? b * g.H + u : g.B * g.H;       // behind the last row: zeros
-        const uint32_t d = dst + r * RW * ROWB;
-        if (wc == c.seam) {
-            tc::tma_load_4d(d, &m.seam_a, ch, 0, 0, y, bar);
-            if (c.n1 + c.skip < RW) tc::tma_load_4d(d + (c.n1 + c.skip) * ROWB, &m.seam_b, ch, c.skip, 0, y, bar);
-        } else if (wc == c.last) {
-            tc::tma_load_4d(d, &m.last, ch, 0, 0, y, bar);
-        } else if (wc >= c.first_wrapped) {
-            tc::tma_load_4d(d, &m.wrapped, ch, 0, wc - c.first_wrapped, y, bar);
-        } else {
-            tc::tma_load_4d(d, &m.row, ch, 0, wc, y, bar);
-        }
-        if (++u >= g.H) u -= g.H;
+    const int y = a < eh ? b * g.H + u : g.B * g.H;       // behind the last row: zeros
+    if (wc == c.seam) {
+        tc::tma_load_4d(dst, &m.seam_a, ch, 0, 0, y, bar);
+        if (c.n1 + c.skip < RW) tc::tma_load_4d(dst + (c.n1 + c.skip) * ROWB, &m.seam_b, ch, c.skip, 0, y, bar);
+    } else if (wc == c.last) {
+        tc::tma_load_4d(dst, &m.last, ch, 0, 0, y, bar);
+    } else if (wc >= c.first_wrapped) {
+        tc::tma_load_4d(dst, &m.wrapped, ch, 0, wc - c.first_wrapped, y, bar);
+    } else {
+        tc::tma_load_4d(dst, &m.row, ch, 0, wc, y, bar);
     }
 }
 
