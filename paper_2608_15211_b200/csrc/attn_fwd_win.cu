@@ -662,7 +662,11 @@ cudaError_t read_fwd_win_status(int* timed_out) {
 #ifndef TERRA_ELEM_F16
 bool fwd_win_supported(const Geo& g) {
     // (head dim 32 with sides up to 16 has a kernel of its own, 0.77 against 1.16 ms on the 510 x 1080 grid with 12 heads)
-    return (g.d == 64 || g.d == 128 || (g.d == 32 && g.w > 16)) && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
+    // Where a window fills little of its slots (side 17 half of them), or has one query tile and little more, the register-tile
+    // kernel with its dense rows is faster: 240 x 360 tokens, 6 x 32, side 17 214 against 487 us, side 20 289 against 384;
+    // 6 x 64, side 9 226 against 312, side 11 166 against 217 (side 12: 266 against 179), side 17 338 against 484 (18: 417 against 412).
+    const bool sparse = g.d == 32 ? g.w <= 20 : g.d == 64 && (g.w <= 11 || g.w == 17);
+    return (g.d == 64 || g.d == 128 || (g.d == 32 && g.w > 16)) && !sparse && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 4 < 0x7fffffffLL;
 }
 
