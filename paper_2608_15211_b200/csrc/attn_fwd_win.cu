@@ -118,7 +118,7 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
 // 8 k + 2 t + e) -> S scale + bias in place, and the rows' maxima.  Pairs on one diagonal share their bias: 7 or 9 reads
 // for 32 scores.  (A thread per row read each score's own entry: the shared-memory pipe then bound the kernel, 1300 to 2500
 // of 4100 to 6800 cycles per 128 x 128 scores and tile.)  `bias`: shared address of the entry of rows g, keys 2 t.
-template <int RW>
+template <int RW, int KC>
 __device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, uint32_t bias, float scale, float (&mx)[4]) {
     constexpr int kRowB = Tab<RW>::kRowF * 4;
     float2 bv[9];
@@ -128,7 +128,7 @@ __device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, uint32_t b
 #pragma unroll
     for (int m = 0; m < 4; ++m)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < KC; ++k) {
             uint32_t* v = &x[m >> 1][16 * u + 4 * k + 2 * (m & 1)];
             const float2 b = bv[RW == 32 ? k - m + 3 : 3 * ((k >> 1) - (m >> 1) + 1) + (k & 1) - (m & 1) + 1];
             float x0, x1;
@@ -139,7 +139,9 @@ __device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, uint32_t b
         }
 }
 
-template <int D, int RW>
+// KC: of every 32 key slots the first 8 KC are worked on (window sides 17 .. 24 in rows of 32 slots leave the last 8 without a
+// token: 3; otherwise 4).  240 x 360 tokens, 6 x 64, side 22: 357 -> 302 us.
+template <int D, int RW, int KC>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
                     const __grid_constant__ WinMaps mq, const __grid_constant__ WinMaps mk, const __grid_constant__ WinMaps mv) {
@@ -234,10 +236,10 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     tmem_ld_frag64(t_s + (16u << 16), x[1]);
                     tmem_ld_wait();
                     float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    add_bias<RW>(x, 0, bias, scale, top);
+                    add_bias<RW, KC>(x, 0, bias, scale, top);
                     bias += 4u * (32 / RW) * Tab<RW>::kRowF;
                     if (2 * j + 1 < td.ku) {
-                        add_bias<RW>(x, 1, bias, scale, top);
+                        add_bias<RW, KC>(x, 1, bias, scale, top);
                         bias += 4u * (32 / RW) * Tab<RW>::kRowF;
                     } else {
                         // 32 slots that do not exist
@@ -284,6 +286,10 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
 #pragma unroll
                             for (int mi = 0; mi < 2; ++mi) {
                                 const int i = 2 * h + mi;
+                                if ((k & 3) >= KC) {
+                                    pk[2 * k + mi] = 0u;
+                                    continue;
+                                }
                                 float x0, x1;
                                 add2(x0, x1, __uint_as_float(x[h][4 * k + 2 * mi]), __uint_as_float(x[h][4 * k + 2 * mi + 1]), -m[i]);
                                 x0 = fast_exp2(x0);
@@ -663,9 +669,9 @@ cudaError_t read_fwd_win_status(int* timed_out) {
 bool fwd_win_supported(const Geo& g) {
     // (head dim 32 with sides up to 16 has a kernel of its own, 0.77 against 1.16 ms on the 510 x 1080 grid with 12 heads)
     // Where a window fills little of its slots (side 17 half of them), or has one query tile and little more, the register-tile
-    // kernel with its dense rows is faster: 240 x 360 tokens, 6 x 32, side 17 214 against 487 us, side 20 289 against 384;
-    // 6 x 64, side 9 226 against 312, side 11 166 against 217 (side 12: 266 against 179), side 17 338 against 484 (18: 417 against 412).
-    const bool sparse = g.d == 32 ? g.w <= 20 : g.d == 64 && (g.w <= 11 || g.w == 17);
+    // kernel with its dense rows is faster: 240 x 360 tokens, 6 x 32, side 17 214 against 487 us, side 22 305 against 319 (side 23: 347 against 308);
+    // 6 x 64, side 9 226 against 312, side 11 166 against 217 (side 12: 266 against 179), side 17 338 against 415 (18: 417 against 361).
+    const bool sparse = g.d == 32 ? g.w <= 22 : g.d == 64 && (g.w <= 11 || g.w == 17);
     return (g.d == 64 || g.d == 128 || (g.d == 32 && g.w > 16)) && !sparse && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 4 < 0x7fffffffLL;
 }
@@ -676,7 +682,7 @@ size_t fwd_win_workspace_bytes(const Geo& g) {
 #endif
 
 namespace {
-template <int D, int RW>
+template <int D, int RW, int KC = 4>
 cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
                        int sm_count, cudaStream_t stream) {
     using L = Lay<D, RW>;
@@ -699,10 +705,10 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
     prof_begin("swin_fwd_win_prep_kernel", stream);
     swin_fwd_win_prep_kernel<RW><<<total / 512 + 1 < 592 ? total / 512 + 1 : 592, 256, 0, stream>>>(g, bias, (float*)workspace);
     count_launch(stream);
-    cudaError_t e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW>, L::kSmemBytes);
+    cudaError_t e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW, KC>, L::kSmemBytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_fwd_win_kernel", stream);
-    e = launch_dependent(swin_fwd_win_kernel<D, RW>, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
+    e = launch_dependent(swin_fwd_win_kernel<D, RW, KC>, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
     count_launch(stream);
     return e;
 }
@@ -710,11 +716,11 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
 
 cudaError_t launch_fwd_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
                            int sm_count, cudaStream_t stream) {
-    const bool wide = win_row_slots(g) == 32;
+    const bool wide = win_row_slots(g) == 32, narrow = g.w <= 24;
     switch (g.d) {
-        case 32: return launch_win<32, 32>(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
-        case 64: return (wide ? launch_win<64, 32> : launch_win<64, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
-        default: return (wide ? launch_win<128, 32> : launch_win<128, 16>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+        case 32: return (narrow ? launch_win<32, 32, 3> : launch_win<32, 32>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+        case 64: return (!wide ? launch_win<64, 16> : narrow ? launch_win<64, 32, 3> : launch_win<64, 32>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+        default: return (!wide ? launch_win<128, 16> : narrow ? launch_win<128, 32, 3> : launch_win<128, 32>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
     }
 }
 
