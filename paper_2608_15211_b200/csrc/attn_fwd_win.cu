@@ -543,7 +543,6 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 const int s_q[2] = {sq.pop(), sq.pop()};
                 for (int c = 0; ok && c < td.nch; ++c) {
                     const int sk = sq.take(), sv = sq.take();
-                    full_use ^= 1u << sv;
                     if (c == 0) wait_full(s_q[0]);
                     wait_full(sk);
                     for (int hf = 0; hf < 2 && 4 * c + 2 * hf < td.ku; ++hf) {
@@ -575,6 +574,10 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                             __syncwarp();
                         }
                     }
+                    // The V tile is not this warp's, but a wait names a phase by parity: a slot's next fill may be waited for only once this
+                    // one is known to have landed.  (Without it, a V tile later than the scores let the next unit's first scores pass
+                    // their wait for the K tile that goes to its slot: head dim 128, 32 x 32 windows, one call in a thousand.)
+                    wait_full(sv);
                 }
                 sq.end_unit(s_q[0], s_q[1]);
             }
@@ -589,6 +592,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             uint32_t full_use = 0;
             unsigned idx = 0, opened[2] = {0, 0};
             bool ok = true;
+            // (Q and K fills need no wait here: a slot that holds V now held them for scores whose products this warp has issued)
             while (ok && next_unit()) {
                 const int s_q[2] = {sq.pop(), sq.pop()};
                 for (int t = 0; t < td.ntq; ++t) full_use ^= 1u << s_q[t];
