@@ -9,9 +9,13 @@
 //   scaled down then), and write P = exp2(S scale + bias - m) over S in 16 bits;
 //   O += P V, accumulated in TMEM.
 // Masks cost the softmax threads nothing: where a window's slots differ in shift-mask label or hold no token, one more
-// 16-wide step of the score product adds -2^30 (fp16) or -2^100 (bf16) to the pairs that must not see one another.  E_q holds
-// a one at the query's label, E_k the penalty at every label but the key's.  One body serves every window: the elementwise
-// code is what bounds the kernel, and two copies of it in one kernel run slower than one.
+// 16-wide step of the score product (bf16 operands in either build) adds 2^64 x -2^64 to the pairs that must not see one
+// another, which leaves the range of fp32: such a score is -inf whatever the scores, the scale and the bias are.  E_q holds 2^64 at
+// the query's label, E_k -2^64 at every label but the key's.  What an infinity cannot be added to, a forbidden score that is
+// +inf or not a number, turns up as NaN in the maximum: the half chunk's scores then go by their labels (drop_forbidden).
+// (Selects by label in every half chunk of the windows that mix them, before or after the load: 256 x 512 tokens, 12 x 64,
+// 32 x 32 windows, one in eight masked, 850 -> 1000 us.)  One body serves every window: the elementwise code is what bounds
+// the kernel, and two copies of it in one kernel run slower than one.
 // Scores and P share three TMEM buffers (head dim 128: two), so that the products of other chunks run under the softmax.
 //
 // What bounds it: MUFU, 16 exponentials per clock and SM (0.40 ms for the 510 x 1080 grid with 12 heads and 16 x 16 windows).
@@ -45,11 +49,8 @@ constexpr int kSoftWarps = 8, kReadWarp0 = 8, kPvWarp = 12, kLoaderWarp = 13, kS
 constexpr int kRegsLaunch = 128, kRegsSoft = 184, kRegsOther = 72;
 static_assert(2 * kRegsSoft + 2 * kRegsOther <= 4 * kRegsLaunch, "register hand-over does not balance");
 constexpr int kTile = 128, kDescs = 8;
-#ifdef TERRA_ELEM_F16
-constexpr uint32_t kMaskQ = 0x7800, kMaskK = 0xF800;           // 2^15, -2^15
-#else
-constexpr uint32_t kMaskQ = 0x5880, kMaskK = 0xD880;           // 2^50, -2^50
-#endif
+constexpr uint32_t kMaskQ = 0x5F80, kMaskK = 0xDF80;           // bf16 2^64, -2^64
+constexpr float kLowest = -3.402823466e38f;                    // a row's reference before its first key
 
 // The bias table by row difference, twice: copy c starts at column difference c - (RW - 1), so that a thread's pairs of keys
 // are read aligned, from the copy of its row's parity; the copies lie 16 banks apart.
@@ -114,8 +115,14 @@ __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
     return v;
 }
 
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+    float d;
+    asm("max.NaN.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 // The thread's scores of one 32-slot key unit (32 query rows x 32 keys a warp; thread 4 g + t holds rows g + 8 m, keys
-// 8 k + 2 t + e) -> S scale + bias in place, and the rows' maxima.  Pairs on one diagonal share their bias: 7 or 9 reads
+// 8 k + 2 t + e) -> S scale + bias in place, and the rows' maxima (NaN if a score is).  Pairs on one diagonal share their bias: 7 or 9 reads
 // for 32 scores.  (A thread per row read each score's own entry: the shared-memory pipe then bound the kernel, 1300 to 2500
 // of 4100 to 6800 cycles per 128 x 128 scores and tile.)  `bias`: shared address of the entry of rows g, keys 2 t.
 template <int RW, int KC>
@@ -135,8 +142,32 @@ __device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, uint32_t b
             fma2(x0, x1, __uint_as_float(v[0]), __uint_as_float(v[1]), scale, b.x, b.y);
             v[0] = __float_as_uint(x0);
             v[1] = __float_as_uint(x1);
-            mx[m] = max3(mx[m], x0, x1);
+            mx[m] = max3_nan(mx[m], x0, x1);
         }
+}
+
+// The scores of a half chunk (key rows `ak` on, `cols` of its columns; 32 query rows a warp, window row `aq` on) whose tokens differ in
+// mask label become -inf, in tensor memory.  Not inlined, and the half chunk starts over from the loop's head: with this code in the
+// middle of the softmax's every unit paid for it (121 x 250 x 2 tokens, 8 x 64, side 32: 285 -> 306 us; so 290).
+template <int RW>
+__device__ __noinline__ void drop_forbidden(uint32_t t_s, int cols, int ak, int aq, int ha, int hb, int gl, int ql) {
+#pragma unroll 1
+    for (int c = 0; c < cols; c += 16)
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+            // 16 keys x 16 queries, each of one window row
+            const bool rows = (ak + c / RW >= ha) == (aq + (RW == 32 ? 0 : h) >= ha);
+            uint32_t r[8];
+            tmem_ld_frag16(t_s + ((16u * h) << 16) + c, r);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int bk = (RW == 32 ? c & 16 : 0) + 8 * (i >> 2) + 2 * ql + (i & 1), bq = (RW == 32 ? 16 * h : 0) + 8 * ((i >> 1) & 1) + gl;
+                r[i] = rows && (bk >= hb) == (bq >= hb) ? r[i] : 0xff800000u;
+            }
+            tmem_st_frag16(t_s + ((16u * h) << 16) + c, r);
+        }
+    tmem_st_wait();
 }
 
 // KC: of every 32 key slots the first 8 KC are worked on (window sides 17 .. 24 in rows of 32 slots leave the last 8 without a
@@ -223,8 +254,9 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             if (ok && t < td.ntq) {
                 const int aq = min((td.tile0 + t) * kTileRows + wq * (32 / RW), td.eh - 1);
                 uint32_t bias = tab0 + 4u * (g.w - 1 - aq + Tab<RW>::kFront) * Tab<RW>::kRowF;
-                float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                float m[4] = {kLowest, kLowest, kLowest, kLowest};     // (finite: a half chunk may hold no key that the row sees)
                 float2 sum[4] = {};
+                int fixed = -1;                          // half chunk whose scores have gone by their labels
                 for (int j = 0; 2 * j < td.ku; ++j) {
                     const unsigned idx = n + j * td.ntq + t, buf = idx % NB;
                     const uint32_t t_s = tq + 64u * buf;
@@ -237,16 +269,20 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     tmem_ld_wait();
                     float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
                     add_bias<RW, KC>(x, 0, bias, scale, top);
-                    bias += 4u * (32 / RW) * Tab<RW>::kRowF;
                     if (2 * j + 1 < td.ku) {
-                        add_bias<RW, KC>(x, 1, bias, scale, top);
-                        bias += 4u * (32 / RW) * Tab<RW>::kRowF;
+                        add_bias<RW, KC>(x, 1, bias + 4u * (32 / RW) * Tab<RW>::kRowF, scale, top);
                     } else {
                         // 32 slots that do not exist
 #pragma unroll
                         for (int i = 16; i < 32; ++i) x[0][i] = x[1][i] = 0xff800000u;
                     }
-                    if (__any_sync(0xffffffffu, top[0] - m[0] > 8.f || top[1] - m[1] > 8.f || top[2] - m[2] > 8.f || top[3] - m[3] > 8.f)) {
+                    if (!__all_sync(0xffffffffu, top[0] - m[0] <= 8.f && top[1] - m[1] <= 8.f && top[2] - m[2] <= 8.f && top[3] - m[3] <= 8.f)) {
+                        if (fixed != j && ((td.ha > 0 && td.ha < td.eh) || (td.hb > 0 && td.hb < td.ew)) &&
+                            __any_sync(0xffffffffu, top[0] != top[0] || top[1] != top[1] || top[2] != top[2] || top[3] != top[3])) {
+                            drop_forbidden<RW>(t_s, 32 * min(2, td.ku - 2 * j), 2 * j * (32 / RW), (td.tile0 + t) * kTileRows + wq * (32 / RW), td.ha, td.hb, gl, ql);
+                            fixed = j--;
+                            continue;
+                        }
                         // raise the reference; O and the sums so far are scaled down, once the products so far are done
                         float f[4];
 #pragma unroll
@@ -299,6 +335,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                             }
                         tmem_st_frag_packed32(t_s + ((16u * h) << 16), pk);
                     }
+                    bias += 4u * (64 / RW) * Tab<RW>::kRowF;
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
@@ -521,7 +558,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             }
         } else if (warp == kScoreWarp) {
             // -------------------------------------------------------------- S = Q K^T
-            constexpr uint32_t kIdS = make_idesc_elem(128, 0, 0, 0);
+            constexpr uint32_t kIdS = make_idesc_elem(128, 0, 0, 0), kIdE = make_idesc_bf16(128, 0, 0, 0);
             const uint64_t d_k = D == 32 ? make_sdesc_sw64(smem0, 512) : make_sdesc_sw128(smem0);
             const uint64_t d_e = make_sdesc_sw64(smem0 + L::kOffE, 512);
             const uint32_t hi = sdesc_hi(d_k), lo = sdesc_lo(d_k), hi_e = sdesc_hi(d_e), lo_e = sdesc_lo(d_e);
@@ -547,7 +584,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     wait_full(sk);
                     for (int hf = 0; hf < 2 && 4 * c + 2 * hf < td.ku; ++hf) {
                         const int left = td.ku - (4 * c + 2 * hf);
-                        const uint32_t id = kIdS + ((left > 1 ? 8u : 4u) << 17);
+                        const uint32_t n = (left > 1 ? 8u : 4u) << 17, id = kIdS + n;
 #pragma unroll
                         for (int t = 0; t < 2; ++t) {
                             if (t >= td.ntq) break;
@@ -566,7 +603,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                                     if (ks == 0) mma_ss_h<false>(dst, a + oa, b + oa, hi, id);
                                     else mma_ss_h<true>(dst, a + oa, b + oa, hi, id);
                                 }
-                                if (td.flags & 4) mma_ss_h<true>(dst, ea, eb, hi_e, id);
+                                if (td.flags & 4) mma_ss_h<true>(dst, ea, eb, hi_e, kIdE + n);
                                 mma_commit(bar(kBS + buf));
                                 if (c == td.nch - 1 && left <= 2) mma_commit(bar(kBEmpty + s_q[t]));
                                 if (t == td.ntq - 1 && (hf == 1 || left <= 2)) mma_commit(bar(kBEmpty + sk));
