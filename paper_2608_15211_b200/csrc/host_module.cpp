@@ -27,6 +27,13 @@ PyObject* on_status = nullptr;          // binding._check: raises the TerraError
 
 struct Failed {};                       // a Python error is set
 
+// Other Python threads run while this one allocates or launches: both wait for the GPU at times (a new segment of the caching
+// allocator, a full launch queue).
+struct NoGil {
+    PyThreadState* state = PyEval_SaveThread();
+    ~NoGil() { PyEval_RestoreThread(state); }
+};
+
 // The descriptor is a ctypes structure; its bytes are read through the buffer protocol.
 struct Desc {
     Py_buffer view{};
@@ -99,9 +106,21 @@ void check(int status) {
 
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// The library call (its pointers are taken before: that may raise).
+template <class F, class... A>
+void launch(F f, A... args) {
+    int status;
+    {
+        NoGil no_gil;
+        status = f(args...);
+    }
+    check(status);
+}
+
 // The caller's tensor, or a new one.
 at::Tensor output(PyObject* o, const char* name, at::ScalarType dtype, at::IntArrayRef shape, const at::Tensor& like) {
     if (o != Py_None) return tensor(o, name);
+    NoGil no_gil;
     return at::detail::empty_cuda(shape, dtype, like.device(), std::nullopt);
 }
 
@@ -113,7 +132,10 @@ at::Tensor workspace(PyObject* o, const Desc& desc, bool backward, const at::Ten
     } else {
         size_t need = 0;
         check(f_workspace(desc.d, backward, &need));
-        if (need) t = at::detail::empty_cuda({(int64_t)need}, at::kByte, like.device(), std::nullopt);
+        if (need) {
+            NoGil no_gil;
+            t = at::detail::empty_cuda({(int64_t)need}, at::kByte, like.device(), std::nullopt);
+        }
     }
     bytes = t.defined() ? t.nbytes() : 0;
     return t;
@@ -161,7 +183,7 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         expect(o, d.act(), all, "o"); expect(lse, at::kFloat, rows, "lse");
         size_t bytes;
         at::Tensor ws = workspace(a[7], d, false, q, bytes);
-        check(f_fwd(d.d, pq, pk, pv, (const float*)pb, ptr(o), (float*)ptr(lse), opt_ptr(ws), bytes, stream()));
+        launch(f_fwd, d.d, pq, pk, pv, (const float*)pb, ptr(o), (float*)ptr(lse), opt_ptr(ws), bytes, stream());
         return tuple({o, lse});
     });
 }
@@ -180,7 +202,7 @@ PyObject* fwd_packed(PyObject*, PyObject* const* a, Py_ssize_t n) {
         expect(o, d.act(), all, "o"); expect(lse, at::kFloat, rows, "lse");
         size_t bytes;
         at::Tensor ws = workspace(a[5], d, false, x, bytes);
-        check(f_fwd_packed(d.d, px, (const float*)pb, ptr(o), (float*)ptr(lse), opt_ptr(ws), bytes, stream()));
+        launch(f_fwd_packed, d.d, px, (const float*)pb, ptr(o), (float*)ptr(lse), opt_ptr(ws), bytes, stream());
         return tuple({o, lse});
     });
 }
@@ -194,7 +216,7 @@ PyObject* fwd_noalloc(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int64_t rows = d.rows(), all = rows * d.d->head_dim;
         expect(q, d.act(), all, "q"); expect(k, d.act(), all, "k"); expect(v, d.act(), all, "v"); expect(o, d.act(), all, "o");
         expect(b, at::kFloat, d.table(), "bias_table"); expect(lse, at::kFloat, rows, "lse");
-        check(f_fwd_noalloc(d.d, ptr(q), ptr(k), ptr(v), (const float*)ptr(b), ptr(o), (float*)ptr(lse), stream()));
+        launch(f_fwd_noalloc, d.d, ptr(q), ptr(k), ptr(v), (const float*)ptr(b), ptr(o), (float*)ptr(lse), stream());
         return tuple({o, lse});
     });
 }
@@ -214,7 +236,7 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
         expect(dq, d.act(), all, "dq"); expect(dk, d.act(), all, "dk"); expect(dv, d.act(), all, "dv"); expect(db, at::kFloat, b.numel(), "dbias");
         size_t bytes;
         at::Tensor ws = workspace(a[12], d, true, q, bytes);
-        check(f_bwd(d.d, pq, pk, pv, (const float*)pb, po, (const float*)pl, pg, ptr(dq), ptr(dk), ptr(dv), (float*)ptr(db), opt_ptr(ws), bytes, stream()));
+        launch(f_bwd, d.d, pq, pk, pv, (const float*)pb, po, (const float*)pl, pg, ptr(dq), ptr(dk), ptr(dv), (float*)ptr(db), opt_ptr(ws), bytes, stream());
         return tuple({dq, dk, dv, db});
     });
 }
@@ -232,7 +254,7 @@ PyObject* bwd_packed(PyObject*, PyObject* const* a, Py_ssize_t n) {
         expect(dx, d.act(), 3 * all, "dqkv"); expect(db, at::kFloat, b.numel(), "dbias");
         size_t bytes;
         at::Tensor ws = workspace(a[8], d, true, x, bytes);
-        check(f_bwd_packed(d.d, px, (const float*)pb, po, (const float*)pl, pg, ptr(dx), (float*)ptr(db), opt_ptr(ws), bytes, stream()));
+        launch(f_bwd_packed, d.d, px, (const float*)pb, po, (const float*)pl, pg, ptr(dx), (float*)ptr(db), opt_ptr(ws), bytes, stream());
         return tuple({dx, db});
     });
 }
