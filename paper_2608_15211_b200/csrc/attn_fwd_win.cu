@@ -61,8 +61,12 @@ struct Tab {
     static __host__ __device__ constexpr int rows(int w) { return 2 * w + 2 * kFront; }
 };
 
+// Full barriers: a slot has one for its Q and K tiles (the score warp waits for each of them) and one for its V tiles (the product warp).
+// A wait names a phase by parity, so nobody may skip a fill of a barrier he waits on: with one barrier for both, a V tile that was
+// later than the scores let the next unit's first scores pass their wait for the K tile that goes to the same slot (head dim 128,
+// 32 x 32 windows: one call in a thousand).  (Waiting for V in the score warp as well: 240 x 360 tokens, 6 x 64, side 18 396 us; so 358.)
 enum { kBFull = 0, kBEmpty = 16, kBS = 32, kBP = 38, kBFree = 44, kBO = 50, kBOFree = 52, kBStat = 54, kBTab = 56, kBBias = 58,
-       kBOne = 59, kBDesc = 61, kBDescFree = kBDesc + kDescs, kBCount = kBDescFree + kDescs };
+       kBOne = 59, kBDesc = 61, kBDescFree = kBDesc + kDescs, kBFullV = kBDescFree + kDescs, kBCount = kBFullV + 16 };
 
 template <int D, int RW>
 struct Lay {
@@ -189,6 +193,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
     if (tid == 0) {
         for (int s = 0; s < L::kSlots; ++s) {
             mbar_init(bar(kBFull + s), 1);
+            mbar_init(bar(kBFullV + s), 1);
             mbar_init(bar(kBEmpty + s), 1);
         }
         for (int b = 0; b < NB; ++b) {
@@ -461,7 +466,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             int e_key = -1, q0 = -1, q1 = -1;        // what the mask operands are made for; Q slots of the last unit
             bool ok = true;
             const int part = lane % kParts, row = lane / kParts;      // lane -> channel part, window row of a tile
-            auto fill = [&](int s, const WinMaps& m, const __nv_bfloat16* src, int a0) {
+            auto fill = [&](int s, int full, const WinMaps& m, const __nv_bfloat16* src, int a0) {
                 ok = ok && mbar_wait_all(bar(kBEmpty + s), ((use >> s) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
                 use ^= 1u << s;
@@ -481,7 +486,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 const uint32_t base = smem0 + s * L::kSlotB;
                 if (win_group_whole<RW>(p.cols, g, td.wr, td.wc, td.eh, a0, 2)) {
                     if (elect_one()) {
-                        mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB);
+                        mbar_arrive_expect_tx(bar(full + s), L::kSlotB);
                         int y0 = td.wr * g.w + a0 + g.sh;
                         if (y0 >= g.H) y0 -= g.H;
                         y0 += td.b * g.H;
@@ -489,14 +494,14 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                         for (int h = 0; h < 2; ++h)
 #pragma unroll
                             for (int pt = 0; pt < kParts; ++pt)
-                                tma_load_4d(base + pt * kTile * kRowB + h * 64 * kRowB, &m.group, td.head * D + pt * L::kPartCh, 0, td.wc, y0 + h * kG, bar(kBFull + s));
+                                tma_load_4d(base + pt * kTile * kRowB + h * 64 * kRowB, &m.group, td.head * D + pt * L::kPartCh, 0, td.wc, y0 + h * kG, bar(full + s));
                     }
                 } else {
-                    if (lane == 0) mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB - (fix ? 2 * kG * kRowB : 0));
+                    if (lane == 0) mbar_arrive_expect_tx(bar(full + s), L::kSlotB - (fix ? 2 * kG * kRowB : 0));
                     __syncwarp();
                     if (row < 2 * kG)
                         load_win_row<RW, kRowB>(m, p.cols, base + part * kTile * kRowB + row * RW * kRowB, g, td.b, td.wr, td.wc, td.eh, a0 + row,
-                                                td.head * D + part * L::kPartCh, bar(kBFull + s));
+                                                td.head * D + part * L::kPartCh, bar(full + s));
                 }
                 __syncwarp();
             };
@@ -546,11 +551,11 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 }
                 q0 = sq.pop();
                 q1 = sq.pop();
-                fill(q0, mq, p.q, td.tile0 * kTileRows);
+                fill(q0, kBFull, mq, p.q, td.tile0 * kTileRows);
                 for (int c = 0; ok && c < td.nch; ++c) {
-                    fill(sq.take(), mk, p.k, c * kTileRows);
-                    if (c == 0 && td.ntq == 2) fill(q1, mq, p.q, (td.tile0 + 1) * kTileRows);
-                    fill(sq.take(), mv, p.v, c * kTileRows);
+                    fill(sq.take(), kBFull, mk, p.k, c * kTileRows);
+                    if (c == 0 && td.ntq == 2) fill(q1, kBFull, mq, p.q, (td.tile0 + 1) * kTileRows);
+                    fill(sq.take(), kBFullV, mv, p.v, c * kTileRows);
                 }
                 sq.end_unit(q0, q1);
                 if (td.ntq < 2) q1 = -1;
@@ -579,7 +584,8 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             while (ok && next_unit()) {
                 const int s_q[2] = {sq.pop(), sq.pop()};
                 for (int c = 0; ok && c < td.nch; ++c) {
-                    const int sk = sq.take(), sv = sq.take();
+                    const int sk = sq.take();
+                    sq.take();                       // (V)
                     if (c == 0) wait_full(s_q[0]);
                     wait_full(sk);
                     for (int hf = 0; hf < 2 && 4 * c + 2 * hf < td.ku; ++hf) {
@@ -611,10 +617,6 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                             __syncwarp();
                         }
                     }
-                    // The V tile is not this warp's, but a wait names a phase by parity: a slot's next fill may be waited for only once this
-                    // one is known to have landed.  (Without it, a V tile later than the scores let the next unit's first scores pass
-                    // their wait for the K tile that goes to its slot: head dim 128, 32 x 32 windows, one call in a thousand.)
-                    wait_full(sv);
                 }
                 sq.end_unit(s_q[0], s_q[1]);
             }
@@ -629,14 +631,12 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             uint32_t full_use = 0;
             unsigned idx = 0, opened[2] = {0, 0};
             bool ok = true;
-            // (Q and K fills need no wait here: a slot that holds V now held them for scores whose products this warp has issued)
             while (ok && next_unit()) {
                 const int s_q[2] = {sq.pop(), sq.pop()};
-                for (int t = 0; t < td.ntq; ++t) full_use ^= 1u << s_q[t];
                 for (int c = 0; ok && c < td.nch; ++c) {
-                    const int sk = sq.take(), sv = sq.take();
-                    full_use ^= 1u << sk;
-                    ok = mbar_wait_all(bar(kBFull + sv), (full_use >> sv) & 1, cta_abort);
+                    sq.take();                       // (K)
+                    const int sv = sq.take();
+                    ok = mbar_wait_all(bar(kBFullV + sv), (full_use >> sv) & 1, cta_abort);
                     full_use ^= 1u << sv;
                     for (int hf = 0; hf < 2 && 4 * c + 2 * hf < td.ku; ++hf) {
                         const int left = td.ku - (4 * c + 2 * hf);

@@ -1,6 +1,6 @@
-"""The window forward's pool of shared-memory slots, on the CPU: a wait names an mbarrier phase by parity, so a role may wait for a slot's
-fill only when it knows that the slot's fill before has landed; otherwise the wait is over at once and the role works on whatever
-the slot holds.  The slots' order is stepped through as the kernel's roles do it, with the waits that the source has."""
+"""The window forward's pool of shared-memory slots, on the CPU: a wait names an mbarrier phase by parity, so a role that waits on a barrier
+has to wait for each of its fills; behind one that it skips and that has not landed, the next wait is over at once and the role works
+on whatever the slot holds.  The slots' order is stepped through as the kernel's roles do it, with the barriers and waits of the source."""
 import os
 import re
 
@@ -14,10 +14,18 @@ def _section(begin, end):
     return text[text.index(begin):text.index(end)]
 
 
-def _score_waits():
-    """Which fills the score warp waits for."""
-    text = _section("- S = Q K^T", "- O += P V")
-    return {"Q0": "wait_full(s_q[0])" in text, "Q1": "wait_full(s_q[1])" in text, "K": "wait_full(sk)" in text, "V": "wait_full(sv)" in text}
+def _barrier(fill):
+    """Which of a slot's full barriers a fill completes."""
+    tensor = {"Q0": "q0, (kBFull\\w*), mq", "Q1": "q1, (kBFull\\w*), mq", "K": r"sq.take\(\), (kBFull\w*), mk", "V": r"sq.take\(\), (kBFull\w*), mv"}[fill]
+    return re.search(r"fill\(" + tensor, open(SOURCE).read())[1]
+
+
+def _waits(section):
+    """The fills that a role waits for, with the barrier it waits on."""
+    names = {"wait_full(s_q[0])": "Q0", "wait_full(s_q[1])": "Q1", "wait_full(sk)": "K", "wait_full(sv)": "V"}
+    found = {fill: re.search(r"bar\((kBFull\w*) \+ s\)", section)[1] for call, fill in names.items() if call in section}
+    direct = re.search(r"mbar_wait_all\(bar\((kBFull\w*) \+ sv\)", section)
+    return {**found, **({"V": direct[1]} if direct else {})}
 
 
 def _slots(head_dim, row_slots):
@@ -51,16 +59,13 @@ RUNS = [[(8, 2)] * 20, [(2, 2)] * 20, [(1, 1)] * 9, [(5, 2), (5, 2), (5, 1)] * 6
 
 @pytest.mark.parametrize("units", RUNS, ids=range(len(RUNS)))
 @pytest.mark.parametrize("head_dim,row_slots", [(32, 32), (64, 16), (64, 32), (128, 16), (128, 32)])
-def test_a_fill_is_waited_for_behind_the_one_before(head_dim, row_slots, units):
-    fills, waits = _fills(_slots(head_dim, row_slots), units), _score_waits()
-    last = {}
-    for slot, fill, unit, chunk in fills:
-        before = last.get(slot)
-        if before is not None:
-            # the score warp: a fill before is known to have landed if it has waited for it
-            if waits[fill]:
-                assert waits[before[0]], f"scores wait for {fill} of unit {unit}, chunk {chunk}, behind {before}, which nothing has waited for"
-            # the product warp waits for V alone: Q and K have landed where it has issued a product of their scores
-            if fill == "V" and before[0] != "V":
-                assert before[1] < unit or (before[0] == "K" and before[2] < chunk), (fill, unit, chunk, before)
-        last[slot] = (fill, unit, chunk)
+def test_a_role_waits_for_every_fill_of_its_barriers(head_dim, row_slots, units):
+    for begin, end in (("- S = Q K^T", "- O += P V"), ("- O += P V", "// teardown")):
+        waits, skipped = _waits(_section(begin, end)), {}
+        assert waits
+        for slot, fill, unit, chunk in _fills(_slots(head_dim, row_slots), units):
+            barrier = (slot, _barrier(fill))
+            if waits.get(fill) == barrier[1]:
+                assert barrier not in skipped, f"{fill} of unit {unit}, chunk {chunk} is waited for behind {skipped[barrier]}, which is not"
+            elif barrier[1] in waits.values():
+                skipped[barrier] = (fill, unit, chunk)
