@@ -1176,6 +1176,8 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     swin_bwd_onepass_prep_kernel<D, RW><<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
         const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, stat);
     count_launch(stream);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const int ctas = sm_count < kMaxCtas ? sm_count : kMaxCtas;
     auto launch = [&](auto kernel, bool inner, long long windows, int slab0, bool overlap) {
         p.inner = inner;
@@ -1198,7 +1200,6 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         return err;
     };
     const long long all = (long long)g.Mh * g.Mw;
-    cudaError_t e = cudaSuccess;
     if constexpr (D == 128) {
         p.row1 = g.Mh;
         p.col1 = g.Mw;

@@ -746,7 +746,9 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
     prof_begin("swin_fwd_win_prep_kernel", stream);
     swin_fwd_win_prep_kernel<RW><<<total / 512 + 1 < 592 ? total / 512 + 1 : 592, 256, 0, stream>>>(g, bias, (float*)workspace);
     count_launch(stream);
-    cudaError_t e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW, KC>, L::kSmemBytes);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW, KC>, L::kSmemBytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_fwd_win_kernel", stream);
     e = launch_dependent(swin_fwd_win_kernel<D, RW, KC>, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
