@@ -1092,7 +1092,8 @@ OnePassPlan bwd_onepass_plan(const Geo& g) {
         if (ls == 0 || t < 0.875 * best) { best = t; p.split_log2 = ls; }
     }
     p.units = items << p.split_log2;
-    const size_t ctas = p.units < 2 * kMaxCtas ? (size_t)p.units : (size_t)(2 * kMaxCtas);       // of both launches
+    const int most = (g.d == 128 ? 1 : 2) * kMaxCtas;    // CTAs of the launches that may overlap (see launch_onepass)
+    const size_t ctas = p.units < most ? (size_t)p.units : (size_t)most;
     const size_t slabs = p.split_log2 ? (size_t)p.units : ctas;
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t table = up(sizeof(float) * (size_t)g.heads * 2 * p.rmax * 2 * p.rw);
