@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import os
 import subprocess
 import sysconfig
@@ -11,6 +12,7 @@ CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libterra_swin.so")
 HOST_SRC = os.path.join(CSRC, "host_module.cpp")
 HOST_PATH = os.path.join(PKG_DIR, "_host.so")
+HOST_TAG_PATH = HOST_PATH + ".tag"          # the Python and torch that the native module was built for
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--shared", "-Xcompiler", "-fPIC", "-lcuda"]
@@ -29,10 +31,23 @@ def _stale() -> bool:
     return any(os.path.getmtime(p) > built for p in deps)
 
 
-def build_host(force: bool = False) -> str:
-    """Compile csrc/host_module.cpp, the attention calls' argument handling, against the installed torch."""
+def _host_tag() -> str:
+    return f"{sysconfig.get_config_var('SOABI')} torch {importlib.metadata.version('torch')}"
+
+
+def _host_stale() -> bool:
+    if not os.path.exists(HOST_PATH) or not os.path.exists(HOST_TAG_PATH):
+        return True
     header = os.path.join(os.path.dirname(PKG_DIR), "include", "terra.h")
-    if not force and os.path.exists(HOST_PATH) and os.path.getmtime(HOST_PATH) >= max(os.path.getmtime(HOST_SRC), os.path.getmtime(header)):
+    if os.path.getmtime(HOST_PATH) < max(os.path.getmtime(HOST_SRC), os.path.getmtime(header)):
+        return True
+    with open(HOST_TAG_PATH) as f:
+        return f.read() != _host_tag()
+
+
+def build_host(force: bool = False) -> str:
+    """Compile csrc/host_module.cpp, the attention calls' argument handling, against the installed Python and torch."""
+    if not force and not _host_stale():
         return HOST_PATH
     import torch
     from torch.utils import cpp_extension
@@ -44,6 +59,8 @@ def build_host(force: bool = False) -> str:
     proc = subprocess.run(cmd, capture_output=True, text=True)
     if proc.returncode != 0:
         raise RuntimeError("g++ failed:\n" + proc.stdout + proc.stderr)
+    with open(HOST_TAG_PATH, "w") as f:
+        f.write(_host_tag())
     return HOST_PATH
 
 
