@@ -346,6 +346,7 @@ swin_bwd_mma_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv
                                 // b_q of one window row a_q, and this half of the block is 32 consecutive offsets b_k of one
                                 // window row a_k.  All pairs with the same b_q - b_k share one table entry: sum each of the
                                 // 47 diagonals, then one global atomic per diagonal.
+                                // (lane l sums diagonal l, rows rr <= l, and, for l < 15, diagonal l + 32, rows rr > l)
                                 const int a_q = slot0 / g.w, bq0 = slot0 - a_q * g.w;
                                 const int k0 = blk * BN + half * 32;
                                 const int a_k = k0 / g.w, bk0 = k0 - a_k * g.w;
@@ -367,25 +368,6 @@ swin_bwd_mma_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv
                                     if (v0 != 0.f) atomicAdd(&dbias[(size_t)(code_r - code_c) * g.heads + head], v0);
                                 }
                             }
-                        } else if (g.w == 32 && r.ew == 32) {
-                            // Full-width 32-wide window: the warp's 16 rows are consecutive offsets b_q of one window row
-                            // a_q, and this half of the block is one window row a_k of keys with b_k = 0..31.  All pairs
-                            // with the same b_q - b_k share one table entry: sum each of the 47 diagonals first, then one
-                            // atomic per diagonal instead of one per pair.
-                            const int a_q = slot0 >> 5, bq0 = slot0 & 31;
-                            const int a_k = 2 * blk + half;
-                            const int row_base = (a_q - a_k) * (2 * g.w - 1) + c0;
-                            // lane l sums diagonal l (rows rr <= l) and, for l < 15, diagonal l + 32 (rows rr > l): 16 loads
-                            // per lane cover all 47 diagonals
-                            float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-                            for (int rr = 0; rr < 16; ++rr) {
-                                const bool first = rr <= lane;
-                                const float val = stage[rr * kStageStride + (first ? 31 - lane + rr : rr - lane - 1)];
-                                if (first) s0 += val; else s1 += val;
-                            }
-                            if (s0 != 0.f) atomicAdd(&s_dbias[row_base + bq0 - 31 + lane], s0);
-                            if (lane < 15 && s1 != 0.f) atomicAdd(&s_dbias[row_base + bq0 + 1 + lane], s1);
                         } else {
                             const int code_c = meta_code(s_meta[cbase(blk) + half * 32 + lane]);
                             for (int rr = 0; rr < 16; ++rr) {
