@@ -1069,8 +1069,9 @@ cudaError_t read_bwd_onepass_status(int* timed_out) {
 #ifndef TERRA_ELEM_F16
 bool bwd_onepass_supported(const Geo& g) {
     // (head dim 32 with sides up to 16 has a kernel of its own, 1.83 against 2.5 ms on the 510 x 1080 grid with 12 heads)
-    // (head dim 64, sides 9 and 10: the register-tile kernels with dense rows, 677 and 571 against 751 and 623 us on 240 x 360 tokens with
-    // 6 heads; side 11: 521 against 526)
+    // Register tiles / this kernel, us, on 240 x 360, 2 x 121 x 250 and 96 x 180 tokens: head dim 64, side 9 676/752 659/719 166/166, 10 572/626 560/601
+    // 146/140; 11 517/537 480/496 140/126 (level), 12 1032/451; head dim 128, side 9 889/800 1215/1130 289/263; head dim 32, side 17 948/967
+    // 1798/1711 389/406 (level), 18 1126/816 2278/1496 468/384.
     return ((g.d == 64 && g.w > 10) || g.d == 128 || (g.d == 32 && g.w > 16)) && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 8 < 0x7fffffffLL;
 }

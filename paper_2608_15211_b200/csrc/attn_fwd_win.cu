@@ -709,10 +709,13 @@ cudaError_t read_fwd_win_status(int* timed_out) {
 #ifndef TERRA_ELEM_F16
 bool fwd_win_supported(const Geo& g) {
     // (head dim 32 with sides up to 16 has a kernel of its own, 0.77 against 1.16 ms on the 510 x 1080 grid with 12 heads)
-    // Where a window fills little of its slots (side 17 half of them), or has one query tile and little more, the register-tile
-    // kernel with its dense rows is faster: 240 x 360 tokens, 6 x 32, side 17 214 against 487 us, side 22 305 against 319 (side 23: 347 against 308);
-    // 6 x 64, side 9 226 against 312, side 11 166 against 217 (side 12: 266 against 179), side 17 338 against 415 (18: 417 against 361).
-    const bool sparse = g.d == 32 ? g.w <= 22 : g.d == 64 && (g.w <= 11 || g.w == 17);
+    // The register-tile kernel packs a window's tokens densely; it is the faster one where a window fills little of the slots of this one.
+    // Register tiles / this kernel, us, on 240 x 360, 2 x 121 x 250 and 96 x 180 tokens:
+    //   head dim 32, side 17 214/495 400/1041 89/235, 22 302/340 556/709 123/159; 23 344/332 664/687 144/140, 24 326/258 611/638 136/126; sides
+    //   above 24 work on all 32 slots of a row: 25 353/430 705/837 154/201, 26 392/402 736/830 164/169; 27 436/386 810/816 175/181, 28 463/342;
+    //   head dim 64, side 9 226/318 212/349 52/80, 11 166/238 156/246 39/56; 12 267/183 248/214 60/46; 17 338/468 318/426 72/95; 18 416/358 379/368 95/84;
+    //   head dim 128, this kernel at every side: 9 283/261 392/369 91/95, 10 242/238 338/328 74/82, 11 207/171 287/269 68/64, 17 400/346 558/486 123/118.
+    const bool sparse = g.d == 32 ? g.w <= 22 || g.w == 25 || g.w == 26 : g.d == 64 && (g.w <= 11 || g.w == 17);
     return (g.d == 64 || g.d == 128 || (g.d == 32 && g.w > 16)) && !sparse && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 4 < 0x7fffffffLL;
 }
