@@ -1,5 +1,5 @@
-// One-pass backward on the tcgen05 tensor cores for windows of more than 64 tokens and of side 9 .. 32, head dims 64 and
-// 128 (head dim 32: sides 17 .. 32), any grid: P and dS of a (window, head) are computed once and feed dQ, dK, dV and dBias.
+// One-pass backward on the tcgen05 tensor cores for window sides 9 .. 32 at head dim 128, 11 .. 32 at 64 and 17 .. 32 at
+// 32, any grid: P and dS of a (window, head) are computed once and feed dQ, dK, dV and dBias.
 //
 // A persistent CTA takes (batch, window, head) units.  Per 128-key tile of a window it keeps K and V in shared memory and
 // streams Q and dO in half chunks of 64 query slots (slots: win_tiles.cuh).  TMEM lanes = keys, columns = queries:
@@ -19,10 +19,10 @@
 // shared-memory load for the bias and a load and a store (or a shuffle, or an atomic) for its gradient.
 // Measured, this kernel and what it needs around it against the kernels it replaces (dK / dV and dQ / dBias kernels that both
 // recomputed P and dS; the latter on mma.sync wherever a window was not a complete 32 x 32 one): 256 x 512 tokens, 12 x 64,
-// 32 x 32 windows 3.0 -> 2.2 ms; 255 x 540, the same 8.8 -> 2.3 ms; 288 x 544, 8 x 128, 16 x 16 windows 3.6 -> 1.2 ms; 64 x 128,
-// 32 x 32 windows 32.2 -> 26.2 ms.  It is bound by the elementwise warps' chain per half chunk (about 5000 cycles for 64 x 128
-// pairs, of which MUFU needs 1024 for two of them), at head dim 128 with 32 x 32 windows by L2: 148 windows in flight restream
-// their Q and dO and hold their dQ slabs, 1 MB each.
+// 32 x 32 windows 3.0 -> 2.1 ms; 255 x 540, the same 8.8 -> 2.2 ms; 288 x 544, 8 x 128, 16 x 16 windows 3.6 -> 1.1 ms; 64 x 128,
+// 32 x 32 windows 32.2 -> 23.9 ms.  It is bound by the elementwise warps' chain per half chunk (issue slots 36 %, tensor pipe 26 %, DRAM 14 %),
+// at head dim 128 with 32 x 32 windows by L2: 148 windows in flight restream their Q and dO and hold their dQ slabs, 1 MB each; on 96 x
+// 160 tokens 7.3 GB are read and 4.0 GB written for 0.9 GB of tensors, and 15 % of L2's sector reads hit.
 // dS^T leaves for shared memory by stmatrix in the layout the dQ product reads.
 //
 // Roles (512 threads): warps 0-3 / 4-7 elementwise on the even / odd half chunks, warps 8-11 read accumulators out of

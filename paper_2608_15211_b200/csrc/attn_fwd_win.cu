@@ -1,12 +1,13 @@
-// Forward shifted-window attention on the tcgen05 tensor cores: window sides 9 .. 32 at head dims 32, 64 and 128, any grid.
+// Forward shifted-window attention on the tcgen05 tensor cores: window sides 9 .. 32 at head dims 64 and 128, 17 .. 32 at head dim 32 (less the
+// sides that fwd_win_supported leaves to the register tiles), any grid.
 //
 // A unit is a pair of 128-row query tiles of one (sample, window, head); a persistent CTA per SM walks over units and streams
 // the window's keys through shared memory in chunks of 128 slots (see win_tiles.cuh: 16 or 32 slots to a window row).  Per
-// chunk and query tile:
-//   S = Q K^T (+ E_q E_k^T, see below), 128 x 128 in TMEM;
-//   the softmax warps, 32 query rows each, take the rows' 128 scores into registers in one go, add the bias, take their exact
-//   maximum, raise the row's reference m when the chunk exceeds it by more than 8 octaves (rare; O and the row sum are
-//   scaled down then), and write P = exp2(S scale + bias - m) over S in 16 bits;
+// half chunk of 64 keys and query tile:
+//   S = Q K^T (+ E_q E_k^T, see below), 128 x 64 in TMEM;
+//   the softmax warps, 32 query rows each, take the rows' 64 scores into registers, add the bias, take the maximum, raise the
+//   row's reference m when the half chunk exceeds it by more than 8 octaves (rare; O and the row sum are scaled down then),
+//   and write P = exp2(S scale + bias - m) over S in 16 bits; the row sum is added up in fp32 before that rounding;
 //   O += P V, accumulated in TMEM.
 // Masks cost the softmax threads nothing: where a window's slots differ in shift-mask label or hold no token, one more
 // 16-wide step of the score product (bf16 operands in either build) adds 2^64 x -2^64 to the pairs that must not see one
@@ -16,9 +17,11 @@
 // (Selects by label in every half chunk of the windows that mix them, before or after the load: 256 x 512 tokens, 12 x 64,
 // 32 x 32 windows, one in eight masked, 850 -> 1000 us.)  One body serves every window: the elementwise code is what bounds
 // the kernel, and two copies of it in one kernel run slower than one.
-// Scores and P share three TMEM buffers (head dim 128: two), so that the products of other chunks run under the softmax.
+// Scores and P share six TMEM buffers (head dim 128: four), so that the products of other half chunks run under the softmax.
 //
-// What bounds it: MUFU, 16 exponentials per clock and SM (0.40 ms for the 510 x 1080 grid with 12 heads and 16 x 16 windows).
+// What bounds it: the softmax warps' chain per half chunk, two warps a scheduler: 0.87 ms for 256 x 512 tokens, 12 x 64, 32 x 32 windows, of
+// which the exponentials need 0.35 (16 a clock and SM); issue slots 40 %, tensor pipe 22 %, DRAM 10 %.  Head dim 128: 7.1 ms for
+// 288 x 544 tokens, 64 x 128 (exponentials 2.2 ms), tensor pipe 39 %.
 //
 // Roles (512 threads): warps 0-3 / 4-7 softmax of the pair's first / second tile, warps 8-11 read O out of TMEM, normalise
 // and store it, warp 12 issues the PV products, warp 13 every copy, warp 14 the scores, warp 15 walks over the units.

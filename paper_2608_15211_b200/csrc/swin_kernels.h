@@ -85,8 +85,7 @@ cudaError_t read_tc_status(int* timed_out, cudaStream_t stream);
 bool tma_row_shape(const Geo& g);
 bool make_row_map(void* cu_tensor_map, const Geo& g, const void* base, int token_stride, int box_tokens, int box_ch = 32);
 
-// tcgen05 forward path for head dim 64 and windows of up to 1024 tokens (keys streamed in chunks, two passes)
-// windows of side 9 .. 32 on any grid (attn_fwd_win.cu)
+// tcgen05 forward path for window sides 9 .. 32 (head dim 32: 17 .. 32) on any grid (attn_fwd_win.cu)
 bool fwd_win_supported(const Geo& g);
 size_t fwd_win_workspace_bytes(const Geo& g);
 cudaError_t launch_fwd_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
@@ -95,6 +94,7 @@ cudaError_t launch_fwd_win_f16(const Geo& g, const void* q, const void* k, const
                                int sm_count, cudaStream_t stream);
 cudaError_t read_fwd_win_status(int* timed_out);
 cudaError_t read_fwd_win_status_f16(int* timed_out);
+// tcgen05 forward path for head dims 64 and 128 and complete windows of side 64 and 128 (keys streamed once in chunks)
 bool fwd_tc64_supported(const Geo& g);
 size_t fwd_tc64_workspace_bytes(const Geo& g);
 cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
@@ -103,8 +103,8 @@ cudaError_t read_fwd_tc64_status(int* timed_out);     // after the stream has be
 // (window sides 64 and 128: whole table rows; `reflect`: the table reflected through its centre)
 cudaError_t launch_bias_prep64(const Geo& g, const float* bias, float* prep, cudaStream_t stream, bool reflect = false);
 
-// tcgen05 key side (dK, dV) of the backward pass for head dim 64 and windows of up to 1024 tokens; `prep` = the
-// tables of launch_bias_prep64, `delta` as for the register-tile kernels
+// tcgen05 key side (dK, dV) of the backward pass for head dims 64 and 128 and complete windows of side 64 and 128; `prep` =
+// the tables of launch_bias_prep64, `delta` as for the register-tile kernels
 bool bwd_kv64_supported(const Geo& g);
 cudaError_t launch_bwd_kv64(const Geo& g, const void* q, const void* k, const void* v, const void* d_o, const float* prep,
                             const float* lse, const float* delta, void* dk, void* dv, int sm_count, cudaStream_t stream);
@@ -115,7 +115,7 @@ cudaError_t launch_bwd_kv64_qside(const Geo& g, const void* q, const void* k, co
                                   const float* prep_reflected, const float* lse, const float* delta, void* dq, float* dbias,
                                   int sm_count, cudaStream_t stream);
 
-// One-pass tcgen05 backward for windows of more than 64 tokens and side <= 32, every head dim, any grid.
+// One-pass tcgen05 backward for window sides 9 .. 32 at head dim 128, 11 .. 32 at 64 and 17 .. 32 at 32, any grid.
 struct OnePassPlan {
     int rw;                  // slots per window row
     int npad, rmax;          // slots of a window rounded up to 128; window rows rounded up to whole key tiles

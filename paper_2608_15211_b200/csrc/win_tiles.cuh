@@ -1,5 +1,5 @@
-// Windows as tiles of slots, loaded by tiled bulk copies (TMA) on ANY grid: shared by the one-pass backward kernel and
-// its host side.
+// Windows as tiles of slots, loaded by tiled bulk copies (TMA) on ANY grid: shared by the window forward, the one-pass
+// backward and their host sides.
 //
 // A window's slots are laid out RW to a window row (RW = 16 for window sides 9 .. 16, 32 for 17 .. 32): slot = RW a + b.
 // Slots with b at or beyond the window's width, or a at or beyond its height, hold no token; the copies fill them with
