@@ -37,6 +37,7 @@
 #include "tc_common.cuh"
 #include "win_tiles.cuh"
 
+#include <cmath>
 #include <cstring>
 
 // fp16 build of this file (through the _f16 wrapper file): names of its own
@@ -62,7 +63,7 @@ constexpr int kTile = 128, kHalf = 64;
 constexpr int kDescs = 8;                                                             // ring of tile descriptors
 constexpr int kScrLine = 160;                                                         // see flush_sums
 
-template <int D, int RW>
+template <int D, int RW, bool ST = false>
 struct Lay {
     static constexpr int kParts = D == 128 ? 2 : 1, kRowB = D >= 64 ? 128 : 64;      // channel parts of a row, bytes of a part's row
     static constexpr int kPartCh = kRowB / 2;
@@ -75,7 +76,7 @@ struct Lay {
     // per half chunk (ring of kTabs): 64 queries' statistics, then the bias rows its pieces meet, twice (the second copy shifted
     // by one entry and 16 banks away, so that lanes with even and odd g read different banks); head dim 128 has no room
     // and reads them from global memory
-    static constexpr bool kTables = D != 128;
+    static constexpr bool kTables = D != 128 && !ST, kGang = ST || (D == 128 && RW == 32);
     static constexpr int kTabs = 4, kBiasRows = kTile / RW + kHalf / RW - 1, kCopyB = kBiasRows * 2 * RW * 4;
     static constexpr int kOffCopy0 = 512, kOffCopy1 = 512 + (kCopyB + 127) / 128 * 128 + 64;
     static constexpr int kTabB = kTables ? (kOffCopy1 + kCopyB + 127) / 128 * 128 : 0;
@@ -94,7 +95,7 @@ struct Lay {
     // dQ: head dim 32 two regions of its own; head dim 64 over P^T and dS^T of buffer 1 (per 128 queries); head dim 128
     // over dP^T of its buffer (per half chunk)
     static constexpr int kColDq = D == 32 ? 448 : D == 64 ? 320 : 64, kStrideDq = D == 32 ? 32 : 128;
-    static constexpr int kResident = D == 32 ? 2 : 0;                                 // windows of that many 128-query chunks keep dQ in TMEM
+    static constexpr int kResident = D == 32 && !ST ? 2 : 0;                                 // windows of that many 128-query chunks keep dQ in TMEM
 };
 
 // barriers (8 bytes each)
@@ -107,16 +108,24 @@ struct Params {
     int split_log2;                  // key tiles of a window are shared by 1 << split_log2 units
     int npad;                        // slots of a full window, rounded up to 128
     int rmax;                        // window rows rounded up to whole key tiles: bias-table rows run from -rmax to rmax - 1
+    int rl;                          // floats of a bias-table row: 2 RW (ST: 64 for every strip of a full window row)
     // The launch's units: first those of the windows (row >= row1, any column), then of (row < row1, column >= col1); a launch of
     // the inner windows has the units of (row < row1, column < col1).
     int row1, col1, inner;
     int slab0;                       // first slab of the launch (two launches may overlap)
     int overlap;                     // the launch runs beside the one before it, which started when its prerequisites were complete
+    // Gangs: `gang` CTAs work on the key tiles of one (window, head) after the other, each on every gang-th of the gang's tiles, and add
+    // to the window's dQ slab in the tiles' order.  flags[slab][event][read-out warp] = number of the next tile that may add
+    // (tiles numbered through the gang's run), flags[slab][events] = windows that are done with the slab.
+    // Where every gang has one window only, the CTAs start at different chunks of its queries (`rotate`) instead of after one another.
+    int gangs, gang, ring, events, rotate;
+    int turn_log2;                   // dQ events that the CTAs take turns by
+    unsigned* flags;
     long long units;
     const float4* rowstat;           // per (b, window, head) and slot pair: (-lse log2 e) x 2, delta x 2
-    const float* bias0;              // [head][2 rmax][2 RW]: bias log2 e at (da + rmax, db + RW), 0 outside the table
+    const float* bias0;              // [head][2 rmax][rl]: bias log2 e at (da + rmax, db + rl / 2), 0 outside the table
     const float* bias1;              // the same, shifted by one entry
-    float* dbias_acc;                // [head][2 rmax][2 RW]
+    float* dbias_acc;                // [head][2 rmax][rl]
     const __nv_bfloat16 *q, *k, *v, *d_o;
     float4* slabs;                   // dQ partial sums: one slab of npad x D floats per CTA (per unit where windows are split)
 };
@@ -144,6 +153,8 @@ struct TileDesc {
     int ha, hb;            // window rows >= ha / columns >= hb carry the other shift-mask label (far outside: none do)
     int flags;             // 1: a tile (0: the end), 2: the unit's first, 4: its last
     int slab;
+    int ns;                // ST: strips of a window row
+    int seq, use, c0;      // gangs: number of the window's first tile, windows before on this slab; first chunk of queries
 };
 
 __device__ __forceinline__ float2 lds_f2(uint32_t addr) {
@@ -255,10 +266,10 @@ __device__ __forceinline__ void step_math(const uint32_t (&rs)[2][8], const uint
 // through shared memory: a line of five groups of 8 floats per g, group = s in order, so that lane l's entry of line g lies at
 // l + 1 + g: one address and immediate offsets, and (lines 40 floats apart) no bank conflicts in either direction.  RW = 32:
 // s = -3 .. 0 behind a group of zeros give diagonals l - 31, s = 0 .. 3 in front of one give l + 1; RW = 16: a round per row
-// difference, s = -1 .. 1 between two groups of zeros, diagonals l - 15.  `acc_row`: floats from piece 0's row to piece 1's.
+// difference, s = -1 .. 1 between two groups of zeros, diagonals l - 15.  `acc`, `acc1`: where the pieces' diagonal -RW would go.
 template <int RW>
-__device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][Piece<RW>::kSums], int lane, float* acc) {
-    constexpr int kRounds = RW == 32 ? 2 : 3, kRow = (32 / RW) * 2 * RW;
+__device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][Piece<RW>::kSums], int lane, float* acc, float* acc1) {
+    constexpr int kRounds = RW == 32 ? 2 : 3;
     const uint32_t w = scr + (lane >> 2) * kScrLine + (lane & 3) * 8, rd = scr + (lane + 1) * 4;
 #pragma unroll
     for (int r = 0; r < kRounds; ++r) {
@@ -288,7 +299,7 @@ __device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const float x = ((v[j][0] + v[j][1]) + (v[j][2] + v[j][3])) + ((v[j][4] + v[j][5]) + (v[j][6] + v[j][7]));
-            float* dst = acc + j * kRow + (RW == 32 ? (r ? 33 : 1) : (r - 1) * 2 * RW + 1) + lane;
+            float* dst = (j ? acc1 : acc) + (RW == 32 ? (r ? 33 : 1) : (r - 1) * 2 * RW + 1) + lane;
             if ((RW == 32 && r == 0) || lane < 31) red_f1(dst, x);
         }
     }
@@ -298,10 +309,10 @@ __device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][
 // `t_s`: S^T (dP^T 64 columns behind it); `t_p`: P^T (dS^T kDsOff behind it).  Head dims 32 and 64: the next step's scores are
 // loaded ahead, pc[0] holds the first piece's tables and the second's follow from shared memory (`tab_b`, `tab_s`).  Head dim
 // 128: pc holds both pieces' tables, whose trip to L2 is the longer one.
-template <int D, int RW, int MASK>
+template <int D, int RW, int MASK, bool ST>
 __device__ __forceinline__ void half_chunk(uint32_t t_s, uint32_t t_p, uint32_t st_addr, Piece<RW> (&pc)[2], uint32_t tab_b, uint32_t tab_s,
                                            const uint32_t (&okm)[2][4], float scale, float2 (&sum)[2][Piece<RW>::kSums], int lane, uint32_t bar_sfree) {
-    using L = Lay<D, RW>;
+    using L = Lay<D, RW, ST>;
     constexpr int kAhead = L::kTables ? 1 : 0;
     uint32_t rs[1 + kAhead][2][8], rp[1 + kAhead][2][8];
     auto ld = [&](int i) {
@@ -340,12 +351,12 @@ __device__ __forceinline__ void half_chunk(uint32_t t_s, uint32_t t_p, uint32_t 
 // dim 128).  Two launches instead of a branch: with both bodies in one kernel the unmasked one ran 1.14 times as long (the
 // elementwise warps are sensitive to what the compiler and the instruction caches make of them), at head dim 128 it is not
 // what bounds the kernel.
-template <int D, int RW, int KIND>
+template <int D, int RW, int KIND, bool ST>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk,
                         __nv_bfloat16* __restrict__ dv, const __grid_constant__ WinMaps mq, const __grid_constant__ WinMaps mk,
                         const __grid_constant__ WinMaps mv, const __grid_constant__ WinMaps mg) {
-    using L = Lay<D, RW>;
+    using L = Lay<D, RW, ST>;
     constexpr int kParts = L::kParts, kRowB = L::kRowB, kG = kHalf / RW;
     extern __shared__ __align__(1024) unsigned char smem[];
     const uint32_t smem0 = smem_u32(smem), bar0 = smem0 + L::kOffBars;
@@ -400,6 +411,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         td.head = d0.x; td.b = d0.y; td.wr = d0.z; td.wc = d0.w;
         td.eh = d1.x; td.ew = d1.y; td.kt = d1.z; td.nch = d1.w;
         td.ha = d2.x; td.hb = d2.y; td.flags = d2.z; td.slab = d2.w;
+        const int4 d3 = src[3];
+        td.ns = ST ? d3.x : 1; td.seq = d3.y; td.use = d3.z; td.c0 = L::kGang ? d3.w : 0;
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kBDescFree + i));
         ++desc_n;
@@ -416,15 +429,16 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         const float scale = g.scale_log2e;
         const uint32_t tq = tmem + ((uint32_t)(32 * wq) << 16);
         const uint32_t t_s = tq + 128u * b, t_p = tq + L::kColP + L::kStrideP * b;
-        const int head_f = 2 * p.rmax * 2 * RW;
+        const int rl = ST ? p.rl : 2 * RW, head_f = 2 * p.rmax * rl;
         // stmatrix: lane l addresses row l % 8 of the four matrices (m, k) = (l / 16, l / 8 % 2)
         const uint32_t st_off = (uint32_t)((32 * wq + 8 * (lane >> 4) + (lane & 7)) * 128 + ((((lane >> 3) & 1) ^ (lane & 7)) << 4));
         const uint32_t scr0 = D == 128 ? smem0 + L::kOffDs + b * L::kDsB + 32 * wq * 128 : smem0 + L::kOffScr + warp * L::kScrB;
         unsigned n = 0;                                      // half chunks of this buffer so far
-        int a_k0, nh, ha, row0, hc = 0;
+        int a_k0, nh, left, ha, row0, hc = 0;
+        int c_k0 = 0;                                        // ST: first column of the warp's keys
         bool masked;
         uint32_t rowbits, qbits, sp;
-        const int lane_e = 2 * t - gl - (gl & 1) + RW;       // the thread's entry within a table row (even: both copies are read in pairs)
+        const int lane_e = 2 * t - gl - (gl & 1) + (ST ? rl / 2 : RW);       // the thread's entry within a table row (even: both copies are read in pairs)
         const float* tbl = ((gl & 1) ? p.bias1 : p.bias0) + lane_e;
         // in a staged table: piece 0's row difference 0 is row 128 / RW - 1 - (the warp's first key row in the tile)
         const uint32_t tab_b0 = smem0 + L::kOffTab + ((gl & 1) ? L::kOffCopy1 : L::kOffCopy0) + ((kTile / RW - 1 - (RW == 32 ? wq : 2 * wq)) * 2 * RW + lane_e) * 4;
@@ -433,34 +447,45 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         // the next tile: what its half chunks have in common
         auto enter_tile = [&]() {
             if (!next_tile()) return false;
-            hc = b;
+            hc = 2 * td.c0 + b;
+            left = td.nch;
             nh = 2 * td.nch;
             ha = td.ha;
             a_k0 = td.kt * (kTile / RW) + (RW == 32 ? wq : 2 * wq);
+            if (ST) {
+                const int u = a_k0;
+                a_k0 = unit_row(u, td.ns);
+                c_k0 = 32 * (u - a_k0 * td.ns);
+            }
             const bool labels = (ha > 0 && ha < td.eh) || (td.hb > 0 && td.hb < td.ew);
-            masked = KIND == 1 || (KIND == 2 && (labels || td.ew < RW || (td.kt + 1) * (kTile / RW) > td.eh));
+            masked = KIND == 1 || (KIND == 2 && (labels || td.ew < td.ns * RW || (td.kt + 1) * (kTile / RW) > td.eh * td.ns));
             rowbits = 0;                                     // bits m: the row holds a key; bits 4 + m: it lies behind hb
             qbits = 0;
             if (masked) {
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
-                    const int a = a_k0 + (RW == 32 ? 0 : m >> 1), bb = gl + 8 * (RW == 32 ? m : m & 1);
+                    const int a = a_k0 + (RW == 32 ? 0 : m >> 1), bb = c_k0 + gl + 8 * (RW == 32 ? m : m & 1);
                     rowbits |= (((a < td.eh && bb < td.ew) ? 1u : 0u) << m) | ((bb >= td.hb ? 16u : 0u) << m);
                     const int q0 = (RW == 32 ? 8 * m : 8 * (m & 1)) + 2 * t;
                     qbits |= ((q0 >= td.hb ? 1u : 0u) | (q0 + 1 >= td.hb ? 2u : 0u)) << (2 * m);
                 }
             }
             // piece 0 of half chunk 0: row difference a_q - a_k = -a_k0
-            row0 = td.head * head_f + (p.rmax - a_k0) * (2 * RW);
+            row0 = td.head * head_f + (p.rmax - a_k0) * rl - c_k0;
             sp = (uint32_t)(((td.b * g.Mh + td.wr) * g.Mw + td.wc) * g.heads + td.head);
             return true;
         };
-        auto bias_ptr = [&]() { return tbl + row0 + hc * kG * (2 * RW); };
+        // floats from there to piece j of half chunk hc
+        auto piece_at = [&](int j) {
+            if (!ST) return (hc * kG + j * (32 / RW)) * (2 * RW);
+            const int u = 2 * hc + j, a = unit_row(u, td.ns);
+            return a * rl + 32 * (u - a * td.ns);
+        };
         auto stat_ptr = [&]() { return p.rowstat + (size_t)sp * (p.npad / 2) + (hc * 32 + t); };
         bool live = enter_tile();
         auto load_tables = [&]() {
-            pc[0].load(bias_ptr(), stat_ptr());
-            pc[1].load(bias_ptr() + (32 / RW) * 2 * RW, stat_ptr() + 16);
+            pc[0].load(tbl + row0 + piece_at(0), stat_ptr());
+            pc[1].load(tbl + row0 + piece_at(1), stat_ptr() + 16);
         };
         if (live && !L::kTables) load_tables();
         while (live) {
@@ -476,11 +501,21 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             tc_fence_after();
             uint32_t okm[2][4] = {};
             if (!masked) {
-                half_chunk<D, RW, KIND == 1 ? 1 : 0>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
+                half_chunk<D, RW, KIND == 1 ? 1 : 0, ST>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
             } else {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const int aq = hc * kG + j * (32 / RW);
+                    int aq = hc * kG + j * (32 / RW);
+                    if (ST) {
+                        const int u = aq;
+                        aq = unit_row(u, td.ns);
+                        qbits = 0;
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            const int q0 = 32 * (u - aq * td.ns) + 8 * m + 2 * t;
+                            qbits |= ((q0 >= td.hb ? 1u : 0u) | (q0 + 1 >= td.hb ? 2u : 0u)) << (2 * m);
+                        }
+                    }
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
                         const bool ka = a_k0 + (RW == 32 ? 0 : m >> 1) >= ha;
@@ -489,7 +524,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                         okm[j][m] = (rowbits & (1u << m)) ? ((rowbits & (16u << m)) ? qbits : ~qbits) & rows : 0u;
                     }
                 }
-                half_chunk<D, RW, KIND == 0 ? 0 : 1>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
+                half_chunk<D, RW, KIND == 0 ? 0 : 1, ST>(t_s, t_p, st_addr, pc, tb, ts, okm, scale, sum, lane, bar(kBSFree + b));
             }
             fence_proxy_async();
             tmem_st_wait();
@@ -500,14 +535,16 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 if (L::kTables) mbar_arrive(bar(kBTabFree + ti));
             }
             // the next half chunk's tables are on their way while the rest is done
-            float* acc = p.dbias_acc + row0 + hc * kG * (2 * RW);
+            float* acc = p.dbias_acc + row0 + piece_at(0) + (ST ? rl / 2 - 32 : 0);
+            float* acc1 = p.dbias_acc + row0 + piece_at(1) + (ST ? rl / 2 - 32 : 0);
             hc += 2;
-            if (hc >= nh) live = enter_tile();
+            if (L::kGang && hc >= nh) hc -= nh;
+            if (--left == 0) live = enter_tile();
             if (live && !L::kTables) load_tables();
             // The bias gradient, while the products are computed.  Head dim 128 has no shared memory to spare: the sums go
             // through the warp's own rows of the dS^T tile once the dQ product has read them.
             if (D == 128 && !mbar_wait_all(bar(kBDq + b), n & 1, cta_abort)) break;
-            flush_sums<RW>(scr0, sum, lane, acc);
+            flush_sums<RW>(scr0, sum, lane, acc, acc1);
             if (D == 128) __syncwarp();
             ++n;
         }
@@ -540,6 +577,55 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 v[4 * i + 3] = __float_as_uint(__uint_as_float(v[4 * i + 3]) + o.w);
             }
         };
+        // Gangs.  A tile adds to a turn's part of its slab when the tile before it has, the window's first tile stores there when the slab's
+        // last window is done with it.  This warp reads and writes the same rows of the slab in every CTA, so it only waits for its like.
+        // The release in front of the signal waits for the adds to arrive; it is left until the next event, when most have.
+        const bool ganged = L::kGang && p.gang > 1;
+        auto flag = [&](int i) { return p.flags + ((size_t)td.slab * (p.events + 1) + i) * 4 + wq; };
+        unsigned* pending = nullptr;
+        unsigned pending_value = 0;
+        // A tile's place in the order of those that add to chunk c: the tiles' own, or (rotate) from round to round of the gang's CTAs and in
+        // each from the one that starts at the chunk, or last in front of it, downwards.
+        auto place = [&](int c) {
+            if (!p.rotate) return td.kt;
+            const int n = min(p.gang, td.nch), j = td.kt % n, round = td.kt - j, in_round = min(n, td.nch - round);
+            const int r = min(in_round - 1, ((c + 1) * n - 1) / td.nch) - j;
+            return round + (r < 0 ? r + in_round : r);
+        };
+        auto signal = [&](unsigned* f, unsigned value) {
+            __syncwarp();
+            if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;\n" ::"l"(f), "r"(value) : "memory");
+        };
+        auto signal_pending = [&]() {
+            if (pending) signal(pending, pending_value);
+            pending = nullptr;
+        };
+        auto await_flag = [&](const unsigned* f, unsigned value) {
+            const long long t0 = clock64();
+            while (true) {
+                unsigned v;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(f) : "memory");
+                if (__all_sync(0xffffffffu, v >= value)) return true;
+                if (__any_sync(0xffffffffu, *cta_abort != 0 || clock64() - t0 > 4000000000LL)) {
+                    *cta_abort = 1;
+                    return false;
+                }
+            }
+        };
+        // in front of event `ev` of a tile that is not a window's only one
+        auto turn = [&](int ev, int at) {
+            signal_pending();
+            const bool starts = (ev & ((1 << p.turn_log2) - 1)) == 0;
+            if (at == 0) return !starts || p.rotate || ev > 0 || await_flag(flag(p.events), td.use);
+            return !starts || await_flag(flag(ev >> p.turn_log2), td.seq + at);
+        };
+        // behind it; `end`: the window's last
+        auto turn_done = [&](int ev, int at, bool end) {
+            if (end || ((ev + 1) & ((1 << p.turn_log2) - 1)) == 0) {
+                pending = flag(ev >> p.turn_log2);
+                pending_value = td.seq + at + 1;
+            }
+        };
         // the accumulator columns are handed back as soon as they are in registers: 64 at a time
         constexpr int kLd = D == 32 ? 1 : 2;
         auto hand_back = [&](int i) {
@@ -549,14 +635,24 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             if (lane == 0) mbar_arrive(bar(i));
         };
         while (ok && next_tile()) {
-            const bool first = td.flags & 2, last = td.flags & 4;
+            bool first = td.flags & 2, last = td.flags & 4;
+            const bool shared = ganged && td.nch > 1;
+            int at = td.kt;
             const size_t sample = (size_t)td.b * g.H * g.W;
             float4* slab = p.slabs + (size_t)td.slab * ((size_t)p.npad * D / 4) + row;
             if (D == 128) {
                 // dQ^T: lanes = channels, columns = the half chunk's queries
-                for (int hc = 0; hc < 2 * td.nch; ++hc, ++n) {
+                for (int i = 0, hc = 2 * td.c0; i < 2 * td.nch; ++i, ++n, hc = hc + 1 == 2 * td.nch ? 0 : hc + 1) {
                     const int b = hc & 1;
-                    ok = mbar_wait_all(bar(kBDq + b), (n >> 1) & 1, cta_abort);
+                    if (shared) {
+                        if (p.rotate) {
+                            at = place(hc >> 1);
+                            first = at == 0;
+                            last = at == td.nch - 1;
+                        }
+                        ok = turn(hc, at);
+                    }
+                    ok = ok && mbar_wait_all(bar(kBDq + b), (n >> 1) & 1, cta_abort);
                     if (!ok) break;
                     tc_fence_after();
                     uint32_t r[2][32];
@@ -573,12 +669,12 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                             const int s0 = hc * kHalf + 32 * hh;
 #pragma unroll
                             for (int jr = 0; jr < 32 / RW; ++jr) {
-                                const int a = s0 / RW + jr;
+                                const int u = s0 / RW + jr, a = ST ? unit_row(u, td.ns) : u, c0 = ST ? 32 * (u - a * td.ns) : 0;
                                 if (a >= td.eh) continue;
-                                int v = td.wc * g.w + g.sw;
+                                int v = td.wc * g.w + c0 + g.sw;
                                 if (v >= g.W) v -= g.W;
-                                __nv_bfloat16* base = dq + (sample + (size_t)win_token(g, td.wr, td.wc, a, 0) - v) * g.ts + td.head * D;
-                                if (v + td.ew <= g.W && td.ew == RW) {
+                                __nv_bfloat16* base = dq + (sample + (size_t)win_token(g, td.wr, td.wc, a, c0) - v) * g.ts + td.head * D;
+                                if (ST ? v + 32 <= g.W && c0 + 32 <= td.ew : v + td.ew <= g.W && td.ew == RW) {
                                     // two lanes exchange halves, so that each stores two channels of every other query
                                     uint32_t* d2 = reinterpret_cast<uint32_t*>(base + (size_t)(v + (row & 1)) * g.ts + (row & ~1));
 #pragma unroll
@@ -591,7 +687,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                                 } else {
 #pragma unroll
                                     for (int i = 0; i < RW; ++i) {
-                                        if (i < td.ew) {
+                                        if (c0 + i < td.ew) {
                                             const uint32_t pkd = pack_elem(__uint_as_float(r[hh][jr * RW + i]) * out_scale, 0.f);
                                             *reinterpret_cast<uint16_t*>(base + (size_t)v * g.ts + row) = (uint16_t)pkd;
                                         }
@@ -601,13 +697,22 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                             }
                         }
                     }
+                    if (shared && !last) turn_done(hc, at, hc == 2 * td.nch - 1);
                 }
             } else {
-                const bool resident = td.nch <= L::kResident;
+                const bool resident = !ganged && td.nch <= L::kResident;
                 if (!resident || last) {
-                    for (int ch = 0; ch < td.nch; ++ch) {
+                    for (int i = 0, ch = td.c0; i < td.nch; ++i, ch = ch + 1 == td.nch ? 0 : ch + 1) {
                         const int r = D == 64 ? 0 : resident ? ch : (int)(n++ & 1);
-                        ok = mbar_wait_all(bar(kBDq + r), (dq_use >> r) & 1, cta_abort);
+                        if (shared) {
+                            if (p.rotate) {
+                                at = place(ch);
+                                first = at == 0;
+                                last = at == td.nch - 1;
+                            }
+                            ok = turn(ch, at);
+                        }
+                        ok = ok && mbar_wait_all(bar(kBDq + r), (dq_use >> r) & 1, cta_abort);
                         if (!ok) break;
                         dq_use ^= 1u << r;
                         tc_fence_after();
@@ -615,7 +720,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
 #pragma unroll
                         for (int q = 0; q < kLd; ++q) tmem_ld32(tl + L::kColDq + L::kStrideDq * r + 32 * q, v[q]);
                         hand_back(kBDqFree + r);
-                        const int slot = ch * kTile + row, a = slot / RW, b = slot % RW;
+                        const int slot = ch * kTile + row, u = slot / RW, a = ST ? unit_row(u, td.ns) : u, b = slot % RW + (ST ? 32 * (u - a * td.ns) : 0);
                         const bool add = !resident && !first, tok = a < td.eh && b < td.ew;
                         uint4* dst = reinterpret_cast<uint4*>(dq + (sample + (tok ? win_token(g, td.wr, td.wc, a, b) : 0)) * g.ts + td.head * D);
 #pragma unroll
@@ -628,16 +733,21 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                                 if (tok) store_scaled32(dst + 4 * q, v[q], out_scale);
                             }
                         }
+                        if (shared && !last) turn_done(ch, at, ch == td.nch - 1);
                     }
                 }
             }
             if (!ok) break;
+            if (shared) {
+                signal_pending();
+                if (!p.rotate && last) signal(flag(p.events), td.use + 1);
+            }
             // ---- dV and dK of the key tile
             ok = mbar_wait_all(bar(kBAcc), na & 1, cta_abort);
             if (!ok) break;
             ++na;
             tc_fence_after();
-            const int slot = td.kt * kTile + row, a = slot / RW, b = slot % RW;
+            const int slot = td.kt * kTile + row, u = slot / RW, a = ST ? unit_row(u, td.ns) : u, b = slot % RW + (ST ? 32 * (u - a * td.ns) : 0);
             const bool tok = a < td.eh && b < td.ew;
             const size_t off = (sample + (tok ? win_token(g, td.wr, td.wc, a, b) : 0)) * g.ts + td.head * D;
 #pragma unroll
@@ -664,7 +774,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             struct { int b, wr, wc; } cur = {0, 0, 0};
             unsigned i = 0;
             bool ok = true;
-            auto put = [&](int flags, int head, int eh, int ew, int kt, int nch, int slab) {
+            auto put = [&](int flags, int head, int eh, int ew, int kt, int nch, int slab, int seq = 0, int use = 0, int c0 = 0) {
                 ok = mbar_wait_all(bar(kBDescFree + i % kDescs), ((i / kDescs) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
                 if (lane == 0) {
@@ -672,6 +782,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     dst[0] = make_int4(head, cur.b, cur.wr, cur.wc);
                     dst[1] = make_int4(eh, ew, kt, nch);
                     dst[2] = make_int4((!g.ph && g.sh > 0) ? g.H - g.sh - cur.wr * g.w : (1 << 20), (!g.pw && g.sw > 0) ? g.W - g.sw - cur.wc * g.w : (1 << 20), flags, slab);
+                    dst[3] = make_int4(strips_of(ew), seq, use, c0);
                     mbar_arrive(bar(kBDesc + i % kDescs));
                 }
                 __syncwarp();
@@ -699,7 +810,9 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     __syncwarp();
                 }
             };
-            for (long long u = blockIdx.x; ok && u < p.units; u += gridDim.x) {
+            const int member = (int)blockIdx.x % p.gang;
+            int seq = 0, windows = 0;                // tiles and windows of several tiles of the gang so far
+            for (long long u = blockIdx.x / p.gang; ok && u < p.units; u += p.gangs) {
                 // unit -> head and share, window, sample (the windows of the launch: see Params)
                 const unsigned hs = (unsigned)g.heads << p.split_log2, bottom = (unsigned)(g.Mh - p.row1) * g.Mw;
                 const unsigned per_row = p.inner ? p.col1 : g.Mw - p.col1, per_sample = p.row1 * per_row + (p.inner ? 0u : bottom);
@@ -715,10 +828,18 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     cur.wc = (p.inner ? 0 : p.col1) + r % per_row;
                 }
                 const int head = hd >> p.split_log2, split = hd - (head << p.split_log2);
-                const int eh = min(g.w, g.H - cur.wr * g.w), ew = min(g.w, g.W - cur.wc * g.w), nch = (eh * RW + kTile - 1) / kTile;
+                const int eh = min(g.w, g.H - cur.wr * g.w), ew = min(g.w, g.W - cur.wc * g.w), nch = (eh * (ST ? strips_of(ew) : 1) * RW + kTile - 1) / kTile;
                 const int kt0 = (split * nch) >> p.split_log2, kt1 = ((split + 1) * nch) >> p.split_log2;
                 // a slab per CTA; where windows are split, per unit in the order of all windows
                 const int slab = p.split_log2 ? (int)((((long long)(cur.b * g.Mh + cur.wr) * g.Mw + cur.wc) * hs) + hd) : p.slab0 + (int)blockIdx.x;
+                if (L::kGang && p.gang > 1) {
+                    for (int kt = (member + p.gang - seq % p.gang) % p.gang; ok && kt < nch; kt += p.gang)
+                        put(1 | (kt == 0 ? 2 : 0) | (kt == nch - 1 ? 4 : 0), head, eh, ew, kt, nch, (int)(blockIdx.x / p.gang) * p.ring + windows % p.ring, seq,
+                            windows / p.ring, p.rotate ? member * nch / min(p.gang, nch) : 0);
+                    seq += nch;
+                    windows += nch > 1;
+                    continue;
+                }
                 for (int kt = kt0; ok && kt < kt1; ++kt) {
                     put(1 | (kt == kt0 ? 2 : 0) | (kt == kt1 - 1 ? 4 : 0), head, eh, ew, kt, nch, slab);
                     if (L::kTables) {
@@ -744,23 +865,48 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 if (!ok) return;
                 use ^= 1u << s;
                 const bool fix = D == 32 && p.cols.skip && td.wc == p.cols.seam;
+                // ST: whether the seam cuts strip u
+                auto cut = [&](int u) { return !ST || u - unit_row(u, td.ns) * td.ns == p.cols.n1 >> 5; };
                 if (D == 32 && fix) {
                     // the seam column's slot n1 cannot be the start of a bulk copy of 64-byte rows (128-byte alignment)
                     for (int i = lane; i < 2 * kG * 4; i += 32) {
-                        const int h = i / (kG * 4), r = (i / 4) % kG, ch = i & 3, a = a0 + (two ? r : h * kG + r);
+                        const int h = i / (kG * 4), r = (i / 4) % kG, ch = i & 3, u = a0 + (two ? r : h * kG + r), a = ST ? unit_row(u, td.ns) : u;
+                        if (!cut(u)) continue;
                         const int tstride = (two && h) ? g.heads * D : g.ts;
                         uint4 val = make_uint4(0, 0, 0, 0);
                         if (a < td.eh && p.cols.n1 < td.ew)
                             val = __ldg(reinterpret_cast<const uint4*>((h ? x1 : x0) + ((size_t)td.b * g.H * g.W + win_token(g, td.wr, td.wc, a, p.cols.n1)) * tstride + td.head * D) + ch);
                         // rows of a K / V tile: both groups in one region; Q and dO: a region each
-                        const int rr = (two ? r : h * kG + r) * RW + p.cols.n1;
+                        const int rr = (two ? r : h * kG + r) * RW + (ST ? p.cols.n1 & 31 : p.cols.n1);
                         *reinterpret_cast<uint4*>(smem + s * L::kSlotB + (two ? h * kHalf * D * 2 : 0) + tile_off<32>(rr, ch)) = val;
                     }
                     fence_proxy_async();
                     __syncwarp();
                 }
                 const uint32_t base = smem0 + s * L::kSlotB;
-                if (win_group_whole<RW>(p.cols, g, td.wr, td.wc, td.eh, a0, two ? 1 : 2)) {
+                if (ST) {
+                    // 64 slots of a window row are one copy where the strips are even in number, a strip one where they are not
+                    const bool whole = (td.ns & 1) == 0 && td.wc != p.cols.seam && td.wc < p.cols.first_wrapped && td.wc != p.cols.last;
+                    if (lane == 0) {
+                        int n = 0;
+                        if (fix) n = two ? 2 * (cut(a0) + cut(a0 + 1)) : cut(a0) + cut(a0 + 1) + cut(a0 + 2) + cut(a0 + 3);
+                        mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB - n * kRowB);
+                    }
+                    __syncwarp();
+                    if (row < (whole ? 2 : 4)) {
+                        const int second = whole ? row : row >> 1, r = whole ? 0 : row & 1;           // of two: the tensor, else the 64-slot group
+                        const int u = a0 + r + (two ? 0 : 2 * second), a = unit_row(u, td.ns), st = u - a * td.ns;
+                        const uint32_t dst = base + r * 32 * kRowB + (two ? second * kHalf * D * 2 + part * kHalf * kRowB : part * kTile * kRowB + second * kHalf * kRowB);
+                        const WinMaps& m = second ? m1 : m0;
+                        if (whole) {
+                            int y = td.wr * g.w + a + g.sh;
+                            if (y >= g.H) y -= g.H;
+                            tma_load_4d(dst, &m.group, td.head * D + part * L::kPartCh, 32 * st, td.wc, a < td.eh ? td.b * g.H + y : g.B * g.H, bar(kBFull + s));
+                        } else {
+                            load_win_strip<kRowB>(m, p.cols, dst, g, td.b, td.wr, td.wc, td.eh, a, st, td.head * D + part * L::kPartCh, bar(kBFull + s));
+                        }
+                    }
+                } else if (win_group_whole<RW>(p.cols, g, td.wr, td.wc, td.eh, a0, two ? 1 : 2)) {
                     // the common case: one thread, one copy per group and channel part
                     if (elect_one()) {
                         mbar_arrive_expect_tx(bar(kBFull + s), L::kSlotB);
@@ -790,7 +936,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 const int sk = sq.pop(), sv = sq.pop();
                 fill(sk, mk, mk, p.k, p.k, td.kt * 2 * kG, false);
                 if (ok) fill(sv, mv, mv, p.v, p.v, td.kt * 2 * kG, false);
-                for (int hc = 0; ok && hc < 2 * td.nch; ++hc) fill(sq.take_half(), mq, mg, p.q, p.d_o, hc * kG, true);
+                for (int i = 0, hc = 2 * td.c0; ok && i < 2 * td.nch; ++i, hc = hc + 1 == 2 * td.nch ? 0 : hc + 1)
+                    fill(sq.take_half(), mq, mg, p.q, p.d_o, hc * kG, true);
                 sq.end_tile(sk, sv);
             }
         } else if (warp == kScoreWarp) {
@@ -868,7 +1015,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             bool ok = true;
             while (ok && next_tile()) {
                 const int sk = sq.pop(), sv = sq.pop();
-                const bool resident = td.nch <= L::kResident, fresh = !resident || (td.flags & 2), ready = !resident || (td.flags & 4);
+                const bool resident = !(L::kGang && p.gang > 1) && td.nch <= L::kResident, fresh = !resident || (td.flags & 2), ready = !resident || (td.flags & 4);
                 const uint32_t acc = tmem + L::kColAcc, kt_lo = lo_tile + sk * (L::kSlotB >> 4);
                 for (int hc = 0; ok && hc < 2 * td.nch; hc += 2, ++n) {
 #pragma unroll
@@ -950,21 +1097,23 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
 // zeroed bias-gradient table.
 constexpr int kStatHeads = 16;
 
-template <int D, int RW>
+template <int D, int RW, bool ST>
 __global__ void __launch_bounds__(256)
 swin_bwd_onepass_prep_kernel(const Geo g, const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ lse,
                              const float* __restrict__ bias, float4* __restrict__ rowstat, float* __restrict__ bias0, float* __restrict__ bias1,
-                             float* __restrict__ dbias_acc, int npad, int rmax, unsigned stat_blocks) {
+                             float* __restrict__ dbias_acc, int npad, int rmax, int rl, unsigned stat_blocks, unsigned* __restrict__ flags, int n_flags) {
     if (blockIdx.x >= stat_blocks) {
-        const int per_head = 2 * rmax * 2 * RW, total = per_head * g.heads, nw = 2 * g.w - 1;
+        for (int i = (blockIdx.x - stat_blocks) * 256 + threadIdx.x; i < n_flags; i += (gridDim.x - stat_blocks) * 256) flags[i] = 0;
+        const int per_head = 2 * rmax * rl, total = per_head * g.heads, nw = 2 * g.w - 1;
         for (int i = (blockIdx.x - stat_blocks) * 256 + threadIdx.x; i < total; i += (gridDim.x - stat_blocks) * 256) {
-            const int head = i / per_head, e = i - head * per_head;
-            const int da = e / (2 * RW) - rmax, db = e % (2 * RW) - RW;
+            // (the larger tables: neighbouring threads read neighbouring heads)
+            const int head = ST ? i % g.heads : i / per_head, e = ST ? i / g.heads : i - head * per_head, at = head * per_head + e;
+            const int da = e / rl - rmax, db = e % rl - rl / 2;
             const bool row = da > -g.w && da < g.w;
             const float* src = bias + ((size_t)(da + g.w - 1) * nw + db + g.w - 1) * g.heads + head;
-            bias0[i] = row && db > -g.w && db < g.w ? kLog2e * __ldg(src) : 0.f;
-            bias1[i] = row && db + 1 > -g.w && db + 1 < g.w ? kLog2e * __ldg(src + g.heads) : 0.f;
-            dbias_acc[i] = 0.f;
+            bias0[at] = row && db > -g.w && db < g.w ? kLog2e * __ldg(src) : 0.f;
+            bias1[at] = row && db + 1 > -g.w && db + 1 < g.w ? kLog2e * __ldg(src + g.heads) : 0.f;
+            dbias_acc[at] = 0.f;
         }
         return;
     }
@@ -981,7 +1130,7 @@ swin_bwd_onepass_prep_kernel(const Geo g, const __nv_bfloat16* __restrict__ o, c
     const int l = threadIdx.x % kLanes;
     for (int r0 = 0; r0 < 64 * nh; r0 += kRowsPass) {
         const int r = r0 + threadIdx.x / kLanes;
-        const int s = r / nh, h = r - s * nh, slot = chunk * 64 + s, a = slot / RW, bb = slot % RW;
+        const int s = r / nh, h = r - s * nh, slot = chunk * 64 + s, u = slot / RW, ns = strips_of(ew), a = ST ? unit_row(u, ns) : u, bb = slot % RW + (ST ? 32 * (u - a * ns) : 0);
         const bool in = r < 64 * nh, tok = in && a < eh && bb < ew;
         float dot = 0.f, nl2 = -INFINITY;
         if (tok) {
@@ -1012,13 +1161,13 @@ swin_bwd_onepass_prep_kernel(const Geo g, const __nv_bfloat16* __restrict__ o, c
 template <int D, int RW>
 __global__ void __launch_bounds__(256)
 swin_bwd_onepass_finish_kernel(const Geo g, const float* __restrict__ dbias_acc, float* __restrict__ dbias, const float4* __restrict__ slabs,
-                               __nv_bfloat16* __restrict__ dq, int npad, int rmax, int split_log2, unsigned bias_blocks) {
+                               __nv_bfloat16* __restrict__ dq, int npad, int rmax, int rl, int split_log2, unsigned bias_blocks) {
     wait_for_prerequisites();
     if (blockIdx.x < bias_blocks) {
         const int nw = 2 * g.w - 1, i = blockIdx.x * 256 + threadIdx.x;
         if (i >= nw * nw * g.heads) return;
         const int head = i % g.heads, r = i / g.heads, da = r / nw - (g.w - 1), db = r % nw - (g.w - 1);
-        dbias[i] = dbias_acc[((size_t)head * 2 * rmax + da + rmax) * 2 * RW + db + RW];
+        dbias[i] = dbias_acc[((size_t)head * 2 * rmax + da + rmax) * rl + db + rl / 2];
         return;
     }
     const int per_item = npad * D / 4, blocks = (per_item + 255) / 256;
@@ -1072,32 +1221,64 @@ bool bwd_onepass_supported(const Geo& g) {
     // Register tiles / this kernel, us, on 240 x 360, 2 x 121 x 250 and 96 x 180 tokens: head dim 64, side 9 676/752 659/719 166/166, 10 572/626 560/601
     // 146/140; 11 517/537 480/496 140/126 (level), 12 1032/451; head dim 128, side 9 889/800 1215/1130 289/263; head dim 32, side 17 948/967
     // 1798/1711 389/406 (level), 18 1126/816 2278/1496 468/384.
+    if (win_strips(g)) return g.w <= kMaxWinW && (long long)g.B * g.H * g.W < 0x7fffffffLL && (long long)g.B * g.Mh * g.Mw * g.heads * 128 < 0x7fffffffLL;
     return ((g.d == 64 && g.w > 10) || g.d == 128 || (g.d == 32 && g.w > 16)) && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 8 < 0x7fffffffLL;
+}
+
+// Gangs (see Params).  The CTAs of a gang read the same Q and dO and add to the same slab a few turns after one another, so these pass
+// between L2 and memory once for kGangMin CTAs or more.  The time of a run in key tiles: the gang's windows times their tiles over its
+// CTAs, plus what its last CTA is behind its first (none where they rotate).  Where a window has more tiles than the gang has CTAs, the first CTA's second
+// tile waits for the last CTA's first: a tile's 2 x tiles half chunks have to hold the gang's lags, and half as much for the unevenness
+// (256 x 640 tokens, 8 x 128, side 64, gangs of 4, 8, 16 and 37: 11.6, 12.9, 14.8 and 19.3 ms; side 128, 7, 9, 18, 37: 43.0, 43.0, 44.2, 47.4).
+static void plan_gangs(OnePassPlan& p, const Geo& g, long long items, int tiles) {
+    p.gangs = kPlanSms;
+    p.gang = p.ring = 1;
+    p.rotate = p.flags = 0;
+    if (!p.strips) return;
+    const double lag = kGangLag / (2.0 * tiles);
+    double best = 0;
+    for (int n = 1; n <= items && n <= kPlanSms / kGangMin; ++n) {
+        const int s = kPlanSms / n;
+        const double slow = s < tiles && 1.5 * lag * s > 1 ? 1.5 * lag * s : 1;
+        const double t = n == items ? (double)((tiles + s - 1) / s) : slow * ((items + n - 1) / n) * tiles / s + lag * s;
+        if (n == 1 || t <= best) { best = t; p.gangs = n; p.gang = s; }
+    }
+    const long long most = (items + p.gangs - 1) / p.gangs * tiles;
+    if (p.gang > most) p.gang = (int)most;
+    p.rotate = items <= p.gangs;
+    if (p.rotate) p.gang = (tiles + (tiles + p.gang - 1) / p.gang - 1) / ((tiles + p.gang - 1) / p.gang);      // as many tiles for each
+    // from a window's first tile to its last one's end, over the time between two windows
+    const int turn = p.gang < tiles ? p.gang : tiles;
+    p.ring = p.rotate ? 1 : (int)std::ceil(((tiles + p.gang - 1) / p.gang + lag * turn) * p.gang / tiles) + 1;
+    p.flags = p.gangs * p.ring * ((p.npad / (g.d == 128 ? 64 : 128)) + 1) * 4;      // (more than the turns need)
 }
 
 OnePassPlan bwd_onepass_plan(const Geo& g) {
     OnePassPlan p;
     p.rw = win_row_slots(g);
     const int kr = kTile / p.rw, rows = g.w < g.H ? g.w : g.H;
-    const int tiles = (rows * p.rw + kTile - 1) / kTile;
+    p.strips = win_strips(g) ? strips_of(g.w) : 0;
+    const int tiles = (rows * (p.strips ? strips_of(g.w < g.W ? g.w : g.W) : 1) * p.rw + kTile - 1) / kTile;
     p.npad = tiles * kTile;
-    p.rmax = (g.w + kr - 1) / kr * kr;
+    p.rl = p.strips ? 64 * p.strips : 2 * p.rw;
+    p.rmax = p.strips ? g.w + 4 : (g.w + kr - 1) / kr * kr;      // (the last key tile's rows reach up to 3 past the window's)
     // Units per window: as many as keep the SMs busy.  The time of a launch is the number of unit rounds x key tiles per
     // unit; splitting costs a sum over slabs, so it has to save an eighth of that time.
     const long long items = (long long)g.B * g.Mh * g.Mw * g.heads;
     p.split_log2 = 0;
     double best = 0;
-    for (int ls = 0; ls <= 3 && (1 << ls) <= tiles; ++ls) {
+    for (int ls = 0; ls <= (p.strips ? 0 : 3) && (1 << ls) <= tiles; ++ls) {
         const double t = (double)(((items << ls) + kPlanSms - 1) / kPlanSms) * ((tiles + (1 << ls) - 1) >> ls);
         if (ls == 0 || t < 0.875 * best) { best = t; p.split_log2 = ls; }
     }
     p.units = items << p.split_log2;
+    plan_gangs(p, g, items, tiles);
     const int most = (g.d == 128 ? 1 : 2) * kMaxCtas;    // CTAs of the launches that may overlap (see launch_onepass)
     const size_t ctas = p.units < most ? (size_t)p.units : (size_t)most;
-    const size_t slabs = p.split_log2 ? (size_t)p.units : ctas;
+    const size_t slabs = p.split_log2 ? (size_t)p.units : p.strips && p.gang > 1 ? (size_t)p.gangs * p.ring : ctas;
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
-    const size_t table = up(sizeof(float) * (size_t)g.heads * 2 * p.rmax * 2 * p.rw);
+    const size_t table = up(sizeof(float) * (size_t)g.heads * 2 * p.rmax * p.rl);
     p.off_bias0 = up(sizeof(float4) * (size_t)g.B * g.Mh * g.Mw * g.heads * (p.npad / 2));
     p.off_bias1 = p.off_bias0 + table;
     p.off_acc = p.off_bias1 + table;
@@ -1105,6 +1286,9 @@ OnePassPlan bwd_onepass_plan(const Geo& g) {
     // a window whose dQ is complete after one key tile, or stays in TMEM, needs no slab
     const bool slab = p.split_log2 > 0 || g.d != 32 ? tiles > 1 : tiles > 2;
     p.bytes = p.off_slabs + (slab ? up(sizeof(float) * slabs * p.npad * g.d) : 0);
+    p.off_flags = p.bytes;
+    if (p.gang > 1 && p.strips) p.bytes += up(sizeof(unsigned) * p.flags);
+    else if (p.gang > 1) p.off_flags = p.off_slabs + sizeof(float) * (size_t)p.gangs * p.ring * p.npad * g.d;      // behind the gangs' slabs (plan_gangs: they fit)
     return p;
 }
 
@@ -1125,6 +1309,7 @@ bool make_win_cols(WinCols* c, const Geo& g) {
 bool make_win_maps(WinMaps* m, const WinCols& c, const Geo& g, const void* base, int ts) {
     std::memset(m, 0, sizeof *m);
     const int rw = win_row_slots(g), box_ch = g.d >= 64 ? 64 : 32;
+    const bool st = win_strips(g);
     auto enc = [&](CUtensorMap* out, int col0, int nb, int ncols, int box_b, int box_rows) {
         const char* b = reinterpret_cast<const char*>(base) + (size_t)col0 * ts * 2;
         return encode_win_map(out, g, b, ts, nb, ncols, box_ch, box_b, box_rows);
@@ -1132,14 +1317,16 @@ bool make_win_maps(WinMaps* m, const WinCols& c, const Geo& g, const void* base,
     int n_main = c.seam >= 0 ? c.seam : c.first_wrapped;
     if (c.last >= 0 && c.last < n_main) n_main = c.last;
     bool ok = true;
-    if (n_main > 0) ok = enc(&m->group, g.sw, g.w, n_main, rw, 64 / rw) && enc(&m->row, g.sw, g.w, n_main, rw, 1);
+    if (n_main > 0) ok = enc(&m->group, g.sw, g.w, n_main, st ? 64 : rw, st ? 1 : 64 / rw) && enc(&m->row, g.sw, g.w, n_main, rw, 1);
     const int w0 = c.n1 > 0 ? g.w - c.n1 : 0;           // token column of the first column behind the seam
     const int n_wrapped = (c.last >= 0 ? c.last : g.Mw) - c.first_wrapped;
     if (ok && n_wrapped > 0) ok = enc(&m->wrapped, w0, g.w, n_wrapped, rw, 1);
     if (ok && c.seam >= 0) {
         const int ew = g.W - c.seam * g.w < g.w ? g.W - c.seam * g.w : g.w;
-        ok = enc(&m->seam_a, g.W - c.n1, c.n1, 1, c.n1, 1);
-        if (ok && c.n1 + c.skip < rw && ew > c.n1) ok = enc(&m->seam_b, 0, ew - c.n1, 1, rw - c.n1 - c.skip, 1);
+        const int cut = st ? c.n1 % 32 : c.n1;          // slots in front of the seam of the row or strip that it cuts
+        if (cut > 0) ok = enc(&m->seam_a, g.W - c.n1, c.n1, 1, cut, 1);
+        if (ok && cut > 0 && cut + c.skip < rw && ew > c.n1) ok = enc(&m->seam_b, 0, ew - c.n1, 1, rw - cut - c.skip, 1);
+        if (ok && st) ok = enc(&m->seam_fa, g.W - c.n1, c.n1, 1, rw, 1) && enc(&m->seam_fb, 0, ew - c.n1, 1, rw, 1);
     }
     if (ok && c.last >= 0) {
         const int col = c.last >= c.first_wrapped ? w0 + (c.last - c.first_wrapped) * g.w : c.last * g.w + g.sw;
@@ -1150,11 +1337,11 @@ bool make_win_maps(WinMaps* m, const WinCols& c, const Geo& g, const void* base,
 #endif  // !TERRA_ELEM_F16
 
 namespace {
-template <int D, int RW>
+template <int D, int RW, bool ST = false>
 cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, const void* k, const void* v, const float* bias, const void* o,
                            const float* lse, const void* d_o, void* dq, void* dk, void* dv, float* dbias, void* workspace, int sm_count,
                            cudaStream_t stream) {
-    using L = Lay<D, RW>;
+    using L = Lay<D, RW, ST>;
     unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
     Params p;
     p.g = g;
@@ -1165,6 +1352,13 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     p.split_log2 = pl.split_log2;
     p.npad = pl.npad;
     p.rmax = pl.rmax;
+    p.rl = pl.rl;
+    p.gang = pl.gang;
+    p.ring = pl.ring;
+    p.rotate = pl.rotate;
+    p.turn_log2 = (D == 128 ? 2 : 1) - pl.rotate;      // 256 queries (rotate: 128)
+    p.events = pl.npad / (D == 128 ? 64 : 128);
+    p.flags = reinterpret_cast<unsigned*>(ws + pl.off_flags);
     p.rowstat = reinterpret_cast<const float4*>(ws);
     p.bias0 = reinterpret_cast<const float*>(ws + pl.off_bias0);
     p.bias1 = reinterpret_cast<const float*>(ws + pl.off_bias1);
@@ -1172,11 +1366,11 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     p.slabs = reinterpret_cast<float4*>(ws + pl.off_slabs);
     p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v; p.d_o = (const __nv_bfloat16*)d_o;
     const unsigned stat = (unsigned)((long long)g.B * g.Mh * g.Mw * (pl.npad / 64) * ((g.heads + kStatHeads - 1) / kStatHeads));
-    const long long table = (long long)g.heads * 2 * pl.rmax * 2 * RW;
+    const long long table = (long long)g.heads * 2 * pl.rmax * pl.rl;
     const unsigned tblocks = (unsigned)(table / 1024 + 1 < 592 ? table / 1024 + 1 : 592);
     prof_begin("swin_bwd_onepass_prep_kernel", stream);
-    swin_bwd_onepass_prep_kernel<D, RW><<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
-        const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, stat);
+    swin_bwd_onepass_prep_kernel<D, RW, ST><<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
+        const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, pl.rl, stat, p.flags, pl.flags);
     count_launch(stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1189,8 +1383,15 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         cudaError_t err = prepare_kernel((const void*)kernel, L::kSmemBytes);
         if (err != cudaSuccess) return err;
         prof_begin(overlap ? "swin_bwd_onepass_kernel<masked>" : "swin_bwd_onepass_kernel", stream);
-        const unsigned grid = (unsigned)(p.units < ctas ? p.units : ctas);
-        if (overlap) {
+        unsigned grid = (unsigned)(p.units < ctas ? p.units : ctas);
+        p.gangs = (int)grid;
+        if (p.gang > 1) {
+            // a device with fewer SMs than planned for: fewer gangs, or a smaller one
+            if (p.gang > ctas) p.gang = ctas;
+            p.gangs = pl.gangs * p.gang <= ctas ? pl.gangs : ctas / p.gang;
+            grid = (unsigned)(p.gangs * p.gang);
+            err = launch_together(kernel, grid, kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
+        } else if (overlap) {
             // needs nothing of the launch before it: its CTAs take the SMs as that one's leave them
             err = launch_dependent(kernel, grid, kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
         } else {
@@ -1202,10 +1403,10 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         return err;
     };
     const long long all = (long long)g.Mh * g.Mw;
-    if constexpr (D == 128) {
+    if constexpr (D == 128 || ST) {
         p.row1 = g.Mh;
         p.col1 = g.Mw;
-        e = launch(swin_bwd_onepass_kernel<D, RW, 2>, true, all, 0, false);
+        e = launch(swin_bwd_onepass_kernel<D, RW, 2, ST>, true, all, 0, false);
     } else {
         // the windows in front of the first row and column that need the mask
         p.row1 = g.w == RW ? g.H / g.w : 0;
@@ -1216,8 +1417,8 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         const long long inner = (long long)p.row1 * p.col1;
         const long long units0 = inner * g.B * g.heads << pl.split_log2;
         const int slabs0 = (int)(units0 < ctas ? units0 : ctas);
-        if (inner > 0) e = launch(swin_bwd_onepass_kernel<D, RW, 0>, true, inner, 0, false);
-        if (e == cudaSuccess && inner < all) e = launch(swin_bwd_onepass_kernel<D, RW, 1>, false, all - inner, slabs0, inner > 0);
+        if (inner > 0) e = launch(swin_bwd_onepass_kernel<D, RW, 0, ST>, true, inner, 0, false);
+        if (e == cudaSuccess && inner < all) e = launch(swin_bwd_onepass_kernel<D, RW, 1, ST>, false, all - inner, slabs0, inner > 0);
     }
     if (e != cudaSuccess) return e;
     const int nw = 2 * g.w - 1;
@@ -1225,7 +1426,7 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     const long long sum_blocks = pl.split_log2 ? (pl.units >> pl.split_log2) * ((pl.npad * D / 4 + 255) / 256) : 0;
     prof_begin("swin_bwd_onepass_finish_kernel", stream);
     e = launch_dependent(swin_bwd_onepass_finish_kernel<D, RW>, (unsigned)(bias_blocks + sum_blocks), 256, 0, stream, g, p.dbias_acc, dbias, p.slabs,
-                         (__nv_bfloat16*)dq, pl.npad, pl.rmax, pl.split_log2, bias_blocks);
+                         (__nv_bfloat16*)dq, pl.npad, pl.rmax, pl.rl, pl.split_log2, bias_blocks);
     count_launch(stream);
     return e;
 }
@@ -1234,7 +1435,8 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
 cudaError_t launch_bwd_onepass(const Geo& g, const void* q, const void* k, const void* v, const float* bias, const void* o, const float* lse,
                                const void* d_o, void* dq, void* dk, void* dv, float* dbias, void* workspace, int sm_count, cudaStream_t stream) {
     const OnePassPlan pl = bwd_onepass_plan(g);
-    auto fn = pl.rw == 16 ? (g.d == 64 ? launch_onepass<64, 16> : launch_onepass<128, 16>)
+    auto fn = pl.strips ? (g.d == 32 ? launch_onepass<32, 32, true> : g.d == 64 ? launch_onepass<64, 32, true> : launch_onepass<128, 32, true>)
+            : pl.rw == 16 ? (g.d == 64 ? launch_onepass<64, 16> : launch_onepass<128, 16>)
                           : (g.d == 32 ? launch_onepass<32, 32> : g.d == 64 ? launch_onepass<64, 32> : launch_onepass<128, 32>);
     return fn(g, pl, q, k, v, bias, o, lse, d_o, dq, dk, dv, dbias, workspace, sm_count, stream);
 }

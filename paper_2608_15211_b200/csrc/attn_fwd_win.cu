@@ -71,15 +71,16 @@ struct Tab {
 enum { kBFull = 0, kBEmpty = 16, kBS = 32, kBP = 38, kBFree = 44, kBO = 50, kBOFree = 52, kBStat = 54, kBTab = 56, kBBias = 58,
        kBOne = 59, kBDesc = 61, kBDescFree = kBDesc + kDescs, kBFullV = kBDescFree + kDescs, kBCount = kBFullV + 16 };
 
-template <int D, int RW>
+template <int D, int RW, bool ST>
 struct Lay {
     static constexpr int kParts = D == 128 ? 2 : 1, kRowB = D >= 64 ? 128 : 64, kPartCh = kRowB / 2;
     static constexpr int kSlotB = kTile * D * 2;                                    // a Q, K or V tile
     static constexpr int kSlots = D == 128 ? (RW == 16 ? 6 : 5) : D == 64 ? 10 : 14;
     static constexpr int kBufs = D == 128 ? 4 : 6, kColO = 64 * kBufs;
     static constexpr int kOffE = kSlots * kSlotB;                                   // E operands, 64 bytes a slot: E_q, then E_k
-    static constexpr int kOffTab = kOffE + 256 * 64;
-    static constexpr int kOffStat = kOffTab + Tab<RW>::rows(RW) * Tab<RW>::kRowF * 4;          // per row of both tiles: m, row sum
+    static constexpr int kEUnits = ST ? 12 : 256 / RW;                              // rows of slots (ST: strips) of the E operands
+    static constexpr int kOffTab = kOffE + kEUnits * RW * 64;
+    static constexpr int kOffStat = kOffTab + (ST ? 0 : Tab<RW>::rows(RW) * Tab<RW>::kRowF * 4);          // per row of both tiles: m, row sum
     static constexpr int kOffDesc = kOffStat + 2 * kTile * 8;
     static constexpr int kOffBars = kOffDesc + kDescs * 64;
     static constexpr int kSmemBytes = kOffBars + 8 * kBCount + 16;
@@ -89,7 +90,8 @@ struct Params {
     Geo g;
     WinCols cols;
     const __nv_bfloat16 *q, *k, *v;
-    const float* tables;         // [head][Tab::rows][Tab::kRowF]
+    const float* tables;         // [head][Tab::rows][Tab::kRowF]; ST: [head][2 w - 1][2][64 strips], read from global memory
+    int strips;                  // ST: strips of a full window row
     int pairs;                   // query tile pairs of a full window
     int head_slow;               // units in head-major order, a run per CTA; else the head is the fastest digit, strided
     long long units;
@@ -100,7 +102,11 @@ struct Unit {
     int eh, ew, tile0, ntq;      // first query tile, 1 or 2 of them
     int ku, nch, ha, hb;         // 32-slot key units, chunks; window rows >= ha / columns >= hb carry the other mask label
     int flags;                   // 1: a unit (0: the end), 2: another head than before, 4: the scores need the mask step
+    int ns;                      // ST: strips of a window row
 };
+
+// ST: rows of strips per row label among the mask operands, so that four strips in a row from any strip on lie in them
+__device__ __forceinline__ int e_rows(int ns) { return ns == 1 ? 4 : ns == 4 ? 1 : 2; }
 
 // FIFO of shared-memory slots: two held for a unit (Q tiles), the others cycle (K, V chunks)
 template <int N>
@@ -132,13 +138,15 @@ __device__ __forceinline__ float max3_nan(float a, float b, float c) {
 // 8 k + 2 t + e) -> S scale + bias in place, and the rows' maxima (NaN if a score is).  Pairs on one diagonal share their bias: 7 or 9 reads
 // for 32 scores.  (A thread per row read each score's own entry: the shared-memory pipe then bound the kernel, 1300 to 2500
 // of 4100 to 6800 cycles per 128 x 128 scores and tile.)  `bias`: shared address of the entry of rows g, keys 2 t.
-template <int RW, int KC>
-__device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, uint32_t bias, float scale, float (&mx)[4]) {
+template <int RW>
+__device__ __forceinline__ void load_bias(float2 (&bv)[RW == 32 ? 7 : 9], uint32_t bias) {
     constexpr int kRowB = Tab<RW>::kRowF * 4;
-    float2 bv[9];
 #pragma unroll
     for (int i = 0; i < (RW == 32 ? 7 : 9); ++i)
         bv[i] = lds_f2(bias + (RW == 32 ? 32 * (i - 3) : (i / 3 - 1) * kRowB + 32 * (i % 3 - 1)));
+}
+template <int RW, int KC>
+__device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, const float2 (&bv)[RW == 32 ? 7 : 9], float scale, float (&mx)[4]) {
 #pragma unroll
     for (int m = 0; m < 4; ++m)
 #pragma unroll
@@ -156,20 +164,23 @@ __device__ __forceinline__ void add_bias(uint32_t (&x)[2][32], int u, uint32_t b
 // The scores of a half chunk (key rows `ak` on, `cols` of its columns; 32 query rows a warp, window row `aq` on) whose tokens differ in
 // mask label become -inf, in tensor memory.  Not inlined, and the half chunk starts over from the loop's head: with this code in the
 // middle of the softmax's every unit paid for it (121 x 250 x 2 tokens, 8 x 64, side 32: 285 -> 306 us; so 290).
-template <int RW>
-__device__ __noinline__ void drop_forbidden(uint32_t t_s, int cols, int ak, int aq, int ha, int hb, int gl, int ql) {
+// ST: `ak` and `aq` are units, `ns` to a window row.
+template <int RW, bool ST>
+__device__ __noinline__ void drop_forbidden(uint32_t t_s, int cols, int ak, int aq, int ha, int hb, int gl, int ql, int ns) {
 #pragma unroll 1
     for (int c = 0; c < cols; c += 16)
 #pragma unroll 1
         for (int h = 0; h < 2; ++h) {
             // 16 keys x 16 queries, each of one window row
-            const bool rows = (ak + c / RW >= ha) == (aq + (RW == 32 ? 0 : h) >= ha);
+            const int uk = ak + c / RW, uq = aq + (RW == 32 ? 0 : h), rk = ST ? unit_row(uk, ns) : uk, rq = ST ? unit_row(uq, ns) : uq;
+            const bool rows = (rk >= ha) == (rq >= ha);
+            const int ck = ST ? 32 * (uk - rk * ns) : 0, cq = ST ? 32 * (uq - rq * ns) : 0;
             uint32_t r[8];
             tmem_ld_frag16(t_s + ((16u * h) << 16) + c, r);
             tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const int bk = (RW == 32 ? c & 16 : 0) + 8 * (i >> 2) + 2 * ql + (i & 1), bq = (RW == 32 ? 16 * h : 0) + 8 * ((i >> 1) & 1) + gl;
+                const int bk = ck + (RW == 32 ? c & 16 : 0) + 8 * (i >> 2) + 2 * ql + (i & 1), bq = cq + (RW == 32 ? 16 * h : 0) + 8 * ((i >> 1) & 1) + gl;
                 r[i] = rows && (bk >= hb) == (bq >= hb) ? r[i] : 0xff800000u;
             }
             tmem_st_frag16(t_s + ((16u * h) << 16) + c, r);
@@ -179,11 +190,11 @@ __device__ __noinline__ void drop_forbidden(uint32_t t_s, int cols, int ak, int 
 
 // KC: of every 32 key slots the first 8 KC are worked on (window sides 17 .. 24 in rows of 32 slots leave the last 8 without a
 // token: 3; otherwise 4).  240 x 360 tokens, 6 x 64, side 22: 357 -> 302 us.
-template <int D, int RW, int KC>
+template <int D, int RW, int KC, bool ST>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
                     const __grid_constant__ WinMaps mq, const __grid_constant__ WinMaps mk, const __grid_constant__ WinMaps mv) {
-    using L = Lay<D, RW>;
+    using L = Lay<D, RW, ST>;
     constexpr int kParts = L::kParts, kRowB = L::kRowB, kG = 64 / RW, NB = L::kBufs, kTileRows = kTile / RW;
     extern __shared__ __align__(1024) unsigned char smem[];
     const uint32_t smem0 = smem_u32(smem), bar0 = smem0 + L::kOffBars;
@@ -240,6 +251,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
         td.eh = d1.x; td.ew = d1.y; td.tile0 = d1.z; td.ntq = d1.w;
         td.ku = d2.x; td.nch = d2.y; td.ha = d2.z; td.hb = d2.w;
         td.flags = src[3].x;
+        if (ST) td.ns = src[3].y;
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kBDescFree + i));
         ++desc_n;
@@ -258,10 +270,30 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
         unsigned n = 0, units = 0, mine = 0, heads = 0, ones = 0;   // half chunks of the CTA; units, those with this tile; tables; 1-tile units
         bool ok = true;
         while (ok && next_unit()) {
-            if (td.flags & 2) ok = mbar_wait_all(bar(kBBias), heads++ & 1, cta_abort);
+            if (!ST && (td.flags & 2)) ok = mbar_wait_all(bar(kBBias), heads++ & 1, cta_abort);
             if (ok && t < td.ntq) {
-                const int aq = min((td.tile0 + t) * kTileRows + wq * (32 / RW), td.eh - 1);
+                const int aq = min((td.tile0 + t) * kTileRows + wq * (32 / RW), (ST ? td.ku : td.eh) - 1);
                 uint32_t bias = tab0 + 4u * (g.w - 1 - aq + Tab<RW>::kFront) * Tab<RW>::kRowF;
+                // ST: the entries of the next half chunk's two key units, from the head's table in L2, are in registers before they are needed
+                float2 bv[ST ? 2 : 1][RW == 32 ? 7 : 9];
+                const float* bp = nullptr;
+                int sk = 0;
+                auto next_bias = [&](int left) {             // key units left
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        if (u < left) {
+#pragma unroll
+                            for (int i = 0; i < 7; ++i) bv[ST ? u : 0][i] = __ldg(reinterpret_cast<const float2*>(bp + 8 * (i - 3)));
+                        }
+                        bp += 32;
+                        if (++sk == td.ns) { sk = 0; bp += 128 * p.strips - 32 * td.ns; }
+                    }
+                };
+                if (ST) {
+                    const int rq = unit_row(aq, td.ns), j0 = 32 * p.strips - 1 + 2 * ql - gl;
+                    bp = p.tables + ((size_t)td.head * (2 * g.w - 1) + g.w - 1 - rq) * (128 * p.strips) + (j0 & 1) * (64 * p.strips) + (j0 & ~1) - 32 * (aq - rq * td.ns);
+                    next_bias(td.ku);
+                }
                 float m[4] = {kLowest, kLowest, kLowest, kLowest};     // (finite: a half chunk may hold no key that the row sees)
                 float2 sum[4] = {};
                 int fixed = -1;                          // half chunk whose scores have gone by their labels
@@ -276,9 +308,11 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     tmem_ld_frag64(t_s + (16u << 16), x[1]);
                     tmem_ld_wait();
                     float top[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                    add_bias<RW, KC>(x, 0, bias, scale, top);
+                    if (!ST) load_bias<RW>(bv[0], bias);
+                    add_bias<RW, KC>(x, 0, bv[0], scale, top);
                     if (2 * j + 1 < td.ku) {
-                        add_bias<RW, KC>(x, 1, bias + 4u * (32 / RW) * Tab<RW>::kRowF, scale, top);
+                        if (!ST) load_bias<RW>(bv[0], bias + 4u * (32 / RW) * Tab<RW>::kRowF);
+                        add_bias<RW, KC>(x, 1, bv[ST ? 1 : 0], scale, top);
                     } else {
                         // 32 slots that do not exist
 #pragma unroll
@@ -287,7 +321,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     if (!__all_sync(0xffffffffu, top[0] - m[0] <= 8.f && top[1] - m[1] <= 8.f && top[2] - m[2] <= 8.f && top[3] - m[3] <= 8.f)) {
                         if (fixed != j && ((td.ha > 0 && td.ha < td.eh) || (td.hb > 0 && td.hb < td.ew)) &&
                             __any_sync(0xffffffffu, top[0] != top[0] || top[1] != top[1] || top[2] != top[2] || top[3] != top[3])) {
-                            drop_forbidden<RW>(t_s, 32 * min(2, td.ku - 2 * j), 2 * j * (32 / RW), (td.tile0 + t) * kTileRows + wq * (32 / RW), td.ha, td.hb, gl, ql);
+                            drop_forbidden<RW, ST>(t_s, 32 * min(2, td.ku - 2 * j), 2 * j * (32 / RW), (td.tile0 + t) * kTileRows + wq * (32 / RW), td.ha, td.hb, gl, ql, ST ? td.ns : 1);
                             fixed = j--;
                             continue;
                         }
@@ -322,6 +356,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                                 }
                         }
                     }
+                    if (ST && 2 * (j + 1) < td.ku) next_bias(td.ku - 2 * (j + 1));
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         uint32_t pk[16];
@@ -388,7 +423,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
                 if (t >= td.ntq) break;
-                const int slot = (td.tile0 + t) * kTile + row, a = slot / RW, bb = slot % RW;
+                const int slot = (td.tile0 + t) * kTile + row, ua = slot / RW, a = ST ? unit_row(ua, td.ns) : ua, bb = slot % RW + (ST ? 32 * (ua - a * td.ns) : 0);
                 ok = mbar_wait_all(bar(kBStat + t), done[t] & 1, cta_abort) && mbar_wait_all(bar(kBO + t), done[t] & 1, cta_abort);
                 if (!ok) break;
                 ++done[t];
@@ -434,13 +469,13 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 if (!ok) return;
                 if (lane == 0) {
                     const int ha = (!g.ph && g.sh > 0) ? g.H - g.sh - wr * g.w : (1 << 20), hb = (!g.pw && g.sw > 0) ? g.W - g.sw - wc * g.w : (1 << 20);
-                    const int nqt = (eh * RW + kTile - 1) / kTile, ku = RW == 32 ? eh : (eh + 1) / 2;
-                    if (ew < RW || (ha > 0 && ha < eh) || (hb > 0 && hb < ew) || (RW == 16 && (eh & 1))) flags |= 4;
+                    const int ns = ST ? strips_of(ew) : 1, nqt = (eh * ns * RW + kTile - 1) / kTile, ku = RW == 32 ? eh * ns : (eh + 1) / 2;
+                    if (ew < ns * RW || (ha > 0 && ha < eh) || (hb > 0 && hb < ew) || (RW == 16 && (eh & 1))) flags |= 4;
                     int4* dst = reinterpret_cast<int4*>(smem + L::kOffDesc + (i % kDescs) * 64);
                     dst[0] = make_int4(head, b, wr, wc);
                     dst[1] = make_int4(eh, ew, tile0, min(2, nqt - tile0));
                     dst[2] = make_int4(ku, (ku + 3) / 4, ha, hb);
-                    dst[3] = make_int4(flags, 0, 0, 0);
+                    dst[3] = make_int4(flags, ns, 0, 0);
                     mbar_arrive(bar(kBDesc + i % kDescs));
                 }
                 __syncwarp();
@@ -455,7 +490,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 else { rest = (unsigned)u / g.heads; head = (unsigned)u - rest * g.heads; }
                 const unsigned win = rest / p.pairs, pair = rest - win * p.pairs, r2 = win / g.Mw, wc = win - r2 * g.Mw, b = r2 / g.Mh, wr = r2 - b * g.Mh;
                 const int eh = min(g.w, g.H - (int)wr * g.w), ew = min(g.w, g.W - (int)wc * g.w);
-                if ((int)pair * 2 * kTileRows >= eh) continue;            // a truncated window has fewer query tiles
+                if ((int)pair * 2 * kTileRows >= eh * (ST ? strips_of(ew) : 1)) continue;            // a truncated window has fewer query tiles
                 put(1 | ((int)head != last_head ? 2 : 0), head, b, wr, wc, eh, ew, pair * 2);
                 last_head = head;
             }
@@ -469,6 +504,12 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             int e_key = -1, q0 = -1, q1 = -1;        // what the mask operands are made for; Q slots of the last unit
             bool ok = true;
             const int part = lane % kParts, row = lane / kParts;      // lane -> channel part, window row of a tile
+            // ST: of the tile's four strips from `a0` on those that the seam cuts
+            auto cut_units = [&](int a0) {
+                int n = 0;
+                for (int u = a0; u < a0 + 4; ++u) n += u - unit_row(u, td.ns) * td.ns == p.cols.n1 >> 5;
+                return n;
+            };
             auto fill = [&](int s, int full, const WinMaps& m, const __nv_bfloat16* src, int a0) {
                 ok = ok && mbar_wait_all(bar(kBEmpty + s), ((use >> s) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
@@ -477,17 +518,34 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 if (D == 32 && fix) {
                     // the seam column's slot n1 cannot be the start of a bulk copy of 64-byte rows (128-byte alignment)
                     for (int i = lane; i < 2 * kG * 4; i += 32) {
-                        const int r = i >> 2, ch = i & 3, a = a0 + r;
+                        const int r = i >> 2, ch = i & 3, a = ST ? unit_row(a0 + r, td.ns) : a0 + r, cut = ST ? p.cols.n1 & 31 : p.cols.n1;
+                        if (ST && a0 + r - a * td.ns != p.cols.n1 >> 5) continue;
                         uint4 val = make_uint4(0, 0, 0, 0);
                         if (a < td.eh && p.cols.n1 < td.ew)
                             val = __ldg(reinterpret_cast<const uint4*>(src + ((size_t)td.b * g.H * g.W + win_token(g, td.wr, td.wc, a, p.cols.n1)) * g.ts + td.head * D) + ch);
-                        *reinterpret_cast<uint4*>(smem + s * L::kSlotB + tile_off<32>(r * RW + p.cols.n1, ch)) = val;
+                        *reinterpret_cast<uint4*>(smem + s * L::kSlotB + tile_off<32>(r * RW + cut, ch)) = val;
                     }
                     fence_proxy_async();
                     __syncwarp();
                 }
                 const uint32_t base = smem0 + s * L::kSlotB;
-                if (win_group_whole<RW>(p.cols, g, td.wr, td.wc, td.eh, a0, 2)) {
+                if (ST) {
+                    // 64 slots of a window row are one copy where the strips are even in number, a strip one where they are not
+                    const bool two = (td.ns & 1) == 0 && td.wc != p.cols.seam && td.wc < p.cols.first_wrapped && td.wc != p.cols.last;
+                    if (lane == 0) mbar_arrive_expect_tx(bar(full + s), L::kSlotB - (fix ? cut_units(a0) * kRowB : 0));
+                    __syncwarp();
+                    if (row < (two ? 2 : 4)) {
+                        const int u = a0 + (two ? 2 : 1) * row, a = unit_row(u, td.ns), st = u - a * td.ns;
+                        const uint32_t dst = base + part * kTile * kRowB + (u - a0) * 32 * kRowB;
+                        if (two) {
+                            int y = td.wr * g.w + a + g.sh;
+                            if (y >= g.H) y -= g.H;
+                            tma_load_4d(dst, &m.group, td.head * D + part * L::kPartCh, 32 * st, td.wc, a < td.eh ? td.b * g.H + y : g.B * g.H, bar(full + s));
+                        } else {
+                            load_win_strip<kRowB>(m, p.cols, dst, g, td.b, td.wr, td.wc, td.eh, a, st, td.head * D + part * L::kPartCh, bar(full + s));
+                        }
+                    }
+                } else if (win_group_whole<RW>(p.cols, g, td.wr, td.wc, td.eh, a0, 2)) {
                     if (elect_one()) {
                         mbar_arrive_expect_tx(bar(full + s), L::kSlotB);
                         int y0 = td.wr * g.w + a0 + g.sh;
@@ -511,7 +569,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             while (ok && next_unit()) {
                 // at most two units ahead of the softmax: the barriers of even and odd units are waited for once per use
                 if (units >= 2) ok = mbar_wait_all(bar(kBTab + (units & 1)), ((units - 2) >> 1) & 1, cta_abort);
-                if (ok && (td.flags & 2)) {
+                if (!ST && ok && (td.flags & 2)) {
                     if (units >= 1) ok = mbar_wait_all(bar(kBTab + ((units - 1) & 1)), ((units - 1) >> 1) & 1, cta_abort);
                     if (ok && elect_one()) {
                         const uint32_t bytes = Tab<RW>::rows(g.w) * Tab<RW>::kRowF * 4;
@@ -522,18 +580,19 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 }
                 if (ok && (td.flags & 4)) {
                     // 32 slots to a row: rows 0-3 carry the first row label, 4-7 the second; a tile starts where its rows change
+                    // ST: e_rows(ns) rows of strips carry the first row label, as many the second
                     const int ha = min(max(td.ha, 0), td.eh), hb = min(max(td.hb, 0), td.ew);
-                    const int key = RW == 32 ? td.ew | hb << 6 : td.ew | hb << 6 | td.eh << 12 | ha << 18;
+                    const int key = ST ? td.ew | hb << 8 : RW == 32 ? td.ew | hb << 6 : td.ew | hb << 6 | td.eh << 12 | ha << 18;
                     if (key != e_key) {
                         e_key = key;
                         // the last unit's scores are done when its Q slots are free
                         if (q0 >= 0) ok = ok && mbar_wait_all(bar(kBEmpty + q0), ((use >> q0) & 1) ^ 1u, cta_abort);
                         if (q1 >= 0) ok = ok && mbar_wait_all(bar(kBEmpty + q1), ((use >> q1) & 1) ^ 1u, cta_abort);
                         if (ok) {
-                            for (int s = lane; s < 256; s += 32) {
-                                const int a = s / RW, b = s % RW;
+                            for (int s = lane; s < L::kEUnits * RW; s += 32) {
+                                const int u = s / RW, a = ST ? unit_row(u, td.ns) : u, b = s % RW + (ST ? 32 * (u - a * td.ns) : 0);
                                 const bool valid = b < td.ew && (RW == 32 || a < td.eh);
-                                const int label = 2 * (RW == 32 ? a >= 4 : a >= ha) + (b >= hb);
+                                const int label = 2 * (RW == 32 ? a >= (ST ? e_rows(td.ns) : 4) : a >= ha) + (b >= hb);
                                 uint32_t eq[2] = {0, 0}, ek[2] = {kMaskK | kMaskK << 16, kMaskK | kMaskK << 16};
                                 if (valid) {
                                     const uint32_t half = (label & 1) ? 0xffff0000u : 0xffffu;
@@ -582,6 +641,10 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             };
             // where the rows from window row a0 on start among the mask operands (16-byte units)
             auto mask_rows = [&](int a0) {
+                if (ST) {
+                    const int a = unit_row(a0, td.ns);
+                    return (uint32_t)(min(max(e_rows(td.ns) - (td.ha - a), 0), e_rows(td.ns)) * td.ns + a0 - a * td.ns) * (RW * 64 / 16);
+                }
                 return RW == 16 ? (uint32_t)a0 * (RW * 64 / 16) : (uint32_t)min(max(4 - (td.ha - a0), 0), 4) * (RW * 64 / 16);
             };
             while (ok && next_unit()) {
@@ -699,6 +762,18 @@ __global__ void swin_fwd_win_prep_kernel(const Geo g, const float* __restrict__ 
     }
 }
 
+// ST: by row difference, two copies (see Params).  Neighbouring threads read neighbouring heads and write a table each.
+__global__ void swin_fwd_win_prep_strips_kernel(const Geo g, const float* __restrict__ bias, float* __restrict__ tables, int strips) {
+    let_dependents_start();
+    const int nw = 2 * g.w - 1, rl = 64 * strips, per_head = nw * 2 * rl;
+    const long long total = (long long)per_head * g.heads;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+        const int e = (int)(i / g.heads), head = (int)(i - (long long)e * g.heads);
+        const int row = e / (2 * rl), f = e - row * 2 * rl, c = f / rl, db = f - c * rl + c - (32 * strips - 1);      // key minus query
+        tables[(size_t)head * per_head + e] = db > -g.w && db < g.w ? __ldg(bias + ((size_t)(nw - 1 - row) * nw + (g.w - 1 - db)) * g.heads + head) * kLog2e : 0.f;
+    }
+}
+
 }  // namespace
 
 cudaError_t read_fwd_win_status(int* timed_out) {
@@ -718,21 +793,24 @@ bool fwd_win_supported(const Geo& g) {
     //   above 24 work on all 32 slots of a row: 25 353/430 705/837 154/201, 26 392/402 736/830 164/169; 27 436/386 810/816 175/181, 28 463/342;
     //   head dim 64, side 9 226/318 212/349 52/80, 11 166/238 156/246 39/56; 12 267/183 248/214 60/46; 17 338/468 318/426 72/95; 18 416/358 379/368 95/84;
     //   head dim 128, this kernel at every side: 9 283/261 392/369 91/95, 10 242/238 338/328 74/82, 11 207/171 287/269 68/64, 17 400/346 558/486 123/118.
+    if (win_strips(g))
+        return g.w <= kMaxWinW && (long long)g.B * g.H * g.W < 0x7fffffffLL && (long long)g.B * g.Mh * g.Mw * g.heads * 64 < 0x7fffffffLL;
     const bool sparse = g.d == 32 ? g.w <= 22 || g.w == 25 || g.w == 26 : g.d == 64 && (g.w <= 11 || g.w == 17);
     return (g.d == 64 || g.d == 128 || (g.d == 32 && g.w > 16)) && !sparse && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 4 < 0x7fffffffLL;
 }
 
 size_t fwd_win_workspace_bytes(const Geo& g) {
+    if (win_strips(g)) return sizeof(float) * (size_t)g.heads * (2 * g.w - 1) * 128 * strips_of(g.w);
     return sizeof(float) * (size_t)g.heads * (win_row_slots(g) == 16 ? Tab<16>::rows(g.w) * Tab<16>::kRowF : Tab<32>::rows(g.w) * Tab<32>::kRowF);
 }
 #endif
 
 namespace {
-template <int D, int RW, int KC = 4>
+template <int D, int RW, int KC = 4, bool ST = false>
 cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
                        int sm_count, cudaStream_t stream) {
-    using L = Lay<D, RW>;
+    using L = Lay<D, RW, ST>;
     Params p;
     p.g = g;
     WinMaps mq, mk, mv;
@@ -740,7 +818,8 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
         return cudaErrorNotSupported;
     p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v;
     p.tables = (const float*)workspace;
-    const int tiles = ((g.w < g.H ? g.w : g.H) * RW + kTile - 1) / kTile;
+    p.strips = ST ? strips_of(g.w) : 1;
+    const int tiles = ((g.w < g.H ? g.w : g.H) * (ST ? strips_of(g.w < g.W ? g.w : g.W) : 1) * RW + kTile - 1) / kTile;
     p.pairs = (tiles + 1) / 2;
     p.units = (long long)g.B * g.Mh * g.Mw * g.heads * p.pairs;
     // A CTA keeps to one head where that leaves no more than 1 SM in 20 idle: neighbouring CTAs then read the heads of the same
@@ -748,16 +827,18 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
     const int bound = sm_count / g.heads * g.heads;
     p.head_slow = bound * 20 < sm_count * 19 && p.units > bound;
     const long long ctas = p.head_slow ? sm_count : bound > 0 ? bound : sm_count;
-    const int total = g.heads * Tab<RW>::rows(g.w) * Tab<RW>::kRowF;
+    const long long total = ST ? (long long)g.heads * (2 * g.w - 1) * 128 * p.strips : g.heads * Tab<RW>::rows(g.w) * Tab<RW>::kRowF;
+    const unsigned pblocks = (unsigned)(total / 512 + 1 < 592 ? total / 512 + 1 : 592);
     prof_begin("swin_fwd_win_prep_kernel", stream);
-    swin_fwd_win_prep_kernel<RW><<<total / 512 + 1 < 592 ? total / 512 + 1 : 592, 256, 0, stream>>>(g, bias, (float*)workspace);
+    if (ST) swin_fwd_win_prep_strips_kernel<<<pblocks, 256, 0, stream>>>(g, bias, (float*)workspace, p.strips);
+    else swin_fwd_win_prep_kernel<RW><<<pblocks, 256, 0, stream>>>(g, bias, (float*)workspace);
     count_launch(stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW, KC>, L::kSmemBytes);
+    e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW, KC, ST>, L::kSmemBytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_fwd_win_kernel", stream);
-    e = launch_dependent(swin_fwd_win_kernel<D, RW, KC>, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
+    e = launch_dependent(swin_fwd_win_kernel<D, RW, KC, ST>, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
     count_launch(stream);
     return e;
 }
@@ -765,6 +846,10 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
 
 cudaError_t launch_fwd_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
                            int sm_count, cudaStream_t stream) {
+    if (win_strips(g)) {
+        auto fn = g.d == 32 ? launch_win<32, 32, 4, true> : g.d == 64 ? launch_win<64, 32, 4, true> : launch_win<128, 32, 4, true>;
+        return fn(g, q, k, v, bias, o, lse, workspace, sm_count, stream);
+    }
     const bool wide = win_row_slots(g) == 32, narrow = g.w <= 24;
     switch (g.d) {
         case 32: return (narrow ? launch_win<32, 32, 3> : launch_win<32, 32>)(g, q, k, v, bias, o, lse, workspace, sm_count, stream);

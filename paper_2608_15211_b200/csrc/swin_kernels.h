@@ -31,6 +31,22 @@ cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Launches `kernel` only when all its CTAs can be on the device together: they wait for one another.
+template <typename... P, typename... A>
+cudaError_t launch_together(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A&&... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Before a kernel's launch: allows it `smem` bytes of dynamic shared memory on the current device and, where `occupancy` is
 // given, says how many CTAs of `threads` threads fit an SM.  Each thread remembers its last few kernels: the two runtime
 // calls cost more host time than the launch of a small kernel.
@@ -119,12 +135,17 @@ cudaError_t launch_bwd_kv64_qside(const Geo& g, const void* q, const void* k, co
 struct OnePassPlan {
     int rw;                  // slots per window row
     int npad, rmax;          // slots of a window rounded up to 128; window rows rounded up to whole key tiles
+    int strips, rl;          // strips of a full window row (0: sides up to 32); floats of a bias-table row
     int split_log2;          // a window's key tiles are shared by 1 << split_log2 units
+    int gangs, gang, ring, rotate;   // or by `gang` CTAs, that add to one slab in turn: `gangs` of them, `ring` slabs each (gang 1: none)
     long long units;
-    size_t off_bias0, off_bias1, off_acc, off_slabs, bytes;      // workspace
+    size_t off_bias0, off_bias1, off_acc, off_slabs, off_flags, bytes;      // workspace
+    int flags;               // ints at off_flags
 };
 constexpr int kPlanSms = 148;          // SM count the plan is made for
 constexpr int kMaxCtas = 160;          // CTAs whose dQ slabs fit the workspace
+constexpr int kGangMin = 4;            // CTAs of a gang at least
+constexpr double kGangLag = 5.5;       // half chunks from a CTA's turn to the next one's
 bool bwd_onepass_supported(const Geo& g);
 OnePassPlan bwd_onepass_plan(const Geo& g);
 cudaError_t launch_bwd_onepass(const Geo& g, const void* q, const void* k, const void* v, const float* bias, const void* o, const float* lse,

@@ -2,6 +2,8 @@
 // backward and their host sides.
 //
 // A window's slots are laid out RW to a window row (RW = 16 for window sides 9 .. 16, 32 for 17 .. 32): slot = RW a + b.
+// Sides 33 .. 128 (ST): a window row is `ns` strips of 32 slots (as many as the window's width needs), row after row: unit = ns a +
+// (strip), slot = 32 unit + b.  A unit is then what a window row is at sides 17 .. 32, to the copies and to the elementwise warps.
 // Slots with b at or beyond the window's width, or a at or beyond its height, hold no token; the copies fill them with
 // zeros.  A tensor is described as [heads * d channels][w columns of a window][window columns][token rows], based at
 // the first token of the shifted frame, so that a box of RW columns reads past the w columns of its window only into
@@ -17,11 +19,13 @@
 namespace terra {
 
 struct WinMaps {
-    CUtensorMap group;       // columns in front of the seam, 64 / RW window rows per copy
-    CUtensorMap row;         // the same, one window row per copy
+    CUtensorMap group;       // columns in front of the seam, 64 / RW window rows per copy (ST: 64 slots of one)
+    CUtensorMap row;         // the same, one window row per copy (ST: a strip of one; so below)
     CUtensorMap wrapped;     // columns behind the seam, one window row
     CUtensorMap seam_a;      // the column cut by the seam: its tokens in front of the seam ...
-    CUtensorMap seam_b;      // ... and behind it, up to slot RW
+    CUtensorMap seam_b;      // ... and behind it, up to slot RW (ST: both of the strip that it cuts)
+    CUtensorMap seam_fa;     // ST: the whole strips in front of the seam ...
+    CUtensorMap seam_fb;     // ... and behind it
     CUtensorMap last;        // a truncated last column (when the seam does not cut it)
 };
 
@@ -34,8 +38,16 @@ struct WinCols {
                              // (a bulk copy must start on a 128-byte boundary), seam_b starts one token later
 };
 
-constexpr int kMaxOnePassW = 32;
+constexpr int kMaxOnePassW = 32, kMaxWinW = 128;
 inline int win_row_slots(const Geo& g) { return g.w <= 16 ? 16 : 32; }
+inline bool win_strips(const Geo& g) { return g.w > 32; }
+
+// ST: strips of a window that is `ew` wide, and the row of a unit (u / ns for u < 2^14)
+__host__ __device__ __forceinline__ int strips_of(int ew) { return (ew + 31) >> 5; }
+__device__ __forceinline__ int unit_row(int u, int ns) {
+    const unsigned inv = ns == 1 ? 65536u : ns == 2 ? 32768u : ns == 3 ? 21846u : 16384u;
+    return (int)(((unsigned)u * inv) >> 16);
+}
 
 // host (attn_fwd_tc.cu, beside the driver's encoder)
 bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_stride, int nb, int ncols, int box_ch, int box_b, int box_rows);
@@ -69,6 +81,32 @@ __device__ __forceinline__ void load_win_row(const WinMaps& m, const WinCols& c,
         tc::tma_load_4d(dst, &m.wrapped, ch, 0, wc - c.first_wrapped, y, bar);
     } else {
         tc::tma_load_4d(dst, &m.row, ch, 0, wc, y, bar);
+    }
+}
+
+// device, ST: strip `s` of window row `a` (32 slots; see load_win_row)
+template <int ROWB>
+__device__ __forceinline__ void load_win_strip(const WinMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
+                                               int a, int s, int ch, uint32_t bar) {
+    int u = wr * g.w + a + g.sh;
+    if (u >= g.H) u -= g.H;
+    const int y = a < eh ? b * g.H + u : g.B * g.H, c0 = 32 * s;
+    if (wc == c.seam) {
+        const int n = c.n1 - c0;                          // slots of the strip in front of the seam
+        if (n >= 32) {
+            tc::tma_load_4d(dst, &m.seam_fa, ch, c0, 0, y, bar);
+        } else if (n <= 0) {
+            tc::tma_load_4d(dst, &m.seam_fb, ch, -n, 0, y, bar);
+        } else {
+            tc::tma_load_4d(dst, &m.seam_a, ch, c0, 0, y, bar);
+            if (n + c.skip < 32) tc::tma_load_4d(dst + (n + c.skip) * ROWB, &m.seam_b, ch, c.skip, 0, y, bar);
+        }
+    } else if (wc == c.last) {
+        tc::tma_load_4d(dst, &m.last, ch, c0, 0, y, bar);
+    } else if (wc >= c.first_wrapped) {
+        tc::tma_load_4d(dst, &m.wrapped, ch, c0, wc - c.first_wrapped, y, bar);
+    } else {
+        tc::tma_load_4d(dst, &m.row, ch, c0, wc, y, bar);
     }
 }
 
