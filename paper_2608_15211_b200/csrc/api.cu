@@ -150,7 +150,6 @@ static bool small_windows(const Geo& g) { return g.w <= 8; }
 
 // (every kernel exists for bf16 and for fp16 activations: `f16` only selects the build of the kernel)
 static bool use_fwd_tc(const Geo& g) { return fwd_tc_supported(g) && !small_windows(g); }
-static bool use_fwd_tc64(const Geo& g) { return fwd_tc64_supported(g) && !force_register_path(); }
 
 static bool use_fwd_win(const Geo& g) { return fwd_win_supported(g) && !force_register_path() && !small_windows(g); }
 
@@ -158,7 +157,6 @@ static size_t fwd_bytes(const Geo& g) {
     if (force_register_path()) return 0;
     if (use_fwd_win(g)) return align_up(fwd_win_workspace_bytes(g), 256);
     if (use_fwd_tc(g)) return align_up(fwd_tc_workspace_bytes(g), 256);
-    if (use_fwd_tc64(g)) return align_up(fwd_tc64_workspace_bytes(g), 256);
     return 0;
 }
 
@@ -173,16 +171,12 @@ static bool force_split_small() {
 
 static bool use_bwd_tc(const Geo& g) { return bwd_tc_supported(g) && !force_register_path() && !small_windows(g); }
 
-static bool use_bwd_kv64(const Geo& g) { return bwd_kv64_supported(g) && !force_register_path(); }
-
 static bool use_bwd_onepass(const Geo& g) { return bwd_onepass_supported(g) && !force_register_path() && !small_windows(g); }
 
 static size_t delta_bytes(const Geo& g) {
     if (use_bwd_onepass(g)) return align_up(bwd_onepass_plan(g).bytes, 256);
     if (use_bwd_tc(g)) return align_up(bwd_tc_workspace_bytes(g), 256);
-    const size_t delta = align_up(sizeof(float) * (size_t)g.B * g.H * g.W * g.heads, 256);
-    // windows of side 64 and 128: the prepared bias tables twice, the second copy reflected for the query side
-    return use_bwd_kv64(g) ? delta + 2 * align_up(fwd_tc64_workspace_bytes(g), 256) : delta;
+    return align_up(sizeof(float) * (size_t)g.B * g.H * g.W * g.heads, 256);                   // delta
 }
 
 // Descriptor check + geometry, and the SM count of the current device, for entry points that live in
@@ -244,9 +238,6 @@ static int fwd_call(const Geo& g, const void* q, const void* k, const void* v,
     cudaStream_t st = (cudaStream_t)stream;
     if (use_fwd_win(g))
         e = g.f16 ? launch_fwd_win_f16(g, q, k, v, bias_table, o, lse, workspace, sms, st) : launch_fwd_win(g, q, k, v, bias_table, o, lse, workspace, sms, st);
-    else if (need > 0 && use_fwd_tc64(g) && !use_fwd_tc(g))
-        e = g.f16 ? launch_fwd_tc64_f16(g, q, k, v, bias_table, o, lse, workspace, sms, st)
-                  : launch_fwd_tc64(g, q, k, v, bias_table, o, lse, workspace, sms, st);
     else if (need > 0)
         e = g.f16 ? launch_fwd_tc_f16(g, q, k, v, bias_table, o, lse, workspace, sms, st)
                   : launch_fwd_tc(g, q, k, v, bias_table, o, lse, workspace, sms, st);
@@ -312,24 +303,6 @@ static int bwd_call(const Geo& g, const void* q, const void* k, const void* v,
     float* delta = reinterpret_cast<float*>(workspace);
     cudaError_t e = g.f16 ? launch_bwd_delta_f16(g, o, d_o, delta, st) : launch_bwd_delta(g, o, d_o, delta, st);
     if (e != cudaSuccess) return cuda_fail(e, "terra_swin_attn_bwd (delta)");
-    if (use_bwd_kv64(g)) {
-        // key side (dK, dV) on tcgen05
-        float* prep = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(workspace) +
-                                               align_up(sizeof(float) * (size_t)g.B * g.H * g.W * g.heads, 256));
-        e = launch_bias_prep64(g, bias_table, prep, st);
-        if (e == cudaSuccess)
-            e = g.f16 ? launch_bwd_kv64_f16(g, q, k, v, d_o, prep, lse, delta, dk, dv, sms, st)
-                      : launch_bwd_kv64(g, q, k, v, d_o, prep, lse, delta, dk, dv, sms, st);
-        if (e == cudaSuccess) {
-            // query side (dQ, dBias): the key-side kernel with the tensors' roles exchanged
-            float* prep_r = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(prep) + align_up(fwd_tc64_workspace_bytes(g), 256));
-            e = launch_bias_prep64(g, bias_table, prep_r, st, true);
-            if (e == cudaSuccess)
-                e = g.f16 ? launch_bwd_kv64_qside_f16(g, q, k, v, d_o, prep_r, lse, delta, dq, dbias, sms, st)
-                          : launch_bwd_kv64_qside(g, q, k, v, d_o, prep_r, lse, delta, dq, dbias, sms, st);
-        }
-        return e == cudaSuccess ? TERRA_OK : cuda_fail(e, "terra_swin_attn_bwd");
-    }
     e = g.f16 ? launch_bwd_mma_f16(g, q, k, v, bias_table, lse, delta, d_o, dq, dk, dv, dbias, sms, st)
               : launch_bwd_mma(g, q, k, v, bias_table, lse, delta, d_o, dq, dk, dv, dbias, sms, st);
     return e == cudaSuccess ? TERRA_OK : cuda_fail(e, "terra_swin_attn_bwd");
@@ -376,25 +349,17 @@ int terra_swin_check(void* stream) {
     int timed_out_bwd = 0;
     e = read_bwd_tc_status(&timed_out_bwd);
     if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
-    int timed_out_64 = 0;
-    e = read_fwd_tc64_status(&timed_out_64);
-    if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
-    int timed_out_kv = 0;
-    e = read_bwd_kv64_status(&timed_out_kv);
-    if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
     // the fp16 builds of the same kernels keep status words of their own
-    int t16[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    int t16[6] = {0, 0, 0, 0, 0, 0};
     e = read_tc_status_f16(&t16[0], (cudaStream_t)stream);
     if (e == cudaSuccess) e = read_bwd_tc_status_f16(&t16[1]);
-    if (e == cudaSuccess) e = read_fwd_tc64_status_f16(&t16[2]);
-    if (e == cudaSuccess) e = read_bwd_kv64_status_f16(&t16[3]);
-    if (e == cudaSuccess) e = read_bwd_onepass_status_f16(&t16[4]);
-    if (e == cudaSuccess) e = read_bwd_onepass_status(&t16[5]);
-    if (e == cudaSuccess) e = read_fwd_win_status_f16(&t16[6]);
-    if (e == cudaSuccess) e = read_fwd_win_status(&t16[7]);
+    if (e == cudaSuccess) e = read_bwd_onepass_status_f16(&t16[2]);
+    if (e == cudaSuccess) e = read_bwd_onepass_status(&t16[3]);
+    if (e == cudaSuccess) e = read_fwd_win_status_f16(&t16[4]);
+    if (e == cudaSuccess) e = read_fwd_win_status(&t16[5]);
     if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
-    const bool any16 = t16[0] || t16[1] || t16[2] || t16[3] || t16[4] || t16[5] || t16[6] || t16[7];
-    return (timed_out || timed_out_bwd || timed_out_64 || timed_out_kv || any16) ? TERRA_ERR_DEVICE_TIMEOUT : TERRA_OK;
+    const bool any16 = t16[0] || t16[1] || t16[2] || t16[3] || t16[4] || t16[5];
+    return (timed_out || timed_out_bwd || any16) ? TERRA_ERR_DEVICE_TIMEOUT : TERRA_OK;
 }
 
 int terra_profile_enable(int on) {

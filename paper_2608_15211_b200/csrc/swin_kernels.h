@@ -72,15 +72,6 @@ cudaError_t launch_bwd_tc_f16(const Geo& g, const void* q, const void* k, const 
                               const void* o, const float* lse, const void* d_o, void* dq, void* dk, void* dv, float* dbias,
                               void* workspace, int sm_count, cudaStream_t stream);
 cudaError_t read_bwd_tc_status_f16(int* timed_out);
-cudaError_t launch_fwd_tc64_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
-                                void* o, float* lse, void* workspace, int sm_count, cudaStream_t stream);
-cudaError_t read_fwd_tc64_status_f16(int* timed_out);
-cudaError_t launch_bwd_kv64_f16(const Geo& g, const void* q, const void* k, const void* v, const void* d_o, const float* prep,
-                                const float* lse, const float* delta, void* dk, void* dv, int sm_count, cudaStream_t stream);
-cudaError_t read_bwd_kv64_status_f16(int* timed_out);
-cudaError_t launch_bwd_kv64_qside_f16(const Geo& g, const void* q, const void* k, const void* v, const void* d_o,
-                                      const float* prep_reflected, const float* lse, const float* delta, void* dq, float* dbias,
-                                      int sm_count, cudaStream_t stream);
 cudaError_t launch_bwd_delta_f16(const Geo& g, const void* o, const void* d_o, float* delta, cudaStream_t stream);
 cudaError_t launch_bwd_mma_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
                                const float* lse, const float* delta, const void* d_o,
@@ -110,27 +101,6 @@ cudaError_t launch_fwd_win_f16(const Geo& g, const void* q, const void* k, const
                                int sm_count, cudaStream_t stream);
 cudaError_t read_fwd_win_status(int* timed_out);
 cudaError_t read_fwd_win_status_f16(int* timed_out);
-// tcgen05 forward path for head dims 64 and 128 and complete windows of side 64 and 128 (keys streamed once in chunks)
-bool fwd_tc64_supported(const Geo& g);
-size_t fwd_tc64_workspace_bytes(const Geo& g);
-cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const void* v, const float* bias,
-                            void* o, float* lse, void* workspace, int sm_count, cudaStream_t stream);
-cudaError_t read_fwd_tc64_status(int* timed_out);     // after the stream has been synchronised
-// (window sides 64 and 128: whole table rows; `reflect`: the table reflected through its centre)
-cudaError_t launch_bias_prep64(const Geo& g, const float* bias, float* prep, cudaStream_t stream, bool reflect = false);
-
-// tcgen05 key side (dK, dV) of the backward pass for head dims 64 and 128 and complete windows of side 64 and 128; `prep` =
-// the tables of launch_bias_prep64, `delta` as for the register-tile kernels
-bool bwd_kv64_supported(const Geo& g);
-cudaError_t launch_bwd_kv64(const Geo& g, const void* q, const void* k, const void* v, const void* d_o, const float* prep,
-                            const float* lse, const float* delta, void* dk, void* dv, int sm_count, cudaStream_t stream);
-cudaError_t read_bwd_kv64_status(int* timed_out);
-// the query side (dQ, dBias) of complete windows of side 64 and 128 with the same kernel; `prep_reflected` = the
-// tables of launch_bias_prep64 with reflect = true; dbias is overwritten
-cudaError_t launch_bwd_kv64_qside(const Geo& g, const void* q, const void* k, const void* v, const void* d_o,
-                                  const float* prep_reflected, const float* lse, const float* delta, void* dq, float* dbias,
-                                  int sm_count, cudaStream_t stream);
-
 // One-pass tcgen05 backward for window sides 9 .. 32 at head dim 128, 11 .. 32 at 64 and 17 .. 32 at 32, any grid.
 struct OnePassPlan {
     int rw;                  // slots per window row
