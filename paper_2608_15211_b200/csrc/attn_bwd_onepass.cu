@@ -76,7 +76,7 @@ struct Lay {
     // per half chunk (ring of kTabs): 64 queries' statistics, then the bias rows its pieces meet, twice (the second copy shifted
     // by one entry and 16 banks away, so that lanes with even and odd g read different banks); head dim 128 has no room
     // and reads them from global memory
-    static constexpr bool kTables = D != 128 && !ST, kGang = ST || (D == 128 && RW == 32);
+    static constexpr bool kTables = D != 128 && !ST, kGang = ST;
     static constexpr int kTabs = 4, kBiasRows = kTile / RW + kHalf / RW - 1, kCopyB = kBiasRows * 2 * RW * 4;
     static constexpr int kOffCopy0 = 512, kOffCopy1 = 512 + (kCopyB + 127) / 128 * 128 + 64;
     static constexpr int kTabB = kTables ? (kOffCopy1 + kCopyB + 127) / 128 * 128 : 0;
@@ -266,9 +266,10 @@ __device__ __forceinline__ void step_math(const uint32_t (&rs)[2][8], const uint
 // through shared memory: a line of five groups of 8 floats per g, group = s in order, so that lane l's entry of line g lies at
 // l + 1 + g: one address and immediate offsets, and (lines 40 floats apart) no bank conflicts in either direction.  RW = 32:
 // s = -3 .. 0 behind a group of zeros give diagonals l - 31, s = 0 .. 3 in front of one give l + 1; RW = 16: a round per row
-// difference, s = -1 .. 1 between two groups of zeros, diagonals l - 15.  `acc`, `acc1`: where the pieces' diagonal -RW would go.
+// difference, s = -1 .. 1 between two groups of zeros, diagonals l - 15.  `acc`: where piece 0's diagonal -RW would go,
+// `acc_row`: floats from there to piece 1's.
 template <int RW>
-__device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][Piece<RW>::kSums], int lane, float* acc, float* acc1) {
+__device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][Piece<RW>::kSums], int lane, float* acc, int acc_row) {
     constexpr int kRounds = RW == 32 ? 2 : 3;
     const uint32_t w = scr + (lane >> 2) * kScrLine + (lane & 3) * 8, rd = scr + (lane + 1) * 4;
 #pragma unroll
@@ -299,7 +300,7 @@ __device__ __forceinline__ void flush_sums(uint32_t scr, const float2 (&sum)[2][
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
             const float x = ((v[j][0] + v[j][1]) + (v[j][2] + v[j][3])) + ((v[j][4] + v[j][5]) + (v[j][6] + v[j][7]));
-            float* dst = (j ? acc1 : acc) + (RW == 32 ? (r ? 33 : 1) : (r - 1) * 2 * RW + 1) + lane;
+            float* dst = acc + j * acc_row + (RW == 32 ? (r ? 33 : 1) : (r - 1) * 2 * RW + 1) + lane;
             if ((RW == 32 && r == 0) || lane < 31) red_f1(dst, x);
         }
     }
@@ -411,8 +412,12 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         td.head = d0.x; td.b = d0.y; td.wr = d0.z; td.wc = d0.w;
         td.eh = d1.x; td.ew = d1.y; td.kt = d1.z; td.nch = d1.w;
         td.ha = d2.x; td.hb = d2.y; td.flags = d2.z; td.slab = d2.w;
-        const int4 d3 = src[3];
-        td.ns = ST ? d3.x : 1; td.seq = d3.y; td.use = d3.z; td.c0 = L::kGang ? d3.w : 0;
+        if (ST) {
+            const int4 d3 = src[3];
+            td.ns = d3.x; td.seq = d3.y; td.use = d3.z; td.c0 = d3.w;
+        } else {
+            td.ns = 1;
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kBDescFree + i));
         ++desc_n;
@@ -447,8 +452,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         // the next tile: what its half chunks have in common
         auto enter_tile = [&]() {
             if (!next_tile()) return false;
-            hc = 2 * td.c0 + b;
-            left = td.nch;
+            hc = ST ? 2 * td.c0 + b : b;
+            if (ST) left = td.nch;
             nh = 2 * td.nch;
             ha = td.ha;
             a_k0 = td.kt * (kTile / RW) + (RW == 32 ? wq : 2 * wq);
@@ -475,17 +480,17 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             sp = (uint32_t)(((td.b * g.Mh + td.wr) * g.Mw + td.wc) * g.heads + td.head);
             return true;
         };
-        // floats from there to piece j of half chunk hc
+        auto bias_ptr = [&]() { return tbl + row0 + hc * kG * (2 * RW); };
+        // ST: floats from row0 to piece j of half chunk hc
         auto piece_at = [&](int j) {
-            if (!ST) return (hc * kG + j * (32 / RW)) * (2 * RW);
             const int u = 2 * hc + j, a = unit_row(u, td.ns);
             return a * rl + 32 * (u - a * td.ns);
         };
         auto stat_ptr = [&]() { return p.rowstat + (size_t)sp * (p.npad / 2) + (hc * 32 + t); };
         bool live = enter_tile();
         auto load_tables = [&]() {
-            pc[0].load(tbl + row0 + piece_at(0), stat_ptr());
-            pc[1].load(tbl + row0 + piece_at(1), stat_ptr() + 16);
+            pc[0].load(ST ? tbl + row0 + piece_at(0) : bias_ptr(), stat_ptr());
+            pc[1].load(ST ? tbl + row0 + piece_at(1) : bias_ptr() + (32 / RW) * 2 * RW, stat_ptr() + 16);
         };
         if (live && !L::kTables) load_tables();
         while (live) {
@@ -535,16 +540,20 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 if (L::kTables) mbar_arrive(bar(kBTabFree + ti));
             }
             // the next half chunk's tables are on their way while the rest is done
-            float* acc = p.dbias_acc + row0 + piece_at(0) + (ST ? rl / 2 - 32 : 0);
-            float* acc1 = p.dbias_acc + row0 + piece_at(1) + (ST ? rl / 2 - 32 : 0);
+            float* acc = p.dbias_acc + row0 + (ST ? piece_at(0) + rl / 2 - 32 : hc * kG * (2 * RW));
+            const int acc_row = ST ? piece_at(1) - piece_at(0) : (32 / RW) * 2 * RW;
             hc += 2;
-            if (L::kGang && hc >= nh) hc -= nh;
-            if (--left == 0) live = enter_tile();
+            if (ST) {
+                if (hc >= nh) hc -= nh;
+                if (--left == 0) live = enter_tile();
+            } else if (hc >= nh) {
+                live = enter_tile();
+            }
             if (live && !L::kTables) load_tables();
             // The bias gradient, while the products are computed.  Head dim 128 has no shared memory to spare: the sums go
             // through the warp's own rows of the dS^T tile once the dQ product has read them.
             if (D == 128 && !mbar_wait_all(bar(kBDq + b), n & 1, cta_abort)) break;
-            flush_sums<RW>(scr0, sum, lane, acc, acc1);
+            flush_sums<RW>(scr0, sum, lane, acc, acc_row);
             if (D == 128) __syncwarp();
             ++n;
         }
@@ -642,8 +651,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             float4* slab = p.slabs + (size_t)td.slab * ((size_t)p.npad * D / 4) + row;
             if (D == 128) {
                 // dQ^T: lanes = channels, columns = the half chunk's queries
-                for (int i = 0, hc = 2 * td.c0; i < 2 * td.nch; ++i, ++n, hc = hc + 1 == 2 * td.nch ? 0 : hc + 1) {
-                    const int b = hc & 1;
+                for (int i = 0; i < 2 * td.nch; ++i, ++n) {
+                    const int b = i & 1, hc = ST && i + 2 * td.c0 >= 2 * td.nch ? i + 2 * td.c0 - 2 * td.nch : ST ? i + 2 * td.c0 : i;
                     if (shared) {
                         if (p.rotate) {
                             at = place(hc >> 1);
@@ -702,7 +711,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             } else {
                 const bool resident = !ganged && td.nch <= L::kResident;
                 if (!resident || last) {
-                    for (int i = 0, ch = td.c0; i < td.nch; ++i, ch = ch + 1 == td.nch ? 0 : ch + 1) {
+                    for (int i = 0; i < td.nch; ++i) {
+                        const int ch = ST && i + td.c0 >= td.nch ? i + td.c0 - td.nch : ST ? i + td.c0 : i;
                         const int r = D == 64 ? 0 : resident ? ch : (int)(n++ & 1);
                         if (shared) {
                             if (p.rotate) {
@@ -782,7 +792,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     dst[0] = make_int4(head, cur.b, cur.wr, cur.wc);
                     dst[1] = make_int4(eh, ew, kt, nch);
                     dst[2] = make_int4((!g.ph && g.sh > 0) ? g.H - g.sh - cur.wr * g.w : (1 << 20), (!g.pw && g.sw > 0) ? g.W - g.sw - cur.wc * g.w : (1 << 20), flags, slab);
-                    dst[3] = make_int4(strips_of(ew), seq, use, c0);
+                    if (ST) dst[3] = make_int4(strips_of(ew), seq, use, c0);
                     mbar_arrive(bar(kBDesc + i % kDescs));
                 }
                 __syncwarp();
@@ -810,9 +820,9 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     __syncwarp();
                 }
             };
-            const int member = (int)blockIdx.x % p.gang;
+            const int member = L::kGang ? (int)blockIdx.x % p.gang : 0;
             int seq = 0, windows = 0;                // tiles and windows of several tiles of the gang so far
-            for (long long u = blockIdx.x / p.gang; ok && u < p.units; u += p.gangs) {
+            for (long long u = L::kGang ? blockIdx.x / p.gang : blockIdx.x; ok && u < p.units; u += L::kGang ? p.gangs : gridDim.x) {
                 // unit -> head and share, window, sample (the windows of the launch: see Params)
                 const unsigned hs = (unsigned)g.heads << p.split_log2, bottom = (unsigned)(g.Mh - p.row1) * g.Mw;
                 const unsigned per_row = p.inner ? p.col1 : g.Mw - p.col1, per_sample = p.row1 * per_row + (p.inner ? 0u : bottom);
@@ -936,8 +946,10 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 const int sk = sq.pop(), sv = sq.pop();
                 fill(sk, mk, mk, p.k, p.k, td.kt * 2 * kG, false);
                 if (ok) fill(sv, mv, mv, p.v, p.v, td.kt * 2 * kG, false);
-                for (int i = 0, hc = 2 * td.c0; ok && i < 2 * td.nch; ++i, hc = hc + 1 == 2 * td.nch ? 0 : hc + 1)
+                for (int i = 0; ok && i < 2 * td.nch; ++i) {
+                    const int hc = ST && i + 2 * td.c0 >= 2 * td.nch ? i + 2 * td.c0 - 2 * td.nch : ST ? i + 2 * td.c0 : i;
                     fill(sq.take_half(), mq, mg, p.q, p.d_o, hc * kG, true);
+                }
                 sq.end_tile(sk, sv);
             }
         } else if (warp == kScoreWarp) {
@@ -1093,7 +1105,8 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
 
 // Everything the kernel above reads besides q, k, v and dO, in one launch.  Blocks [0, stat_blocks): per slot of a window
 // -lse log2 e and delta = rowsum(dO O), by windows and slots (slots without a token: -inf and 0), 64 slots x up to 16 heads
-// a block; bound by the reads of O and dO.  The other blocks: the bias tables by row difference and diagonal, and the
+// a block: as many as leave four blocks an SM.  Bound by the reads of O and dO, on small grids by the chain of a
+// block's reads (42 x 42 tokens, 13 x 128, side 21: 16 heads a block 29 us; so 10).  The other blocks: the bias tables by row difference and diagonal, and the
 // zeroed bias-gradient table.
 constexpr int kStatHeads = 16;
 
@@ -1101,7 +1114,7 @@ template <int D, int RW, bool ST>
 __global__ void __launch_bounds__(256)
 swin_bwd_onepass_prep_kernel(const Geo g, const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ lse,
                              const float* __restrict__ bias, float4* __restrict__ rowstat, float* __restrict__ bias0, float* __restrict__ bias1,
-                             float* __restrict__ dbias_acc, int npad, int rmax, int rl, unsigned stat_blocks, unsigned* __restrict__ flags, int n_flags) {
+                             float* __restrict__ dbias_acc, int npad, int rmax, int rl, unsigned stat_blocks, int block_heads, unsigned* __restrict__ flags, int n_flags) {
     if (blockIdx.x >= stat_blocks) {
         for (int i = (blockIdx.x - stat_blocks) * 256 + threadIdx.x; i < n_flags; i += (gridDim.x - stat_blocks) * 256) flags[i] = 0;
         const int per_head = 2 * rmax * rl, total = per_head * g.heads, nw = 2 * g.w - 1;
@@ -1119,14 +1132,14 @@ swin_bwd_onepass_prep_kernel(const Geo g, const __nv_bfloat16* __restrict__ o, c
     }
     constexpr int kLanes = D / 8, kRowsPass = 256 / kLanes;
     __shared__ float4 st[kStatHeads][33];
-    const unsigned hgroups = (g.heads + kStatHeads - 1) / kStatHeads, chunks = npad / 64;
+    const unsigned hgroups = (g.heads + block_heads - 1) / block_heads, chunks = npad / 64;
     unsigned x = blockIdx.x;
-    const int h0 = (int)(x % hgroups) * kStatHeads;
+    const int h0 = (int)(x % hgroups) * block_heads;
     x /= hgroups;
     const int chunk = (int)(x % chunks);
     x /= chunks;
     const int wc = (int)(x % g.Mw), wr = (int)(x / g.Mw % g.Mh), b = (int)(x / g.Mw / g.Mh);
-    const int nh = min(kStatHeads, g.heads - h0), eh = min(g.w, g.H - wr * g.w), ew = min(g.w, g.W - wc * g.w);
+    const int nh = min(block_heads, g.heads - h0), eh = min(g.w, g.H - wr * g.w), ew = min(g.w, g.W - wc * g.w);
     const int l = threadIdx.x % kLanes;
     for (int r0 = 0; r0 < 64 * nh; r0 += kRowsPass) {
         const int r = r0 + threadIdx.x / kLanes;
@@ -1365,12 +1378,15 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     p.dbias_acc = reinterpret_cast<float*>(ws + pl.off_acc);
     p.slabs = reinterpret_cast<float4*>(ws + pl.off_slabs);
     p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v; p.d_o = (const __nv_bfloat16*)d_o;
-    const unsigned stat = (unsigned)((long long)g.B * g.Mh * g.Mw * (pl.npad / 64) * ((g.heads + kStatHeads - 1) / kStatHeads));
+    int block_heads = kStatHeads;
+    const long long stat_chunks = (long long)g.B * g.Mh * g.Mw * (pl.npad / 64);
+    while (block_heads > 1 && stat_chunks * ((g.heads + block_heads - 1) / block_heads) < 4 * kPlanSms) block_heads /= 2;
+    const unsigned stat = (unsigned)(stat_chunks * ((g.heads + block_heads - 1) / block_heads));
     const long long table = (long long)g.heads * 2 * pl.rmax * pl.rl;
     const unsigned tblocks = (unsigned)(table / 1024 + 1 < 592 ? table / 1024 + 1 : 592);
     prof_begin("swin_bwd_onepass_prep_kernel", stream);
     swin_bwd_onepass_prep_kernel<D, RW, ST><<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
-        const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, pl.rl, stat, p.flags, pl.flags);
+        const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, pl.rl, stat, block_heads, p.flags, pl.flags);
     count_launch(stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
