@@ -273,12 +273,18 @@ swin_fwd_mma_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv
 // (batch, window); a window is one 64-row tile of Q, K and V, 8 slots to a window row (slot = 8 a + b).  No online softmax: the
 // whole score row is in registers.
 // These shapes should be bound by HBM, but a CTA's chain (copies, products, softmax, stores) is several times as long as the
-// copies take, so what counts is how many CTAs an SM holds: tiles are not double-buffered (8 x 128 channels: 4 CTAs of 50 KB),
+// copies take, so what counts is how many CTAs an SM holds, and at head dims 32 and 64, where two sets of tiles leave room for five and four,
+// that the next window's copies run under a window's chain (one set, 6 and 5 CTAs: 536 x 1008 tokens, 6 x 32 214 us, so 200;
+// 2 x 213 x 613, 6 x 64 169 us, so 154).  At head dim 128 one set (4 CTAs of 50 KB);
 // the bias entries that a thread needs (a window row further down is a row further up in the table: 18 for 32 scores) stay in its
-// registers for the whole run, a warp's output takes the place of its own Q rows, and a window costs two barriers.
+// registers for the whole run, a warp's output takes the place of its own Q rows, and a window costs two barriers (two sets: one).
 // 288 x 544 tokens, 8 x 128: 353 -> 232 us (85 % of the copy bandwidth); 128 x 256, 6 x 32: 27 -> 20 us.
 template <int D>
-__global__ void __launch_bounds__(NTHREADS, D == 128 ? 4 : D == 64 ? 5 : 6)
+constexpr bool kSmallTwice = D != 128;
+template <int D>
+constexpr size_t kSmallFwdSmem = (kSmallTwice<D> ? 6 : 3) * (size_t)BN * D * 2;
+template <int D>
+__global__ void __launch_bounds__(NTHREADS, D == 32 ? 5 : 4)
 swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
                       const __nv_bfloat16* __restrict__ v, const float* __restrict__ bias,
                       __nv_bfloat16* __restrict__ o, float* __restrict__ lse, int ctas_per_head) {
@@ -288,8 +294,6 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
     constexpr int TILE_BYTES = BN * D * 2;
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* s_q = smem;
-    unsigned char* s_k = smem + TILE_BYTES;
-    unsigned char* s_v = smem + 2 * TILE_BYTES;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int gq = lane >> 2, tq = lane & 3;
@@ -305,21 +309,21 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
     };
     // each warp copies its own 16 rows (window rows 2 warp and 2 warp + 1) of the three tiles
     const int crow = 16 * warp + lane / CPR, cchunk = lane % CPR;
-    auto issue_loads = [&](const ItemCursor& c) {
+    auto issue_loads = [&](const ItemCursor& c, unsigned char* tiles) {
         const int eh = min(g.w, g.H - c.wr * g.w), ew = min(g.w, g.W - c.wc * g.w);
 #pragma unroll
         for (int i = 0; i < 16 / RPI; ++i) {
             const int row = crow + i * RPI, a = row >> 3, b = row & 7;
             const bool ok = a < eh && b < ew;
             const size_t off = ok ? token(c, a, b) * g.ts + head * D + cchunk * 8 : 0;
-            const uint32_t dst = smem_u32(s_q + tile_off<D>(row, cchunk));
+            const uint32_t dst = smem_u32(tiles + tile_off<D>(row, cchunk));
             cp_async16(dst, q + off, ok ? 16 : 0);
             cp_async16(dst + TILE_BYTES, k + off, ok ? 16 : 0);
             cp_async16(dst + 2 * TILE_BYTES, v + off, ok ? 16 : 0);
         }
         cp_async_commit();
     };
-    if (cur.b < g.B) issue_loads(cur);
+    if (cur.b < g.B) issue_loads(cur, s_q);
 
     // bias log2 e between query row (2 warp + h, gq) and key (nt, 2 tq + e): entry [h - nt + 7][e]
     float bv[9][2];
@@ -339,6 +343,11 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
         const int hb = (!g.pw && g.sw > 0) ? min(max(g.W - g.sw - cur.wc * g.w, 0), 8) : 8;
         cp_async_wait<0>();
         __syncthreads();
+        unsigned char *const s_k = s_q + TILE_BYTES, *const s_v = s_q + 2 * TILE_BYTES;
+        ItemCursor next = cur;
+        cursor_advance(next, 1, g.Mw, g.Mh);
+        unsigned char* const s_next = kSmallTwice<D> ? (s_q == smem ? smem + 3 * TILE_BYTES : smem) : smem;
+        if (kSmallTwice<D> && next.b < g.B) issue_loads(next, s_next);
 
         // S = Q K^T for the warp's 16 query rows
         float acc_s[BN / 8][4];
@@ -449,9 +458,12 @@ swin_fwd_small_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __
             if (a < eh && b < ew)
                 *reinterpret_cast<uint4*>(o + (token(cur, a, b) * g.heads + head) * D + cchunk * 8) = *reinterpret_cast<const uint4*>(s_q + tile_off<D>(row, cchunk));
         }
-        cursor_advance(cur, 1, g.Mw, g.Mh);
-        __syncthreads();   // the tiles are free for the next window
-        if (cur.b < g.B) issue_loads(cur);
+        cur = next;
+        s_q = s_next;
+        if (!kSmallTwice<D>) {
+            __syncthreads();   // the tiles are free for the next window
+            if (cur.b < g.B) issue_loads(cur, s_q);
+        }
     }
 }
 
@@ -469,7 +481,7 @@ cudaError_t TERRA_ELEM_FN(launch_fwd_mma)(const Geo& g, const void* q, const voi
                            void* o, float* lse, int sm_count, cudaStream_t stream) {
     if (g.w <= 8) {
         auto kern = g.d == 32 ? swin_fwd_small_kernel<32> : g.d == 64 ? swin_fwd_small_kernel<64> : swin_fwd_small_kernel<128>;
-        const size_t smem = 3 * (size_t)BN * g.d * 2;
+        const size_t smem = g.d == 32 ? kSmallFwdSmem<32> : g.d == 64 ? kSmallFwdSmem<64> : kSmallFwdSmem<128>;
         int occ = 0;
         cudaError_t e = prepare_kernel((const void*)kern, smem, NTHREADS, &occ);
         if (e != cudaSuccess) return e;
