@@ -1,7 +1,7 @@
 // Forward shifted-window attention on the tcgen05 tensor cores: window sides 9 .. 32 at head dims 64 and 128, 17 .. 32 at head dim 32 (less the
 // sides that fwd_win_supported leaves to the register tiles), any grid.
 //
-// A unit is a pair of 128-row query tiles of one (sample, window, head); a persistent CTA per SM walks over units and streams
+// A unit is a pair of 128-row query tiles of one (sample, window, head), on small grids one tile; a persistent CTA per SM walks over units and streams
 // the window's keys through shared memory in chunks of 128 slots (see win_tiles.cuh: 16 or 32 slots to a window row).  Per
 // half chunk of 64 keys and query tile:
 //   S = Q K^T (+ E_q E_k^T, see below), 128 x 64 in TMEM;
@@ -92,7 +92,9 @@ struct Params {
     const __nv_bfloat16 *q, *k, *v;
     const float* tables;         // [head][Tab::rows][Tab::kRowF]; ST: [head][2 w - 1][2][64 strips], read from global memory
     int strips;                  // ST: strips of a full window row
-    int pairs;                   // query tile pairs of a full window
+    int tiles;                   // query tiles of a unit: 2, or 1 where that leaves every unit a CTA
+    int units_win, units_row;    // units of a window of full height, and of one of the last, truncated window row
+    int rows;                    // window rows of full height
     int head_slow;               // units in head-major order, a run per CTA; else the head is the fastest digit, strided
     long long units;
 };
@@ -473,7 +475,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     if (ew < ns * RW || (ha > 0 && ha < eh) || (hb > 0 && hb < ew) || (RW == 16 && (eh & 1))) flags |= 4;
                     int4* dst = reinterpret_cast<int4*>(smem + L::kOffDesc + (i % kDescs) * 64);
                     dst[0] = make_int4(head, b, wr, wc);
-                    dst[1] = make_int4(eh, ew, tile0, min(2, nqt - tile0));
+                    dst[1] = make_int4(eh, ew, tile0, min(p.tiles, nqt - tile0));
                     dst[2] = make_int4(ku, (ku + 3) / 4, ha, hb);
                     dst[3] = make_int4(flags, ns, 0, 0);
                     mbar_arrive(bar(kBDesc + i % kDescs));
@@ -488,10 +490,13 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 unsigned rest, head;
                 if (p.head_slow) { head = (unsigned)u / per_head; rest = (unsigned)u - head * per_head; }
                 else { rest = (unsigned)u / g.heads; head = (unsigned)u - rest * g.heads; }
-                const unsigned win = rest / p.pairs, pair = rest - win * p.pairs, r2 = win / g.Mw, wc = win - r2 * g.Mw, b = r2 / g.Mh, wr = r2 - b * g.Mh;
+                // sample, then the windows of full height, then the last row's
+                const unsigned full = (unsigned)p.rows * g.Mw * p.units_win, per_sample = full + (unsigned)(g.Mh - p.rows) * g.Mw * p.units_row;
+                const unsigned b = rest / per_sample, in = rest - b * per_sample, each = in < full ? p.units_win : p.units_row, at = in < full ? in : in - full;
+                const unsigned win = at / each, unit = at - win * each, row = win / g.Mw, wc = win - row * g.Mw, wr = in < full ? row : p.rows;
                 const int eh = min(g.w, g.H - (int)wr * g.w), ew = min(g.w, g.W - (int)wc * g.w);
-                if ((int)pair * 2 * kTileRows >= eh * (ST ? strips_of(ew) : 1)) continue;            // a truncated window has fewer query tiles
-                put(1 | ((int)head != last_head ? 2 : 0), head, b, wr, wc, eh, ew, pair * 2);
+                if (ST && (int)unit * p.tiles * kTileRows >= eh * strips_of(ew)) continue;            // a truncated window has fewer query tiles
+                put(1 | ((int)head != last_head ? 2 : 0), head, b, wr, wc, eh, ew, unit * p.tiles);
                 last_head = head;
             }
             if (ok) put(0, 0, 0, 0, 0, 1, 1, 0);
@@ -819,9 +824,18 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
     p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v;
     p.tables = (const float*)workspace;
     p.strips = ST ? strips_of(g.w) : 1;
-    const int tiles = ((g.w < g.H ? g.w : g.H) * (ST ? strips_of(g.w < g.W ? g.w : g.W) : 1) * RW + kTile - 1) / kTile;
-    p.pairs = (tiles + 1) / 2;
-    p.units = (long long)g.B * g.Mh * g.Mw * g.heads * p.pairs;
+    const int row_slots = (ST ? strips_of(g.w < g.W ? g.w : g.W) : 1) * RW;
+    auto tiles_of = [&](int rows) { return (rows * row_slots + kTile - 1) / kTile; };
+    p.rows = g.H / g.w;
+    auto plan = [&](int tiles) {
+        p.tiles = tiles;
+        p.units_win = (tiles_of(g.w) + tiles - 1) / tiles;
+        p.units_row = (tiles_of(g.H - p.rows * g.w) + tiles - 1) / tiles;
+        p.units = (long long)g.B * g.Mw * g.heads * ((long long)p.rows * p.units_win + (g.Mh - p.rows) * p.units_row);
+    };
+    // One tile a unit has a unit's chain to itself: two thirds of a pair's time (32 x 64 tokens, 4 x 32, side 32: 27.7 -> 23.6 us a call).
+    plan(1);
+    if (p.units > sm_count) plan(2);
     // A CTA keeps to one head where that leaves no more than 1 SM in 20 idle: neighbouring CTAs then read the heads of the same
     // tokens at the same time.  Otherwise each CTA takes a run of the units in head-major order.
     const int bound = sm_count / g.heads * g.heads;
