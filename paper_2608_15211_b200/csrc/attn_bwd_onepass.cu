@@ -1142,11 +1142,11 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
 // zeroed bias-gradient table.
 constexpr int kStatHeads = 16;
 
-template <int D, int RW, bool ST>
+template <int D, int RW, bool ST, bool FEW>
 __global__ void __launch_bounds__(256)
 swin_bwd_onepass_prep_kernel(const Geo g, const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o, const float* __restrict__ lse,
                              const float* __restrict__ bias, float4* __restrict__ rowstat, float* __restrict__ bias0, float* __restrict__ bias1,
-                             float* __restrict__ dbias_acc, int npad, int rmax, int rl, unsigned stat_blocks, int block_heads, unsigned* __restrict__ flags, int n_flags) {
+                             float* __restrict__ dbias_acc, int npad, int rmax, int rl, unsigned stat_blocks, int few_heads, unsigned* __restrict__ flags, int n_flags) {
     if (blockIdx.x >= stat_blocks) {
         for (int i = (blockIdx.x - stat_blocks) * 256 + threadIdx.x; i < n_flags; i += (gridDim.x - stat_blocks) * 256) flags[i] = 0;
         const int per_head = 2 * rmax * rl, total = per_head * g.heads, nw = 2 * g.w - 1;
@@ -1164,6 +1164,7 @@ swin_bwd_onepass_prep_kernel(const Geo g, const __nv_bfloat16* __restrict__ o, c
     }
     constexpr int kLanes = D / 8, kRowsPass = 256 / kLanes;
     __shared__ float4 st[kStatHeads][33];
+    const int block_heads = FEW ? few_heads : kStatHeads;
     const unsigned hgroups = (g.heads + block_heads - 1) / block_heads, chunks = npad / 64;
     unsigned x = blockIdx.x;
     const int h0 = (int)(x % hgroups) * block_heads;
@@ -1417,7 +1418,8 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     const long long table = (long long)g.heads * 2 * pl.rmax * pl.rl;
     const unsigned tblocks = (unsigned)(table / 1024 + 1 < 592 ? table / 1024 + 1 : 592);
     prof_begin("swin_bwd_onepass_prep_kernel", stream);
-    swin_bwd_onepass_prep_kernel<D, RW, ST><<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
+    const auto prep = block_heads < kStatHeads ? swin_bwd_onepass_prep_kernel<D, RW, ST, true> : swin_bwd_onepass_prep_kernel<D, RW, ST, false>;
+    prep<<<stat + tblocks, 256, 0, stream>>>(g, (const __nv_bfloat16*)o, (const __nv_bfloat16*)d_o, lse, bias,
         const_cast<float4*>(p.rowstat), const_cast<float*>(p.bias0), const_cast<float*>(p.bias1), p.dbias_acc, pl.npad, pl.rmax, pl.rl, stat, block_heads, p.flags, pl.flags);
     count_launch(stream);
     cudaError_t e = cudaGetLastError();
