@@ -57,8 +57,11 @@ using namespace tc;
 
 constexpr int kThreads = 512;
 constexpr int kWorkWarps = 8, kReadWarp0 = 8, kProductWarp = 12, kLoaderWarp = 13, kScoreWarp = 14, kPlanWarp = 15;
-constexpr int kRegsLaunch = 128, kRegsWork = 168, kRegsRead = 104, kRegsOther = 72;
+// Registers a thread: at launch, then of the elementwise, read-out and other warps.  The read-out's 64 accumulator values and addresses
+// need 120 (with 104 it spilled: 111 x 398 tokens, 12 x 128, side 64 5.1 ms, so 4.3; 288 x 544, 8 x 128, side 16 950 us, so 914).
+constexpr int kRegsLaunch = 128, kRegsWork = 160, kRegsRead = 120, kRegsOther = 72;
 static_assert(2 * kRegsWork + kRegsRead + kRegsOther <= 4 * kRegsLaunch, "register hand-over does not balance");
+static_assert(kRegsWork >= kRegsLaunch && kRegsRead <= kRegsLaunch && kRegsOther <= kRegsLaunch, "only the elementwise warps take registers");
 constexpr int kTile = 128, kHalf = 64;
 constexpr int kDescs = 8;                                                             // ring of tile descriptors
 constexpr int kScrLine = 160;                                                         // see flush_sums
@@ -76,6 +79,8 @@ struct Lay {
     // per half chunk (ring of kTabs): 64 queries' statistics, then the bias rows its pieces meet, twice (the second copy shifted
     // by one entry and 16 banks away, so that lanes with even and odd g read different banks); head dim 128 has no room
     // and reads them from global memory
+    // windows that are two parts (see part_tiles) as such; at head dim 32 what it takes costs all windows 5 % (2 x 256 x 544, 13 x 32, side 32)
+    static constexpr bool kTwo = ST || D != 32;
     static constexpr bool kTables = D != 128 && !ST, kGang = ST;
     static constexpr int kTabs = 4, kBiasRows = kTile / RW + kHalf / RW - 1, kCopyB = kBiasRows * 2 * RW * 4;
     static constexpr int kOffCopy0 = 512, kOffCopy1 = 512 + (kCopyB + 127) / 128 * 128 + 64;
@@ -112,6 +117,7 @@ struct Params {
     // The launch's units: first those of the windows (row >= row1, any column), then of (row < row1, column >= col1); a launch of
     // the inner windows has the units of (row < row1, column < col1).
     int row1, col1, inner;
+    int part_row, part_ha;           // the window row whose windows may be two parts, -1: none (see part_tiles), and the second part's first row
     int slab0;                       // first slab of the launch (two launches may overlap)
     int overlap;                     // the launch runs beside the one before it, which started when its prerequisites were complete
     // Gangs: `gang` CTAs work on the key tiles of one (window, head) after the other, each on every gang-th of the gang's tiles, and add
@@ -149,7 +155,8 @@ struct SlotQueue {
 // A key tile of a unit, as the planning warp hands it to the other roles.
 struct TileDesc {
     int head, b, wr, wc;
-    int eh, ew, kt, nch;
+    int eh, ew, kt;
+    int nch, q0;           // chunks of 128 queries that the tile meets, and the first of them (see part_tiles)
     int ha, hb;            // window rows >= ha / columns >= hb carry the other shift-mask label (far outside: none do)
     int flags;             // 1: a tile (0: the end), 2: the unit's first, 4: its last
     int slab;
@@ -440,7 +447,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         const int4* src = reinterpret_cast<const int4*>(smem + L::kOffDesc + i * 64);
         const int4 d0 = src[0], d1 = src[1], d2 = src[2];
         td.head = d0.x; td.b = d0.y; td.wr = d0.z; td.wc = d0.w;
-        td.eh = d1.x; td.ew = d1.y; td.kt = d1.z; td.nch = d1.w;
+        td.eh = d1.x; td.ew = d1.y; td.kt = d1.z; td.nch = d1.w & 0xffff; td.q0 = L::kTwo ? d1.w >> 16 : 0;
         td.ha = d2.x; td.hb = d2.y; td.flags = d2.z; td.slab = d2.w;
         if (ST) {
             const int4 d3 = src[3];
@@ -482,9 +489,9 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         // the next tile: what its half chunks have in common
         auto enter_tile = [&]() {
             if (!next_tile()) return false;
-            hc = ST ? 2 * td.c0 + b : b;
+            hc = 2 * td.q0 + (ST ? 2 * td.c0 + b : b);
             if (ST) left = td.nch;
-            nh = 2 * td.nch;
+            nh = 2 * (td.q0 + td.nch);
             ha = td.ha;
             a_k0 = td.kt * (kTile / RW) + (RW == 32 ? wq : 2 * wq);
             if (ST) {
@@ -492,7 +499,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 a_k0 = unit_row(u, td.ns);
                 c_k0 = 32 * (u - a_k0 * td.ns);
             }
-            const bool labels = (ha > 0 && ha < td.eh) || (td.hb > 0 && td.hb < td.ew);
+            const bool labels = (ha > 0 && ha < td.eh && (!L::kTwo || part_tiles(ha, td.eh, td.ns * RW) == 0)) || (td.hb > 0 && td.hb < td.ew);
             masked = KIND == 1 || (KIND == 2 && (labels || td.ew < td.ns * RW || (td.kt + 1) * (kTile / RW) > td.eh * td.ns));
             rowbits = 0;                                     // bits m: the row holds a key; bits 4 + m: it lies behind hb
             qbits = 0;
@@ -574,7 +581,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             const int acc_row = ST ? piece_at(1) - piece_at(0) : (32 / RW) * 2 * RW;
             hc += 2;
             if (ST) {
-                if (hc >= nh) hc -= nh;
+                if (hc >= nh) hc -= 2 * td.nch;
                 if (--left == 0) live = enter_tile();
             } else if (hc >= nh) {
                 live = enter_tile();
@@ -626,8 +633,9 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         // A tile's place in the order of those that add to chunk c: the tiles' own, or (rotate) from round to round of the gang's CTAs and in
         // each from the one that starts at the chunk, or last in front of it, downwards.
         auto place = [&](int c) {
-            if (!p.rotate) return td.kt;
-            const int n = min(p.gang, td.nch), j = td.kt % n, round = td.kt - j, in_round = min(n, td.nch - round);
+            const int kt = td.kt - td.q0;
+            if (!p.rotate) return kt;
+            const int n = min(p.gang, td.nch), j = kt % n, round = kt - j, in_round = min(n, td.nch - round);
             const int r = min(in_round - 1, ((c + 1) * n - 1) / td.nch) - j;
             return round + (r < 0 ? r + in_round : r);
         };
@@ -676,20 +684,22 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         while (ok && next_tile()) {
             bool first = td.flags & 2, last = td.flags & 4;
             const bool shared = ganged && td.nch > 1;
-            int at = td.kt;
+            int at = td.kt - td.q0;
             const size_t sample = (size_t)td.b * g.H * g.W;
-            float4* slab = p.slabs + (size_t)td.slab * ((size_t)p.npad * D / 4) + row;
+            float4* slab = p.slabs + ((size_t)td.slab * p.npad + td.q0 * kTile) * (D / 4) + row;
+            const int u0 = td.q0 * (kTile / RW);                 // the part's first window row (ST: strip)
             if (D == 128) {
                 // dQ^T: lanes = channels, columns = the half chunk's queries
                 for (int i = 0; i < 2 * td.nch; ++i, ++n) {
-                    const int b = i & 1, hc = ST && i + 2 * td.c0 >= 2 * td.nch ? i + 2 * td.c0 - 2 * td.nch : ST ? i + 2 * td.c0 : i;
+                    const int b = i & 1, rel = ST && i + 2 * td.c0 >= 2 * td.nch ? i + 2 * td.c0 - 2 * td.nch : ST ? i + 2 * td.c0 : i;
+                    const int ev = ST && p.rotate ? 2 * td.q0 + rel : rel;       // (rotate: both parts of a window use one slab)
                     if (shared) {
                         if (p.rotate) {
-                            at = place(hc >> 1);
+                            at = place(rel >> 1);
                             first = at == 0;
                             last = at == td.nch - 1;
                         }
-                        ok = turn(hc, at);
+                        ok = turn(ev, at);
                     }
                     ok = ok && mbar_wait_all(bar(kBDq + b), (n >> 1) & 1, cta_abort);
                     if (!ok) break;
@@ -700,15 +710,15 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     hand_back(kBDqFree + b);
 #pragma unroll
                     for (int hh = 0; hh < 2; ++hh) {
-                        float4* s4 = slab + (hc * 16 + hh * 8) * 128;
+                        float4* s4 = slab + (rel * 16 + hh * 8) * 128;
                         if (!last || split) {
                             to_slab(s4, r[hh], !first);
                         } else {
                             if (!first) from_slab(s4, r[hh]);
-                            const int s0 = hc * kHalf + 32 * hh;
+                            const int s0 = rel * kHalf + 32 * hh;
 #pragma unroll
                             for (int jr = 0; jr < 32 / RW; ++jr) {
-                                const int u = s0 / RW + jr, a = ST ? unit_row(u, td.ns) : u, c0 = ST ? 32 * (u - a * td.ns) : 0;
+                                const int u = u0 + s0 / RW + jr, a = ST ? unit_row(u, td.ns) : u, c0 = ST ? 32 * (u - a * td.ns) : 0;
                                 if (a >= td.eh) continue;
                                 int v = td.wc * g.w + c0 + g.sw;
                                 if (v >= g.W) v -= g.W;
@@ -736,21 +746,22 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                             }
                         }
                     }
-                    if (shared && !last) turn_done(hc, at, hc == 2 * td.nch - 1);
+                    if (shared && !last) turn_done(ev, at, rel == 2 * td.nch - 1);
                 }
             } else {
                 const bool resident = !ganged && td.nch <= L::kResident;
                 if (!resident || last) {
                     for (int i = 0; i < td.nch; ++i) {
-                        const int ch = ST && i + td.c0 >= td.nch ? i + td.c0 - td.nch : ST ? i + td.c0 : i;
-                        const int r = D == 64 ? 0 : resident ? ch : (int)(n++ & 1);
+                        const int rel = ST && i + td.c0 >= td.nch ? i + td.c0 - td.nch : ST ? i + td.c0 : i;
+                        const int ev = ST && p.rotate ? td.q0 + rel : rel;
+                        const int r = D == 64 ? 0 : resident ? rel : (int)(n++ & 1);
                         if (shared) {
                             if (p.rotate) {
-                                at = place(ch);
+                                at = place(rel);
                                 first = at == 0;
                                 last = at == td.nch - 1;
                             }
-                            ok = turn(ch, at);
+                            ok = turn(ev, at);
                         }
                         ok = ok && mbar_wait_all(bar(kBDq + r), (dq_use >> r) & 1, cta_abort);
                         if (!ok) break;
@@ -760,12 +771,12 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
 #pragma unroll
                         for (int q = 0; q < kLd; ++q) tmem_ld32(tl + L::kColDq + L::kStrideDq * r + 32 * q, v[q]);
                         hand_back(kBDqFree + r);
-                        const int slot = ch * kTile + row, u = slot / RW, a = ST ? unit_row(u, td.ns) : u, b = slot % RW + (ST ? 32 * (u - a * td.ns) : 0);
+                        const int slot = rel * kTile + row, u = u0 + slot / RW, a = ST ? unit_row(u, td.ns) : u, b = slot % RW + (ST ? 32 * (u - a * td.ns) : 0);
                         const bool add = !resident && !first, tok = a < td.eh && b < td.ew;
                         uint4* dst = reinterpret_cast<uint4*>(dq + (sample + (tok ? win_token(g, td.wr, td.wc, a, b) : 0)) * g.ts + td.head * D);
 #pragma unroll
                         for (int q = 0; q < kLd; ++q) {
-                            float4* s4 = slab + (ch * (D / 4) + q * 8) * 128;
+                            float4* s4 = slab + (rel * (D / 4) + q * 8) * 128;
                             if (!last || split) {
                                 to_slab(s4, v[q], add);
                             } else {
@@ -774,7 +785,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                                 else if (tok) store_scaled32(dst + 4 * q, v[q], out_scale);
                             }
                         }
-                        if (shared && !last) turn_done(ch, at, ch == td.nch - 1);
+                        if (shared && !last) turn_done(ev, at, rel == td.nch - 1);
                     }
                 }
             }
@@ -816,13 +827,13 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             struct { int b, wr, wc; } cur = {0, 0, 0};
             unsigned i = 0;
             bool ok = true;
-            auto put = [&](int flags, int head, int eh, int ew, int kt, int nch, int slab, int seq = 0, int use = 0, int c0 = 0) {
+            auto put = [&](int flags, int head, int eh, int ew, int kt, int nch, int q0, int slab, int seq = 0, int use = 0, int c0 = 0) {
                 ok = mbar_wait_all(bar(kBDescFree + i % kDescs), ((i / kDescs) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
                 if (lane == 0) {
                     int4* dst = reinterpret_cast<int4*>(smem + L::kOffDesc + (i % kDescs) * 64);
                     dst[0] = make_int4(head, cur.b, cur.wr, cur.wc);
-                    dst[1] = make_int4(eh, ew, kt, nch);
+                    dst[1] = make_int4(eh, ew, kt, nch | q0 << 16);
                     dst[2] = make_int4((!g.ph && g.sh > 0) ? g.H - g.sh - cur.wr * g.w : (1 << 20), (!g.pw && g.sw > 0) ? g.W - g.sw - cur.wc * g.w : (1 << 20), flags, slab);
                     if (ST) dst[3] = make_int4(strips_of(ew), seq, use, c0);
                     mbar_arrive(bar(kBDesc + i % kDescs));
@@ -833,12 +844,12 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             // The tables of the tile in front of the last one put: each of its copies takes this warp a few hundred cycles, and
             // the loading warp has as many of its own (with both on one warp it was what the score warp waited for).
             unsigned n = 0;                          // half chunks so far
-            int t_head = 0, t_kt = 0, t_nch = 0, t_win = 0;
+            int t_head = 0, t_kt = 0, t_nch = 0, t_q0 = 0, t_win = 0;
             auto tables = [&]() {
                 // bias rows of half chunk hc: row differences from hc kG - (kt + 1) (128 / RW) + 1 on
                 const size_t rows0 = ((size_t)t_head * 2 * p.rmax + p.rmax + 1 - (t_kt + 1) * (kTile / RW)) * (2 * RW);
                 const float4* stat = p.rowstat + ((size_t)t_win * g.heads + t_head) * (p.npad / 2);
-                for (int hc = 0; ok && hc < 2 * t_nch; ++hc, ++n) {
+                for (int hc = 2 * t_q0; ok && hc < 2 * (t_q0 + t_nch); ++hc, ++n) {
                     const int r = (int)(n % L::kTabs);
                     ok = mbar_wait_all(bar(kBTabFree + r), ((n / L::kTabs) & 1) ^ 1u, cta_abort);
                     if (!ok) break;
@@ -874,23 +885,30 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 const int kt0 = (split * nch) >> p.split_log2, kt1 = ((split + 1) * nch) >> p.split_log2;
                 // a slab per CTA; where windows are split, per unit in the order of all windows
                 const int slab = p.split_log2 ? (int)((((long long)(cur.b * g.Mh + cur.wr) * g.Mw + cur.wc) * hs) + hd) : p.slab0 + (int)blockIdx.x;
+                // where the window is two, a part's tiles meet its own queries only
+                const int t0 = !L::kTwo || cur.wr != p.part_row ? 0 : ST ? part_tiles(p.part_ha, eh, strips_of(ew) * RW) : p.part_ha * RW / kTile;
                 if (L::kGang && p.gang > 1) {
-                    for (int kt = (member + p.gang - seq % p.gang) % p.gang; ok && kt < nch; kt += p.gang)
-                        put(1 | (kt == 0 ? 2 : 0) | (kt == nch - 1 ? 4 : 0), head, eh, ew, kt, nch, (int)(blockIdx.x / p.gang) * p.ring + windows % p.ring, seq,
-                            windows / p.ring, p.rotate ? member * nch / min(p.gang, nch) : 0);
-                    seq += nch;
-                    windows += nch > 1;
+                    for (int q0 = 0; q0 < nch;) {
+                        const int tn = q0 == 0 && t0 > 0 ? t0 : nch - q0, ranks = min(p.gang, tn);
+                        for (int kt = (member + p.gang - seq % p.gang) % p.gang; ok && kt < tn; kt += p.gang)
+                            put(1 | (kt == 0 ? 2 : 0) | (kt == tn - 1 ? 4 : 0), head, eh, ew, q0 + kt, tn, q0, (int)(blockIdx.x / p.gang) * p.ring + windows % p.ring, seq,
+                                windows / p.ring, p.rotate ? kt % ranks * tn / ranks : 0);
+                        seq += tn;
+                        windows += tn > 1;
+                        q0 += tn;
+                    }
                     continue;
                 }
                 for (int kt = kt0; ok && kt < kt1; ++kt) {
-                    put(1 | (kt == kt0 ? 2 : 0) | (kt == kt1 - 1 ? 4 : 0), head, eh, ew, kt, nch, slab);
+                    const int q0 = t0 > 0 && kt >= t0 ? t0 : 0, q1 = t0 > 0 && kt < t0 ? t0 : nch;
+                    put(1 | (kt == max(kt0, q0) ? 2 : 0) | (kt == min(kt1, q1) - 1 ? 4 : 0), head, eh, ew, kt, q1 - q0, q0, slab);
                     if (L::kTables) {
                         tables();
-                        t_head = head; t_kt = kt; t_nch = nch; t_win = (cur.b * g.Mh + cur.wr) * g.Mw + cur.wc;
+                        t_head = head; t_kt = kt; t_nch = q1 - q0; t_q0 = q0; t_win = (cur.b * g.Mh + cur.wr) * g.Mw + cur.wc;
                     }
                 }
             }
-            if (ok) put(0, 0, 0, 0, 0, 0, 0);
+            if (ok) put(0, 0, 0, 0, 0, 0, 0, 0);
             if (L::kTables) tables();
         } else if (warp == kLoaderWarp) {
             // -------------------------------------------------------------- copies.  One warp fills every slot: a wait names a
@@ -979,7 +997,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 fill(sk, mk, mk, p.k, p.k, td.kt * 2 * kG, false);
                 if (ok) fill(sv, mv, mv, p.v, p.v, td.kt * 2 * kG, false);
                 for (int i = 0; ok && i < 2 * td.nch; ++i) {
-                    const int hc = ST && i + 2 * td.c0 >= 2 * td.nch ? i + 2 * td.c0 - 2 * td.nch : ST ? i + 2 * td.c0 : i;
+                    const int hc = 2 * td.q0 + (ST && i + 2 * td.c0 >= 2 * td.nch ? i + 2 * td.c0 - 2 * td.nch : ST ? i + 2 * td.c0 : i);
                     fill(sq.take_half(), mq, mg, p.q, p.d_o, hc * kG, true);
                 }
                 sq.end_tile(sk, sv);
@@ -1227,9 +1245,11 @@ swin_bwd_onepass_finish_kernel(const Geo g, const float* __restrict__ dbias_acc,
     const int row = i & 127, cg = i >> 7;
     const int slot0 = D == 128 ? 4 * cg : (cg / (D / 4)) * kTile + row;
     if (i >= per_item || slot0 >= nch * kTile) return;
+    const int t0 = Lay<D, RW>::kTwo ? part_tiles((!g.ph && g.sh > 0) ? g.H - g.sh - wr * g.w : (1 << 20), eh, RW) : 0;
+    const int c_lo = t0 > 0 && slot0 >= t0 * kTile ? t0 : 0, c_hi = t0 > 0 && slot0 < t0 * kTile ? t0 : nch;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int s = 0; s < (1 << split_log2); ++s) {
-        if (((s * nch) >> split_log2) == (((s + 1) * nch) >> split_log2)) continue;
+        if (max((s * nch) >> split_log2, c_lo) >= min(((s + 1) * nch) >> split_log2, c_hi)) continue;       // none of its tiles meets the chunk
         const float4 t = __ldcg(slabs + ((item << split_log2) + s) * per_item + i);
         v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
     }
@@ -1399,6 +1419,9 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     p.npad = pl.npad;
     p.rmax = pl.rmax;
     p.rl = pl.rl;
+    p.part_ha = !g.ph && g.sh > 0 ? (g.H - g.sh) % g.w : 0;
+    p.part_row = (g.H - g.sh) / g.w;
+    if (p.part_ha == 0 || (!ST && part_tiles(p.part_ha, g.H - p.part_row * g.w < g.w ? g.H - p.part_row * g.w : g.w, RW) == 0)) p.part_row = -1;
     p.gang = pl.gang;
     p.ring = pl.ring;
     p.rotate = pl.rotate;
@@ -1461,7 +1484,8 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         // the windows in front of the first row and column that need the mask
         p.row1 = g.w == RW ? g.H / g.w : 0;
         p.col1 = g.w == RW ? g.W / g.w : 0;
-        if (!g.ph && g.sh > 0 && (g.H - g.sh) % g.w && (g.H - g.sh) / g.w < p.row1) p.row1 = (g.H - g.sh) / g.w;
+        // (a row of windows that are two each needs none)
+        if (!g.ph && g.sh > 0 && (g.H - g.sh) % g.w && (g.H - g.sh) / g.w < p.row1 && (!L::kTwo || part_tiles((g.H - g.sh) % g.w, g.w, RW) == 0)) p.row1 = (g.H - g.sh) / g.w;
         if (!g.pw && g.sw > 0 && (g.W - g.sw) % g.w && (g.W - g.sw) / g.w < p.col1) p.col1 = (g.W - g.sw) / g.w;
         if (p.row1 == 0 || p.col1 == 0) p.row1 = p.col1 = 0;
         const long long inner = (long long)p.row1 * p.col1;

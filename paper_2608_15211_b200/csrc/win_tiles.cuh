@@ -110,6 +110,10 @@ __device__ __forceinline__ void load_win_strip(const WinMaps& m, const WinCols& 
     }
 }
 
+// A window whose rows from `ha` on carry another mask label than those before is two windows where a 128-slot tile ends between them: the
+// tiles of one part see none of the other's.  The first part's tiles, 0 where the window is one.  `row_slots`: slots of a window row.
+__host__ __device__ __forceinline__ int part_tiles(int ha, int eh, int row_slots) { return ha > 0 && ha < eh && ha * row_slots % 128 == 0 ? ha * row_slots / 128 : 0; }
+
 // slot (a, b) of a window -> grid token
 __device__ __forceinline__ int win_token(const Geo& g, int wr, int wc, int a, int b) {
     int u = wr * g.w + a + g.sh;
