@@ -95,6 +95,7 @@ struct Params {
     int tiles;                   // query tiles of a unit: 2, or 1 where that leaves every unit a CTA
     int units_win, units_row;    // units of a window of full height, and of one of the last, truncated window row
     int rows;                    // window rows of full height
+    int part_row, part_ha;       // the window row whose windows may be two parts, -1: none (see part_tiles), and the second part's first row
     int head_slow;               // units in head-major order, a run per CTA; else the head is the fastest digit, strided
     long long units;
 };
@@ -105,6 +106,7 @@ struct Unit {
     int ku, nch, ha, hb;         // 32-slot key units, chunks; window rows >= ha / columns >= hb carry the other mask label
     int flags;                   // 1: a unit (0: the end), 2: another head than before, 4: the scores need the mask step
     int ns;                      // ST: strips of a window row
+    int c0;                      // first chunk of keys
 };
 
 // ST: rows of strips per row label among the mask operands, so that four strips in a row from any strip on lie in them
@@ -252,8 +254,9 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
         td.head = d0.x; td.b = d0.y; td.wr = d0.z; td.wc = d0.w;
         td.eh = d1.x; td.ew = d1.y; td.tile0 = d1.z; td.ntq = d1.w;
         td.ku = d2.x; td.nch = d2.y; td.ha = d2.z; td.hb = d2.w;
-        td.flags = src[3].x;
-        if (ST) td.ns = src[3].y;
+        const int4 d3 = src[3];
+        td.flags = d3.x; td.c0 = d3.z;
+        if (ST) td.ns = d3.y;
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kBDescFree + i));
         ++desc_n;
@@ -275,7 +278,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             if (!ST && (td.flags & 2)) ok = mbar_wait_all(bar(kBBias), heads++ & 1, cta_abort);
             if (ok && t < td.ntq) {
                 const int aq = min((td.tile0 + t) * kTileRows + wq * (32 / RW), (ST ? td.ku : td.eh) - 1);
-                uint32_t bias = tab0 + 4u * (g.w - 1 - aq + Tab<RW>::kFront) * Tab<RW>::kRowF;
+                uint32_t bias = tab0 + 4u * (g.w - 1 - aq + Tab<RW>::kFront + td.c0 * kTileRows) * Tab<RW>::kRowF;
                 // ST: the entries of the next half chunk's two key units, from the head's table in L2, are in registers before they are needed
                 float2 bv[ST ? 2 : 1][RW == 32 ? 7 : 9];
                 const float* bp = nullptr;
@@ -294,13 +297,17 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 if (ST) {
                     const int rq = unit_row(aq, td.ns), j0 = 32 * p.strips - 1 + 2 * ql - gl;
                     bp = p.tables + ((size_t)td.head * (2 * g.w - 1) + g.w - 1 - rq) * (128 * p.strips) + (j0 & 1) * (64 * p.strips) + (j0 & ~1) - 32 * (aq - rq * td.ns);
-                    next_bias(td.ku);
+                    const int rk = unit_row(4 * td.c0, td.ns);
+                    sk = 4 * td.c0 - rk * td.ns;
+                    bp += rk * 128 * p.strips + 32 * sk;
+                    next_bias(td.ku - 4 * td.c0);
                 }
                 float m[4] = {kLowest, kLowest, kLowest, kLowest};     // (finite: a half chunk may hold no key that the row sees)
                 float2 sum[4] = {};
                 int fixed = -1;                          // half chunk whose scores have gone by their labels
-                for (int j = 0; 2 * j < td.ku; ++j) {
-                    const unsigned idx = n + j * td.ntq + t, buf = idx % NB;
+                const int j0 = 2 * td.c0;
+                for (int j = j0; 2 * j < td.ku; ++j) {
+                    const unsigned idx = n + (j - j0) * td.ntq + t, buf = idx % NB;
                     const uint32_t t_s = tq + 64u * buf;
                     ok = mbar_wait_all(bar(kBS + buf), (idx / NB) & 1, cta_abort);
                     if (!ok) break;
@@ -339,7 +346,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                             sum[i].x *= f[i];
                             sum[i].y *= f[i];
                         }
-                        if (j > 0) {
+                        if (j > j0) {
                             // (the buffer of the last product cannot be freed again before this half chunk's product)
                             const unsigned last = idx - td.ntq;
                             ok = mbar_wait_all(bar(kBFree + last % NB), (last / NB) & 1, cta_abort);
@@ -412,7 +419,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             }
             if (lane == 0) mbar_arrive(bar(kBTab + (units & 1)));
             ++units;
-            n += ((td.ku + 1) >> 1) * td.ntq;
+            n += (((td.ku + 1) >> 1) - 2 * td.c0) * td.ntq;
         }
     } else if (warp < kPvWarp) {
         // ------------------------------------------------------------------ O: normalise and store
@@ -466,18 +473,20 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             unsigned i = 0;
             int last_head = -1;
             bool ok = true;
-            auto put = [&](int flags, int head, int b, int wr, int wc, int eh, int ew, int tile0) {
+            auto put = [&](int flags, int head, int b, int wr, int wc, int eh, int ew, int tile0, int t0) {
                 ok = mbar_wait_all(bar(kBDescFree + i % kDescs), ((i / kDescs) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
                 if (lane == 0) {
                     const int ha = (!g.ph && g.sh > 0) ? g.H - g.sh - wr * g.w : (1 << 20), hb = (!g.pw && g.sw > 0) ? g.W - g.sw - wc * g.w : (1 << 20);
-                    const int ns = ST ? strips_of(ew) : 1, nqt = (eh * ns * RW + kTile - 1) / kTile, ku = RW == 32 ? eh * ns : (eh + 1) / 2;
-                    if (ew < ns * RW || (ha > 0 && ha < eh) || (hb > 0 && hb < ew) || (RW == 16 && (eh & 1))) flags |= 4;
+                    const int ns = ST ? strips_of(ew) : 1, nqt = (eh * ns * RW + kTile - 1) / kTile, ku_all = RW == 32 ? eh * ns : (eh + 1) / 2;
+                    // a window of two parts: the part's keys (t0: the second part's first tile)
+                    const int c0 = t0 > 0 && tile0 >= t0 ? t0 : 0, ku = t0 > 0 && tile0 < t0 ? 4 * t0 : ku_all;
+                    if (ew < ns * RW || (ha > 0 && ha < eh && t0 == 0) || (hb > 0 && hb < ew) || (RW == 16 && (eh & 1))) flags |= 4;
                     int4* dst = reinterpret_cast<int4*>(smem + L::kOffDesc + (i % kDescs) * 64);
                     dst[0] = make_int4(head, b, wr, wc);
                     dst[1] = make_int4(eh, ew, tile0, min(p.tiles, nqt - tile0));
                     dst[2] = make_int4(ku, (ku + 3) / 4, ha, hb);
-                    dst[3] = make_int4(flags, ns, 0, 0);
+                    dst[3] = make_int4(flags, ns, c0, 0);
                     mbar_arrive(bar(kBDesc + i % kDescs));
                 }
                 __syncwarp();
@@ -496,10 +505,13 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 const unsigned win = at / each, unit = at - win * each, row = win / g.Mw, wc = win - row * g.Mw, wr = in < full ? row : p.rows;
                 const int eh = min(g.w, g.H - (int)wr * g.w), ew = min(g.w, g.W - (int)wc * g.w);
                 if (ST && (int)unit * p.tiles * kTileRows >= eh * strips_of(ew)) continue;            // a truncated window has fewer query tiles
-                put(1 | ((int)head != last_head ? 2 : 0), head, b, wr, wc, eh, ew, unit * p.tiles);
+                // (not where a pair of tiles would be of either part: one after the other, 288 x 544 tokens, 8 x 128, side 16, took 341 us; as one window 300)
+                int t0 = (int)wr != p.part_row ? 0 : part_tiles(p.part_ha, eh, (ST ? strips_of(ew) : 1) * RW);
+                if (t0 & (p.tiles - 1)) t0 = 0;
+                put(1 | ((int)head != last_head ? 2 : 0), head, b, wr, wc, eh, ew, unit * p.tiles, t0);
                 last_head = head;
             }
-            if (ok) put(0, 0, 0, 0, 0, 1, 1, 0);
+            if (ok) put(0, 0, 0, 0, 0, 1, 1, 0, 0);
         } else if (warp == kLoaderWarp) {
             // -------------------------------------------------------------- copies, bias tables, mask operands
             SlotQueue<L::kSlots> sq;
@@ -619,9 +631,9 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 q0 = sq.pop();
                 q1 = sq.pop();
                 fill(q0, kBFull, mq, p.q, td.tile0 * kTileRows);
-                for (int c = 0; ok && c < td.nch; ++c) {
+                for (int c = td.c0; ok && c < td.nch; ++c) {
                     fill(sq.take(), kBFull, mk, p.k, c * kTileRows);
-                    if (c == 0 && td.ntq == 2) fill(q1, kBFull, mq, p.q, (td.tile0 + 1) * kTileRows);
+                    if (c == td.c0 && td.ntq == 2) fill(q1, kBFull, mq, p.q, (td.tile0 + 1) * kTileRows);
                     fill(sq.take(), kBFullV, mv, p.v, c * kTileRows);
                 }
                 sq.end_unit(q0, q1);
@@ -654,10 +666,10 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             };
             while (ok && next_unit()) {
                 const int s_q[2] = {sq.pop(), sq.pop()};
-                for (int c = 0; ok && c < td.nch; ++c) {
+                for (int c = td.c0; ok && c < td.nch; ++c) {
                     const int sk = sq.take();
                     sq.take();                       // (V)
-                    if (c == 0) wait_full(s_q[0]);
+                    if (c == td.c0) wait_full(s_q[0]);
                     wait_full(sk);
                     for (int hf = 0; hf < 2 && 4 * c + 2 * hf < td.ku; ++hf) {
                         const int left = td.ku - (4 * c + 2 * hf);
@@ -666,7 +678,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                         for (int t = 0; t < 2; ++t) {
                             if (t >= td.ntq) break;
                             const unsigned buf = idx % NB;
-                            if (t == 1 && c == 0 && hf == 0) wait_full(s_q[1]);
+                            if (t == 1 && c == td.c0 && hf == 0) wait_full(s_q[1]);
                             ok = ok && mbar_wait_all(bar(kBFree + buf), ((idx / NB) & 1) ^ 1u, cta_abort);
                             if (!ok) break;
                             ++idx;
@@ -704,7 +716,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
             bool ok = true;
             while (ok && next_unit()) {
                 const int s_q[2] = {sq.pop(), sq.pop()};
-                for (int c = 0; ok && c < td.nch; ++c) {
+                for (int c = td.c0; ok && c < td.nch; ++c) {
                     sq.take();                       // (K)
                     const int sv = sq.take();
                     ok = mbar_wait_all(bar(kBFullV + sv), (full_use >> sv) & 1, cta_abort);
@@ -715,7 +727,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                         for (int t = 0; t < 2; ++t) {
                             if (t >= td.ntq) break;
                             const unsigned buf = idx % NB;
-                            const bool first = c == 0 && hf == 0;
+                            const bool first = c == td.c0 && hf == 0;
                             ok = ok && mbar_wait_all(bar(kBP + buf), (idx / NB) & 1, cta_abort);
                             if (first) {
                                 ok = ok && mbar_wait_all(bar(kBOFree + t), (opened[t] & 1) ^ 1u, cta_abort);
@@ -833,6 +845,8 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
         p.units_row = (tiles_of(g.H - p.rows * g.w) + tiles - 1) / tiles;
         p.units = (long long)g.B * g.Mw * g.heads * ((long long)p.rows * p.units_win + (g.Mh - p.rows) * p.units_row);
     };
+    p.part_ha = !g.ph && g.sh > 0 ? (g.H - g.sh) % g.w : 0;
+    p.part_row = p.part_ha > 0 ? (g.H - g.sh) / g.w : -1;
     // One tile a unit has a unit's chain to itself: two thirds of a pair's time (32 x 64 tokens, 4 x 32, side 32: 27.7 -> 23.6 us a call).
     plan(1);
     if (p.units > sm_count) plan(2);
