@@ -1,5 +1,5 @@
-// One-pass backward on the tcgen05 tensor cores for window sides 9 .. 32 at head dim 128, 11 .. 32 at 64 and 17 .. 32 at
-// 32, any grid: P and dS of a (window, head) are computed once and feed dQ, dK, dV and dBias.
+// One-pass backward on the tcgen05 tensor cores for window sides 9 .. 128 at head dim 128, 11 .. 128 at 64 and 17 .. 128 at 32, any grid:
+// P and dS of a (window, head) are computed once and feed dQ, dK, dV and dBias.
 //
 // A persistent CTA takes (batch, window, head) units.  Per 128-key tile of a window it keeps K and V in shared memory and
 // streams Q and dO in half chunks of 64 query slots (slots: win_tiles.cuh).  TMEM lanes = keys, columns = queries:
@@ -11,6 +11,8 @@
 // dQ sums over the window's key tiles: in TMEM where it fits (head dim 32, windows of at most 256 slots), else in a slab of
 // fp32 that belongs to the CTA (one thread adds to one address, in key-tile order, so the sum has a fixed order).  Few
 // (window, head) units: a window's key tiles are split over 2, 4 or 8 CTAs with a slab each.
+// Sides above 32 (ST): window rows in strips of 32 slots (win_tiles.cuh), a strip taking the place of a row; bias and statistics from L2; gangs of
+// CTAs share a window (Params).  Of a window whose mask label changes between two tiles each part is a window (part_tiles).
 //
 // The elementwise warps read and write TMEM in the fragment layout of mma.m16n8 (tcgen05.ld.16x256b): a thread holds 4 key
 // rows x 8 query columns of every 32 x 32 block, at key offsets g + 8 m and query offsets 8 k + 2 t + e (g = lane / 4,
@@ -20,7 +22,7 @@
 // Measured, this kernel and what it needs around it against the kernels it replaces (dK / dV and dQ / dBias kernels that both
 // recomputed P and dS; the latter on mma.sync wherever a window was not a complete 32 x 32 one): 256 x 512 tokens, 12 x 64,
 // 32 x 32 windows 3.0 -> 2.1 ms; 255 x 540, the same 8.8 -> 2.2 ms; 288 x 544, 8 x 128, 16 x 16 windows 3.6 -> 1.1 ms; 64 x 128,
-// 32 x 32 windows 32.2 -> 23.9 ms.  It is bound by the elementwise warps' chain per half chunk (issue slots 36 %, tensor pipe 26 %, DRAM 14 %),
+// 32 x 32 windows 32.2 -> 23.2 ms; 256 x 640, 8 x 128, 128 x 128 windows 51 -> 32 ms; 111 x 398, 12 x 128, side 64 25.4 -> 4.2 ms.  It is bound by the elementwise warps' chain per half chunk (issue slots 36 %, tensor pipe 26 %, DRAM 14 %),
 // at head dim 128 with 32 x 32 windows by L2: 148 windows in flight restream their Q and dO and hold their dQ slabs, 1 MB each; on 96 x
 // 160 tokens 7.3 GB are read and 4.0 GB written for 0.9 GB of tensors, and 15 % of L2's sector reads hit.
 // dS^T leaves for shared memory by stmatrix in the layout the dQ product reads.
@@ -58,10 +60,15 @@ using namespace tc;
 constexpr int kThreads = 512;
 constexpr int kWorkWarps = 8, kReadWarp0 = 8, kProductWarp = 12, kLoaderWarp = 13, kScoreWarp = 14, kPlanWarp = 15;
 // Registers a thread: at launch, then of the elementwise, read-out and other warps.  The read-out's 64 accumulator values and addresses
-// need 120 (with 104 it spilled: 111 x 398 tokens, 12 x 128, side 64 5.1 ms, so 4.3; 288 x 544, 8 x 128, side 16 950 us, so 914).
-constexpr int kRegsLaunch = 128, kRegsWork = 160, kRegsRead = 120, kRegsOther = 72;
-static_assert(2 * kRegsWork + kRegsRead + kRegsOther <= 4 * kRegsLaunch, "register hand-over does not balance");
-static_assert(kRegsWork >= kRegsLaunch && kRegsRead <= kRegsLaunch && kRegsOther <= kRegsLaunch, "only the elementwise warps take registers");
+// need 120 at head dims 64 and 128 and with strips (with 104 it spilled: 111 x 398 tokens, 12 x 128, side 64 5.1 ms, so 4.3; 288 x 544, 8 x 128, side 16 950 us, so 914).
+// At head dim 32 the elementwise warps keep them (2 x 256 x 544, 13 heads, side 32: 3085 -> 3033).
+constexpr int kRegsLaunch = 128, kRegsOther = 72;
+template <int D, bool ST>
+struct Regs {
+    static constexpr int kWork = D == 32 && !ST ? 168 : 160, kRead = D == 32 && !ST ? 104 : 120;
+    static_assert(2 * kWork + kRead + kRegsOther <= 4 * kRegsLaunch, "register hand-over does not balance");
+    static_assert(kWork >= kRegsLaunch && kRead <= kRegsLaunch && kRegsOther <= kRegsLaunch, "only the elementwise warps take registers");
+};
 constexpr int kTile = 128, kHalf = 64;
 constexpr int kDescs = 8;                                                             // ring of tile descriptors
 constexpr int kScrLine = 160;                                                         // see flush_sums
@@ -447,7 +454,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         const int4* src = reinterpret_cast<const int4*>(smem + L::kOffDesc + i * 64);
         const int4 d0 = src[0], d1 = src[1], d2 = src[2];
         td.head = d0.x; td.b = d0.y; td.wr = d0.z; td.wc = d0.w;
-        td.eh = d1.x; td.ew = d1.y; td.kt = d1.z; td.nch = d1.w & 0xffff; td.q0 = L::kTwo ? d1.w >> 16 : 0;
+        td.eh = d1.x; td.ew = d1.y; td.kt = d1.z; td.nch = L::kTwo ? d1.w & 0xffff : d1.w; td.q0 = L::kTwo ? d1.w >> 16 : 0;
         td.ha = d2.x; td.hb = d2.y; td.flags = d2.z; td.slab = d2.w;
         if (ST) {
             const int4 d3 = src[3];
@@ -466,7 +473,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
 
     if (warp < kWorkWarps) {
         // ------------------------------------------------------------------ elementwise: the half chunks of buffer b
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kRegsWork));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(Regs<D, ST>::kWork));
         const int b = warp >> 2, wq = warp & 3, gl = lane >> 2, t = lane & 3;
         const float scale = g.scale_log2e;
         const uint32_t tq = tmem + ((uint32_t)(32 * wq) << 16);
@@ -596,7 +603,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         }
     } else if (warp < kProductWarp) {
         // ------------------------------------------------------------------ read-out
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kRegsRead));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(Regs<D, ST>::kRead));
         const int wq = warp & 3, row = 32 * wq + lane;          // TMEM lane
         const uint32_t tl = tmem + ((uint32_t)(32 * wq) << 16);
         const float out_scale = g.scale_log2e * kLn2;
@@ -833,7 +840,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 if (lane == 0) {
                     int4* dst = reinterpret_cast<int4*>(smem + L::kOffDesc + (i % kDescs) * 64);
                     dst[0] = make_int4(head, cur.b, cur.wr, cur.wc);
-                    dst[1] = make_int4(eh, ew, kt, nch | q0 << 16);
+                    dst[1] = make_int4(eh, ew, kt, L::kTwo ? nch | q0 << 16 : nch);
                     dst[2] = make_int4((!g.ph && g.sh > 0) ? g.H - g.sh - cur.wr * g.w : (1 << 20), (!g.pw && g.sw > 0) ? g.W - g.sw - cur.wc * g.w : (1 << 20), flags, slab);
                     if (ST) dst[3] = make_int4(strips_of(ew), seq, use, c0);
                     mbar_arrive(bar(kBDesc + i % kDescs));
@@ -1246,12 +1253,19 @@ swin_bwd_onepass_finish_kernel(const Geo g, const float* __restrict__ dbias_acc,
     const int slot0 = D == 128 ? 4 * cg : (cg / (D / 4)) * kTile + row;
     if (i >= per_item || slot0 >= nch * kTile) return;
     const int t0 = Lay<D, RW>::kTwo ? part_tiles((!g.ph && g.sh > 0) ? g.H - g.sh - wr * g.w : (1 << 20), eh, RW) : 0;
-    const int c_lo = t0 > 0 && slot0 >= t0 * kTile ? t0 : 0, c_hi = t0 > 0 && slot0 < t0 * kTile ? t0 : nch;
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = 0; s < (1 << split_log2); ++s) {
-        if (max((s * nch) >> split_log2, c_lo) >= min(((s + 1) * nch) >> split_log2, c_hi)) continue;       // none of its tiles meets the chunk
+    auto add = [&](int s) {
         const float4 t = __ldcg(slabs + ((item << split_log2) + s) * per_item + i);
         v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w;
+    };
+    if (t0 == 0) {
+        for (int s = 0; s < (1 << split_log2); ++s)
+            if (((s * nch) >> split_log2) != (((s + 1) * nch) >> split_log2)) add(s);
+    } else {
+        // two parts: the slabs of those whose tiles meet the chunk
+        const int c_lo = slot0 >= t0 * kTile ? t0 : 0, c_hi = slot0 < t0 * kTile ? t0 : nch;
+        for (int s = 0; s < (1 << split_log2); ++s)
+            if (max((s * nch) >> split_log2, c_lo) < min(((s + 1) * nch) >> split_log2, c_hi)) add(s);
     }
     const float f = g.scale_log2e * kLn2;
     const uint32_t lo = pack_elem(v.x * f, v.y * f), hi = pack_elem(v.z * f, v.w * f);
@@ -1459,9 +1473,16 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         unsigned grid = (unsigned)(p.units < ctas ? p.units : ctas);
         p.gangs = (int)grid;
         if (p.gang > 1) {
-            // a device with fewer SMs than planned for: fewer gangs, or a smaller one
-            if (p.gang > ctas) p.gang = ctas;
-            p.gangs = pl.gangs * p.gang <= ctas ? pl.gangs : ctas / p.gang;
+            // a device with fewer SMs than planned for: smaller gangs, then fewer; with several windows a gang its CTAs go after one another
+            p.gangs = pl.gangs;
+            if (p.gangs * p.gang > ctas) {
+                p.gang = ctas / p.gangs > 2 ? ctas / p.gangs : 2;
+                p.gangs = p.gangs < ctas / p.gang ? p.gangs : ctas / p.gang;
+            }
+            if (p.rotate && p.gangs < p.units) {
+                p.rotate = 0;
+                p.turn_log2 = D == 128 ? 2 : 1;
+            }
             grid = (unsigned)(p.gangs * p.gang);
             err = launch_together(kernel, grid, kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
         } else if (overlap) {

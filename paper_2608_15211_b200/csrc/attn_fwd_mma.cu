@@ -6,7 +6,7 @@
 // contiguous grid all happen here; nothing window-major is ever written to global memory.
 // The file is compiled for bf16 and, through attn_fwd_mma_f16.cu, for fp16 activations.
 // The first kernel covers every window class (truncated edges, the split latitude-wrap row, every side and head dim); what runs
-// there is sides 33 .. 128 that the tcgen05 kernels do not take.
+// there is the sides that fill little of the tcgen05 kernels' slots, the forward without a workspace and TERRA_REGISTER_PATH=1.
 #include "swin_common.cuh"
 #include "swin_kernels.h"
 

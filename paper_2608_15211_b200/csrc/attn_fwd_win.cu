@@ -1,4 +1,4 @@
-// Forward shifted-window attention on the tcgen05 tensor cores: window sides 9 .. 32 at head dims 64 and 128, 17 .. 32 at head dim 32 (less the
+// Forward shifted-window attention on the tcgen05 tensor cores: window sides 9 .. 128 at head dims 64 and 128, 17 .. 128 at head dim 32 (less the
 // sides that fwd_win_supported leaves to the register tiles), any grid.
 //
 // A unit is a pair of 128-row query tiles of one (sample, window, head), on small grids one tile; a persistent CTA per SM walks over units and streams
@@ -18,6 +18,10 @@
 // 32 x 32 windows, one in eight masked, 850 -> 1000 us.)  One body serves every window: the elementwise code is what bounds
 // the kernel, and two copies of it in one kernel run slower than one.
 // Scores and P share six TMEM buffers (head dim 128: four), so that the products of other half chunks run under the softmax.
+// Sides above 32 (ST): window rows in strips of 32 slots (win_tiles.cuh), a strip in the place of a row.  The bias table of a head (0.5 MB at side
+// 128) stays in L2: a thread has the 14 entries of its next half chunk in registers before it needs them (256 x 640 tokens, 8 x 128, side 128: 13.6
+// ms, with table rows staged in shared memory per 128 keys 14.4; 111 x 398, 12 x 128, side 64, on mma.sync 6.75, so 1.3 ms).  Of a window whose
+// mask label changes between two tiles each part is a window (part_tiles): 13.6 -> 10.6 ms at shift 64.
 //
 // What bounds it: the softmax warps' chain per half chunk, two warps a scheduler: 0.87 ms for 256 x 512 tokens, 12 x 64, 32 x 32 windows, of
 // which the exponentials need 0.35 (16 a clock and SM); issue slots 40 %, tensor pipe 22 %, DRAM 10 %.  Head dim 128: 7.1 ms for

@@ -92,7 +92,7 @@ cudaError_t read_tc_status(int* timed_out, cudaStream_t stream);
 bool tma_row_shape(const Geo& g);
 bool make_row_map(void* cu_tensor_map, const Geo& g, const void* base, int token_stride, int box_tokens, int box_ch = 32);
 
-// tcgen05 forward path for window sides 9 .. 32 (head dim 32: 17 .. 32) on any grid (attn_fwd_win.cu)
+// tcgen05 forward path for window sides 9 .. 128 (head dim 32: 17 .. 128) on any grid (attn_fwd_win.cu)
 bool fwd_win_supported(const Geo& g);
 size_t fwd_win_workspace_bytes(const Geo& g);
 cudaError_t launch_fwd_win(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
@@ -101,7 +101,7 @@ cudaError_t launch_fwd_win_f16(const Geo& g, const void* q, const void* k, const
                                int sm_count, cudaStream_t stream);
 cudaError_t read_fwd_win_status(int* timed_out);
 cudaError_t read_fwd_win_status_f16(int* timed_out);
-// One-pass tcgen05 backward for window sides 9 .. 32 at head dim 128, 11 .. 32 at 64 and 17 .. 32 at 32, any grid.
+// One-pass tcgen05 backward for window sides 9 .. 128 at head dim 128, 11 .. 128 at 64 and 17 .. 128 at 32, any grid.
 struct OnePassPlan {
     int rw;                  // slots per window row
     int npad, rmax;          // slots of a window rounded up to 128; window rows rounded up to whole key tiles
