@@ -110,6 +110,9 @@ struct Lay {
     static constexpr int kResident = D == 32 && !ST ? 2 : 0;                                 // windows of that many 128-query chunks keep dQ in TMEM
 };
 
+template <bool ST>
+using Maps = std::conditional_t<ST, WinStripMaps, WinMaps>;
+
 // barriers (8 bytes each)
 constexpr int kBFull = 0, kBEmpty = 16, kBSdp = 32, kBSFree = 34, kBDs = 36, kBPFree = 38, kBDq = 40, kBDqFree = 42, kBAcc = 44, kBAccFree = 45,
               kBDesc = 46, kBDescFree = kBDesc + kDescs, kBTab = kBDescFree + kDescs, kBTabFree = kBTab + 4, kBCount = kBTabFree + 4;
@@ -398,8 +401,8 @@ __device__ __forceinline__ void half_chunk(uint32_t t_s, uint32_t t_p, uint32_t 
 template <int D, int RW, int KIND, bool ST>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ dq, __nv_bfloat16* __restrict__ dk,
-                        __nv_bfloat16* __restrict__ dv, const __grid_constant__ WinMaps mq, const __grid_constant__ WinMaps mk,
-                        const __grid_constant__ WinMaps mv, const __grid_constant__ WinMaps mg) {
+                        __nv_bfloat16* __restrict__ dv, const __grid_constant__ Maps<ST> mq, const __grid_constant__ Maps<ST> mk,
+                        const __grid_constant__ Maps<ST> mv, const __grid_constant__ Maps<ST> mg) {
     using L = Lay<D, RW, ST>;
     constexpr int kParts = L::kParts, kRowB = L::kRowB, kG = kHalf / RW;
     constexpr bool kExchange = D == 32 && KIND == 0;
@@ -927,7 +930,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
             // lane -> channel part, window row of a tile or of the two half chunks
             const int part = lane % kParts, row = lane / kParts;
             // one slot; `two`: Q and dO of a half chunk (else the two 64-slot groups of a K or V tile); a0 = first window row
-            auto fill = [&](int s, const WinMaps& m0, const WinMaps& m1, const __nv_bfloat16* x0, const __nv_bfloat16* x1, int a0, bool two) {
+            auto fill = [&](int s, const Maps<ST>& m0, const Maps<ST>& m1, const __nv_bfloat16* x0, const __nv_bfloat16* x1, int a0, bool two) {
                 ok = mbar_wait_all(bar(kBEmpty + s), ((use >> s) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
                 use ^= 1u << s;
@@ -951,7 +954,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                     __syncwarp();
                 }
                 const uint32_t base = smem0 + s * L::kSlotB;
-                if (ST) {
+                if constexpr (ST) {
                     // 64 slots of a window row are one copy where the strips are even in number, a strip one where they are not
                     const bool whole = (td.ns & 1) == 0 && td.wc != p.cols.seam && td.wc < p.cols.first_wrapped && td.wc != p.cols.last;
                     if (lane == 0) {
@@ -964,7 +967,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                         const int second = whole ? row : row >> 1, r = whole ? 0 : row & 1;           // of two: the tensor, else the 64-slot group
                         const int u = a0 + r + (two ? 0 : 2 * second), a = unit_row(u, td.ns), st = u - a * td.ns;
                         const uint32_t dst = base + r * 32 * kRowB + (two ? second * kHalf * D * 2 + part * kHalf * kRowB : part * kTile * kRowB + second * kHalf * kRowB);
-                        const WinMaps& m = second ? m1 : m0;
+                        const Maps<ST>& m = second ? m1 : m0;
                         if (whole) {
                             int y = td.wr * g.w + a + g.sh;
                             if (y >= g.H) y -= g.H;
@@ -1406,13 +1409,21 @@ bool make_win_maps(WinMaps* m, const WinCols& c, const Geo& g, const void* base,
         const int cut = st ? c.n1 % 32 : c.n1;          // slots in front of the seam of the row or strip that it cuts
         if (cut > 0) ok = enc(&m->seam_a, g.W - c.n1, c.n1, 1, cut, 1);
         if (ok && cut > 0 && cut + c.skip < rw && ew > c.n1) ok = enc(&m->seam_b, 0, ew - c.n1, 1, rw - cut - c.skip, 1);
-        if (ok && st) ok = enc(&m->seam_fa, g.W - c.n1, c.n1, 1, rw, 1) && enc(&m->seam_fb, 0, ew - c.n1, 1, rw, 1);
     }
     if (ok && c.last >= 0) {
         const int col = c.last >= c.first_wrapped ? w0 + (c.last - c.first_wrapped) * g.w : c.last * g.w + g.sw;
         ok = enc(&m->last, col, g.W - c.last * g.w, 1, rw, 1);
     }
     return ok;
+}
+
+bool make_win_maps(WinStripMaps* m, const WinCols& c, const Geo& g, const void* base, int ts) {
+    std::memset(m, 0, sizeof *m);
+    if (!make_win_maps(static_cast<WinMaps*>(m), c, g, base, ts)) return false;
+    if (c.seam < 0) return true;
+    const int ew = g.W - c.seam * g.w < g.w ? g.W - c.seam * g.w : g.w, box_ch = g.d >= 64 ? 64 : 32;
+    const char* b = reinterpret_cast<const char*>(base);
+    return encode_win_map(&m->seam_fa, g, b + (size_t)(g.W - c.n1) * ts * 2, ts, c.n1, 1, box_ch, 32, 1) && encode_win_map(&m->seam_fb, g, b, ts, ew - c.n1, 1, box_ch, 32, 1);
 }
 #endif  // !TERRA_ELEM_F16
 
@@ -1425,7 +1436,7 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
     Params p;
     p.g = g;
-    WinMaps mq, mk, mv, mg;
+    Maps<ST> mq, mk, mv, mg;
     if (!make_win_cols(&p.cols, g) || !make_win_maps(&mq, p.cols, g, q, g.ts) || !make_win_maps(&mk, p.cols, g, k, g.ts) ||
         !make_win_maps(&mv, p.cols, g, v, g.ts) || !make_win_maps(&mg, p.cols, g, d_o, g.heads * g.d))
         return cudaErrorNotSupported;

@@ -116,6 +116,9 @@ struct Unit {
 // ST: rows of strips per row label among the mask operands, so that four strips in a row from any strip on lie in them
 __device__ __forceinline__ int e_rows(int ns) { return ns == 1 ? 4 : ns == 4 ? 1 : 2; }
 
+template <bool ST>
+using Maps = std::conditional_t<ST, WinStripMaps, WinMaps>;
+
 // FIFO of shared-memory slots: two held for a unit (Q tiles), the others cycle (K, V chunks)
 template <int N>
 struct SlotQueue {
@@ -201,7 +204,7 @@ __device__ __noinline__ void drop_forbidden(uint32_t t_s, int cols, int ak, int 
 template <int D, int RW, int KC, bool ST>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
-                    const __grid_constant__ WinMaps mq, const __grid_constant__ WinMaps mk, const __grid_constant__ WinMaps mv) {
+                    const __grid_constant__ Maps<ST> mq, const __grid_constant__ Maps<ST> mk, const __grid_constant__ Maps<ST> mv) {
     using L = Lay<D, RW, ST>;
     constexpr int kParts = L::kParts, kRowB = L::kRowB, kG = 64 / RW, NB = L::kBufs, kTileRows = kTile / RW;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -531,7 +534,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 for (int u = a0; u < a0 + 4; ++u) n += u - unit_row(u, td.ns) * td.ns == p.cols.n1 >> 5;
                 return n;
             };
-            auto fill = [&](int s, int full, const WinMaps& m, const __nv_bfloat16* src, int a0) {
+            auto fill = [&](int s, int full, const Maps<ST>& m, const __nv_bfloat16* src, int a0) {
                 ok = ok && mbar_wait_all(bar(kBEmpty + s), ((use >> s) & 1) ^ 1u, cta_abort);
                 if (!ok) return;
                 use ^= 1u << s;
@@ -550,7 +553,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                     __syncwarp();
                 }
                 const uint32_t base = smem0 + s * L::kSlotB;
-                if (ST) {
+                if constexpr (ST) {
                     // 64 slots of a window row are one copy where the strips are even in number, a strip one where they are not
                     const bool two = (td.ns & 1) == 0 && td.wc != p.cols.seam && td.wc < p.cols.first_wrapped && td.wc != p.cols.last;
                     if (lane == 0) mbar_arrive_expect_tx(bar(full + s), L::kSlotB - (fix ? cut_units(a0) * kRowB : 0));
@@ -834,7 +837,7 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
     using L = Lay<D, RW, ST>;
     Params p;
     p.g = g;
-    WinMaps mq, mk, mv;
+    Maps<ST> mq, mk, mv;
     if (!make_win_cols(&p.cols, g) || !make_win_maps(&mq, p.cols, g, q, g.ts) || !make_win_maps(&mk, p.cols, g, k, g.ts) || !make_win_maps(&mv, p.cols, g, v, g.ts))
         return cudaErrorNotSupported;
     p.q = (const __nv_bfloat16*)q; p.k = (const __nv_bfloat16*)k; p.v = (const __nv_bfloat16*)v;

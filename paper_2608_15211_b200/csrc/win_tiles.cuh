@@ -13,6 +13,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "swin_common.cuh"
 #include "tc_common.cuh"
 
@@ -24,9 +26,13 @@ struct WinMaps {
     CUtensorMap wrapped;     // columns behind the seam, one window row
     CUtensorMap seam_a;      // the column cut by the seam: its tokens in front of the seam ...
     CUtensorMap seam_b;      // ... and behind it, up to slot RW (ST: both of the strip that it cuts)
+    CUtensorMap last;        // a truncated last column (when the seam does not cut it)
+};
+
+// (apart: with them in every kernel's arguments, four tensors' maps leave the 4 KB that a launch passes at once, and a small call took 3 us longer)
+struct WinStripMaps : WinMaps {
     CUtensorMap seam_fa;     // ST: the whole strips in front of the seam ...
     CUtensorMap seam_fb;     // ... and behind it
-    CUtensorMap last;        // a truncated last column (when the seam does not cut it)
 };
 
 struct WinCols {
@@ -54,6 +60,7 @@ bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_
 // host (attn_bwd_onepass.cu): false if the driver's encoder is not available
 bool make_win_cols(WinCols* c, const Geo& g);
 bool make_win_maps(WinMaps* m, const WinCols& c, const Geo& g, const void* base, int token_stride);
+bool make_win_maps(WinStripMaps* m, const WinCols& c, const Geo& g, const void* base, int token_stride);
 
 // device: whether the `groups` 64-slot groups from window row `a0` on are one copy each (map `group`)
 template <int RW>
@@ -86,7 +93,7 @@ __device__ __forceinline__ void load_win_row(const WinMaps& m, const WinCols& c,
 
 // device, ST: strip `s` of window row `a` (32 slots; see load_win_row)
 template <int ROWB>
-__device__ __forceinline__ void load_win_strip(const WinMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
+__device__ __forceinline__ void load_win_strip(const WinStripMaps& m, const WinCols& c, uint32_t dst, const Geo& g, int b, int wr, int wc, int eh,
                                                int a, int s, int ch, uint32_t bar) {
     int u = wr * g.w + a + g.sh;
     if (u >= g.H) u -= g.H;
