@@ -1462,6 +1462,7 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     int block_heads = kStatHeads;
     const long long stat_chunks = (long long)g.B * g.Mh * g.Mw * (pl.npad / 64);
     while (block_heads > 1 && stat_chunks * ((g.heads + block_heads - 1) / block_heads) < 4 * kPlanSms) block_heads /= 2;
+    if (g.heads <= block_heads) block_heads = kStatHeads;               // (no more blocks by it)
     const unsigned stat = (unsigned)(stat_chunks * ((g.heads + block_heads - 1) / block_heads));
     const long long table = (long long)g.heads * 2 * pl.rmax * pl.rl;
     const unsigned tblocks = (unsigned)(table / 1024 + 1 < 592 ? table / 1024 + 1 : 592);
