@@ -1334,7 +1334,7 @@ static void plan_gangs(OnePassPlan& p, const Geo& g, long long items, int tiles)
     // from a window's first tile to its last one's end, over the time between two windows
     const int turn = p.gang < tiles ? p.gang : tiles;
     p.ring = p.rotate ? 1 : (int)std::ceil(((tiles + p.gang - 1) / p.gang + lag * turn) * p.gang / tiles) + 1;
-    p.flags = p.gangs * p.ring * ((p.npad / (g.d == 128 ? 64 : 128)) + 1) * 4;      // (more than the turns need)
+    p.flags = p.gang > 1 ? p.gangs * p.ring * ((p.npad / (g.d == 128 ? 64 : 128)) + 1) * 4 : 0;      // (more than the turns need; a gang of one takes none)
 }
 
 OnePassPlan bwd_onepass_plan(const Geo& g) {
@@ -1370,8 +1370,7 @@ OnePassPlan bwd_onepass_plan(const Geo& g) {
     const bool slab = p.split_log2 > 0 || g.d != 32 ? tiles > 1 : tiles > 2;
     p.bytes = p.off_slabs + (slab ? up(sizeof(float) * slabs * p.npad * g.d) : 0);
     p.off_flags = p.bytes;
-    if (p.gang > 1 && p.strips) p.bytes += up(sizeof(unsigned) * p.flags);
-    else if (p.gang > 1) p.off_flags = p.off_slabs + sizeof(float) * (size_t)p.gangs * p.ring * p.npad * g.d;      // behind the gangs' slabs (plan_gangs: they fit)
+    p.bytes += up(sizeof(unsigned) * p.flags);
     return p;
 }
 

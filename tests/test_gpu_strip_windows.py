@@ -58,3 +58,40 @@ def test_strips_under_capture():
     for i in range(3):
         assert torch.equal(grads[i], ref[i])
     assert (grads[3] - ref[3]).norm() <= 1e-5 * ref[3].norm()        # float atomics: 32-bit sums in another order
+
+
+# windows of one key tile, which no gang shares
+TIGHT = [(1, 4, 32, 8, 64, 64, 2, 7, 0, 1), (1, 1, 100, 3, 128, 64, 0, 32, 0, 1), (1, 4, 32, 2, 32, 33, 0, 0, 0, 1)]
+
+
+@pytest.mark.parametrize("case", TIGHT, ids=["_".join(map(str, c)) for c in TIGHT])
+def test_nothing_is_written_behind_the_workspace(case):
+    """Both calls with exactly the workspace they ask for, inside a larger buffer."""
+    cfg = small_config("strips", *case)
+    x = make_inputs(cfg)
+    xg = {k: v.cuda() for k, v in x.items()}
+    d = terra.make_desc(cfg)
+    need = [terra.terra_swin_workspace_bytes(d, backward) for backward in (False, True)]
+    guard = 1 << 20
+    buf = torch.full((2 * guard + max(need),), 0xA5, dtype=torch.uint8, device="cuda")
+
+    def workspace(n):
+        buf.fill_(0xA5)
+        return buf[guard:guard + n]
+
+    def untouched(n):
+        return bool((buf[:guard] == 0xA5).all()) and bool((buf[guard + n:] == 0xA5).all())
+
+    o, lse = terra.terra_swin_attn_fwd(d, xg["q"], xg["k"], xg["v"], xg["bias"], workspace=workspace(need[0]))
+    assert untouched(need[0])
+    got = terra.terra_swin_attn_bwd(d, xg["q"], xg["k"], xg["v"], xg["bias"], o, lse, xg["do"], workspace=workspace(need[1]))
+    assert untouched(need[1])
+    terra.terra_swin_check()
+    table = x["bias"].double().numpy()
+    ref_o, ref_lse = oracle.attn_fwd(cfg, x["q"], x["k"], x["v"], table)
+    ref = oracle.attn_bwd(cfg, x["q"], x["k"], x["v"], x["do"], table)
+    tok = oracle.selection_tokens(cfg, None)
+    gate("o", gpu_rows(o, cfg, tok), ref_o)
+    gate("lse", gpu_rows(lse, cfg, tok), ref_lse)
+    for i, name in enumerate(("dq", "dk", "dv", "dbias")):
+        gate(name, gpu_rows(got[i], cfg, tok) if i < 3 else got[i].cpu().double().numpy(), ref[i])

@@ -1,0 +1,27 @@
+"""The one-pass backward's plan over the sides and grids that it takes, on the CPU: what the kernels write into the workspace lies in it."""
+from tests._host_program import run_host_program
+
+SWEEP = """
+int main() {
+    const int heights[] = {1, 2, 3, 4, 5, 8, 16, 33, 64, 100, 128, 130, 260}, widths[] = {1, 20, 32, 33, 64, 96, 97, 128, 129, 700, 5000};
+    const int sides[] = {11, 16, 17, 32, 33, 34, 40, 64, 65, 96, 97, 128};
+    long long n = 0, bad = 0;
+    for (int B : {1, 3}) for (int H : heights) for (int W : widths) for (int heads : {1, 2, 3, 8, 12, 37, 64, 148}) for (int d : {32, 64, 128}) for (int w : sides) {
+        terra_swin_desc desc = {B, H, W, heads, d, w, 0, 0, 0, 1, 0.f, TERRA_DTYPE_BF16};
+        Geo g;
+        if (resolve_attention_geo(&desc, &g) != TERRA_OK || !bwd_onepass_supported(g)) continue;
+        const OnePassPlan p = bwd_onepass_plan(g);
+        ++n;
+        const bool flags = p.off_flags >= p.off_slabs && p.off_flags + 4 * (size_t)p.flags <= p.bytes;
+        if (!flags && bad++ < 10)
+            std::printf("B %d, %d x %d, %d x %d, side %d: gangs %d of %d, flags from %zu to %zu of %zu\\n", B, H, W, heads, d, w, p.gangs, p.gang,
+                        p.off_flags, p.off_flags + 4 * (size_t)p.flags, p.bytes);
+    }
+    std::printf("%lld plans, %lld bad\\n", n, bad);
+    return bad != 0 || n == 0;
+}
+"""
+
+
+def test_flags_lie_in_the_workspace(tmp_path):
+    run_host_program(tmp_path, SWEEP)
