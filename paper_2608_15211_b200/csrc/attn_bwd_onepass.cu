@@ -1366,8 +1366,8 @@ OnePassPlan bwd_onepass_plan(const Geo& g) {
     p.off_bias1 = p.off_bias0 + table;
     p.off_acc = p.off_bias1 + table;
     p.off_slabs = p.off_acc + table;
-    // a window whose dQ is complete after one key tile, or stays in TMEM, needs no slab
-    const bool slab = p.split_log2 > 0 || g.d != 32 ? tiles > 1 : tiles > 2;
+    // a window whose dQ is complete after one key tile, or stays in TMEM (head dim 32 without strips: Lay::kResident), needs no slab
+    const bool slab = p.split_log2 > 0 || g.d != 32 || p.strips ? tiles > 1 : tiles > 2;
     p.bytes = p.off_slabs + (slab ? up(sizeof(float) * slabs * p.npad * g.d) : 0);
     p.off_flags = p.bytes;
     p.bytes += up(sizeof(unsigned) * p.flags);

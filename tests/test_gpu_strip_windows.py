@@ -60,8 +60,9 @@ def test_strips_under_capture():
     assert (grads[3] - ref[3]).norm() <= 1e-5 * ref[3].norm()        # float atomics: 32-bit sums in another order
 
 
-# windows of one key tile, which no gang shares
-TIGHT = [(1, 4, 32, 8, 64, 64, 2, 7, 0, 1), (1, 1, 100, 3, 128, 64, 0, 32, 0, 1), (1, 4, 32, 2, 32, 33, 0, 0, 0, 1)]
+# windows of one key tile, which no gang shares, and of two (head dim 32: with a slab, unlike below side 33), with fewer and more windows than gangs
+TIGHT = [(1, 4, 32, 8, 64, 64, 2, 7, 0, 1), (1, 1, 100, 3, 128, 64, 0, 32, 0, 1), (1, 4, 32, 2, 32, 33, 0, 0, 0, 1),
+         (1, 4, 64, 2, 32, 64, 2, 32, 0, 1), (1, 8, 30, 3, 32, 48, 4, 0, 0, 1), (1, 4, 5000, 12, 32, 64, 2, 32, 0, 1)]
 
 
 @pytest.mark.parametrize("case", TIGHT, ids=["_".join(map(str, c)) for c in TIGHT])

@@ -12,10 +12,15 @@ int main() {
         if (resolve_attention_geo(&desc, &g) != TERRA_OK || !bwd_onepass_supported(g)) continue;
         const OnePassPlan p = bwd_onepass_plan(g);
         ++n;
+        // dQ slabs: of every unit where windows are split, of every gang's ring, else of the CTAs of the launches that may run at the same time
+        const int tiles = p.npad / 128;
+        const bool uses = tiles > (d == 32 && !p.strips && p.split_log2 == 0 ? 2 : 1);
+        const long long ctas = std::min<long long>(p.units, (d == 128 || p.strips ? 1 : 2) * kMaxCtas);
+        const size_t slabs = !uses ? 0 : p.split_log2 ? p.units : p.gang > 1 ? (long long)p.gangs * p.ring : ctas, end = p.off_slabs + 4 * slabs * p.npad * d;
         const bool flags = p.off_flags >= p.off_slabs && p.off_flags + 4 * (size_t)p.flags <= p.bytes;
-        if (!flags && bad++ < 10)
-            std::printf("B %d, %d x %d, %d x %d, side %d: gangs %d of %d, flags from %zu to %zu of %zu\\n", B, H, W, heads, d, w, p.gangs, p.gang,
-                        p.off_flags, p.off_flags + 4 * (size_t)p.flags, p.bytes);
+        if ((!flags || end > (p.flags ? p.off_flags : p.bytes)) && bad++ < 10)
+            std::printf("B %d, %d x %d, %d x %d, side %d: gangs %d of %d, slabs from %zu to %zu, flags from %zu to %zu of %zu\\n", B, H, W, heads, d, w, p.gangs, p.gang,
+                        p.off_slabs, end, p.off_flags, p.off_flags + 4 * (size_t)p.flags, p.bytes);
     }
     std::printf("%lld plans, %lld bad\\n", n, bad);
     return bad != 0 || n == 0;
@@ -23,5 +28,5 @@ int main() {
 """
 
 
-def test_flags_lie_in_the_workspace(tmp_path):
+def test_slabs_and_flags_lie_in_the_workspace(tmp_path):
     run_host_program(tmp_path, SWEEP)
