@@ -125,7 +125,7 @@ __device__ __forceinline__ void scatter_rows(const unsigned char* tile, __nv_bfl
 // KV = false: CTA owns 64 queries (own tiles Q, dO; streams K, V) -> dQ, dBias
 constexpr int kStageStride = 40;   // floats per row of the dS staging tile (32 columns used)
 
-// BIG = windows of more than 1024 tokens (window sides 33 .. 128): the slot tables cover the CTA's own 64 rows plus
+// BIG = window sides 33 .. 128: the slot tables cover the CTA's own 64 rows plus
 // the streamed block in flight (two stages) instead of the whole window, the bias is read from the caller's table in
 // global memory, and the bias gradient goes to global memory with atomics (summed over diagonals first where the
 // window is complete along its width).
@@ -732,11 +732,12 @@ swin_bwd_delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* 
     if (row < rows && chunk == 0) delta[row] = acc;
 }
 
-// Row stride (floats) of the summed-dS image, or 0 when the window is too large for it.  The stride is
+// Row stride (floats) of the summed-dS image, or 0 when the window is too large for it, or the side (the image is binned into the
+// bias gradient's table in shared memory, which sides above 32 have not, however few rows the grid has).  The stride is
 // 8 mod 32 so that the 16 lanes of one 8-byte access wave hit 32 different banks.
 int acc_stride_for(const Geo& g) {
     int npad_max = ((g.nmax + BN - 1) / BN) * BN;
-    return npad_max <= 256 ? npad_max + 8 : 0;
+    return g.w <= 32 && npad_max <= 256 ? npad_max + 8 : 0;
 }
 
 size_t bwd_smem_bytes(const Geo& g, bool query_side) {
