@@ -1299,7 +1299,16 @@ cudaError_t read_bwd_onepass_status(int* timed_out) {
 }
 
 #ifndef TERRA_ELEM_F16
+// Bias-table rows run from -table_rmax to table_rmax - 1 and are table_rl floats long.
+static int table_rmax(const Geo& g) {
+    const int kr = kTile / win_row_slots(g);
+    return win_strips(g) ? g.w + 4 : (g.w + kr - 1) / kr * kr;      // (strips: the last key tile's rows reach up to 3 past the window's)
+}
+static int table_rl(const Geo& g) { return win_strips(g) ? 64 * strips_of(g.w) : 2 * win_row_slots(g); }
+
 bool bwd_onepass_supported(const Geo& g) {
+    // entries of the bias tables are numbered in 32 bits, with room for a loop that steps past the last (side 128: 31759 heads)
+    if ((long long)g.heads * 2 * table_rmax(g) * table_rl(g) > 0x7ff00000LL) return false;
     // (head dim 32 with sides up to 16 has a kernel of its own, 1.83 against 2.5 ms on the 510 x 1080 grid with 12 heads)
     // Register tiles / this kernel, us, on 240 x 360, 2 x 121 x 250 and 96 x 180 tokens: head dim 64, side 9 676/752 659/719 166/166, 10 572/626 560/601
     // 146/140; 11 517/537 480/496 140/126 (level), 12 1032/451; head dim 128, side 9 889/800 1215/1130 289/263; head dim 32, side 17 948/967
@@ -1340,12 +1349,12 @@ static void plan_gangs(OnePassPlan& p, const Geo& g, long long items, int tiles)
 OnePassPlan bwd_onepass_plan(const Geo& g) {
     OnePassPlan p;
     p.rw = win_row_slots(g);
-    const int kr = kTile / p.rw, rows = g.w < g.H ? g.w : g.H;
+    const int rows = g.w < g.H ? g.w : g.H;
     p.strips = win_strips(g) ? strips_of(g.w) : 0;
     const int tiles = (rows * (p.strips ? strips_of(g.w < g.W ? g.w : g.W) : 1) * p.rw + kTile - 1) / kTile;
     p.npad = tiles * kTile;
-    p.rl = p.strips ? 64 * p.strips : 2 * p.rw;
-    p.rmax = p.strips ? g.w + 4 : (g.w + kr - 1) / kr * kr;      // (the last key tile's rows reach up to 3 past the window's)
+    p.rl = table_rl(g);
+    p.rmax = table_rmax(g);
     // Units per window: as many as keep the SMs busy.  The time of a launch is the number of unit rounds x key tiles per
     // unit; splitting costs a sum over slabs, so it has to save an eighth of that time.
     const long long items = (long long)g.B * g.Mh * g.Mw * g.heads;

@@ -1,4 +1,6 @@
 """The one-pass backward's plan over the sides and grids that it takes, on the CPU: what the kernels write into the workspace lies in it."""
+import paper_2608_15211_b200 as terra
+from paper_2608_15211_b200.workloads import small_config
 from tests._host_program import run_host_program
 
 SWEEP = """
@@ -30,3 +32,14 @@ int main() {
 
 def test_slabs_and_flags_lie_in_the_workspace(tmp_path):
     run_host_program(tmp_path, SWEEP)
+
+
+def test_more_heads_than_the_tables_entries_can_be_numbered_for():
+    """Head counts behind which 32 bits do not number the entries of the one-pass backward's bias tables take the register tiles, whose workspace
+    is a float per token and head."""
+    for window, per_head in ((128, 2 * 132 * 256), (33, 2 * 37 * 128), (32, 2 * 32 * 64)):
+        most = (2**31 - 2**20) // per_head
+        for heads, tables in ((most, True), (most + 1, False), (2 * most, False)):
+            desc = terra.make_desc(small_config("heads", 1, 1, 2, heads, 128, window, 0, 0))
+            need, delta = terra.terra_swin_workspace_bytes(desc, True), 4 * 2 * heads
+            assert need > 3 * 4 * per_head * heads if tables else delta <= need < delta + 256
