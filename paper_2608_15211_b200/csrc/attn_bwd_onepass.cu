@@ -1313,7 +1313,14 @@ bool bwd_onepass_supported(const Geo& g) {
     // Register tiles / this kernel, us, on 240 x 360, 2 x 121 x 250 and 96 x 180 tokens: head dim 64, side 9 676/752 659/719 166/166, 10 572/626 560/601
     // 146/140; 11 517/537 480/496 140/126 (level), 12 1032/451; head dim 128, side 9 889/800 1215/1130 289/263; head dim 32, side 17 948/967
     // 1798/1711 389/406 (level), 18 1126/816 2278/1496 468/384.
-    if (win_strips(g)) return g.w <= kMaxWinW && (long long)g.B * g.H * g.W < 0x7fffffffLL && (long long)g.B * g.Mh * g.Mw * g.heads * 128 < 0x7fffffffLL;
+    // Strips: where the windows' work in them (strip_work) is at most 10, 9 and 7 times the dense one at head dims 32, 64 and 128: all but windows of
+    // few columns.  Register tiles / strips, us: 240 x 360, 6 x 32, side 33 7573/2785; 200 x 64 x 1, 6 x 32, side 64 220/8166; 8 x 128 x 4, 12 x 128, side 64
+    // 400/2952; 200 x 8 x 8, 4 x 128, side 40 159/374.  On 1662 shapes strips alone were more than 5 % slower on 243, the rule is wrong on 45.
+    if (win_strips(g)) {
+        const StripWork x = strip_work(g);
+        if (x.strips > (g.d == 32 ? 10 : g.d == 64 ? 9 : 7) * x.dense) return false;
+        return g.w <= kMaxWinW && (long long)g.B * g.H * g.W < 0x7fffffffLL && (long long)g.B * g.Mh * g.Mw * g.heads * 128 < 0x7fffffffLL;
+    }
     return ((g.d == 64 && g.w > 10) || g.d == 128 || (g.d == 32 && g.w > 16)) && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 8 < 0x7fffffffLL;
 }

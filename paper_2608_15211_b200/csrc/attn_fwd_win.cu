@@ -817,8 +817,18 @@ bool fwd_win_supported(const Geo& g) {
     //   above 24 work on all 32 slots of a row: 25 353/430 705/837 154/201, 26 392/402 736/830 164/169; 27 436/386 810/816 175/181, 28 463/342;
     //   head dim 64, side 9 226/318 212/349 52/80, 11 166/238 156/246 39/56; 12 267/183 248/214 60/46; 17 338/468 318/426 72/95; 18 416/358 379/368 95/84;
     //   head dim 128, this kernel at every side: 9 283/261 392/369 91/95, 10 242/238 338/328 74/82, 11 207/171 287/269 68/64, 17 400/346 558/486 123/118.
-    if (win_strips(g))
+    // Strips: where the windows' work in them (strip_work) is at most 2.8 times the dense one at head dim 32, 6 times at 64 and 128, and the largest
+    // window has more than 5, 4 and 2 blocks of 64 tokens (below, the two launches and a 128-slot tile's chain cost more than the register
+    // tiles take in all).  Register tiles / strips, us, 6 x 32 channels: side 33 1020/1408 686/1019 216/306, 36 1183/1359 795/902 242/265, 38 1240/1388
+    // 856/953 248/249, 40 1410/1304 966/1078 258/238, 44 1677/1394 1124/871 364/286; 6 x 64: side 33 1360/1260 916/931 287/296, 36 1584/1178 1066/849 324/247;
+    // 4 x 128: side 33 1463/999 983/726 306/247.  Side 64 on narrow and low grids: 200 x 64 x 1, 6 x 32 23/3868; 200 x 8 x 8, 6 x 64 29/86.  On 1662
+    // shapes of sides 33 .. 128 strips alone were more than 5 % slower on 574, by the rule the wrong one of the two is taken on 92.
+    if (win_strips(g)) {
+        const StripWork x = strip_work(g);
+        const int blocks = (g.nmax + 63) / 64;
+        if (g.d == 32 ? blocks <= 5 || 10 * x.strips > 28 * x.dense : blocks <= (g.d == 64 ? 4 : 2) || x.strips > 6 * x.dense) return false;
         return g.w <= kMaxWinW && (long long)g.B * g.H * g.W < 0x7fffffffLL && (long long)g.B * g.Mh * g.Mw * g.heads * 64 < 0x7fffffffLL;
+    }
     const bool sparse = g.d == 32 ? g.w <= 22 || g.w == 25 || g.w == 26 : g.d == 64 && (g.w <= 11 || g.w == 17);
     return (g.d == 64 || g.d == 128 || (g.d == 32 && g.w > 16)) && !sparse && g.w > 8 && g.w <= kMaxOnePassW && (long long)g.B * g.H * g.W < 0x7fffffffLL &&
            (long long)g.B * g.Mh * g.Mw * g.heads * 4 < 0x7fffffffLL;

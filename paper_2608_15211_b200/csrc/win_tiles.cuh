@@ -55,6 +55,22 @@ __device__ __forceinline__ int unit_row(int u, int ns) {
     return (int)(((unsigned)u * inv) >> 16);
 }
 
+// host: what the windows of a (sample, head) hold in blocks of 64 x 64 pairs, as register tiles count them (`dense`) and in strips (`strips`: 64
+// keys x 128 queries are two, and a 128-slot tile costs four of its own)
+struct StripWork { long long dense, strips; };
+inline StripWork strip_work(const Geo& g) {
+    StripWork x = {0, 0};
+    const int rows[2] = {g.H / g.w, g.H % g.w ? 1 : 0}, cols[2] = {g.W / g.w, g.W % g.w ? 1 : 0};
+    for (int i = 0; i < 2; ++i)
+        for (int j = 0; j < 2; ++j) {
+            const long long eh = i ? g.H % g.w : g.w, ew = j ? g.W % g.w : g.w, n = (long long)rows[i] * cols[j];
+            const long long blocks = (eh * ew + 63) / 64, units = eh * ((ew + 31) / 32), tiles = (units + 3) / 4;
+            x.dense += n * blocks * blocks;
+            x.strips += n * 2 * tiles * ((units + 1) / 2 + 2);
+        }
+    return x;
+}
+
 // host (attn_fwd_tc.cu, beside the driver's encoder)
 bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_stride, int nb, int ncols, int box_ch, int box_b, int box_rows);
 // host (attn_bwd_onepass.cu): false if the driver's encoder is not available

@@ -16,6 +16,8 @@ CASES = [
     (1, 33, 33, 1, 64, 33, 0, 0, 1, 1), (1, 40, 70, 2, 32, 33, 5, 16, 0, 1), (2, 64, 64, 1, 128, 64, 20, 32, 0, 0), (1, 70, 90, 1, 32, 65, 31, 25, 0, 1),
     (1, 96, 100, 1, 64, 96, 50, 33, 0, 0), (1, 45, 230, 1, 128, 100, 3, 65, 1, 1), (1, 128, 30, 1, 64, 128, 64, 7, 0, 0), (1, 3, 128, 2, 32, 128, 1, 64, 0, 1),
     (3, 35, 140, 7, 64, 40, 20, 20, 0, 1), (1, 130, 66, 3, 128, 64, 32, 16, 0, 1), (1, 34, 1, 1, 128, 128, 0, 0, 0, 1),
+    # on the register tiles, forward or in both directions: windows that fill little of their strips
+    (1, 68, 70, 2, 32, 34, 17, 9, 0, 1), (3, 64, 3, 2, 64, 64, 20, 1, 0, 1), (2, 8, 8, 1, 128, 40, 4, 0, 1, 0), (1, 5, 60, 2, 32, 64, 2, 7, 0, 0),
 ]
 
 
