@@ -149,9 +149,12 @@ static bool force_register_path() {
 static bool small_windows(const Geo& g) { return g.w <= 8; }
 
 // (every kernel exists for bf16 and for fp16 activations: `f16` only selects the build of the kernel)
-static bool use_fwd_tc(const Geo& g) { return fwd_tc_supported(g) && !small_windows(g); }
+// Forward: windows of at most 64 tokens, whatever the side, are one block of the register tiles, as terra_swin_attn_fwd_noalloc has it, which
+// promises the same bits.  Register tiles / tcgen05 kernels, us: 4 x 16 tokens, 6 x 32, side 16 10/17, 3 x 7000 33/56, 200 x 8 x 8, side 24 21/77; 6 x 64,
+// 2 x 2000, side 32 16/24, 3 x 7000, side 16 45/91; 4 x 128, 3 x 7000, side 20 47/62, 200 x 8 x 8, side 16 31/42.  (138 such shapes, 1.3 to 4.2 times.)
+static bool use_fwd_tc(const Geo& g) { return fwd_tc_supported(g) && g.nmax > 64; }
 
-static bool use_fwd_win(const Geo& g) { return fwd_win_supported(g) && !force_register_path() && !small_windows(g); }
+static bool use_fwd_win(const Geo& g) { return fwd_win_supported(g) && !force_register_path() && g.nmax > 64; }
 
 static size_t fwd_bytes(const Geo& g) {
     if (force_register_path()) return 0;

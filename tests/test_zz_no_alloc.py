@@ -76,3 +76,16 @@ def test_noalloc_forward_on_a_shape_without_scratch_and_its_limit():
     with pytest.raises(terra.TerraError) as e:
         terra.terra_swin_attn_fwd_noalloc(d, x["q"], x["k"], x["v"], x["bias"], o, lse)
     assert e.value.status == 7
+
+
+@pytest.mark.parametrize("case", [(1, 4, 16, 3, 32, 16, 2, 8), (2, 6, 10, 2, 32, 24, 3, 5), (1, 2, 70, 2, 64, 32, 1, 16), (3, 8, 8, 2, 64, 12, 0, 6), (1, 5, 12, 2, 128, 20, 2, 7),
+                                  (2, 8, 8, 1, 128, 40, 4, 4)], ids=lambda c: "_".join(map(str, c)))
+def test_windows_of_at_most_64_tokens_are_bit_equal_whatever_the_side(case):
+    cfg = small_config("na5", *case)
+    x = {k: v.cuda() for k, v in make_inputs(cfg, extra=4).items()}
+    d = terra.make_desc(cfg)
+    o_ref, lse_ref = terra.terra_swin_attn_fwd(d, x["q"], x["k"], x["v"], x["bias"])
+    o, lse = torch.full_like(o_ref, float("nan")), torch.full_like(lse_ref, float("nan"))
+    _call_noalloc(d, x, o, lse)
+    assert torch.equal(o, o_ref)
+    assert torch.equal(lse, lse_ref)
