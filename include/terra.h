@@ -121,6 +121,9 @@ int terra_swin_attn_fwd(const terra_swin_desc* desc, const void* q, const void* 
  *                                                       with window <= 16; with atomics, hence in no fixed
  *                                                       order, for the other shapes)
  *   workspace         >= terra_swin_workspace_bytes(desc, 1) bytes
+ * Sides above 32 are worked on by CTAs that add to one sum in turn, in a cooperative launch of up to one CTA per SM.  On a
+ * stream or in a process that may use a part of the SMs only there are fewer of them; dq, dk and dv are then sums in
+ * another (still fixed) order.
  */
 int terra_swin_attn_bwd(const terra_swin_desc* desc, const void* q, const void* k, const void* v,
                         const float* bias_table, const void* o, const float* lse, const void* d_o,

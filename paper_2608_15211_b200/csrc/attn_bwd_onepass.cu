@@ -1353,6 +1353,39 @@ static void plan_gangs(OnePassPlan& p, const Geo& g, long long items, int tiles)
     p.flags = p.gang > 1 ? p.gangs * p.ring * ((p.npad / (g.d == 128 ? 64 : 128)) + 1) * 4 : 0;      // (more than the turns need; a gang of one takes none)
 }
 
+// The plan's gangs on `ctas` CTAs at a time: smaller gangs, then fewer; with several windows a gang its CTAs go after one another.  On one CTA the
+// windows have it in turn, with a slab of the first gang's.
+GangShape fit_gangs(const OnePassPlan& p, long long units, int ctas) {
+    GangShape s = {p.gangs, p.gang, p.rotate};
+    if (s.gangs * s.gang > ctas) {
+        s.gang = ctas / s.gangs > 2 ? ctas / s.gangs : ctas < 2 ? 1 : 2;
+        s.gangs = s.gangs < ctas / s.gang ? s.gangs : ctas / s.gang;
+    }
+    if (s.gangs < units || s.gang == 1) s.rotate = 0;
+    return s;
+}
+
+// SMs that a launch in `stream` may use: a green context's stream has a part of the device.
+int sms_of_stream(cudaStream_t stream, int device_sms) {
+    using GreenOfStream = CUresult (*)(CUstream, CUgreenCtx*);
+    using ResourceOfGreen = CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+    struct Entries { GreenOfStream green; ResourceOfGreen resource; };
+    static const Entries e = [] {
+        Entries x = {nullptr, nullptr};
+        void *a = nullptr, *b = nullptr;
+        cudaDriverEntryPointQueryResult qa, qb;
+        if (cudaGetDriverEntryPoint("cuStreamGetGreenCtx", &a, cudaEnableDefault, &qa) == cudaSuccess && qa == cudaDriverEntryPointSuccess &&
+            cudaGetDriverEntryPoint("cuGreenCtxGetDevResource", &b, cudaEnableDefault, &qb) == cudaSuccess && qb == cudaDriverEntryPointSuccess)
+            x = {reinterpret_cast<GreenOfStream>(a), reinterpret_cast<ResourceOfGreen>(b)};
+        return x;
+    }();
+    CUgreenCtx ctx = nullptr;
+    CUdevResource r;
+    if (!e.green || e.green(stream, &ctx) != CUDA_SUCCESS || !ctx || e.resource(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS) return device_sms;
+    const int sms = (int)r.sm.smCount;
+    return sms < 1 || sms > device_sms ? device_sms : sms;
+}
+
 OnePassPlan bwd_onepass_plan(const Geo& g) {
     OnePassPlan p;
     p.rw = win_row_slots(g);
@@ -1465,7 +1498,7 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
     p.gang = pl.gang;
     p.ring = pl.ring;
     p.rotate = pl.rotate;
-    p.turn_log2 = (D == 128 ? 2 : 1) - pl.rotate;      // 256 queries (rotate: 128)
+    p.turn_log2 = 0;
     p.events = pl.npad / (D == 128 ? 64 : 128);
     p.flags = reinterpret_cast<unsigned*>(ws + pl.off_flags);
     p.rowstat = reinterpret_cast<const float4*>(ws);
@@ -1500,18 +1533,19 @@ cudaError_t launch_onepass(const Geo& g, const OnePassPlan& pl, const void* q, c
         unsigned grid = (unsigned)(p.units < ctas ? p.units : ctas);
         p.gangs = (int)grid;
         if (p.gang > 1) {
-            // a device with fewer SMs than planned for: smaller gangs, then fewer; with several windows a gang its CTAs go after one another
-            p.gangs = pl.gangs;
-            if (p.gangs * p.gang > ctas) {
-                p.gang = ctas / p.gangs > 2 ? ctas / p.gangs : 2;
-                p.gangs = p.gangs < ctas / p.gang ? p.gangs : ctas / p.gang;
+            // as many CTAs as can be on the device together, or on the part of it that the stream or the process may use: a partition that
+            // the query does not see refuses the launch
+            for (int most = sms_of_stream(stream, ctas);; most = (int)grid / 2) {
+                const GangShape fit = fit_gangs(pl, p.units, most);
+                p.gangs = fit.gangs;
+                p.gang = fit.gang;
+                p.rotate = fit.rotate;
+                p.turn_log2 = (D == 128 ? 2 : 1) - p.rotate;      // 256 queries (rotate: 128)
+                grid = (unsigned)(p.gangs * p.gang);
+                err = launch_together(kernel, grid, kThreads, L::kSmemBytes, stream, p.gang > 1, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
+                if (err != cudaErrorCooperativeLaunchTooLarge) break;
+                cudaGetLastError();
             }
-            if (p.rotate && p.gangs < p.units) {
-                p.rotate = 0;
-                p.turn_log2 = D == 128 ? 2 : 1;
-            }
-            grid = (unsigned)(p.gangs * p.gang);
-            err = launch_together(kernel, grid, kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);
         } else if (overlap) {
             // needs nothing of the launch before it: its CTAs take the SMs as that one's leave them
             err = launch_dependent(kernel, grid, kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)dq, (__nv_bfloat16*)dk, (__nv_bfloat16*)dv, mq, mk, mv, mg);

@@ -31,12 +31,12 @@ cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-// Launches `kernel` only when all its CTAs can be on the device together: they wait for one another.
+// Launches `kernel`, where its CTAs wait for one another (`together`) only if all can be on the device at the same time.
 template <typename... P, typename... A>
-cudaError_t launch_together(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, A&&... args) {
+cudaError_t launch_together(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, bool together, A&&... args) {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeCooperative;
-    attr.val.cooperative = 1;
+    attr.val.cooperative = together;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
@@ -118,6 +118,9 @@ constexpr int kGangMin = 4;            // CTAs of a gang at least
 constexpr double kGangLag = 5.5;       // half chunks from a CTA's turn to the next one's
 bool bwd_onepass_supported(const Geo& g);
 OnePassPlan bwd_onepass_plan(const Geo& g);
+struct GangShape { int gangs, gang, rotate; };
+GangShape fit_gangs(const OnePassPlan& p, long long units, int ctas);
+int sms_of_stream(cudaStream_t stream, int device_sms);
 cudaError_t launch_bwd_onepass(const Geo& g, const void* q, const void* k, const void* v, const float* bias, const void* o, const float* lse,
                                const void* d_o, void* dq, void* dk, void* dv, float* dbias, void* workspace, int sm_count, cudaStream_t stream);
 cudaError_t launch_bwd_onepass_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias, const void* o, const float* lse,

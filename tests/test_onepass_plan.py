@@ -23,6 +23,14 @@ int main() {
         if ((!flags || end > (p.flags ? p.off_flags : p.bytes)) && bad++ < 10)
             std::printf("B %d, %d x %d, %d x %d, side %d: gangs %d of %d, slabs from %zu to %zu, flags from %zu to %zu of %zu\\n", B, H, W, heads, d, w, p.gangs, p.gang,
                         p.off_slabs, end, p.off_flags, p.off_flags + 4 * (size_t)p.flags, p.bytes);
+        // on fewer SMs: CTAs that fit, slabs and flags of the plan, and CTAs that start at different chunks only where no gang has a second window
+        for (int ctas : {1, 2, 3, 8, 16, 37, 72, 100, 147, 148, 160}) {
+            if (p.gang < 2) break;
+            const GangShape s = fit_gangs(p, p.units, ctas);
+            const bool fits = s.gangs >= 1 && s.gang >= 1 && s.gangs * s.gang <= ctas && s.gangs <= p.gangs && s.gang <= p.gang && (!s.rotate || s.gangs >= p.units) &&
+                              (s.gang > 1 || ctas == 1) && (ctas < p.gangs * p.gang || (s.gangs == p.gangs && s.gang == p.gang && s.rotate == p.rotate));
+            if (!fits && bad++ < 10) std::printf("%d CTAs for %d gangs of %d: %d of %d\\n", ctas, p.gangs, p.gang, s.gangs, s.gang);
+        }
     }
     std::printf("%lld plans, %lld bad\\n", n, bad);
     return bad != 0 || n == 0;
