@@ -201,7 +201,9 @@ __device__ __noinline__ void drop_forbidden(uint32_t t_s, int cols, int ak, int 
 
 // KC: of every 32 key slots the first 8 KC are worked on (window sides 17 .. 24 in rows of 32 slots leave the last 8 without a
 // token: 3; otherwise 4).  240 x 360 tokens, 6 x 64, side 22: 357 -> 302 us.
-template <int D, int RW, int KC, bool ST>
+// TWO: windows of two parts (part_tiles) as such.  Of its own below side 33: the code for it cost grids without such windows 1 to 5 % (108 x 230 tokens,
+// 30 x 128, side 9 685 us, so 648; 2 x 299 x 796, 2 x 64, side 13 333, so 327; 2 x 299 x 796, 2 x 128, side 12 499, so 479).
+template <int D, int RW, int KC, bool ST, bool TWO>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict__ o, float* __restrict__ lse,
                     const __grid_constant__ Maps<ST> mq, const __grid_constant__ Maps<ST> mk, const __grid_constant__ Maps<ST> mv) {
@@ -262,7 +264,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
         td.eh = d1.x; td.ew = d1.y; td.tile0 = d1.z; td.ntq = d1.w;
         td.ku = d2.x; td.nch = d2.y; td.ha = d2.z; td.hb = d2.w;
         const int4 d3 = src[3];
-        td.flags = d3.x; td.c0 = d3.z;
+        td.flags = d3.x; td.c0 = TWO ? d3.z : 0;
         if (ST) td.ns = d3.y;
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kBDescFree + i));
@@ -513,7 +515,7 @@ swin_fwd_win_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restrict_
                 const int eh = min(g.w, g.H - (int)wr * g.w), ew = min(g.w, g.W - (int)wc * g.w);
                 if (ST && (int)unit * p.tiles * kTileRows >= eh * strips_of(ew)) continue;            // a truncated window has fewer query tiles
                 // (not where a pair of tiles would be of either part: one after the other, 288 x 544 tokens, 8 x 128, side 16, took 341 us; as one window 300)
-                int t0 = (int)wr != p.part_row ? 0 : part_tiles(p.part_ha, eh, (ST ? strips_of(ew) : 1) * RW);
+                int t0 = !TWO || (int)wr != p.part_row ? 0 : part_tiles(p.part_ha, eh, (ST ? strips_of(ew) : 1) * RW);
                 if (t0 & (p.tiles - 1)) t0 = 0;
                 put(1 | ((int)head != last_head ? 2 : 0), head, b, wr, wc, eh, ew, unit * p.tiles, t0);
                 last_head = head;
@@ -880,10 +882,12 @@ cudaError_t launch_win(const Geo& g, const void* q, const void* k, const void* v
     count_launch(stream);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = prepare_kernel((const void*)swin_fwd_win_kernel<D, RW, KC, ST>, L::kSmemBytes);
+    const int part = p.part_row < 0 ? 0 : part_tiles(p.part_ha, g.H - p.part_row * g.w < g.w ? g.H - p.part_row * g.w : g.w, RW);
+    const auto kernel = ST || (part > 0 && part % p.tiles == 0) ? swin_fwd_win_kernel<D, RW, KC, ST, true> : swin_fwd_win_kernel<D, RW, KC, ST, ST>;
+    e = prepare_kernel((const void*)kernel, L::kSmemBytes);
     if (e != cudaSuccess) return e;
     prof_begin("swin_fwd_win_kernel", stream);
-    e = launch_dependent(swin_fwd_win_kernel<D, RW, KC, ST>, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
+    e = launch_dependent(kernel, (unsigned)(p.units < ctas ? p.units : ctas), kThreads, L::kSmemBytes, stream, p, (__nv_bfloat16*)o, lse, mq, mk, mv);
     count_launch(stream);
     return e;
 }

@@ -16,6 +16,8 @@ CASES = [
     (2, 27, 30, 2, 64, 9, 4, 3, 0, 1), (1, 41, 50, 2, 128, 13, 6, 5, 0, 0), (1, 48, 80, 3, 128, 16, 0, 0, 0, 1), (2, 80, 70, 5, 64, 17, 8, 9, 1, 0),
     (2, 45, 50, 2, 64, 20, 10, 10, 0, 1), (1, 70, 45, 2, 64, 31, 20, 30, 0, 0), (1, 60, 73, 3, 32, 24, 12, 12, 0, 1), (1, 40, 55, 2, 32, 17, 8, 21, 1, 0),
     (2, 96, 128, 6, 128, 32, 16, 16, 0, 1), (1, 160, 176, 12, 64, 16, 8, 8, 0, 1), (1, 3, 40, 1, 64, 32, 1, 7, 0, 1), (1, 33, 40, 150, 32, 32, 1, 7, 0, 1),
+    # a label that changes between two tiles: windows of two parts, a tile a unit (16 slots to a row), and pairs of tiles of one part and of both (32)
+    (1, 16, 64, 3, 64, 16, 8, 8, 0, 1), (2, 30, 50, 2, 128, 15, 7, 3, 0, 0), (1, 48, 50, 2, 32, 24, 12, 5, 0, 1), (1, 64, 96, 30, 64, 32, 16, 16, 0, 1), (1, 64, 96, 30, 128, 24, 4, 0, 0, 0),
 ]
 
 
