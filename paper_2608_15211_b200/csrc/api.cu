@@ -156,8 +156,11 @@ static bool use_fwd_tc(const Geo& g) { return fwd_tc_supported(g) && g.nmax > 64
 
 static bool use_fwd_win(const Geo& g) { return fwd_win_supported(g) && !force_register_path() && g.nmax > 64; }
 
+static bool use_fwd_tc64(const Geo& g) { return fwd_tc64_pays(g) && !force_register_path(); }
+
 static size_t fwd_bytes(const Geo& g) {
     if (force_register_path()) return 0;
+    if (use_fwd_tc64(g)) return align_up(fwd_tc64_workspace_bytes(g), 256);
     if (use_fwd_win(g)) return align_up(fwd_win_workspace_bytes(g), 256);
     if (use_fwd_tc(g)) return align_up(fwd_tc_workspace_bytes(g), 256);
     return 0;
@@ -239,7 +242,10 @@ static int fwd_call(const Geo& g, const void* q, const void* k, const void* v,
     if (rc) return rc;
     cudaError_t e;
     cudaStream_t st = (cudaStream_t)stream;
-    if (use_fwd_win(g))
+    if (use_fwd_tc64(g))
+        e = g.f16 ? launch_fwd_tc64_f16(g, q, k, v, bias_table, o, lse, workspace, sms, st)
+                  : launch_fwd_tc64(g, q, k, v, bias_table, o, lse, workspace, sms, st);
+    else if (use_fwd_win(g))
         e = g.f16 ? launch_fwd_win_f16(g, q, k, v, bias_table, o, lse, workspace, sms, st) : launch_fwd_win(g, q, k, v, bias_table, o, lse, workspace, sms, st);
     else if (need > 0)
         e = g.f16 ? launch_fwd_tc_f16(g, q, k, v, bias_table, o, lse, workspace, sms, st)
@@ -353,15 +359,18 @@ int terra_swin_check(void* stream) {
     e = read_bwd_tc_status(&timed_out_bwd);
     if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
     // the fp16 builds of the same kernels keep status words of their own
-    int t16[6] = {0, 0, 0, 0, 0, 0};
+    int t16[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     e = read_tc_status_f16(&t16[0], (cudaStream_t)stream);
     if (e == cudaSuccess) e = read_bwd_tc_status_f16(&t16[1]);
     if (e == cudaSuccess) e = read_bwd_onepass_status_f16(&t16[2]);
     if (e == cudaSuccess) e = read_bwd_onepass_status(&t16[3]);
     if (e == cudaSuccess) e = read_fwd_win_status_f16(&t16[4]);
     if (e == cudaSuccess) e = read_fwd_win_status(&t16[5]);
+    if (e == cudaSuccess) e = read_fwd_tc64_status_f16(&t16[6]);
+    if (e == cudaSuccess) e = read_fwd_tc64_status(&t16[7]);
     if (e != cudaSuccess) return cuda_fail(e, "terra_swin_check");
-    const bool any16 = t16[0] || t16[1] || t16[2] || t16[3] || t16[4] || t16[5];
+    bool any16 = false;
+    for (int t : t16) any16 = any16 || t;
     return (timed_out || timed_out_bwd || any16) ? TERRA_ERR_DEVICE_TIMEOUT : TERRA_OK;
 }
 

@@ -26,6 +26,7 @@
 #include "swin_common.cuh"
 #include "swin_kernels.h"
 #include "tc_common.cuh"
+#include "tma_rows.cuh"
 #include "win_tiles.cuh"
 
 // fp16 build of this file (through attn_fwd_tc_f16.cu): the kernel, its launcher and its status word get names of
@@ -932,6 +933,17 @@ bool encode_win_map(CUtensorMap* map, const Geo& g, const void* base, int token_
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                box_ch == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool make_row_maps3(RowMaps3* maps, const Geo& g, const void* base, int token_stride, int part_cols) {
+    for (int i = 0; i < 3; ++i)
+        if (!make_row_map(&maps->m[i], g, base, token_stride, 32 >> i, part_cols)) return false;
+    // boxes of 64 and 128 tokens (a box may not be longer than the token axis)
+    for (int i = 3; i < 5; ++i) {
+        const int box = (long long)g.B * g.H * g.W >= (8 << i) ? (8 << i) : 32;
+        if (!make_row_map(&maps->m[i], g, base, token_stride, box, part_cols)) return false;
+    }
+    return true;
 }
 
 size_t fwd_tc_workspace_bytes(const Geo& g) { return (size_t)g.heads * kFwdBiasFloats * sizeof(float); }

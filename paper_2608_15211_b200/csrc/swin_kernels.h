@@ -101,6 +101,15 @@ cudaError_t launch_fwd_win_f16(const Geo& g, const void* q, const void* k, const
                                int sm_count, cudaStream_t stream);
 cudaError_t read_fwd_win_status(int* timed_out);
 cudaError_t read_fwd_win_status_f16(int* timed_out);
+// tcgen05 forward path for head dims 64 and 128 and many complete windows of side 64 and 128 without mask labels (attn_fwd_tc64.cu)
+bool fwd_tc64_pays(const Geo& g);
+size_t fwd_tc64_workspace_bytes(const Geo& g);
+cudaError_t launch_fwd_tc64(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
+                            int sm_count, cudaStream_t stream);
+cudaError_t launch_fwd_tc64_f16(const Geo& g, const void* q, const void* k, const void* v, const float* bias, void* o, float* lse, void* workspace,
+                                int sm_count, cudaStream_t stream);
+cudaError_t read_fwd_tc64_status(int* timed_out);     // after the stream has been synchronised
+cudaError_t read_fwd_tc64_status_f16(int* timed_out);
 // One-pass tcgen05 backward for window sides 9 .. 128 at head dim 128, 11 .. 128 at 64 and 17 .. 128 at 32, any grid.
 struct OnePassPlan {
     int rw;                  // slots per window row
