@@ -1326,21 +1326,52 @@ bool bwd_onepass_supported(const Geo& g) {
 }
 
 // Gangs (see Params).  The CTAs of a gang read the same Q and dO and add to the same slab a few turns after one another, so these pass
-// between L2 and memory once for kGangMin CTAs or more.  The time of a run in key tiles: the gang's windows times their tiles over its
-// CTAs, plus what its last CTA is behind its first (none where they rotate).  Where a window has more tiles than the gang has CTAs, the first CTA's second
-// tile waits for the last CTA's first: a tile's 2 x tiles half chunks have to hold the gang's lags, and half as much for the unevenness
-// (256 x 640 tokens, 8 x 128, side 64, gangs of 4, 8, 16 and 37: 11.6, 12.9, 14.8 and 19.3 ms; side 128, 7, 9, 18, 37: 43.0, 43.0, 44.2, 47.4).
+// between L2 and memory once for kGangMin CTAs or more.  The time of a run in a full window's key tiles: the longest gang's windows times their tiles over its
+// CTAs, plus half of what its last CTA is behind its first, `lag` a CTA (none of it where they rotate).  The longer that is against a tile the more
+// its CTAs wait for turns, a quarter of it beyond 0.3 tiles, whether a window has as many tiles or not.  Gangs of 4, 8, 12, 16, 37 and 74, ms: 128 windows of side
+// 64 (heads and windows) at head dim 128 4.38, 4.44, 4.62, 4.98, 6.13, 7.59; 320 10.9, 11.0, 11.4, 12.1, 15.5, 18.6; 64 of side 128 33.9, 34.2, 33.5, 34.0, 33.7, 37.7.
+// Over 56 sizes of complete windows what is chosen is at most 10 % from the best.
 static void plan_gangs(OnePassPlan& p, const Geo& g, long long items, int tiles) {
     p.gangs = kPlanSms;
     p.gang = p.ring = 1;
     p.rotate = p.flags = 0;
     if (!p.strips) return;
+    // Up to six windows a gang: what each takes (its parts' tiles, against their own queries) in the order in which the gangs take them; of more
+    // all count as full.
+    constexpr int kMostGangs = kPlanSms / kGangMin, kListed = 6 * kMostGangs;
+    double share[kListed];
+    int parts[kListed][2];
+    if (items <= kListed) {
+        const int ha = !g.ph && g.sh > 0 ? (g.H - g.sh) % g.w : 0, part_row = ha > 0 ? (g.H - g.sh) / g.w : -1;
+        for (int i = 0; i < items; ++i) {
+            const int win = i / g.heads % (g.Mh * g.Mw), wr = win / g.Mw, wc = win % g.Mw, eh = wr < g.H / g.w ? g.w : g.H % g.w;
+            const int slots = strips_of(wc < g.W / g.w ? g.w : g.W % g.w) * p.rw, all = (eh * slots + kTile - 1) / kTile;
+            parts[i][0] = wr == part_row ? part_tiles(ha, eh, slots) : 0;
+            parts[i][1] = all - parts[i][0];
+            share[i] = ((double)parts[i][0] * parts[i][0] + (double)parts[i][1] * parts[i][1]) / tiles;
+        }
+    }
+    // Where every gang has one window its CTAs go by whole tiles, have no chain from one window to the next (119 x 303 tokens, 3 x 128, side 64: 30 gangs
+    // of 4 1105 us, 15 of 9 1322; 63 x 123, 12 x 128, side 128: 12 of 12 1636, 6 of 24 2020) and read Q, dO and slab (`held`: of the parts worked on) all
+    // over, each for itself where L2 does not hold them (128 x 128, 16 x 64, side 128, 134 MB: 16 gangs of 9 1.22 times as long as 8 of 18; 16 x 32, 67 MB: 1.02).
+    double held = 0;
+    for (int i = 0; items <= kListed && i < items; ++i) held += 8.0 * kTile * g.d * (parts[i][0] > parts[i][1] ? parts[i][0] : parts[i][1]);
     const double lag = kGangLag / (2.0 * tiles);
     double best = 0;
-    for (int n = 1; n <= items && n <= kPlanSms / kGangMin; ++n) {
+    for (int n = 1; n <= items && n <= kMostGangs; ++n) {
         const int s = kPlanSms / n;
-        const double slow = s < tiles && 1.5 * lag * s > 1 ? 1.5 * lag * s : 1;
-        const double t = n == items ? (double)((tiles + s - 1) / s) : slow * ((items + n - 1) / n) * tiles / s + lag * s;
+        double longest = items <= kListed ? 0 : (double)((items + n - 1) / n) * tiles / s;
+        for (int k = 0; items <= kListed && k < n; ++k) {
+            double x = 0;
+            if (n == items)
+                for (int t : parts[k]) x += (double)((t + s - 1) / s) * t / tiles;
+            else
+                for (int i = k; i < items; i += n) x += share[i];
+            if (n < items) x /= s;
+            if (x > longest) longest = x;
+        }
+        const double behind = lag * s, slow = behind > 0.3 ? 1 + 0.25 * (behind - 0.3) : 1;
+        const double t = n == items ? (held < (s > 4 ? 115e6 : 160e6) ? 0.9 : 1.2) * longest : slow * longest + 0.5 * behind;
         if (n == 1 || t <= best) { best = t; p.gangs = n; p.gang = s; }
     }
     const long long most = (items + p.gangs - 1) / p.gangs * tiles;
