@@ -640,15 +640,7 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
         auto flag = [&](int i) { return p.flags + ((size_t)td.slab * (p.events + 1) + i) * 4 + wq; };
         unsigned* pending = nullptr;
         unsigned pending_value = 0;
-        // A tile's place in the order of those that add to chunk c: the tiles' own, or (rotate) from round to round of the gang's CTAs and in
-        // each from the one that starts at the chunk, or last in front of it, downwards.
-        auto place = [&](int c) {
-            const int kt = td.kt - td.q0;
-            if (!p.rotate) return kt;
-            const int n = min(p.gang, td.nch), j = kt % n, round = kt - j, in_round = min(n, td.nch - round);
-            const int r = min(in_round - 1, ((c + 1) * n - 1) / td.nch) - j;
-            return round + (r < 0 ? r + in_round : r);
-        };
+        auto place = [&](int c) { return gang_place(td.kt - td.q0, c, td.nch, p.gang, p.rotate); };
         auto signal = [&](unsigned* f, unsigned value) {
             __syncwarp();
             if (lane == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;\n" ::"l"(f), "r"(value) : "memory");
@@ -899,10 +891,10 @@ swin_bwd_onepass_kernel(const __grid_constant__ Params p, __nv_bfloat16* __restr
                 const int t0 = !L::kTwo || cur.wr != p.part_row ? 0 : ST ? part_tiles(p.part_ha, eh, strips_of(ew) * RW) : p.part_ha * RW / kTile;
                 if (L::kGang && p.gang > 1) {
                     for (int q0 = 0; q0 < nch;) {
-                        const int tn = q0 == 0 && t0 > 0 ? t0 : nch - q0, ranks = min(p.gang, tn);
-                        for (int kt = (member + p.gang - seq % p.gang) % p.gang; ok && kt < tn; kt += p.gang)
+                        const int tn = q0 == 0 && t0 > 0 ? t0 : nch - q0;
+                        for (int kt = gang_first_tile(member, seq, p.gang); ok && kt < tn; kt += p.gang)
                             put(1 | (kt == 0 ? 2 : 0) | (kt == tn - 1 ? 4 : 0), head, eh, ew, q0 + kt, tn, q0, (int)(blockIdx.x / p.gang) * p.ring + windows % p.ring, seq,
-                                windows / p.ring, p.rotate ? kt % ranks * tn / ranks : 0);
+                                windows / p.ring, gang_first_chunk(kt, tn, p.gang, p.rotate));
                         seq += tn;
                         windows += tn > 1;
                         q0 += tn;

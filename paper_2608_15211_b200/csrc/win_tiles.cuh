@@ -137,6 +137,23 @@ __device__ __forceinline__ void load_win_strip(const WinStripMaps& m, const WinC
 // tiles of one part see none of the other's.  The first part's tiles, 0 where the window is one.  `row_slots`: slots of a window row.
 __host__ __device__ __forceinline__ int part_tiles(int ha, int eh, int row_slots) { return ha > 0 && ha < eh && ha * row_slots % 128 == 0 ? ha * row_slots / 128 : 0; }
 
+// Gangs of the one-pass backward (attn_bwd_onepass.cu), whose CTAs share the key tiles of a window (or of a part of one), `tiles` of them.
+// The first tile that CTA `member` takes, where `seq` tiles were dealt before; then every gang-th.
+__host__ __device__ __forceinline__ int gang_first_tile(int member, int seq, int gang) { return (member + gang - seq % gang) % gang; }
+// The chunk of queries that tile `kt` starts at.
+__host__ __device__ __forceinline__ int gang_first_chunk(int kt, int tiles, int gang, bool rotate) {
+    const int ranks = gang < tiles ? gang : tiles;
+    return rotate ? kt % ranks * tiles / ranks : 0;
+}
+// A tile's place in the order of those that add to chunk c: the tiles' own, or (rotate) from round to round of the gang's CTAs and in
+// each from the one that starts at the chunk, or last in front of it, downwards.
+__host__ __device__ __forceinline__ int gang_place(int kt, int c, int tiles, int gang, bool rotate) {
+    if (!rotate) return kt;
+    const int n = gang < tiles ? gang : tiles, j = kt % n, round = kt - j, in_round = n < tiles - round ? n : tiles - round;
+    const int last = ((c + 1) * n - 1) / tiles, r = (last < in_round - 1 ? last : in_round - 1) - j;
+    return round + (r < 0 ? r + in_round : r);
+}
+
 // slot (a, b) of a window -> grid token
 __device__ __forceinline__ int win_token(const Geo& g, int wr, int wc, int a, int b) {
     int u = wr * g.w + a + g.sh;
