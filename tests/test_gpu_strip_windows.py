@@ -20,9 +20,12 @@ CASES = [
     (1, 68, 70, 2, 32, 34, 17, 9, 0, 1), (3, 64, 3, 2, 64, 64, 20, 1, 0, 1), (2, 8, 8, 1, 128, 40, 4, 0, 1, 0), (1, 5, 60, 2, 32, 64, 2, 7, 0, 0),
 ]
 
+# gangs that take one window after another, more than their ring has slabs (tests/test_onepass_plan.py), whole ones, ones of two parts and truncated ones
+GANGS = [(1, 12, 64, 200, 32, 64, 6, 32, 0, 1), (1, 12, 66, 150, 128, 64, 6, 32, 0, 1), (1, 24, 80, 100, 128, 40, 12, 20, 0, 1), (2, 20, 70, 75, 64, 64, 10, 20, 0, 0)]
+
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16], ids=["bf16", "fp16"])
-@pytest.mark.parametrize("case", CASES, ids=["_".join(map(str, c)) for c in CASES])
+@pytest.mark.parametrize("case", CASES + GANGS, ids=["_".join(map(str, c)) for c in CASES + GANGS])
 def test_strip_windows(case, dtype):
     cfg = small_config("strips", *case)
     x = {k: v.to(dtype) if v.dtype == torch.bfloat16 else v * 25.0 for k, v in make_inputs(cfg).items()}

@@ -2,6 +2,7 @@
 import paper_2608_15211_b200 as terra
 from paper_2608_15211_b200.workloads import small_config
 from tests._host_program import run_host_program
+from tests.test_gpu_strip_windows import GANGS
 
 SWEEP = """
 int main() {
@@ -40,6 +41,28 @@ int main() {
 
 def test_slabs_and_flags_lie_in_the_workspace(tmp_path):
     run_host_program(tmp_path, SWEEP)
+
+
+RING = """
+int main(int argc, char** argv) {
+    for (int i = 1; i + 9 < argc; i += 10) {
+        int x[10];
+        for (int j = 0; j < 10; ++j) x[j] = std::atoi(argv[i + j]);
+        terra_swin_desc desc = {x[0], x[1], x[2], x[3], x[4], x[5], x[6], x[7], x[8], x[9], 0.f, TERRA_DTYPE_BF16};
+        Geo g;
+        if (resolve_attention_geo(&desc, &g) != TERRA_OK || !bwd_onepass_supported(g)) return 1;
+        const OnePassPlan p = bwd_onepass_plan(g);
+        if (p.gang < 2 || p.rotate || p.units <= (long long)p.gangs * p.ring)
+            return std::printf("%lld windows, gangs %d of %d, ring %d, rotate %d\\n", p.units, p.gangs, p.gang, p.ring, p.rotate), 1;
+    }
+    return 0;
+}
+"""
+
+
+def test_gang_cases_go_round_their_rings(tmp_path):
+    """The GPU cases of that name have more windows for every gang than it has slabs."""
+    run_host_program(tmp_path, RING, *(v for case in GANGS for v in case))
 
 
 def test_more_heads_than_the_tables_entries_can_be_numbered_for():

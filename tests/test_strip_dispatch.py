@@ -23,3 +23,20 @@ def test_route(case, forward, backward):
         delta = -(-4 * B * H * W * heads // 256) * 256
         assert (terra.terra_swin_workspace_bytes(desc, False) > 0) == forward
         assert (terra.terra_swin_workspace_bytes(desc, True) > delta) == backward
+
+
+OWN = [
+    # B, H, W, heads, head_dim, window, shift_h, shift_w, periodic_h, periodic_w: complete windows of side 64 and 128 on their own forward kernel or not
+    ((1, 64, 640, 1, 64, 64, 0, 8, 0, 1), True), ((1, 64, 576, 1, 64, 64, 0, 8, 0, 1), False), ((1, 128, 256, 16, 128, 128, 64, 64, 1, 1), True),
+    ((1, 128, 256, 16, 128, 128, 64, 64, 0, 1), False), ((1, 128, 256, 16, 128, 128, 0, 64, 0, 0), False), ((1, 128, 256, 16, 128, 128, 0, 60, 0, 1), False),
+    ((1, 64, 64, 40, 64, 64, 0, 0, 0, 1), False), ((1, 64, 64, 37, 64, 64, 0, 0, 0, 1), True), ((1, 64, 64, 149, 64, 64, 0, 0, 0, 1), False),
+    ((1, 128, 256, 16, 32, 128, 0, 64, 0, 1), False), ((1, 128, 320, 16, 128, 96, 0, 64, 0, 1), False),
+]
+
+
+@pytest.mark.parametrize("case, own", OWN, ids=["_".join(map(str, c[0])) for c in OWN])
+def test_complete_windows_route(case, own):
+    desc = terra.make_desc(small_config("route", *case))
+    heads, window = case[3], case[5]
+    prepared = -(-4 * heads * ((2 * window - 1) * 2 * window + 4) // 256) * 256          # that kernel's tables; strips' are larger
+    assert (terra.terra_swin_workspace_bytes(desc, False) == prepared) == own
