@@ -15,7 +15,7 @@
 // Row maximum: windows without mask labels use the upper bound max_j(raw score) * scale + max(bias) over the key
 // slots that hold a token (softmax is shift invariant, so the result is the same; only the exponent range
 // matters: the bound exceeds the true maximum by at most the spread of the head's bias table, and a head whose
-// table spreads over more than 64 octaves takes the exact path); windows that mix shift-mask labels take the
+// table spreads over more than kBoundSpread octaves takes the exact path); windows that mix shift-mask labels take the
 // exact maximum over the keys the row may see.
 // Every mbarrier wait is bounded; on expiry the CTA raises an abort flag, all roles leave their loops,
 // TMEM is released and the host reads the device status word.
@@ -824,7 +824,7 @@ swin_fwd_tc_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __nv_
 //   table[(da + w - 1) * cs + (db + w - 1)] = T[(da + w - 1) * (2w - 1) + (db + w - 1), head] * log2(e)
 //   for |da|, |db| < w (unused gaps 0), table[2 c0 + 1 .. 3 c0 + 1] = -inf (where key slots without a
 //   token point), and the head's largest entry in the last float (+inf instead if the head's entries spread over
-//   more than 64 octaves: the forward kernel then takes exact row maxima).
+//   more than kBoundSpread octaves: the forward kernel then takes exact row maxima).
 __global__ void __launch_bounds__(256)
 swin_fwd_bias_prep_kernel(const float* __restrict__ bias, float* __restrict__ prep, int w, int heads, int cs) {
     let_dependents_start();
@@ -857,7 +857,7 @@ swin_fwd_bias_prep_kernel(const float* __restrict__ bias, float* __restrict__ pr
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int i = 1; i < 8; ++i) { mx = fmaxf(mx, red[i]); mn = fminf(mn, red_mn[i]); }
-        dst[kFwdBiasFloats - 1] = (mx - mn <= 64.f) ? mx : INFINITY;
+        dst[kFwdBiasFloats - 1] = (mx - mn <= kBoundSpread) ? mx : INFINITY;
     }
     wait_for_prerequisites();      // what depends on this launch also depends on the one before it
 }

@@ -165,6 +165,14 @@ __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
     __half2 v = __floats2half2_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
 }
+// Forward kernels that bound a row's maximum by max(raw score) scale + max(bias): how far, in octaves, a head's bias entries may spread for it.  A row's own
+// maximum lies up to that far below the bound, and so do its P, which have to stay numbers of the elements' type (fp16: 2^-14 at least without loss).
+#ifdef TERRA_ELEM_F16
+constexpr float kBoundSpread = 8.f;
+#else
+constexpr float kBoundSpread = 64.f;
+#endif
+
 // The kernel files are compiled twice, for bf16 and (with TERRA_ELEM_F16 defined by a one-line wrapper file) for fp16
 // activations: same code, the element type enters through these operations, the tcgen05 instruction descriptor's
 // operand formats (make_idesc_elem) and the name suffix.

@@ -58,3 +58,23 @@ def test_fp16_descriptor_refuses_bf16_tensors_and_the_other_way_round():
     h = {k: (v.to(torch.float16) if v.dtype == torch.bfloat16 else v) for k, v in x.items()}
     with pytest.raises(ValueError):
         terra.terra_swin_attn_fwd(terra.make_desc(cfg), h["q"], h["k"], h["v"], h["bias"])
+
+
+# one entry of the bias table far above the others: the one row of a window that meets it has a much larger maximum than the rest
+LONE = [(1, 32, 48, 2, 32, 16, 0, 8, 0, 1), (1, 45, 70, 2, 32, 14, 7, 0, 0, 1), (1, 30, 40, 2, 32, 9, 0, 0, 0, 1)]
+
+
+@pytest.mark.parametrize("case", LONE, ids=["_".join(map(str, c)) for c in LONE])
+@pytest.mark.parametrize("entry", [4.0, 7.0, 20.0, 40.0])
+def test_a_lone_large_bias_entry(case, entry):
+    cfg = small_config("lone", *case)
+    x = {k: v.half() if v.dtype == torch.bfloat16 else v.clone() for k, v in make_inputs(cfg).items()}
+    x["bias"][0, :] = entry
+    xg = {k: v.cuda() for k, v in x.items()}
+    o, lse = terra.terra_swin_attn_fwd(terra.make_desc(cfg, dtype=torch.float16), xg["q"], xg["k"], xg["v"], xg["bias"])
+    terra.terra_swin_check()
+    sel = [0] if cfg.window > 32 else None
+    ref_o, ref_lse = oracle.attn_fwd(cfg, x["q"], x["k"], x["v"], x["bias"].double().numpy(), sel=sel)
+    tok = oracle.selection_tokens(cfg, sel)
+    gate("o", gpu_rows(o, cfg, tok), ref_o)
+    gate("lse", gpu_rows(lse, cfg, tok), ref_lse)
