@@ -5,12 +5,11 @@
 // The window's keys are streamed once, in chunks of 128, through a ring of shared-memory slots.  Per chunk:
 //   S = Q K_c^T                                                        (SS MMAs into the tile's columns)
 //   online softmax: the softmax threads take the chunk's maximum (the bound max_j(raw) * scale + max(bias); for heads
-//   whose bias table spreads over more than 64 octaves the exact one), raise the
+//   whose bias table spreads over more than kBoundSpread octaves the exact one), raise the
 //   row's reference m when the chunk exceeds it by more than 8 octaves (then O and the row sum are scaled down in
 //   tensor memory), and write P = exp2(S * scale + bias - m) back over S in the elements' 16 bits;
-//   O += P [V_c | 1]                                                   (A from TMEM; at head dim 64, 16 columns of
-//   ones behind V make the accumulator's columns 64..79 carry the row sums; at head dim 128 tensor memory has no
-//   columns left for them and the softmax threads add the row sums themselves).
+//   O += P V_c                                                         (A from TMEM; the softmax threads add up the row
+//   sums, in fp32 before P is rounded).
 // Roles: warps 0-3 / 4-7 softmax warpgroups (one thread per query row of the pair's first / second tile),
 // warp 8 issues every tcgen05.mma (whole warp runs the loop, one elected lane issues), warp 9 fetches Q and K rows, warp 10
 // the V rows, with tiled bulk copies, undoing the roll; warp 11 has no work.  A row is kept as head dim / 32 parts of 32
@@ -57,25 +56,22 @@ constexpr int kBiasFloats = 6048;                     // place of the staged tab
 constexpr int kColO = 128;
 
 // Shared-memory plan per head dim D (64 or 128): a row is kept as D / 32 parts of 32 columns, each part a region in the
-// 64-byte-swizzled operand layout.  Head dim 64: two Q stages, three ring slots of K | V | ones.  Head dim 128: rows
-// are twice as long, so one Q stage and two ring slots of K | V, and no ones block: tensor memory has no columns
-// left for the row sums next to a 128-column accumulator, the softmax threads add them up themselves.
+// 64-byte-swizzled operand layout.  Head dim 64: two Q stages, three ring slots of K | V.  Head dim 128: rows
+// are twice as long, so one Q stage and two ring slots.
 template <int D>
 struct Lay {
     static constexpr int kParts = D / 32;
-    static constexpr bool kOnes = D == 64;
     static constexpr int kQStages = D == 64 ? 2 : 1, kSlots = D == 64 ? 3 : 2;
     static constexpr int kQStageBytes = kParts * kQPart;
-    static constexpr int kOffK = 0, kOffV = kParts * kKPart, kOffOnes = 2 * kParts * kKPart;
-    static constexpr int kSlotBytes = (2 * kParts + (kOnes ? 1 : 0)) * kKPart;
+    static constexpr int kOffK = 0, kOffV = kParts * kKPart;
+    static constexpr int kSlotBytes = 2 * kParts * kKPart;
     static constexpr int kOffSlots = kQStages * kQStageBytes;
     static constexpr int kOffRowTok = kOffSlots + kSlots * kSlotBytes;             // per Q stage: the 256 rows' tokens
     static constexpr int kOffBias = kOffRowTok + kQStages * 1024;
     static constexpr int kOffBars = ((kOffBias + kBiasFloats * 4 + 1023) / 1024) * 1024;
     static constexpr int kSmemBytes = kOffBars + 1024;
-    static constexpr int kNO = kOnes ? D + 16 : D;    // columns of the PV product
     static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
-    static_assert(kColO + kNO <= 256, "tensor memory columns of one query tile");
+    static_assert(kColO + D <= 256, "tensor memory columns of one query tile");
 };
 
 struct Item {
@@ -148,7 +144,6 @@ __device__ __forceinline__ void load_bias_row32(float (&bv)[32], uint32_t top) {
     bv[30] = lds_f32_at<4>(bb);
     bv[31] = lds_f32_at<0>(bb);
 }
-template <bool SUM>
 __device__ __forceinline__ void softmax_cols32_row(const uint32_t (&r)[32], uint32_t (&pk)[16], uint32_t top, float scale, float neg_m, float (&sum)[2]) {
     float bv[32];
     load_bias_row32(bv, top);
@@ -160,7 +155,7 @@ __device__ __forceinline__ void softmax_cols32_row(const uint32_t (&r)[32], uint
         add2(x0, x1, x0, x1, neg_m);
         const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
         pk[e2] = pack_elem(p0, p1);
-        if (SUM) add2vv(sum[0], sum[1], sum[0], sum[1], p0, p1);
+        add2vv(sum[0], sum[1], sum[0], sum[1], p0, p1);
     }
 }
 
@@ -218,8 +213,6 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
     constexpr int kParts = L::kParts, kQStages = L::kQStages, kSlots = L::kSlots, kQStageBytes = L::kQStageBytes;
     constexpr int kOffK = L::kOffK, kOffV = L::kOffV, kSlotBytes = L::kSlotBytes, kOffSlots = L::kOffSlots;
     constexpr int kOffRowTok = L::kOffRowTok, kOffBias = L::kOffBias, kOffBars = L::kOffBars;
-    constexpr int kNO = L::kNO;
-    constexpr bool kSum = !L::kOnes;                    // row sums of P are added up by the softmax threads
     extern __shared__ __align__(1024) unsigned char smem[];
     const uint32_t smem0 = smem_u32(smem);
     const uint32_t bar0 = smem0 + kOffBars;
@@ -264,17 +257,10 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
         *cta_abort = 0;
         fence_barrier_init();
     }
-    // the head's prepared bias table; the ones block of every ring slot (first 16 bf16 of a row = 1)
+    // the head's prepared bias table
     const int lw = 31 - __clz(g.w);                         // w = 1 << lw
     const int rows_floats = (2 * g.w - 1) * 2 * g.w + 4;    // floats of one head's prepared table
     if (tid == 0) reinterpret_cast<float*>(smem + kOffBias)[kBiasFloats - 1] = bias_prep[(size_t)(head + 1) * rows_floats - 1];
-    if (L::kOnes) {
-        for (int i = tid; i < kSlots * kChunk * 4; i += kThreads) {
-            const int s = i / (kChunk * 4), rem = i - s * (kChunk * 4), row = rem >> 2, chunk = rem & 3;
-            const uint32_t val = chunk < 2 ? kElemOnesPair : 0u;
-            *reinterpret_cast<uint4*>(smem + kOffSlots + s * kSlotBytes + L::kOffOnes + tile_off<32>(row, chunk)) = make_uint4(val, val, val, val);
-        }
-    }
     fence_proxy_async();
     if (warp == kMmaWarp) {
         tmem_alloc(smem_u32(tmem_slot), 512);
@@ -390,7 +376,7 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
         }
     } else {
         // ------------------------------------------------------------------ MMA issuer
-        const uint32_t idesc_pv = make_idesc_elem(128, kNO, 0, 1);
+        const uint32_t idesc_pv = make_idesc_elem(128, D, 0, 1);
         int kuse = 0;
         long long ru = 0;
         int n_p[2] = {0, 0}, n_items_t[2] = {0, 0};
@@ -532,8 +518,8 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
             // Online softmax, chunk by chunk: P is formed against a reference m that is at least the row's maximum so
             // far minus 8 octaves; only when a chunk's maximum exceeds the reference by more than that is the reference
             // raised and the accumulated O (with the row sum) scaled down by 2^(old - new).  The
-            // chunk maximum is the bound max_j(raw) * scale + max(bias); for heads whose bias table spreads over more than 64
-            // octaves it is the exact maximum.
+            // chunk maximum is the bound max_j(raw) * scale + max(bias); for heads whose bias table spreads over more than
+            // kBoundSpread octaves it is the exact maximum.
             float m = -INFINITY;
             float psum[2] = {0.f, 0.f};
             for (int c = 0; c < x.nch; ++c) {
@@ -575,7 +561,7 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                     // one waits for this thread's arrival below: O is this thread's to modify
                     const float f = rescale ? fast_exp2(m - mc) : 1.f;
 #pragma unroll 1
-                    for (int oc = 0; oc < kNO; oc += 16) {
+                    for (int oc = 0; oc < D; oc += 16) {
                         uint32_t ro[16];
                         tmem_ld16(t_s + kColO + oc, ro);
                         tmem_ld_wait();
@@ -595,12 +581,12 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
                     uint32_t pk[16];
                     tmem_ld_wait();
                     if (i + 1 < nfull) tmem_ld32(t_s + 32 * (i + 1), rb);
-                    softmax_cols32_row<kSum>(ra, pk, row_top(stage, i), scale, neg_m, psum);
+                    softmax_cols32_row(ra, pk, row_top(stage, i), scale, neg_m, psum);
                     tmem_st16(t_s + 16 * i, pk);
                     if (i + 1 < nfull) {
                         tmem_ld_wait();
                         if (i + 2 < nfull) tmem_ld32(t_s + 32 * (i + 2), ra);
-                        softmax_cols32_row<kSum>(rb, pk, row_top(stage, i + 1), scale, neg_m, psum);
+                        softmax_cols32_row(rb, pk, row_top(stage, i + 1), scale, neg_m, psum);
                         tmem_st16(t_s + 16 * (i + 1), pk);
                     }
                 }
@@ -613,44 +599,25 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
             if (!mbar_wait_all(bar_oready(wg), n_o & 1, cta_abort)) break;
             ++n_o;
             tc_fence_after();
-            if (!kSum) {
-                uint32_t ro[32], ro2[32], rsum;
-                tmem_ld32(t_s + kColO, ro);
-                tmem_ld32(t_s + kColO + 32, ro2);
-                tmem_ld1(t_s + kColO + D, rsum);
-                tmem_ld_wait();
-                tc_fence_before();
-                mbar_arrive(bar_ofree(wg));
-                if (tok >= 0) {
-                    const float sum = __uint_as_float(rsum);
-                    const size_t row_off = ((size_t)x.b * HW + (size_t)tok) * g.heads + head;
-                    lse[row_off] = (m + log2f(sum)) * kLn2;
-                    const float inv = 1.f / sum;
-                    uint4* dst = reinterpret_cast<uint4*>(o + row_off * D);
-                    store_o32(dst, ro, inv);
-                    store_o32(dst + 4, ro2, inv);
-                }
-            } else {
-                // the accumulator's 128 columns in two rounds of 64, to keep the registers in hand
-                const float sum = psum[0] + psum[1];
-                const float inv = 1.f / sum;
-                const size_t row_off = ((size_t)x.b * HW + (size_t)(tok >= 0 ? tok : 0)) * g.heads + head;
-                uint4* dst = reinterpret_cast<uint4*>(o + row_off * D);
-                if (tok >= 0) lse[row_off] = (m + log2f(sum)) * kLn2;
+            // the accumulator's columns in rounds of 64, to keep the registers in hand
+            const float sum = psum[0] + psum[1];
+            const float inv = 1.f / sum;
+            const size_t row_off = ((size_t)x.b * HW + (size_t)(tok >= 0 ? tok : 0)) * g.heads + head;
+            uint4* dst = reinterpret_cast<uint4*>(o + row_off * D);
+            if (tok >= 0) lse[row_off] = (m + log2f(sum)) * kLn2;
 #pragma unroll
-                for (int hq = 0; hq < D / 64; ++hq) {
-                    uint32_t ro[32], ro2[32];
-                    tmem_ld32(t_s + kColO + 64 * hq, ro);
-                    tmem_ld32(t_s + kColO + 64 * hq + 32, ro2);
-                    tmem_ld_wait();
-                    if (hq == D / 64 - 1) {
-                        tc_fence_before();
-                        mbar_arrive(bar_ofree(wg));
-                    }
-                    if (tok >= 0) {
-                        store_o32(dst + 8 * hq, ro, inv);
-                        store_o32(dst + 8 * hq + 4, ro2, inv);
-                    }
+            for (int hq = 0; hq < D / 64; ++hq) {
+                uint32_t ro[32], ro2[32];
+                tmem_ld32(t_s + kColO + 64 * hq, ro);
+                tmem_ld32(t_s + kColO + 64 * hq + 32, ro2);
+                tmem_ld_wait();
+                if (hq == D / 64 - 1) {
+                    tc_fence_before();
+                    mbar_arrive(bar_ofree(wg));
+                }
+                if (tok >= 0) {
+                    store_o32(dst + 8 * hq, ro, inv);
+                    store_o32(dst + 8 * hq + 4, ro2, inv);
                 }
             }
         }
@@ -666,7 +633,7 @@ swin_fwd_tc64_kernel(const Geo g, const __nv_bfloat16* __restrict__ q, const __n
 }
 
 // The prepared bias table, per head: (2w - 1) table rows of 2w floats (the last one padding), log2 e times the caller's entries, and four more
-// floats, the last of which is the head's largest entry (+inf instead if the head's entries spread over more than 64 octaves).
+// floats, the last of which is the head's largest entry (+inf instead if the head's entries spread over more than kBoundSpread octaves).
 __global__ void __launch_bounds__(256)
 swin_fwd_bias_prep64_kernel(const float* __restrict__ bias, float* __restrict__ prep, int w, int heads) {
     const int head = blockIdx.x;
@@ -694,9 +661,9 @@ swin_fwd_bias_prep64_kernel(const float* __restrict__ bias, float* __restrict__ 
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int i = 1; i < 8; ++i) { mx = fmaxf(mx, red[i]); mn = fminf(mn, red_mn[i]); }
-        // a table that spreads over more than 64 octaves makes the bound max(raw) * scale + max(bias) on the row
+        // a table that spreads over more makes the bound max(raw) * scale + max(bias) on the row
         // maximum too loose for the exponent range: +inf here tells the forward kernel to take exact row maxima
-        dst[total - 1] = (mx - mn <= 64.f) ? mx : INFINITY;
+        dst[total - 1] = (mx - mn <= kBoundSpread) ? mx : INFINITY;
     }
 }
 

@@ -61,7 +61,7 @@ def test_fp16_descriptor_refuses_bf16_tensors_and_the_other_way_round():
 
 
 # one entry of the bias table far above the others: the one row of a window that meets it has a much larger maximum than the rest
-LONE = [(1, 32, 48, 2, 32, 16, 0, 8, 0, 1), (1, 45, 70, 2, 32, 14, 7, 0, 0, 1), (1, 30, 40, 2, 32, 9, 0, 0, 0, 1)]
+LONE = [(1, 32, 48, 2, 32, 16, 0, 8, 0, 1), (1, 45, 70, 2, 32, 14, 7, 0, 0, 1), (1, 30, 40, 2, 32, 9, 0, 0, 0, 1), (1, 64, 640, 1, 64, 64, 0, 8, 0, 1), (1, 64, 448, 2, 128, 64, 0, 40, 0, 1)]
 
 
 @pytest.mark.parametrize("case", LONE, ids=["_".join(map(str, c)) for c in LONE])
