@@ -456,7 +456,7 @@ def main():
         # two-kernel backward paths 4d each (key side: dV, dK; query side: dP, dQ).
         pairs = wk["score_elements"]
         d = cfg.head_dim
-        kernel_flop = {"swin_fwd_tc_kernel": 4 * d * pairs, "swin_fwd_mma_kernel": 4 * d * pairs,
+        kernel_flop = {"swin_fwd_tc_kernel": 4 * d * pairs, "swin_fwd_tc64_kernel": 4 * d * pairs, "swin_fwd_mma_kernel": 4 * d * pairs,
                        "swin_fwd_small_kernel": 4 * d * pairs, "swin_fwd_win_kernel": 4 * d * pairs, "swin_bwd_onepass_kernel": 8 * d * pairs,
                        "swin_bwd_fused_kernel": 8 * d * pairs, "swin_bwd_small_kernel": 8 * d * pairs,
                        "swin_bwd_mma_kernel<key tiles>": 4 * d * pairs, "swin_bwd_mma_kernel<query tiles>": 4 * d * pairs,

@@ -6,7 +6,7 @@
 // contiguous grid all happen here; nothing window-major is ever written to global memory.
 // The file is compiled for bf16 and, through attn_fwd_mma_f16.cu, for fp16 activations.
 // The first kernel covers every window class (truncated edges, the split latitude-wrap row, every side and head dim); what runs
-// there is the sides that fill little of the tcgen05 kernels' slots, the forward without a workspace and TERRA_REGISTER_PATH=1.
+// there is the sides and grids that fill little of the tcgen05 kernels' slots, windows of at most 64 tokens, the forward without a workspace and TERRA_REGISTER_PATH=1.
 #include "swin_common.cuh"
 #include "swin_kernels.h"
 
@@ -35,7 +35,7 @@ __device__ __forceinline__ void load_rows(unsigned char* s_tile, const __nv_bflo
     }
 }
 
-// BIG = windows of more than 1024 tokens (window sides 33 .. 128): the slot tables of a whole window and the head's
+// BIG = window sides 33 .. 128 (up to 16 384 tokens a window): the slot tables of a whole window and the head's
 // bias table no longer fit shared memory, so the tables cover the CTA's 64 query rows plus the key block in flight
 // (two stages) and the bias is read from the caller's table in global memory.
 template <int D, bool BIG>

@@ -1,5 +1,5 @@
 // Forward shifted-window attention on the tcgen05 tensor cores: window sides 9 .. 128 at head dims 64 and 128, 17 .. 128 at head dim 32 (less the
-// sides that fwd_win_supported leaves to the register tiles), any grid.
+// sides and, above 32, the grids that fwd_win_supported leaves to the register tiles, and the complete windows of attn_fwd_tc64.cu), any grid.
 //
 // A unit is a pair of 128-row query tiles of one (sample, window, head), on small grids one tile; a persistent CTA per SM walks over units and streams
 // the window's keys through shared memory in chunks of 128 slots (see win_tiles.cuh: 16 or 32 slots to a window row).  Per
