@@ -1352,8 +1352,9 @@ static void plan_gangs(OnePassPlan& p, const Geo& g, long long items, int tiles)
     double best = 0;
     for (int n = 1; n <= items && n <= kMostGangs; ++n) {
         const int s = kPlanSms / n;
+        const double behind = lag * s, slow = behind > 0.3 ? 1 + 0.25 * (behind - 0.3) : 1;
         double longest = items <= kListed ? 0 : (double)((items + n - 1) / n) * tiles / s;
-        for (int k = 0; items <= kListed && k < n; ++k) {
+        for (int k = 0; items <= kListed && k < n && (n == 1 || n == items || slow * longest <= best); ++k) {      // (no further than until it is longer)
             double x = 0;
             if (n == items)
                 for (int t : parts[k]) x += (double)((t + s - 1) / s) * t / tiles;
@@ -1362,7 +1363,6 @@ static void plan_gangs(OnePassPlan& p, const Geo& g, long long items, int tiles)
             if (n < items) x /= s;
             if (x > longest) longest = x;
         }
-        const double behind = lag * s, slow = behind > 0.3 ? 1 + 0.25 * (behind - 0.3) : 1;
         const double t = n == items ? (held < (s > 4 ? 115e6 : 160e6) ? 0.9 : 1.2) * longest : slow * longest + 0.5 * behind;
         if (n == 1 || t <= best) { best = t; p.gangs = n; p.gang = s; }
     }
